@@ -73,8 +73,8 @@ typedef enum {
                                         of the proposal MLP (set with turboreg_set_proposal_model) */
 /* flags */
 #define TURBOREG_FLAG_SC2_BITSET 0x1u  /* SC^2 by bitset AND+popcount on CUDA cores
-                                          instead of the tcgen05 FP8 GEMM (same integers) */
-#define TURBOREG_FLAG_SC2_GEMM 0x40u   /* SC^2 by the tcgen05 FP8 GEMM.  Without either flag a single
+                                          instead of the tcgen05 FP4 GEMM (same integers) */
+#define TURBOREG_FLAG_SC2_GEMM 0x40u   /* SC^2 by the tcgen05 FP4 GEMM.  Without either flag a single
                                           problem with N <= 5120 (and pair MMAs available) gets the
                                           path chosen on the device after the compatibility graph,
                                           from N and the edge count (the CUDA-core path up to about
@@ -135,8 +135,7 @@ void turboreg_default_params(turboreg_params* p, float tau, int32_t k1, float in
  * max_n correspondences and batches of up to max_batch problems whose total
  * correspondence count is at most max_n * max_batch.  `cuda_stream` is a
  * cudaStream_t to run on, or NULL to let the context create its own.  The
- * device workspace (about 3.1 * max_n^2 bytes plus 2.3 * max_n^2 bytes per
- * batched problem slot) is allocated here, never inside register calls.
+ * device workspace (about 2.6 * max_n^2 bytes per batched problem slot) is allocated here, never inside register calls.
  * On success *out receives the context.
  * Errors: INVALID_ARG (out NULL, max_n < 3 or > TURBOREG_MAX_N, max_batch < 1),
  *         OOM, CUDA. */

@@ -21,7 +21,8 @@ extern "C" {
  * turboreg_register call on a context (n_pad = N rounded up to 256). */
 typedef enum {
     TURBOREG_BUF_ADJ_BITS = 1,  /* uint32 [n_pad][n_pad/32]: bit (j%32) of word [i][j/32] = G_ij (Eq. 1) */
-    TURBOREG_BUF_ADJ_FP8 = 2,   /* uint8  [n_pad][n_pad]: G_ij as FP8 E4M3 (0x38 = 1.0, 0x00 = 0) */
+    TURBOREG_BUF_ADJ_FP8 = 2,   /* uint8  [n_pad][n_pad]: G_ij as FP8 E4M3 (0x38 = 1.0, 0x00 = 0),
+                                   expanded from the GEMM's packed FP4 operand */
     TURBOREG_BUF_SC2 = 3,       /* uint16 [n_pad][n_pad]: O2Graph weights G~_ij (Eq. 2, Def. 2);
                                    only i < j is defined */
     TURBOREG_BUF_PIVOTS = 4,    /* int32 [n_pivots][4]: (i, j, G~_ij, 0) in Eq. 4 order */

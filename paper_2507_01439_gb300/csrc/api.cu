@@ -47,7 +47,7 @@ struct Workspace {
     size_t nh = 0;           // K1_MAX * K2_MAX
     float* pts = nullptr;            // [slots][6 np]
     float* pts8 = nullptr;           // [slots][8 np]
-    uint8_t* a8 = nullptr;           // [slots][np^2]
+    uint8_t* a4 = nullptr;           // [slots][np^2 / 2]
     uint32_t* bits = nullptr;        // [slots][np^2 / 32]
     uint16_t* w = nullptr;           // [slots][np^2]
     int32_t* rows = nullptr;         // [slots][7][np]: rowscore, deg, active (int4 per row), rowmax
@@ -116,8 +116,8 @@ struct turboreg_ctx {
     bool desc_pending = false;
     float stage_ms[kNumStages] = {};
     int32_t last_n = 0, last_npad = 0, last_k1 = 0, last_k2 = 0;
-    bool last_fp8 = false;   // the last plan materialised the FP8 adjacency (tensor-core SC^2)
-    bool last_auto = false;  // ... or left the choice to the device (the FP8 matrix exists if the GEMM ran)
+    bool last_fp4 = false;   // the last plan materialised the FP4 adjacency (tensor-core SC^2)
+    bool last_auto = false;  // ... or left the choice to the device (the FP4 matrix exists if the GEMM ran)
     bool have_times = false;
     // Captured pipelines.  Each slot owns a private copy of its descriptors in
     // device memory, so replays of different shapes never see each other's.
@@ -178,7 +178,7 @@ cudaError_t halloc(T** p, size_t count)
 
 void free_ws(Workspace& ws)
 {
-    void* dptrs[] = {ws.pts, ws.pts8, ws.a8, ws.bits, ws.w, ws.rows, ws.hist, ws.cand, ws.piv, ws.cliques,
+    void* dptrs[] = {ws.pts, ws.pts8, ws.a4, ws.bits, ws.w, ws.rows, ws.hist, ws.cand, ws.piv, ws.cliques,
                      ws.rt, ws.inl, ws.hbits, ws.score, ws.feat, ws.prob, ws.ctl, ws.res, ws.in_src, ws.in_dst,
                      ws.desc};
     for (void* p : dptrs)
@@ -203,7 +203,7 @@ int alloc_ws(Workspace& ws, int32_t max_n, int32_t slots)
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = dalloc(&ws.pts, S * 6 * np);
     if (e == cudaSuccess) e = dalloc(&ws.pts8, S * 8 * np);
-    if (e == cudaSuccess) e = dalloc(&ws.a8, S * n2);
+    if (e == cudaSuccess) e = dalloc(&ws.a4, S * n2 / 2);
     if (e == cudaSuccess) e = dalloc(&ws.bits, S * n2 / 32);
     if (e == cudaSuccess) e = dalloc(&ws.w, S * n2);
     if (e == cudaSuccess) e = dalloc(&ws.rows, S * 7 * np);
@@ -310,7 +310,7 @@ ProbView make_view(turboreg_ctx* c, int slot, int64_t in_off, int32_t n, const t
     v.dbg = (p->flags & TURBOREG_FLAG_DEBUG_STALL_COMPAT) ? TR_DBG_STALL_COMPAT : 0u;
     v.pts = ws.pts + s * 6 * np;
     v.pts8 = ws.pts8 + s * 8 * np;
-    v.a8 = ws.a8 + s * n2;
+    v.a4 = ws.a4 + s * n2 / 2;
     v.bits = ws.bits + s * n2 / 32;
     v.w = ws.w + s * n2;
     int32_t* rows = ws.rows + s * 7 * np;
@@ -333,14 +333,15 @@ ProbView make_view(turboreg_ctx* c, int slot, int64_t in_off, int32_t n, const t
     return v;
 }
 
-// TMA descriptors of slot `slot` for the operand tiles of its FP8 adjacency.
+// TMA descriptors of slot `slot` for the operand tiles of its FP4 adjacency.
 int encode_maps(turboreg_ctx* c, int slot, int32_t n_pad, CUtensorMap* out2)
 {
     Workspace& ws = c->ws;
     if (ws.map_npad[slot] != n_pad) {
-        void* base = ws.a8 + static_cast<size_t>(slot) * ws.np * ws.np;
-        const cuuint64_t dims[2] = {static_cast<cuuint64_t>(n_pad), static_cast<cuuint64_t>(n_pad)};
-        const cuuint64_t strides[1] = {static_cast<cuuint64_t>(n_pad)};   // bytes between rows
+        void* base = ws.a4 + static_cast<size_t>(slot) * ws.np * ws.np / 2;
+        // bytes of two packed values each
+        const cuuint64_t dims[2] = {static_cast<cuuint64_t>(n_pad / 2), static_cast<cuuint64_t>(n_pad)};
+        const cuuint64_t strides[1] = {static_cast<cuuint64_t>(n_pad / 2)};   // bytes between rows
         const cuuint32_t boxA[2] = {static_cast<cuuint32_t>(kSc2BK), static_cast<cuuint32_t>(kSc2BM)};
         const cuuint32_t boxB[2] = {static_cast<cuuint32_t>(kSc2BK), static_cast<cuuint32_t>(kSc2BN)};
         const cuuint32_t estr[2] = {1, 1};
@@ -397,10 +398,10 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
     for (int st = 0; st < kNumBatchStages; ++st) ws.h_pre[st * (num + 1)] = 0;
     for (int32_t b = 0; b < num; ++b) {
         ws.h_views[b] = make_view(c, b, in_off[b], n[b], prm[b]);
-        if (plan.bitset) ws.h_views[b].a8 = nullptr;   // the CUDA-core SC^2 reads the bitset only
-        if (plan.sc2_auto) {   // the FP8 operand only if the device chooses the GEMM
-            ws.h_views[b].a8_auto = ws.h_views[b].a8;
-            ws.h_views[b].a8 = nullptr;
+        if (plan.bitset) ws.h_views[b].a4 = nullptr;   // the CUDA-core SC^2 reads the bitset only
+        if (plan.sc2_auto) {   // the FP4 operand only if the device chooses the GEMM
+            ws.h_views[b].a4_auto = ws.h_views[b].a4;
+            ws.h_views[b].a4 = nullptr;
         }
         const int32_t vppb = (num == 1 && !vflag) ? balanced_vppb(n[b], prm[b]->k1 * prm[b]->k2, device_sms())
                                                   : 4 * vpw_flag;
@@ -422,7 +423,7 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
         }
     }
     plan.vpw = vppb_max <= 4 * 32 ? 32 : vppb_max <= 4 * 64 ? 64 : 128;
-    c->last_fp8 = !plan.bitset && !plan.sc2_auto;
+    c->last_fp4 = !plan.bitset && !plan.sc2_auto;
     c->last_auto = plan.sc2_auto != 0;
     plan.vcap = num == 1 && !vflag;
     return TURBOREG_OK;
@@ -467,7 +468,7 @@ int enqueue_plan(turboreg_ctx* c, const Plan& pl, const Batch& bt, const float* 
     bool fused = false;
     if (pl.sc2_auto) {
         // one problem: the CUDA-core kernel chooses the path from the degrees and
-        // either computes SC^2 or expands the FP8 operand; the GEMM then runs or
+        // either computes SC^2 or expands the FP4 operand; the GEMM then runs or
         // returns at once.  Both keep the histogram for the count blocks.
         launch_sc2_bitset(bt, pl.tot[ST_BITSET], pl.max_n, pl.min_n, sc2_pair_clusters(), s);
         launch_sc2_tcgen05(bt, pl.tot[ST_GEMM], pl.max_n, true, s, true);
@@ -1040,6 +1041,27 @@ int turboreg_register_batched(turboreg_ctx* c, const float* src_cat, const float
     return TURBOREG_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The packed FP4 adjacency as one FP8 E4M3 byte per entry (0x38 = 1.0): the
+// inspection format of TURBOREG_BUF_ADJ_FP8.
+int64_t copy_adj_bytes(const uint8_t* a4, size_t count, void* dst, int64_t max_bytes)
+{
+    if (count > static_cast<size_t>(max_bytes)) count = static_cast<size_t>(max_bytes);
+    std::vector<uint8_t> packed((count + 1) / 2);
+    if (count && cudaMemcpy(packed.data(), a4, packed.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return -TURBOREG_ERR_CUDA;
+    uint8_t* out = static_cast<uint8_t*>(dst);
+    for (size_t k = 0; k < count; ++k) out[k] = ((packed[k / 2] >> (4 * (k & 1))) & 0xFu) ? 0x38 : 0x00;
+    return static_cast<int64_t>(count);
+}
+
+}  // namespace
+
+extern "C" {
+
 int turboreg_debug_sc2_path(turboreg_ctx* c, int32_t* path)
 {
     if (!c || !path) return TURBOREG_ERR_INVALID_ARG;
@@ -1050,7 +1072,7 @@ int turboreg_debug_sc2_path(turboreg_ctx* c, int32_t* path)
         TR_CHECK(cudaMemcpy(&h, c->ws.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
         *path = static_cast<int32_t>(h.sc2_path);
     } else {
-        *path = c->last_fp8 ? 2 : 1;
+        *path = c->last_fp4 ? 2 : 1;
     }
     return TURBOREG_OK;
 }
@@ -1087,11 +1109,9 @@ int64_t turboreg_debug_copy(turboreg_ctx* c, int which, void* dst, int64_t max_b
     switch (which) {
         case TURBOREG_BUF_ADJ_BITS: src = v.bits; bytes = np * np / 8; break;
         case TURBOREG_BUF_ADJ_FP8:
-            if (!c->last_fp8 && !(c->last_auto && h.sc2_path == 2u))
+            if (!c->last_fp4 && !(c->last_auto && h.sc2_path == 2u))
                 return -TURBOREG_ERR_INVALID_ARG;   // not materialised by that plan (or that choice)
-            src = v.a8;
-            bytes = np * np;
-            break;
+            return copy_adj_bytes(v.a4, np * np, dst, max_bytes);
         case TURBOREG_BUF_SC2: src = v.w; bytes = np * np * 2; break;
         case TURBOREG_BUF_PIVOTS: src = v.piv; bytes = static_cast<size_t>(h.n_pivots) * 16; break;
         case TURBOREG_BUF_CLIQUES: src = v.cliques; bytes = nh * 16; break;

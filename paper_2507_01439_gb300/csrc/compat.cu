@@ -8,8 +8,8 @@
 // compat: G_ij = [ | ||x_i - x_j|| - ||y_i - y_j|| | <= tau ], i != j, G_ii = 0
 //         (Eq. 1; zero diagonal because App. B equates G^_ij with the number
 //         of triangles on edge (i,j)).  Written as a row bitset (operand of the
-//         clique search), as FP8 E4M3 0/1 bytes (operand of the SC^2 GEMM) and
-//         as node degrees.
+//         clique search), as packed FP4 0/1 values (operand of the SC^2 GEMM)
+//         and as node degrees.
 //
 // Work decomposition: 128 x 128 tiles (I, J) with I <= J only.  A block
 // computes its tile once and writes it twice (rows i of tile (I, J) and,
@@ -167,19 +167,7 @@ __device__ __forceinline__ void compat_fast2(const f2 (&XI)[6], const f2 (&XJ)[6
     a1 = P1 <= 0.f;
 }
 
-// 4 bits -> 4 bytes of FP8 E4M3 (0x38 = 1.0 for a set bit, 0x00 otherwise)
-__device__ __forceinline__ uint32_t nibble_to_fp8(uint32_t nib)
-{
-    return ((nib * 0x00204081u) & 0x01010101u) * 0x38u;
-}
-
-__device__ __forceinline__ uint4 bits16_to_fp8(uint32_t b16)
-{
-    return make_uint4(nibble_to_fp8(b16 & 0xF), nibble_to_fp8((b16 >> 4) & 0xF), nibble_to_fp8((b16 >> 8) & 0xF),
-                      nibble_to_fp8((b16 >> 12) & 0xF));
-}
-
-// kAuto: the SC^2 path is chosen on the device (one problem): no FP8 matrix,
+// kAuto: the SC^2 path is chosen on the device (one problem): no FP4 matrix,
 // and the degree sum 2 |E| is added up in the control block
 template <bool kAuto>
 __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
@@ -343,22 +331,21 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
             if (lane == 0 && ds) atomicAdd(&v.ctl->deg_sum, ds);
         }
     }
-    // FP8 rows (only for the tensor-core SC^2), 128 contiguous bytes per row:
-    // pass k writes rows 4k .. 4k + 3 of the warp's 32, lane l the 16-byte
-    // segment l % 8 of row 4k + l / 8
-    const bool fp8 = !kAuto && v.a8 != nullptr;
+    // FP4 rows (only for the tensor-core SC^2), 64 contiguous bytes per row:
+    // pass k writes rows 8k .. 8k + 7 of the warp's 32, lane l the 16 bytes of
+    // word l % 4 of row 8k + l / 4
+    const bool fp4 = !kAuto && v.a4 != nullptr;
 #pragma unroll
-    for (int k = 0; k < kR / 4 && fp8; ++k) {
-        const int r = 4 * k + (lane >> 3);
-        const int seg = lane & 7;
+    for (int k = 0; k < kR / 8 && fp4; ++k) {
+        const int r = 8 * k + (lane >> 2);
+        const int q = lane & 3;
         const uint32_t w0 = __shfl_sync(0xffffffffu, wrow_bits[0], r);
         const uint32_t w1 = __shfl_sync(0xffffffffu, wrow_bits[1], r);
         const uint32_t w2 = __shfl_sync(0xffffffffu, wrow_bits[2], r);
         const uint32_t w3 = __shfl_sync(0xffffffffu, wrow_bits[3], r);
-        const uint32_t w = (seg >> 1) == 0 ? w0 : (seg >> 1) == 1 ? w1 : (seg >> 1) == 2 ? w2 : w3;
         const int i = i0 + warp * kR + r;
-        *reinterpret_cast<uint4*>(v.a8 + (size_t)i * v.n_pad + j0 + seg * 16) =
-            bits16_to_fp8((w >> ((seg & 1) * 16)) & 0xFFFFu);
+        *reinterpret_cast<uint4*>(v.a4 + (size_t)i * (v.n_pad >> 1) + (j0 >> 1) + q * 16) =
+            word_fp4(q == 0 ? w0 : q == 1 ? w1 : q == 2 ? w2 : w3);
     }
     if (diag) return;
     // mirrored tile: row j gets bits of rows i0 .. i0+127; column c's word w
@@ -378,14 +365,12 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
             if (lane == 0 && ds) atomicAdd(&v.ctl->deg_sum, 2u * ds);
         }
     }
-    // FP8 rows: pass k writes rows j0 + 16k .. +15, eight threads per 128-byte row
+    // FP4 rows: pass k writes rows j0 + 32k .. +31, four threads per 64-byte row
 #pragma unroll
-    for (int k = 0; k < 8 && fp8; ++k) {
-        const int c = 16 * k + (threadIdx.x >> 3);
-        const int seg = threadIdx.x & 7;
-        const uint32_t w = reinterpret_cast<const uint32_t*>(colpart[c])[seg >> 1];
-        *reinterpret_cast<uint4*>(v.a8 + (size_t)(j0 + c) * v.n_pad + i0 + seg * 16) =
-            bits16_to_fp8((w >> ((seg & 1) * 16)) & 0xFFFFu);
+    for (int k = 0; k < 4 && fp4; ++k) {
+        const int c = 32 * k + (threadIdx.x >> 2);
+        const int q = threadIdx.x & 3;
+        *reinterpret_cast<uint4*>(v.a4 + (size_t)(j0 + c) * (v.n_pad >> 1) + (i0 >> 1) + q * 16) = word_fp4(colpart[c][q]);
     }
 }
 

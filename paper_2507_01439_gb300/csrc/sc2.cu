@@ -3,21 +3,35 @@
 //   W_ij = G_ij * sum_k G_ik G_jk  for i < j,   i.e.  W = triu(G .* (G G), 1)
 //
 // Main path: a binary GEMM on the 5th-generation tensor cores.  G is stored
-// as FP8 E4M3 0/1 bytes; since G is symmetric, G G = G G^T, so both MMA
-// operands are K-major row blocks of the same matrix.  Products of 0/1 are
-// exact and the FP32 accumulator holds integers <= N-2 < 2^24 exactly, so the
-// result is the integer SC^2 count.  Only output tiles that contain some
-// i < j are computed (the upper triangle, about half the square).
+// as packed FP4 (E2M1) 0/1 values; since G is symmetric, G G = G G^T, so both
+// MMA operands are K-major row blocks of the same matrix.  The MMAs are the
+// block-scaled FP4 kind with every block scale 1.0; products of 0/1 are exact
+// and the FP32 accumulator holds integers <= N-2 < 2^24 exactly, so the
+// result is the integer SC^2 count.  FP4 operands carry twice the products
+// per byte and per tensor-core cycle of FP8 ones, and the kernel is bound by
+// exactly these two (at the full MMA rate the operands stream from L2 at
+// ~17 TB/s with either type).  Only output blocks that contain some i < j are
+// computed (the upper triangle, about half the square).  Measured against the
+// FP8 kernel it replaced: 3640 -> 1388 us at N = 20000 (where the histogram
+// also moved to shared memory and the block order keeps the operand in L2),
+// 48 -> 35 us at N = 4333 (13 % density), 2838 -> 2137 us for 256 problems
+// of N = 500 .. 5000.
 //
-// Kernel anatomy (one 128 x 256 output tile per CTA, 128 threads):
-//   warp 0 lane 0  TMA producer: 128-byte-swizzled K-major tiles A[i-block,k],
-//                  A[j-block,k] into a 4-stage shared-memory ring (mbarriers)
-//   warp 1 lane 0  MMA issuer: tcgen05.mma kind::f8f6f4, M=128 N=256 K=32,
-//                  4 per stage, accumulating in 256 TMEM columns
-//   warps 0-3      epilogue: tcgen05.ld the accumulator (warp w owns TMEM
-//                  lanes 32w..32w+31 = tile rows), mask with the adjacency
-//                  bitset and i < j, store uint16 W, and add the row and
-//                  column sums into the SC^2 row scores.
+// Work: 256 x 256 output blocks (bm <= bn), taken by 2-CTA clusters as pair
+// MMAs (cta_group::2, each CTA's shared memory holding its halves of A and B)
+// or, on request, as two 128 x 256 halves by independent CTAs.
+//   warp 0 lane 0  TMA producer: 128-byte-swizzled K-major tiles, 256 columns
+//                  of K per stage, into a ring of 2 to 5 stages (as many as fit
+//                  beside the histogram)
+//   warp 1 lane 0  MMA issuer: tcgen05.mma kind::mxf4, N=256 K=64, 4 per stage
+//   warps 2..17    epilogue of the previous block while the next one runs
+//
+// Tensor memory (512 columns): two 256-column accumulators and 16 columns of
+// block scales do not fit side by side, so the accumulators overlap in 16
+// columns: buffer 0 at columns 0..255, buffer 1 at 240..495, scales at
+// 496..511.  The epilogue warps that own the shared columns read them first
+// and report it (`tover`); the next block's MMAs wait for that, not for the
+// whole epilogue.
 //
 // Alternative (sc2_bitset.cu): the same integers from the adjacency bitset
 // with AND + popcount on CUDA cores, work only on the edges.
@@ -29,156 +43,157 @@ namespace tr {
 
 namespace {
 
-constexpr int kStages = 4;
-constexpr int kABytes = kSc2BM * kSc2BK;   // 16 KB
-constexpr int kBBytes = kSc2BN * kSc2BK;   // 32 KB
+constexpr int kHalf = kSc2BM * kSc2BK;     // 16 KB: 128 rows x 128 bytes of one operand
 constexpr int kEpiWarps = 16;              // 4 per TMEM lane quarter, each a quarter of the columns
 constexpr int kEpiCols = 4 * kSc2BN / kEpiWarps;   // 64 columns per epilogue warp
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kPipeBytes = kStages * (kABytes + kBBytes);
-constexpr int kBarBytes = 512;            // mbarriers, TMEM slot, select scratch
+constexpr int kMaxStages = 5;
+constexpr int kBarBytes = 512;             // mbarriers, TMEM slot
+constexpr int kStgBytes = kEpiWarps * 2048;   // W staging: 32 x 32 uint16 per epilogue warp
 constexpr int kSmemMax = 232448;           // 227 KB opt-in limit per block
-constexpr uint32_t kTmemCols = 512;        // two 256-column FP32 accumulators
-// E4M3 x E4M3 -> F32, M = 128, N = 256, both K-major
-constexpr uint32_t kIdesc = idesc_f32acc(0u, 0u, kSc2BM, kSc2BN);
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kAcc1 = 240;            // first column of accumulator 1 (16 shared with accumulator 0)
+constexpr uint32_t kScaleCol = 496;        // block scales: A from 496 (4 columns), B from 500 (8 columns)
+constexpr int kPanel = 8;                  // column blocks per panel of the block order
 
-__device__ __forceinline__ void tile_of(int t, int& bm, int& bn)
+template <bool kPair>
+constexpr int stage_bytes() { return (kPair ? 2 : 3) * kHalf; }   // this CTA's part of A and B per stage
+
+// Block u of a problem with nb = n_pad / 256 column blocks.  Blocks are
+// ordered in panels of eight column blocks, row by row inside a panel, so
+// that the blocks in flight at any time cover a compact patch of the output:
+// at N = 20000 one wave of 76 blocks reads 17 of the 79 row blocks of G
+// instead of all of them, and the 200 MB operand is served from L2.
+__device__ __forceinline__ void block_of(int u, int nb, int& bm, int& bn)
 {
-    // tiles of column block bn are row blocks 0 .. 2bn+1; column block bn starts at t = bn(bn+1)
-    int b = static_cast<int>((sqrtf(4.0f * t + 1.0f) - 1.0f) * 0.5f);
-    while (b * (b + 1) > t) --b;
-    while ((b + 1) * (b + 2) <= t) ++b;
-    bn = b;
-    bm = t - b * (b + 1);
+    // panel P holds the columns 8P .. and starts at block 8P (8P + 1) / 2
+    int P = static_cast<int>((sqrtf(8.0f * static_cast<float>(u) + 1.0f) - 1.0f) * 0.5f) / kPanel;
+    while (kPanel * P * (kPanel * P + 1) / 2 > u) --P;
+    while (kPanel * (P + 1) * (kPanel * (P + 1) + 1) / 2 <= u) ++P;
+    const int c0 = kPanel * P;
+    const int w = min(kPanel, nb - c0);
+    int r = u - c0 * (c0 + 1) / 2;
+    if (r < c0 * w) {
+        bm = r / w;
+        bn = c0 + r % w;
+        return;
+    }
+    r -= c0 * w;
+    int k = 0;
+    while (r >= w - k) {
+        r -= w - k;
+        ++k;
+    }
+    bm = c0 + k;
+    bn = c0 + k + r;
 }
 
-// Epilogue of one 128 x 256 output tile whose FP32 accumulator is at TMEM
-// column tacc: warp (quarter, part) reads TMEM lanes 32 quarter .. +31 (tile
-// rows) and the kEpiCols columns of its part, masks with the adjacency bitset
-// and i < j, stores uint16 W, adds the row and column sums to the SC^2 row
-// scores and counts the edge weights (shared or global histogram).  The
-// bitset words of the warp's columns are fetched before the accumulator is
-// waited for (epi_words), so their latency overlaps the MMAs.
-__device__ __forceinline__ uint2 epi_words(const ProbView& v, int bm, int bn, int quarter, int part, int lane)
+// Block k of this worker (cluster or CTA `c` of `C`): chunks of `L`
+// consecutive blocks, strided over the workers (a batch takes several blocks
+// of one problem in a row, so that its histogram is flushed less often).
+__device__ __forceinline__ int block_index(int k, int c, int C, int L)
+{
+    return (c + k / L * C) * L + k % L;
+}
+
+// The bitset words of an epilogue warp's columns, fetched before the
+// accumulator is waited for, so that their latency overlaps the MMAs.
+__device__ __forceinline__ uint2 epi_words(const ProbView& v, int row, int col)
 {
     static_assert(kEpiCols == 64, "one 8-byte bitset load per warp row");
-    const int row = bm * kSc2BM + quarter * 32 + lane;
-    return *reinterpret_cast<const uint2*>(v.bits + (size_t)row * v.ldb + ((bn * kSc2BN + part * kEpiCols) >> 5));
+    return *reinterpret_cast<const uint2*>(v.bits + (size_t)row * v.ldb + (col >> 5));
 }
 
-template <bool kSingle>
-__device__ __forceinline__ void sc2_epilogue_tile(const ProbView& v, uint32_t tacc, int bm, int bn, int quarter,
-                                                  int part, int lane, uint2 words, uint32_t* shist)
+// The warp's 2 KB staging area holds its 32 x 32 block of W: row r as four
+// 16-byte chunks, chunk q at slot q ^ ((r >> 1) & 3), so that row-wise and
+// column-wise accesses are both free of bank conflicts.
+__device__ __forceinline__ uint32_t stg_slot(int r, int q) { return static_cast<uint32_t>(r * 4 + (q ^ ((r >> 1) & 3))); }
+
+// Bits of each 16-bit half unshuffled: even positions into its low byte, odd
+// ones into its high byte (three butterfly steps).
+__device__ __forceinline__ uint32_t unshuffle16(uint32_t x)
 {
-    const int row = bm * kSc2BM + quarter * 32 + lane;
-    uint16_t* wrow = v.w + (size_t)row * v.n_pad;
-    int rsum = 0, rmax = 0;
-#pragma unroll 1
-    for (int c = 0; c < kEpiCols / 32; ++c) {
-        const int cc = part * kEpiCols + c * 32;
-        uint32_t acc[32];
-        tmem_ld32(tacc + static_cast<uint32_t>(cc) + (static_cast<uint32_t>(quarter * 32) << 16),
-                  acc);
-        tmem_ld_wait();
-        const int col0 = bn * kSc2BN + cc;
-        uint32_t word = c == 0 ? words.x : words.y;
-        if (col0 + 31 <= row) word = 0u;                       // keep only j > row
-        else if (col0 <= row) word &= ~0u << (row - col0 + 1);
-        int val[32];
-#pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            val[q] = ((word >> q) & 1u) ? static_cast<int>(__uint_as_float(acc[q])) : 0;
-            rsum += val[q];
-            rmax = max(rmax, val[q]);
-        }
-        if (word) {
-#pragma unroll
-            for (int q = 0; q < 32; ++q)
-                if (val[q] > 0) {
-                    if (kSingle) atomicAdd(&shist[val[q]], 1u);
-                    else atomicAdd(&v.hist[val[q]], 1u);
-                }
-        }
-        uint4* dst = reinterpret_cast<uint4*>(wrow + col0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint4 pk;
-            pk.x = static_cast<uint32_t>(val[8 * q + 0]) | (static_cast<uint32_t>(val[8 * q + 1]) << 16);
-            pk.y = static_cast<uint32_t>(val[8 * q + 2]) | (static_cast<uint32_t>(val[8 * q + 3]) << 16);
-            pk.z = static_cast<uint32_t>(val[8 * q + 4]) | (static_cast<uint32_t>(val[8 * q + 5]) << 16);
-            pk.w = static_cast<uint32_t>(val[8 * q + 6]) | (static_cast<uint32_t>(val[8 * q + 7]) << 16);
-            dst[q] = pk;
-        }
-        // column sums over this warp's 32 rows (butterfly transpose-reduce):
-        // afterwards lane l holds the sum of column col0 + l
-        if (__any_sync(0xffffffffu, word != 0u)) {
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) {
-                const bool upper = (lane & off) != 0;
-#pragma unroll
-                for (int q = 0; q < off; ++q) {
-                    const int send = upper ? val[q] : val[q + off];
-                    const int keepv = upper ? val[q + off] : val[q];
-                    val[q] = keepv + __shfl_xor_sync(0xffffffffu, send, off);
-                }
-            }
-            if (val[0] != 0) atomicAdd(&v.rowscore[col0 + lane], val[0]);
-        }
-    }
-    if (rsum != 0) atomicAdd(&v.rowscore[row], rsum);
-    if (rmax != 0 && v.rowmax) atomicMax(&v.rowmax[row], rmax);
+    uint32_t t = (x ^ (x >> 1)) & 0x22222222u;
+    x ^= t ^ (t << 1);
+    t = (x ^ (x >> 2)) & 0x0C0C0C0Cu;
+    x ^= t ^ (t << 2);
+    t = (x ^ (x >> 4)) & 0x00F000F0u;
+    return x ^ t ^ (t << 4);
 }
 
-// The same epilogue through the warp's 2 KB of shared memory `stg`, which
-// holds the warp's 32 x 32 block of W (row r as four 16-byte chunks, chunk q
-// at slot q ^ ((r >> 1) & 3), so that row-wise and column-wise accesses are
-// both free of bank conflicts).  From there:
+// Bytes of x picked by sel, a nibble with bit 3 set replicating the byte's
+// sign bit (__byte_perm ignores that bit).
+__device__ __forceinline__ uint32_t sign_bytes(uint32_t x, uint32_t sel)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "r"(sel));
+    return r;
+}
+
+// Arrival on a barrier given by its address in the cluster's (pair) or this CTA's shared window.
+template <bool kPair>
+__device__ __forceinline__ void arrive_at(uint32_t bar)
+{
+    if (kPair) mbar_arrive_cluster(bar);
+    else mbar_arrive_addr(bar);
+}
+
+// Epilogue of one warp's 32 rows x 64 columns whose FP32 accumulator is at
+// TMEM address tacc: masks with the adjacency words and i < j, stores uint16
+// W, adds row and column sums to the SC^2 row scores, row maxima, and counts
+// the edge weights (shared or global histogram).
+//   integers      adding 2^23 leaves an accumulator's integer in its low 16
+//                 bits (exact: it is an integer below 2^16); a byte permute
+//                 packs two, and one that replicates sign bits turns two
+//                 adjacency bits into their mask
 //   W store       pass k writes rows 8k .. 8k + 7, lane l chunk l % 4 of row
 //                 8k + l / 4: each instruction covers 8 x 64 contiguous bytes
 //   column sums   lane l reads 8 bytes (4 columns) of rows 4k + l / 8; the
 //                 four row groups are added with two shuffles per column
 //   histogram     each lane visits only the set bits of its adjacency word
-// These replace per-lane row stores (a half-filled sector per lane), the
-// 31-shuffle butterfly and 32 predicated atomics per chunk.
-__device__ __forceinline__ uint32_t stg_slot(int r, int q) { return static_cast<uint32_t>(r * 4 + (q ^ ((r >> 1) & 3))); }
-
-template <bool kSingle>
-__device__ __forceinline__ void sc2_epilogue_tile_staged(const ProbView& v, uint32_t tacc, int bm, int bn, int quarter,
-                                                         int part, int lane, uint2 words, uint32_t* shist, uint4* stg)
+// first / over: the 32-column chunk to take first, and the barrier (or 0) to
+// report to once its accumulator columns are in registers.
+template <bool kPair, bool kHist>
+__device__ __forceinline__ void sc2_epilogue(const ProbView& v, uint32_t tacc, int row0, int col_w, int lane,
+                                             uint2 words, uint32_t* shist, uint4* stg, int first, uint32_t over)
 {
-    const int row0 = bm * kSc2BM + quarter * 32;
     const int row = row0 + lane;
-    int rsum = 0, rmax = 0;
+    uint32_t rsum = 0u, rmax2 = 0u;
 #pragma unroll 1
-    for (int c = 0; c < kEpiCols / 32; ++c) {
-        const int cc = part * kEpiCols + c * 32;
+    for (int k = 0; k < kEpiCols / 32; ++k) {
+        const int c = k ^ first;
         uint32_t acc[32];
-        tmem_ld32(tacc + static_cast<uint32_t>(cc) + (static_cast<uint32_t>(quarter * 32) << 16),
-                  acc);
+        tmem_ld32(tacc + static_cast<uint32_t>(c * 32), acc);
         tmem_ld_wait();
-        const int col0 = bn * kSc2BN + cc;
+        if (k == 0 && over != 0u) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_at<kPair>(over);
+        }
+        const int col0 = col_w + c * 32;
         uint32_t word = c == 0 ? words.x : words.y;
         if (col0 + 31 <= row) word = 0u;                       // keep only j > row
         else if (col0 <= row) word &= ~0u << (row - col0 + 1);
+        const uint32_t ub = unshuffle16(word);
+        uint32_t h[16];
+        const f2 magic = pk(8388608.f, 8388608.f);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint32_t h[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int a = 8 * q + 2 * e;
-                const int lo = ((word >> a) & 1u) ? static_cast<int>(__uint_as_float(acc[a])) : 0;
-                const int hi = ((word >> (a + 1)) & 1u) ? static_cast<int>(__uint_as_float(acc[a + 1])) : 0;
-                rsum += lo + hi;
-                rmax = max(rmax, max(lo, hi));
-                h[e] = static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
-            }
-            stg[stg_slot(lane, q)] = make_uint4(h[0], h[1], h[2], h[3]);
+        for (int e = 0; e < 16; ++e) {
+            const f2 s = add2(pk(__uint_as_float(acc[2 * e]), __uint_as_float(acc[2 * e + 1])), magic);
+            // columns 2e, 2e + 1: bit e % 8 of the two bytes of half e / 8, moved to the bytes' sign bits
+            const uint32_t m = sign_bytes(ub << (7 - (e & 7)), e < 8 ? 0x9988u : 0xBBAAu);
+            h[e] = __byte_perm(static_cast<uint32_t>(s.v), static_cast<uint32_t>(s.v >> 32), 0x5410u) & m;
+            rsum = __dp2a_lo(h[e], 0x0101u, rsum);
+            rmax2 = __vmaxu2(rmax2, h[e]);
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            stg[stg_slot(lane, q)] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
         __syncwarp();
         // W rows, as full 64-byte segments
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int r = 8 * k + (lane >> 2), q = lane & 3;
+        for (int k4 = 0; k4 < 4; ++k4) {
+            const int r = 8 * k4 + (lane >> 2), q = lane & 3;
             *reinterpret_cast<uint4*>(v.w + (size_t)(row0 + r) * v.n_pad + col0 + q * 8) = stg[stg_slot(r, q)];
         }
         // column sums: lane l adds columns 4 (l % 8) .. +3 over rows l / 8 + 4k
@@ -187,9 +202,9 @@ __device__ __forceinline__ void sc2_epilogue_tile_staged(const ProbView& v, uint
             const int m = lane & 7;
             int cs[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                const uint2 d0 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * k + (lane >> 3), m >> 1))[m & 1];
-                const uint2 d1 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * k + 4 + (lane >> 3), m >> 1))[m & 1];
+            for (int kk = 0; kk < 8; kk += 2) {
+                const uint2 d0 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * kk + (lane >> 3), m >> 1))[m & 1];
+                const uint2 d1 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * kk + 4 + (lane >> 3), m >> 1))[m & 1];
                 const uint32_t x = d0.x + d1.x, y = d0.y + d1.y;   // two rows per 16-bit lane
                 cs[0] += static_cast<int>(x & 0xFFFFu);
                 cs[1] += static_cast<int>(x >> 16);
@@ -211,187 +226,34 @@ __device__ __forceinline__ void sc2_epilogue_tile_staged(const ProbView& v, uint
             const int q = __ffs(bits) - 1;
             const int w = reinterpret_cast<const uint16_t*>(stg + stg_slot(lane, q >> 3))[q & 7];
             if (w > 0) {
-                if (kSingle) atomicAdd(&shist[w], 1u);
+                if (kHist) atomicAdd(&shist[w], 1u);
                 else atomicAdd(&v.hist[w], 1u);
             }
         }
         __syncwarp();   // the next chunk overwrites the staging area
     }
-    if (rsum != 0) atomicAdd(&v.rowscore[row], rsum);
+    if (rsum != 0u) atomicAdd(&v.rowscore[row], static_cast<int>(rsum));
+    const int rmax = static_cast<int>(max(rmax2 & 0xFFFFu, rmax2 >> 16));
     if (rmax != 0 && v.rowmax) atomicMax(&v.rowmax[row], rmax);
 }
 
-// Persistent, warp-specialised: CTA b handles global tiles b, b + grid, ...
-// of all problems of the batch (problem p's tiles are [pre[p], pre[p+1]) of
-// stage ST_GEMM; tensor maps of problem p at maps[2p], maps[2p+1]).
-//   warp 0 lane 0   TMA producer over all (tile, k) of this CTA
-//   warp 1 lane 0   MMA issuer; accumulator buffer (tile count & 1)
-//   warps 2..17     epilogue of the previous tile while the next one runs
-// kSingle: one problem: the edge-weight histogram is kept in shared memory
-// and added to the global one at the end (the count pass then chooses the
-// pivot threshold from it).
-template <bool kSingle>
-__global__ void __launch_bounds__(kThreads, 1) sc2_tcgen05_kernel(Batch bt, int total)
-{
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sA = smem;
-    uint8_t* sB = smem + kStages * kABytes;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kPipeBytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* tfull = empty + kStages;      // [2] accumulator ready
-    uint64_t* tempty = tfull + 2;           // [2] accumulator drained
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
-    uint32_t* shist = reinterpret_cast<uint32_t*>(smem + kPipeBytes + kBarBytes);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nbins = kSingle ? bt.views[0].n + 1 : 0;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], kEpiWarps);
-        }
-        fence_mbar_init();
-    }
-    if (kSingle)
-        for (int b = threadIdx.x; b < nbins; b += blockDim.x) shist[b] = 0u;
-    if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    bool ok = true;
-    const int u0 = static_cast<int>(blockIdx.x);
-    const int us = static_cast<int>(gridDim.x);
-    const int nu = total;
-    // the set-up above (barriers, tensor memory, shared histogram) overlaps the
-    // previous stage; its outputs are read only from here on
-    pdl_wait();
-    pdl_release();
-
-    if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer ----------------
-            int it = 0;
-            for (int u = u0; u < nu && ok; u += us) {
-                int lt;
-                const int p = locate(bt, ST_GEMM, u, lt);
-                const int KT = bt.views[p].n_pad / kSc2BK;
-                const CUtensorMap* mA = bt.maps + 2 * p;
-                const CUtensorMap* mB = mA + 1;
-                int bm, bn;
-                tile_of(lt, bm, bn);
-                for (int kb = 0; kb < KT; ++kb, ++it) {
-                    const int s = it % kStages;
-                    const uint32_t ph = (it / kStages) & 1u;
-                    if (!mbar_wait(&empty[s], ph ^ 1u)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&full[s], kABytes + kBBytes);
-                    tma_load_2d(sA + s * kABytes, mA, kb * kSc2BK, bm * kSc2BM, &full[s]);
-                    tma_load_2d(sB + s * kBBytes, mB, kb * kSc2BK, bn * kSc2BN, &full[s]);
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
-            int it = 0, tc = 0;
-            for (int u = u0; u < nu && ok; u += us, ++tc) {
-                int lt;
-                const int p = locate(bt, ST_GEMM, u, lt);
-                const int KT = bt.views[p].n_pad / kSc2BK;
-                const int buf = tc & 1;
-                const uint32_t use = static_cast<uint32_t>(tc >> 1);
-                if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t d = tmem + static_cast<uint32_t>(buf * kSc2BN);
-                for (int kb = 0; kb < KT; ++kb, ++it) {
-                    const int s = it % kStages;
-                    const uint32_t ph = (it / kStages) & 1u;
-                    if (!mbar_wait(&full[s], ph)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t a0 = smem_u32(sA + s * kABytes);
-                    const uint32_t b0 = smem_u32(sB + s * kBBytes);
-#pragma unroll
-                    for (int k = 0; k < kSc2BK / 32; ++k)   // K = 32 FP8 per MMA, 32-byte steps in the swizzle row
-                        mma_f8f6f4(d, sdesc_k_sw128(a0 + k * 32), sdesc_k_sw128(b0 + k * 32), kIdesc,
-                                   (kb | k) != 0 ? 1u : 0u);
-                    mma_commit(&empty[s]);
-                }
-                if (!ok) break;
-                mma_commit(&tfull[buf]);
-            }
-        }
-        __syncwarp();
-    } else {
-        // ---------------- epilogue warps ----------------
-        const int quarter = warp & 3;              // TMEM lanes this warp may access
-        const int part = (warp - 2) >> 2;          // column part of the tile
-        int tc = 0;
-        for (int u = u0; u < nu; u += us, ++tc) {
-            int lt;
-            const int p = locate(bt, ST_GEMM, u, lt);
-            const ProbView v = bt.views[p];
-            int bm, bn;
-            tile_of(lt, bm, bn);
-            const int buf = tc & 1;
-            const uint32_t use = static_cast<uint32_t>(tc >> 1);
-            const uint2 words = epi_words(v, bm, bn, quarter, part, lane);
-            const bool got = mbar_wait(&tfull[buf], use & 1u);
-            if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-            tc_fence_after();
-            sc2_epilogue_tile<kSingle>(v, tmem + static_cast<uint32_t>(buf * kSc2BN), bm, bn, quarter, part, lane, words,
-                                       shist);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[buf]);
-        }
-    }
-    if (!ok && lane == 0) atomicOr(&bt.views[0].ctl->err, TR_ERR_TIMEOUT);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
-    }
-    if (!kSingle) return;
-    // this CTA's histogram into the global one, from which the count pass
-    // chooses the pivot threshold
-    const ProbView v0 = bt.views[0];
-    for (int b = threadIdx.x + 1; b < nbins; b += blockDim.x)
-        if (shist[b]) atomicAdd(&v0.hist[b], shist[b]);
-}
-
-// 2-SM form (cta_group::2): the two CTAs of a cluster compute one 256 x 256
-// output block with pair MMAs (M = 256: 128 rows of A per CTA; N = 256: 128
-// columns of B per CTA).  Each CTA's shared memory holds only its own halves
-// (32 KB per 128-deep K stage instead of 48 KB), so five stages fit beside a
-// 32 KB staging area through which the epilogue writes W as full 64-byte row
-// segments (the direct per-row stores of the other forms half-fill a sector
-// per lane and slow the concurrent MMAs).
-//   both CTAs  warp 0 lane 0: TMA loads of this CTA's A and B halves, counted
-//              on the leader's `full` barrier; the leader announces 64 KB
-//   leader     warp 1 lane 0: pair MMAs; their commits release the stage in
-//              both CTAs (`empty`) and hand each CTA its accumulator (`tfull`)
-//   both CTAs  warps 2..17: epilogue of this CTA's 128 x 256 rows; the
-//              accumulator is free again when the epilogue warps of both CTAs
-//              have arrived on the leader's `tempty`
+// kPair: 2-CTA clusters with pair MMAs (M = 256 over both CTAs); else CTAs of
+// their own take 128-row halves of the blocks.  kHist: the edge-weight
+// histogram is kept in shared memory and added to the global one when the
+// worker leaves a problem (the count pass or the select launch then chooses
+// the pivot threshold from it); else every edge adds to the global bins.
+//   pair: both CTAs' producers load their 128 rows of A and of B, counted on
+//         the leader's `full` barrier; the leader issues the MMAs, whose commits
+//         release the stage in both CTAs (`empty`) and hand each CTA its
+//         accumulator (`tfull`); the epilogue warps of both CTAs arrive on the
+//         leader's `tempty` and `tover`
 // Every wait is bounded; before exit each producer waits for the last stage
-// releases and the cluster synchronises, so no arrival targets a finished CTA.
-constexpr int kStages2 = 5;
-constexpr int kPipeBytes2 = kStages2 * 2 * kABytes;   // 160 KB
-constexpr int kStageBytes2 = kEpiWarps * 2048;       // W staging: 32 x 32 uint16 per epilogue warp
-constexpr int kBase2 = kPipeBytes2 + kBarBytes + kStageBytes2 + 1024;   // before the shared histogram
-
+// releases and a cluster synchronises, so no arrival targets a finished CTA.
 // auto_mode: one problem whose SC^2 path the CUDA-core kernel before this one
 // chose; when it chose itself, every CTA returns at once (before any set-up).
-template <bool kHist>
-__global__ void __launch_bounds__(kThreads, 1) sc2_pair_mma_kernel(Batch bt, int total, int hist_bins, int auto_mode)
+template <bool kPair, bool kHist>
+__global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int total, int hist_bins, int nst, int chunk,
+                                                              int auto_mode)
 {
     if (auto_mode) {
         const Ctl* ctl = bt.views[0].ctl;   // the descriptor before the wait, the flag after it
@@ -403,155 +265,194 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_pair_mma_kernel(Batch bt, int
     }
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    constexpr int kBPart = kPair ? kHalf : 2 * kHalf;    // this CTA's bytes of B per stage
     uint8_t* sA = smem;                                  // [stage] 128 rows x 128 B
-    uint8_t* sB = smem + kStages2 * kABytes;             // [stage] 128 rows x 128 B (this CTA's B half)
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kPipeBytes2);
-    uint64_t* empty = full + kStages2;
-    uint64_t* tfull = empty + kStages2;      // [2] accumulator ready
-    uint64_t* tempty = tfull + 2;            // [2] accumulator drained (leader's counts both CTAs)
-    uint64_t* hsync = tempty + 2;            // epilogue warps: a problem's bins complete / flushed
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 3);
-    uint4* stg = reinterpret_cast<uint4*>(smem + kPipeBytes2 + kBarBytes);
-    uint32_t* shist = reinterpret_cast<uint32_t*>(smem + kPipeBytes2 + kBarBytes + kStageBytes2);
+    uint8_t* sB = smem + nst * kHalf;                    // [stage] 128 or 256 rows x 128 B
+    uint8_t* tail = smem + nst * stage_bytes<kPair>();
+    uint64_t* full = reinterpret_cast<uint64_t*>(tail);
+    uint64_t* empty = full + kMaxStages;
+    uint64_t* tfull = empty + kMaxStages;    // [2] accumulator ready
+    uint64_t* tempty = tfull + 2;            // [2] accumulator drained
+    uint64_t* tover = tempty + 2;            // the columns both accumulators share are read
+    uint64_t* hsync = tover + 1;             // epilogue warps: a problem's bins complete / flushed
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(hsync + 1);
+    uint4* stg = reinterpret_cast<uint4*>(tail + kBarBytes);
+    uint32_t* shist = reinterpret_cast<uint32_t*>(tail + kBarBytes + kStgBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nbins = kHist ? hist_bins : 0;
-    const uint32_t rank = cluster_ctarank();
+    const uint32_t rank = kPair ? cluster_ctarank() : 0u;
     const bool leader = rank == 0;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages2; ++s) {
+        for (int s = 0; s < nst; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], 2 * kEpiWarps);
+            mbar_init(&tempty[b], (kPair ? 2 : 1) * kEpiWarps);
         }
+        mbar_init(tover, (kPair ? 2 : 1) * 4);
         mbar_init(hsync, kEpiWarps);
         fence_mbar_init();
     }
     if (kHist)
         for (int b = threadIdx.x; b < nbins; b += blockDim.x) shist[b] = 0u;
-    if (warp == 0) tmem_alloc_pair(tmem_slot, kTmemCols);
+    if (warp == 0) {
+        if (kPair) tmem_alloc_pair(tmem_slot, kTmemCols);
+        else tmem_alloc(tmem_slot, kTmemCols);
+    }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();   // both CTAs' barriers and tensor memory are ready
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (warp >= 4 && warp < 8) {   // warps 4..7: TMEM lane quarters 0..3; every block scale is 1.0 (E8M0 127)
+        tmem_st16(tmem + kScaleCol + (static_cast<uint32_t>((warp & 3) * 32) << 16), 0x7F7F7F7Fu);
+        tmem_st_wait();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (kPair) cluster_sync_all();   // both CTAs' barriers and tensor memory are ready
+    tc_fence_after();
     bool ok = true;
-    const int u0 = static_cast<int>(blockIdx.x >> 1);
-    const int us = static_cast<int>(gridDim.x >> 1);
-    const int nu = total >> 1;
-    const uint32_t full_l = mapa_shared(&full[0], 0);      // leader's barriers, cluster addresses
-    const uint32_t tempty_l = mapa_shared(&tempty[0], 0);
+    // worker (cluster or CTA) c of C; a pair takes whole blocks, a CTA halves of them
+    const int c = static_cast<int>(kPair ? blockIdx.x >> 1 : blockIdx.x);
+    const int C = static_cast<int>(kPair ? gridDim.x >> 1 : gridDim.x);
+    const int nu = kPair ? total >> 1 : total;
+    const uint32_t full_l = kPair ? mapa_shared(&full[0], 0) : 0u;      // leader's barriers, cluster addresses
+    const uint32_t tempty_l = kPair ? mapa_shared(&tempty[0], 0) : smem_u32(&tempty[0]);
+    const uint32_t tover_l = kPair ? mapa_shared(tover, 0) : smem_u32(tover);
+    // block u of the launch -> problem, column blocks and this CTA's row / column offsets
+    auto place = [&](int u, int& p, int& nk, int& row0, int& colb) {
+        int lt;
+        p = locate(bt, ST_GEMM, kPair ? 2 * u : u, lt);
+        const int nb = bt.views[p].n_pad / kSc2BN;
+        int bm, bn;
+        block_of(lt >> 1, nb, bm, bn);
+        nk = nb;   // K stages of 256 columns
+        row0 = bm * kSc2BN + (kPair ? static_cast<int>(rank) : lt & 1) * kSc2BM;
+        colb = bn * kSc2BN;
+    };
+    // the set-up above (barriers, tensor memory, shared histogram) overlaps the
+    // previous stage; its outputs are read only from here on
     pdl_wait();
     pdl_release();
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---------------- TMA producer (both CTAs) ----------------
-            int it = 0;
-            for (int u = u0; u < nu && ok; u += us) {
-                const int t = 2 * u + static_cast<int>(rank);
-                int lt;
-                const int p = locate(bt, ST_GEMM, t, lt);
-                const int KT = bt.views[p].n_pad / kSc2BK;
-                const CUtensorMap* mA = bt.maps + 2 * p;   // 128-row boxes
-                int bm, bn;
-                tile_of(lt, bm, bn);
-                for (int kb = 0; kb < KT; ++kb, ++it) {
-                    const int s = it % kStages2;
-                    const uint32_t ph = (it / kStages2) & 1u;
+            // ---------------- TMA producer ----------------
+            int s = 0;
+            uint32_t ph = 0u;
+            for (int k = 0; ok; ++k) {
+                const int u = block_index(k, c, C, chunk);
+                if (u >= nu) break;
+                int p, nk, row0, colb;
+                place(u, p, nk, row0, colb);
+                const CUtensorMap* mA = bt.maps + 2 * p;   // 128-row boxes; + 1: 256-row boxes
+                for (int kb = 0; kb < nk; ++kb) {
                     if (!mbar_wait(&empty[s], ph ^ 1u)) { ok = false; break; }
-                    if (leader) mbar_arrive_expect_tx(&full[s], 4 * kABytes);   // both CTAs' A and B halves
-                    const uint32_t bar = full_l + static_cast<uint32_t>(s * sizeof(uint64_t));
-                    tma_load_2d_pair(sA + s * kABytes, mA, kb * kSc2BK, bm * kSc2BM, bar);
-                    tma_load_2d_pair(sB + s * kABytes, mA, kb * kSc2BK, bn * kSc2BN + static_cast<int>(rank) * kSc2BM, bar);
+                    if (kPair) {
+                        if (leader) mbar_arrive_expect_tx(&full[s], 4 * kHalf);   // both CTAs' A and B halves
+                        const uint32_t bar = full_l + static_cast<uint32_t>(s * sizeof(uint64_t));
+                        tma_load_2d_pair(sA + s * kHalf, mA, kb * kSc2BK, row0, bar);
+                        tma_load_2d_pair(sB + s * kHalf, mA, kb * kSc2BK, colb + static_cast<int>(rank) * kSc2BM, bar);
+                    } else {
+                        mbar_arrive_expect_tx(&full[s], 3 * kHalf);
+                        tma_load_2d(sA + s * kHalf, mA, kb * kSc2BK, row0, &full[s]);
+                        tma_load_2d(sB + s * kBPart, mA + 1, kb * kSc2BK, colb, &full[s]);
+                    }
+                    if (++s == nst) { s = 0; ph ^= 1u; }
                 }
             }
-            // tail: the leader's last releases of every stage have arrived here
-            for (int q = 0; q < kStages2; ++q, ++it) {
-                const int s = it % kStages2;
-                const uint32_t ph = (it / kStages2) & 1u;
+            // tail: the last releases of every stage have arrived here
+            for (int q = 0; kPair && q < nst; ++q) {
                 if (!mbar_wait(&empty[s], ph ^ 1u)) { ok = false; break; }
+                if (++s == nst) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0 && leader) {
-            // ---------------- pair MMA issuer (leader) ----------------
-            constexpr uint32_t kIdesc2 = idesc_f32acc(0u, 0u, 2 * kSc2BM, kSc2BN);   // M = 256, N = 256
-            int it = 0, tc = 0;
-            for (int u = u0; u < nu && ok; u += us, ++tc) {
-                const int t = 2 * u;
-                int lt;
-                const int p = locate(bt, ST_GEMM, t, lt);
-                const int KT = bt.views[p].n_pad / kSc2BK;
-                const int buf = tc & 1;
-                const uint32_t use = static_cast<uint32_t>(tc >> 1);
-                if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u)) { ok = false; break; }
+            // ---------------- MMA issuer (a pair's leader) ----------------
+            constexpr uint32_t kIdesc = idesc_mxf4(kPair ? 2 * kSc2BM : kSc2BM, kSc2BN);
+            const uint32_t sfa = tmem + kScaleCol, sfb = tmem + kScaleCol + 4;
+            int s = 0;
+            uint32_t ph = 0u;
+            for (int k = 0; ok; ++k) {
+                const int u = block_index(k, c, C, chunk);
+                if (u >= nu) break;
+                int p, nk, row0, colb;
+                place(u, p, nk, row0, colb);
+                const int buf = k & 1;
+                const uint32_t use = static_cast<uint32_t>(k >> 1);
+                // this accumulator drained, and the previous one's shared columns read
+                if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u) ||
+                    (k > 0 && !mbar_wait(tover, static_cast<uint32_t>(k - 1) & 1u))) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t d = tmem + static_cast<uint32_t>(buf * kSc2BN);
-                for (int kb = 0; kb < KT; ++kb, ++it) {
-                    const int s = it % kStages2;
-                    const uint32_t ph = (it / kStages2) & 1u;
+                const uint32_t d = tmem + (buf ? kAcc1 : 0u);
+                for (int kb = 0; kb < nk; ++kb) {
                     if (!mbar_wait(&full[s], ph)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a0 = smem_u32(sA + s * kABytes);
-                    const uint32_t b0 = smem_u32(sB + s * kABytes);
+                    const uint32_t a0 = smem_u32(sA + s * kHalf);
+                    const uint32_t b0 = smem_u32(sB + s * kBPart);
 #pragma unroll
-                    for (int k = 0; k < kSc2BK / 32; ++k)
-                        mma_f8f6f4_pair(d, sdesc_k_sw128(a0 + k * 32), sdesc_k_sw128(b0 + k * 32), kIdesc2,
-                                        (kb | k) != 0 ? 1u : 0u);
-                    mma_commit_pair_mc(&empty[s], 0x3);
+                    for (int q = 0; q < kSc2BK / 32; ++q)   // K = 64 FP4 (32 bytes) per MMA
+                        mma_mxf4<kPair>(d, sdesc_k_sw128(a0 + q * 32), sdesc_k_sw128(b0 + q * 32), kIdesc, sfa, sfb,
+                                        (kb | q) != 0 ? 1u : 0u);
+                    if (kPair) mma_commit_pair_mc(&empty[s], 0x3);
+                    else mma_commit(&empty[s]);
+                    if (++s == nst) { s = 0; ph ^= 1u; }
                 }
                 if (!ok) break;
-                mma_commit_pair_mc(&tfull[buf], 0x3);
+                if (kPair) mma_commit_pair_mc(&tfull[buf], 0x3);
+                else mma_commit(&tfull[buf]);
             }
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue warps (both CTAs) ----------------
-        const int quarter = warp & 3;
-        const int part = (warp - 2) >> 2;
-        int tc = 0;
-        for (int u = u0; u < nu; u += us, ++tc) {
-            const int t = 2 * u + static_cast<int>(rank);
-            int lt;
-            const int p = locate(bt, ST_GEMM, t, lt);
+        // ---------------- epilogue warps ----------------
+        const int quarter = warp & 3;              // TMEM lanes this warp may access
+        const int part = (warp - 2) >> 2;          // column part of the block
+        const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
+        for (int k = 0;; ++k) {
+            const int u = block_index(k, c, C, chunk);
+            if (u >= nu) break;
+            int p, nk, row0, colb;
+            place(u, p, nk, row0, colb);
             const ProbView v = bt.views[p];
-            int bm, bn;
-            tile_of(lt, bm, bn);
-            const int buf = tc & 1;
-            const uint32_t use = static_cast<uint32_t>(tc >> 1);
-            const uint2 words = epi_words(v, bm, bn, quarter, part, lane);
-            // a batch: whether this CTA's next block belongs to another problem
+            const int buf = k & 1;
+            const uint32_t use = static_cast<uint32_t>(k >> 1);
+            const int r0 = row0 + quarter * 32, cw = colb + part * kEpiCols;
+            const uint2 words = epi_words(v, r0 + lane, cw);
+            // a batch: whether this worker's next block belongs to another problem
             bool flush_after = false;
-            if (kHist && u + us < nu) {
+            const int un = block_index(k + 1, c, C, chunk);
+            if (kHist && un < nu) {
                 int ltn;
-                flush_after = locate(bt, ST_GEMM, 2 * (u + us) + static_cast<int>(rank), ltn) != p;
+                flush_after = locate(bt, ST_GEMM, kPair ? 2 * un : un, ltn) != p;
             }
             const bool got = mbar_wait(&tfull[buf], use & 1u);
             if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
             tc_fence_after();
-            sc2_epilogue_tile_staged<kHist>(v, tmem + static_cast<uint32_t>(buf * kSc2BN), bm, bn, quarter, part,
-                                            lane, words, shist, stg + (warp - 2) * 128);
+            // the shared columns: the last 16 of accumulator 0, the first 16 of accumulator 1
+            const bool owner = buf == 0 ? part == 3 : part == 0;
+            sc2_epilogue<kPair, kHist>(v, tmem + (buf ? kAcc1 : 0u) + static_cast<uint32_t>(part * kEpiCols) + lane_off, r0, cw,
+                                lane, words, shist, stg + (warp - 2) * 128, buf == 0 && part == 3 ? 1 : 0,
+                                owner ? tover_l : 0u);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(tempty_l + static_cast<uint32_t>(buf * sizeof(uint64_t)));
+            if (lane == 0) arrive_at<kPair>(tempty_l + static_cast<uint32_t>(buf * sizeof(uint64_t)));
             if (flush_after) {
                 // the epilogue warps add this problem's bins to its global
                 // histogram and clear them (a rendezvous before and after)
-                const ProbView* vf = bt.views + p;
-                const int nf = vf->n;
-                uint32_t* hf = vf->hist;
+                const int nf = v.n;
                 if (lane == 0) mbar_arrive(hsync);
                 if (!__all_sync(0xffffffffu, mbar_wait(hsync, 0u))) { ok = false; break; }
                 for (int b = (warp - 2) * 32 + lane + 1; b <= nf; b += 32 * kEpiWarps) {
                     const uint32_t h = shist[b];
                     if (h) {
-                        atomicAdd(hf + b, h);
+                        atomicAdd(v.hist + b, h);
                         shist[b] = 0u;
                     }
                 }
@@ -564,14 +465,17 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_pair_mma_kernel(Batch bt, int
     if (!ok && lane == 0) atomicOr(&bt.views[0].ctl->err, TR_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
-    // the problem of this cluster's last block (both CTAs of a cluster take the
+    // the problem of this worker's last block (both CTAs of a cluster take the
     // same blocks): its bins are still in shared memory
     int p_last = -1;
-    if (u0 < nu) {
+    if (c * chunk < nu) {
+        const int nc = (nu + chunk - 1) / chunk;
+        const int lc = c + (nc - 1 - c) / C * C;
+        const int ul = min(nu, (lc + 1) * chunk) - 1;
         int lt;
-        p_last = locate(bt, ST_GEMM, 2 * (u0 + ((nu - 1 - u0) / us) * us), lt);
+        p_last = locate(bt, ST_GEMM, kPair ? 2 * ul : ul, lt);
     }
-    if (kHist && !leader && p_last >= 0) {
+    if (kPair && kHist && !leader && p_last >= 0) {
         // the peer's histogram into the leader's (distributed shared memory), so
         // that one CTA per cluster adds to the global bins
         const uint32_t lead_hist = mapa_shared(shist, 0);
@@ -580,14 +484,15 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_pair_mma_kernel(Batch bt, int
             if (h) red_add_cluster(lead_hist + 4u * static_cast<uint32_t>(b), h);
         }
     }
-    cluster_sync_all();   // neither CTA exits or frees tensor memory while the other may still use it;
-                          // orders the peer's additions before the leader's flush
+    if (kPair) cluster_sync_all();   // neither CTA exits or frees tensor memory while the other may still use it;
+                                     // orders the peer's additions before the leader's flush
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem, kTmemCols);
+        if (kPair) tmem_dealloc_pair(tmem, kTmemCols);
+        else tmem_dealloc(tmem, kTmemCols);
     }
     if (!kHist || !leader || p_last < 0) return;
-    // the cluster's histogram into the global one, from which the count pass
+    // the worker's histogram into the global one, from which the count pass
     // (one problem) or the select launch (a batch) chooses the pivot threshold
     const ProbView vl = bt.views[p_last];
     for (int b = threadIdx.x + 1; b <= vl.n; b += blockDim.x)
@@ -597,28 +502,59 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_pair_mma_kernel(Batch bt, int
 int g_sc2_sms = 0;
 int g_sc2_pair_clusters = 0;   // co-resident 2-CTA clusters of the pair kernels (0: use single CTAs)
 
-// kHist: the blocks keep the edge-weight histogram in shared memory
-// (hist_bins bins)
-template <bool kHist>
-cudaError_t launch_pair(const Batch& b, int total_tiles, size_t smem, int hist_bins, cudaStream_t s, int auto_mode)
+template <bool kPair>
+size_t smem_bytes(int nst, int bins)
 {
-    int grid = 2 * g_sc2_pair_clusters;
-    if (grid > total_tiles) grid = total_tiles;   // total_tiles is even
+    return static_cast<size_t>(nst) * stage_bytes<kPair>() + kBarBytes + kStgBytes + 1024 + static_cast<size_t>(bins) * 4;
+}
+
+// Ring stages beside `bins` histogram bins (at most kMaxStages; 0: fewer than two fit).
+template <bool kPair>
+int stages_for(int bins)
+{
+    int nst = kMaxStages;
+    while (nst > 1 && smem_bytes<kPair>(nst, bins) > static_cast<size_t>(kSmemMax)) --nst;
+    return nst > 1 ? nst : 0;
+}
+
+// Blocks a worker takes in a row: one for a single problem; in a batch up to
+// four, while that leaves every worker at least 16 chunks.
+int chunk_for(const Batch& b, int units, int workers)
+{
+    if (b.num == 1) return 1;
+    const int l = units / (workers * 16);
+    return l < 1 ? 1 : l > 4 ? 4 : l;
+}
+
+template <bool kPair, bool kHist>
+cudaError_t launch_mma(const Batch& b, int total_tiles, int bins, cudaStream_t s, int auto_mode)
+{
+    const int nst = stages_for<kPair>(bins);
+    const int units = kPair ? total_tiles / 2 : total_tiles;
+    int workers = kPair ? g_sc2_pair_clusters : device_sms();
+    const int chunk = chunk_for(b, units, workers);
+    if (workers > units) workers = units;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.gridDim = dim3(static_cast<unsigned>(kPair ? 2 * workers : workers));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = smem_bytes<kPair>(nst, bins);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, sc2_pair_mma_kernel<kHist>, b, total_tiles, hist_bins, auto_mode);
+    cfg.numAttrs = kPair ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, sc2_mma_kernel<kPair, kHist>, b, total_tiles, bins, nst, chunk, auto_mode);
+}
+
+template <bool kPair, bool kHist>
+cudaError_t mma_attr()
+{
+    return cudaFuncSetAttribute(sc2_mma_kernel<kPair, kHist>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
 }
 
 }  // namespace
@@ -632,16 +568,9 @@ cudaError_t sc2_tcgen05_setup()
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sc2_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sc2_tcgen05_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemMax);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sc2_tcgen05_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kPipeBytes + kBarBytes + 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sc2_pair_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sc2_pair_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBase2);
+    if (e == cudaSuccess) e = mma_attr<true, true>();
+    if (e == cudaSuccess) e = mma_attr<false, true>();
+    if (e == cudaSuccess) e = mma_attr<false, false>();
     if (e == cudaSuccess) {
         // how many 2-CTA clusters fit at once with the largest shared-memory request
         cudaLaunchConfig_t cfg = {};
@@ -656,7 +585,7 @@ cudaError_t sc2_tcgen05_setup()
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, sc2_pair_mma_kernel<true>, &cfg) == cudaSuccess)
+        if (cudaOccupancyMaxActiveClusters(&nc, sc2_mma_kernel<true, true>, &cfg) == cudaSuccess)
             g_sc2_pair_clusters = nc;
         else
             cudaGetLastError();   // no cluster support: the single-CTA kernel is used
@@ -664,28 +593,23 @@ cudaError_t sc2_tcgen05_setup()
     return e;
 }
 
-// A single problem keeps its histogram in shared memory when it fits; a
-// batch (or a very large problem) uses global atomics.
+// The bins of any problem the library takes fit beside two stages of the pair
+// form (131 KB at N = 32768); the single-CTA form's larger stages leave room
+// for N up to about 24 800, above which its edges add to the global bins.
 bool launch_sc2_tcgen05(const Batch& b, int total_tiles, int max_n, bool pair_mma, cudaStream_t s, bool auto_mode)
 {
-    const bool pair = pair_mma && g_sc2_pair_clusters > 0;
-    const int sms = g_sc2_sms > 0 ? g_sc2_sms : 148;
-    const int grid = total_tiles < sms ? total_tiles : sms;
-    const size_t base = pair ? static_cast<size_t>(kBase2) : static_cast<size_t>(kPipeBytes + kBarBytes + 1024);
-    const size_t hist = static_cast<size_t>(max_n + 1) * 4;
-    const bool fits = base + hist <= static_cast<size_t>(kSmemMax);
-    const bool single = b.num == 1 && fits;
-    if (pair) {
-        if (fits)
-            launch_pair<true>(b, total_tiles, base + hist, max_n + 1, s, auto_mode ? 1 : 0);
-        else
-            launch_pair<false>(b, total_tiles, base, 0, s, auto_mode ? 1 : 0);
-    } else if (single) {
-        launch_pdl(sc2_tcgen05_kernel<true>, grid, kThreads, base + hist, s, b, total_tiles);
+    const int bins = max_n + 1;
+    if (pair_mma && g_sc2_pair_clusters > 0) {
+        static_assert(2 * stage_bytes<true>() + kBarBytes + kStgBytes + 1024 + (TURBOREG_MAX_N + 1) * 4 <= kSmemMax,
+                      "the largest histogram fits beside two stages");
+        launch_mma<true, true>(b, total_tiles, bins, s, auto_mode ? 1 : 0);
+    } else if (stages_for<false>(bins) > 0) {
+        launch_mma<false, true>(b, total_tiles, bins, s, 0);
     } else {
-        launch_pdl(sc2_tcgen05_kernel<false>, grid, kThreads, base, s, b, total_tiles);
+        launch_mma<false, false>(b, total_tiles, 0, s, 0);
+        return false;
     }
-    return single;
+    return b.num == 1;
 }
 
 

@@ -248,7 +248,7 @@ __device__ __forceinline__ uint32_t and_popc(const uint4 (&a)[NQ], const uint4 (
 // between (fewer units per CTA for smaller N), and always the faster one up
 // to n_pad = 2048; the tensor-core GEMM: 12.5 + waves x K-stages x 0.368 (its
 // 2-CTA clusters over the 256 x 256 upper-triangle tiles, 0.368 us per
-// 128-deep stage) plus 4 (n_pad / 5120)^2 for the FP8 matrix it then needs.
+// 128-deep stage) plus 4 (n_pad / 5120)^2 for the FP4 matrix it then needs.
 __device__ __forceinline__ bool sc2_bitset_faster(int n_pad, unsigned long long deg_sum, int clusters)
 {
     if (n_pad <= 2048) return true;
@@ -263,18 +263,9 @@ __device__ __forceinline__ bool sc2_bitset_faster(int n_pad, unsigned long long 
     return t_bitset <= t_gemm;
 }
 
-// 4 adjacency bits -> 4 bytes of FP8 E4M3 (0x38 = 1.0 for a set bit, 0 otherwise)
-__device__ __forceinline__ uint32_t nib_fp8(uint32_t nib) { return ((nib * 0x00204081u) & 0x01010101u) * 0x38u; }
-
-__device__ __forceinline__ uint4 half_word_fp8(uint32_t b16)
-{
-    return make_uint4(nib_fp8(b16 & 0xFu), nib_fp8((b16 >> 4) & 0xFu), nib_fp8((b16 >> 8) & 0xFu),
-                      nib_fp8((b16 >> 12) & 0xFu));
-}
-
 // auto_clusters > 0: one problem whose SC^2 path is chosen here (the GEMM's
 // co-resident 2-CTA clusters); if the GEMM is the faster path, the CTAs expand
-// the bitset into its FP8 operand and leave the rest to it.
+// the bitset into its FP4 operand and leave the rest to it.
 template <int NQ, bool kExact, bool kCsa>
 __global__ void __launch_bounds__(kLThreads, 1)
     sc2_bitset_lane_kernel(Batch bt, int total, int ldb_max, int hist_bins, int auto_clusters)
@@ -369,15 +360,12 @@ __global__ void __launch_bounds__(kLThreads, 1)
                 if (early_cols) landed &= mbar_wait(&cols_full[half], 0u);
                 if (!landed) atomicOr(&v0.ctl->err, TR_ERR_TIMEOUT);
             }
-            // the GEMM's FP8 operand from the bitset: word q of the matrix -> 32 bytes
+            // the GEMM's FP4 operand from the bitset: word q of the matrix -> 16 bytes
             const size_t words = static_cast<size_t>(v0.n_pad) * v0.ldb;
             for (size_t q = static_cast<size_t>(blockIdx.x) * kLThreads + tid; q < words;
                  q += static_cast<size_t>(gridDim.x) * kLThreads) {
-                const uint32_t w = __ldcg(v0.bits + q);
-                const size_t row = q / static_cast<size_t>(v0.ldb), col = (q % static_cast<size_t>(v0.ldb)) * 32;
-                uint4* dst = reinterpret_cast<uint4*>(v0.a8_auto + row * v0.n_pad + col);
-                dst[0] = half_word_fp8(w & 0xFFFFu);
-                dst[1] = half_word_fp8(w >> 16);
+                // (rows of both are contiguous, so word q of the bitset is 16 bytes at 16 q)
+                reinterpret_cast<uint4*>(v0.a4_auto)[q] = word_fp4(__ldcg(v0.bits + q));
             }
             return;
         }

@@ -60,6 +60,21 @@ __device__ __forceinline__ uint64_t globaltimer()
     return t;
 }
 
+// 8 adjacency bits -> 8 packed FP4 (E2M1) values, 0x2 = 1.0 for a set bit: the
+// bits are spread to the low bits of the nibbles, then moved up by one.
+__device__ __forceinline__ uint32_t byte_fp4(uint32_t b)
+{
+    b = (b | (b << 12)) & 0x000F000Fu;
+    b = (b | (b << 6)) & 0x03030303u;
+    return ((b << 1) | (b << 4)) & 0x22222222u;
+}
+
+// 32 adjacency bits -> 16 bytes of packed FP4 values
+__device__ __forceinline__ uint4 word_fp4(uint32_t w)
+{
+    return make_uint4(byte_fp4(w & 0xFFu), byte_fp4((w >> 8) & 0xFFu), byte_fp4((w >> 16) & 0xFFu), byte_fp4(w >> 24));
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier
 // ---------------------------------------------------------------------------
@@ -82,6 +97,12 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// The same on a barrier given by its address in this CTA's shared window.
+__device__ __forceinline__ void mbar_arrive_addr(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
@@ -312,24 +333,12 @@ __device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr)
     return d;
 }
 
-// Instruction descriptor (kind::f16 / kind::f8f6f4 layout): D format [4,6)
+// Instruction descriptor (kind::f16 layout): D format [4,6)
 // (1 = F32), A format [7,10), B format [10,13), A/B major bits 15/16 (0 = K),
 // N >> 3 at [17,23), M >> 4 at [24,29).
 __host__ __device__ constexpr uint32_t idesc_f32acc(uint32_t afmt, uint32_t bfmt, uint32_t M, uint32_t N)
 {
     return (1u << 4) | (afmt << 7) | (bfmt << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
-}
-
-// D[tmem] (+)= A[smem] * B[smem]^T, FP8/FP6/FP4 operands, one CTA.
-__device__ __forceinline__ void mma_f8f6f4(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                           uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // D[tmem] (+)= A * B^T with 16-bit (f16 / bf16) operands, one CTA.
@@ -344,19 +353,40 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
         : "memory");
 }
 
-// D[tmem] (+)= A * B^T over a CTA pair (cta_group::2): issued by one thread of
-// the leader CTA; A's M = 256 rows are this CTA's 128 and the peer's 128 at the
-// same shared-memory offset, B's N columns likewise, and each CTA's tensor
-// memory holds its 128 rows of D.
-__device__ __forceinline__ void mma_f8f6f4_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                uint32_t accumulate)
+// Instruction descriptor of kind::mxf4: A format [7,10) and B format [10,12)
+// (1 = E2M1), N >> 3 at [17,23), scale format bit 23 (1 = E8M0), M >> 4 at
+// [24,29); scale-factor ids 0, K = 64 (bit 31 clear).
+__host__ __device__ constexpr uint32_t idesc_mxf4(uint32_t M, uint32_t N)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    return (1u << 7) | (1u << 10) | ((N >> 3) << 17) | (1u << 23) | ((M >> 4) << 24);
+}
+
+// D[tmem] (+)= A[smem] * B[smem]^T with packed FP4 (E2M1) operands, K = 64,
+// one E8M0 scale per 32 elements of K at tensor-memory columns sfa (A) and
+// sfb (B).  kPair: over a CTA pair (cta_group::2), issued by one thread of
+// the leader CTA; A's M = 256 rows are this CTA's 128 and the peer's 128 at
+// the same shared-memory offset, B's N columns likewise, and each CTA's
+// tensor memory holds its 128 rows of D (and its own copy of the scales).
+template <bool kPair>
+__device__ __forceinline__ void mma_mxf4(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t sfa,
+                                         uint32_t sfb, uint32_t accumulate)
+{
+    if constexpr (kPair)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(
+                tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(
+                tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb)
+            : "memory");
 }
 
 // Arrive on the mbarrier at `bar`'s offset in every CTA of `mask` when all
@@ -393,6 +423,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
         : "r"(taddr)
         : "memory");
 }
+
+// Store `x` to 16 consecutive 32-bit TMEM columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, uint32_t x)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(
+            taddr),
+        "r"(x)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 

@@ -17,7 +17,7 @@ struct Ctl;
 struct ProbView {
     int64_t in_off;      // first match of this problem in the (concatenated) input arrays
     int32_t n;           // correspondences
-    int32_t n_pad;       // n rounded up to 256 (GEMM tile multiple); leading dimension of a8 and w
+    int32_t n_pad;       // n rounded up to 256 (GEMM tile multiple); leading dimension of w, in elements of a4
     int32_t ldb;         // words per bitset row = n_pad / 32
     int32_t k1, k2;      // Eq. 4 / Eq. 7
     float tau;           // Eq. 1 threshold
@@ -27,13 +27,13 @@ struct ProbView {
     int32_t scoring;     // TURBOREG_SCORE_IN / _MAE / _MSE
     int32_t vppb;        // verification tile: matches per block (<= 4 x the kernel's points per warp)
     uint32_t dbg;        // failure injection for tests (TR_DBG_*), 0 in normal use
-    uint8_t* a8_auto;    // non-null: the SC^2 path is chosen on the device from the degrees (one
-                         // problem, n_pad <= 5120); a8 is then null, so the compatibility kernel
-                         // writes the bitset only, and the FP8 matrix is expanded into a8_auto
+    uint8_t* a4_auto;    // non-null: the SC^2 path is chosen on the device from the degrees (one
+                         // problem, n_pad <= 5120); a4 is then null, so the compatibility kernel
+                         // writes the bitset only, and the FP4 matrix is expanded into a4_auto
                          // if the tensor-core GEMM is chosen
     float* pts;          // [6][n_pad]
     float* pts8;         // [n_pad][8] = (x0, x1, x2, y0, y1, y2, 0, 0)
-    uint8_t* a8;         // [n_pad][n_pad] FP8 E4M3 0/1 adjacency
+    uint8_t* a4;         // [n_pad][n_pad / 2] packed FP4 (E2M1) 0/1 adjacency, element 2k in the low nibble
     uint32_t* bits;      // [n_pad][ldb] adjacency bitset
     uint16_t* w;         // [n_pad][n_pad] O2Graph weights (i < j only)
     int32_t* rowscore;   // [n_pad] SC^2 row sums
@@ -184,7 +184,7 @@ void launch_topk_single(const ProbView& v, cudaStream_t s);
 
 constexpr int kSc2BM = 128;   // GEMM tile rows  (TMEM lanes)
 constexpr int kSc2BN = 256;   // GEMM tile cols  (TMEM columns)
-constexpr int kSc2BK = 128;   // K bytes per pipeline stage (one 128-byte swizzle row)
+constexpr int kSc2BK = 128;   // K bytes per pipeline stage (one 128-byte swizzle row, 256 FP4 values)
 constexpr int kSc2AutoMaxNpad = 5120;   // the device-side choice of the SC^2 path: n_pad <= 5120
 constexpr int kSc2BitsetAlwaysNpad = 2048;   // ... below which the CUDA-core path is taken directly
 
