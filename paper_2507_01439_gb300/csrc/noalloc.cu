@@ -7,13 +7,13 @@
 // the device and take unbounded time.  turboreg_select_pivots_noalloc gives
 // them the pivot-selection stage with every scratch buffer it needs placed in
 // one fixed array in the library's own device memory (kScratchBytes, about
-// 225 KB, loaded with the module and held by every GPU that loads the library
+// 257 KB, loaded with the module and held by every GPU that loads the library
 // until the process exits).  The caller passes the weight matrix and the output buffers;
 // nothing is allocated or freed, by this code or by any library it calls.
 //
 // The scratch is shared by every call: the histogram and the control block
 // (which holds the active-row and slot counters) are cleared with
-// cudaMemsetAsync at the start of each call, and two calls whose work overlaps on the GPU (different streams, or
+// one cudaMemsetAsync at the start of each call, and two calls whose work overlaps on the GPU (different streams, or
 // different host threads) race on it.  Serialise calls per device.
 //
 // In host code the name g_pivot_scratch only stands in for the array; its
@@ -53,7 +53,8 @@ constexpr size_t kOffCtl = 0;
 constexpr size_t kOffHist = align256(sizeof(Ctl));
 constexpr size_t kOffActive = kOffHist + align256(sizeof(uint32_t) * (kMaxN + 1));
 constexpr size_t kOffCand = kOffActive + align256(sizeof(int4) * kMaxN);
-constexpr size_t kScratchBytes = kOffCand + align256(sizeof(uint64_t) * kMaxK1);
+constexpr size_t kOffRowmax = kOffCand + align256(sizeof(uint64_t) * kMaxK1);
+constexpr size_t kScratchBytes = kOffRowmax + align256(sizeof(int32_t) * kMaxN);
 
 static __device__ __align__(256) uint8_t g_pivot_scratch[kScratchBytes];
 
@@ -136,16 +137,15 @@ extern "C" int turboreg_select_pivots_noalloc(const uint16_t* w_dev, int32_t n, 
     v.hist = reinterpret_cast<uint32_t*>(scr + kOffHist);
     v.active = reinterpret_cast<int4*>(scr + kOffActive);
     v.cand = reinterpret_cast<uint64_t*>(scr + kOffCand);
+    v.rowmax = reinterpret_cast<int32_t*>(scr + kOffRowmax);   // rows with an edge: written by the histogram
     v.piv = reinterpret_cast<int4*>(pivots_dev);
 
-    // the previous call's contents stay in the array: clear what must start at zero
-    cudaError_t e = cudaMemsetAsync(scr + kOffCtl, 0, sizeof(Ctl), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(v.hist, 0, sizeof(uint32_t) * (n + 1), s);
+    // the previous call's contents stay in the array: clear what must start at
+    // zero (the control block and, behind it, the histogram)
+    cudaError_t e = cudaMemsetAsync(scr + kOffCtl, 0, kOffHist + sizeof(uint32_t) * (n + 1), s);
     if (e != cudaSuccess) return TURBOREG_ERR_CUDA;
-    launch_topk_single(v, s);
+    launch_topk_single(v, n_pivots_dev, s);
     e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(n_pivots_dev, &v.ctl->n_pivots, sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) {
         std::fprintf(stderr, "turboreg_select_pivots_noalloc: %s\n", cudaGetErrorString(e));
         return TURBOREG_ERR_CUDA;

@@ -7,12 +7,12 @@
 //
 // Exact radix-style selection; the selected set, and so the pivots, do not
 // depend on the order in which blocks run:
-//   hist    histogram of edge weights (built by the SC^2 GEMM epilogue, or
-//           by hist_kernel for the CUDA-core SC^2 path and for callers)
+//   hist    histogram of edge weights (built by the SC^2 pass; by hist_kernel
+//           for the learned weights and for a caller's matrix, there with the
+//           row maxima)
 //   select  alpha = K1-th largest weight, c_gt = #{W > alpha}, m = K1' - c_gt
 //           ties still needed (K1' = min(K1, |E+|)): every count block for
-//           one problem whose histogram the GEMM completed, else one block
-//           per problem of the select launch
+//           one problem, else one block per problem of the select launch
 //   count   blocks of eight row pairs (i, n-1-i): #{j : W_ij > alpha} and
 //           #{j : W_ij == alpha}; rows with such edges join the active list
 //           (rows whose largest weight, recorded by the SC^2 pass, is below
@@ -35,7 +35,6 @@ namespace tr {
 namespace {
 
 constexpr int kHistSmemMaxBins = 24576;   // 96 KB of shared bins; larger N uses global atomics
-constexpr int kHistRowsPerBlock = 64;     // 8 warps x 8 rows
 constexpr int kCountThreads = 256;
 constexpr int kCountPairs = 8;            // row pairs per count block
 
@@ -57,93 +56,6 @@ __device__ __forceinline__ float learned_row_bound(const ProbView& v, int i)
     return __fmul_rn(__fmul_rn(static_cast<float>(__ldcg(v.rowmax + i)), __ldcg(v.prob + i)), pmax);
 }
 
-// Iterate row i's upper-triangle entries j in (i, n) in chunks of 8 uint16
-// (16-byte loads); lane l takes chunks c0 + l, c0 + l + 32, ..., two loads in
-// flight per lane.  Chunks whose 8 weights are all zero are skipped.
-template <typename F>
-__device__ __forceinline__ void for_row_chunks(const ProbView& v, int i, int lane, F&& f)
-{
-    if (i + 1 >= v.n) return;
-    const uint16_t* wrow = v.w + (size_t)i * v.n_pad;
-    const int c0 = (i + 1) >> 3, c1 = (v.n - 1) >> 3;
-    for (int c = c0 + lane; c <= c1; c += 64) {
-        const int cb = c + 32;
-        const uint4 qa = *reinterpret_cast<const uint4*>(wrow + c * 8);
-        const uint4 qb = cb <= c1 ? *reinterpret_cast<const uint4*>(wrow + cb * 8) : make_uint4(0, 0, 0, 0);
-        const uint32_t u[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int j = (e < 8 ? c : cb) * 8 + (e & 7);
-            const int w = (u[e >> 1] >> ((e & 1) * 16)) & 0xFFFF;
-            if (u[e >> 1] == 0u) continue;
-            f(j, (j > i && j < v.n) ? pivot_weight(v, i, j, w) : 0);
-        }
-    }
-}
-
-// Histogram of edge weights (used when SC^2 comes from the CUDA-core path or
-// from a caller): 64 rows per block, shared-memory bins when they fit.  A
-// caller's weight above n - 2 (no SC^2 count can be larger; the bins end at
-// n) is not counted: it sets TR_ERR_BAD_WEIGHT, and the select kernel then
-// selects nothing.
-template <class VS, bool kSmem>
-__global__ void __launch_bounds__(256) hist_kernel(VS vs)
-{
-    int lb;
-    const ProbView v = vs.get(ST_HIST, blockIdx.x, lb);   // launch descriptors: before the wait
-    pdl_wait();
-    pdl_release();
-    extern __shared__ uint32_t sh[];
-    const int nb = v.n + 1;
-    if (kSmem) {
-        for (int q = threadIdx.x; q < nb; q += blockDim.x) sh[q] = 0;
-        __syncthreads();
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int r = 0; r < kHistRowsPerBlock / 8; ++r) {
-        const int i = lb * kHistRowsPerBlock + warp * (kHistRowsPerBlock / 8) + r;
-        if (i >= v.n) break;
-        // learned weights: a row whose bound is below 1 holds only zeros (not counted)
-        if (!(learned_row_bound(v, i) >= 1.f)) continue;
-        for_row_chunks(v, i, lane, [&](int, int w) {
-            if (VS::kCallerWeights && w > v.n - 2) {
-                atomicOr(&v.ctl->err, TR_ERR_BAD_WEIGHT);
-            } else if (w > 0) {
-                if (kSmem) atomicAdd(&sh[w], 1u);
-                else atomicAdd(&v.hist[w], 1u);
-            }
-        });
-    }
-    if (kSmem) {
-        __syncthreads();
-        for (int q = threadIdx.x; q < nb; q += blockDim.x)
-            if (sh[q]) atomicAdd(&v.hist[q], sh[q]);
-    }
-}
-
-template <class VS>
-__global__ void __launch_bounds__(1024) select_kernel(VS vs)
-{
-    int lb;
-    const ProbView v = vs.get(ST_SELECT, blockIdx.x, lb);   // launch descriptors: before the wait
-    pdl_wait();
-    pdl_release();
-    __shared__ int sbuf[33];
-    if (VS::kCallerWeights && (v.ctl->err & TR_ERR_BAD_WEIGHT) != 0u) {
-        // out-of-range weights: select nothing, so that the count, emit and
-        // rank passes write no candidate (rank reports the error)
-        if (threadIdx.x == 0) {
-            v.ctl->n_edges = 0;
-            v.ctl->n_sel = 0;
-            v.ctl->alpha = 0x7FFFFFFF;
-            v.ctl->c_gt = 0;
-            v.ctl->m_ties = 0;
-        }
-        return;
-    }
-    select_alpha(v, sbuf);
-}
-
 // Zero the weights of a 16-byte chunk (8 entries, columns 8c .. 8c+7) outside
 // the row's upper part (row, n): only a row's first and last chunks have any.
 __device__ __forceinline__ uint4 mask_chunk(uint4 q, int c, int row, int n)
@@ -157,6 +69,163 @@ __device__ __forceinline__ uint4 mask_chunk(uint4 q, int c, int row, int n)
     return make_uint4(wd[0], wd[1], wd[2], wd[3]);
 }
 
+// Eight row pairs (p, n-1-p) of a block, whose upper-triangle parts hold about
+// n/8 16-byte chunks per pair, so that every group has about the same span of
+// rows; entry k: pair 8 g + k / 2, side k % 2.
+struct RowGroup {
+    int row[16], c0[16], off[17];   // row, its first chunk, first chunk number in the group
+};
+
+// Row of entry t (< 16) of group g; false when the entry holds no edge.
+__device__ __forceinline__ bool group_row(int g, int t, int n, int& row)
+{
+    const int p = g * kCountPairs + (t >> 1);
+    row = (t & 1) ? n - 1 - p : p;
+    return t < 16 && p < (n + 1) / 2 && !((t & 1) && row == p) && row + 1 < n;
+}
+
+// The group's chunk numbering over its rows marked `act`, by one warp (lane t < 32).
+__device__ __forceinline__ void group_offsets(RowGroup& sg, int t, int row, bool act, int n)
+{
+    const int c0 = (row + 1) >> 3;
+    const int len = act ? ((n - 1) >> 3) - c0 + 1 : 0;
+    int incl = len;
+#pragma unroll
+    for (int off = 1; off < 16; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (t >= off) incl += y;
+    }
+    if (t < 16) {
+        sg.row[t] = row;
+        sg.c0[t] = c0;
+        sg.off[t] = incl - len;
+    }
+    if (t == 15) sg.off[16] = incl;
+}
+
+// The group's chunks spread over all the block's threads, eight 16-byte loads
+// in flight each: f(k, row, c, weights) for chunk c of entry k, entries outside
+// the upper part zeroed.
+template <typename F>
+__device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGroup& sg, F&& f)
+{
+    const int tot = sg.off[16];
+    for (int base = threadIdx.x; base < tot; base += 8 * kCountThreads) {
+        uint4 q[8];
+        int kk[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int x = base + u * kCountThreads;
+            int k = 0;
+#pragma unroll
+            for (int m = 1; m < 16; ++m) k += sg.off[m] <= x ? 1 : 0;
+            kk[u] = k;
+            q[u] = x < tot ? *reinterpret_cast<const uint4*>(v.w + (size_t)sg.row[k] * v.n_pad +
+                                                             (size_t)(sg.c0[k] + x - sg.off[k]) * 8)
+                           : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int x = base + u * kCountThreads;
+            if (x >= tot) break;
+            const int k = kk[u];
+            const int row = sg.row[k], c = sg.c0[k] + x - sg.off[k];
+            f(k, row, c, mask_chunk(q[u], c, row, v.n));
+        }
+    }
+}
+
+// Histogram of edge weights, for the learned weights and for a caller's
+// matrix: the count pass's groups of row pairs (all rows read, in one or a few
+// rounds of eight loads per thread), shared-memory bins when they fit.  It
+// reads the upper triangle once; bound by the instructions on the non-zero
+// words.  One warp per row with two loads in flight and 64 rows per block (79
+// blocks, a chain of 80 load rounds per warp) took 196 us at n = 5000; the
+// whole selection call went from 231 to 49 us, a learned batch of 32 problems
+// from 1075 to 951 us.
+// A caller's weight above n - 2 (no SC^2 count can be larger; the bins end at
+// n) is not counted: it sets TR_ERR_BAD_WEIGHT, and nothing is selected then;
+// a caller's row maxima are recorded, so that the count pass skips rows.
+template <class VS, bool kSmem>
+__global__ void __launch_bounds__(kCountThreads, 3) hist_kernel(VS vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_HIST, blockIdx.x, lb);   // launch descriptors: before the wait
+    extern __shared__ uint32_t sh[];
+    __shared__ RowGroup sg;
+    __shared__ uint32_t smax[16];
+    const int n = v.n, t = threadIdx.x;
+    if (kSmem)
+        for (int q = t; q <= n; q += kCountThreads) sh[q] = 0;
+    pdl_wait();
+    pdl_release();
+    const bool learned = v.prob != nullptr;
+    const int groups = count_blocks(n), stride = hist_blocks(n);
+    bool bad = false;
+    for (int g = lb; g < groups; g += stride) {
+        __syncthreads();   // the bins are cleared; the previous group's list is consumed
+        int row;
+        bool act = group_row(g, t, n, row);
+        if (t < 32) {
+            // learned weights: a row whose bound is below 1 holds only zeros (not counted)
+            if (act && learned) act = learned_row_bound(v, row) >= 1.f;
+            group_offsets(sg, t, row, act, n);
+            if (t < 16) smax[t] = 0u;
+        }
+        __syncthreads();
+        int kcur = -1;
+        uint32_t mx = 0u;   // running maximum of entry kcur's weights, two 16-bit halves
+        auto flush_max = [&]() {
+            const uint32_t m = max(mx & 0xFFFFu, mx >> 16);
+            if (m) atomicMax(&smax[kcur], m);
+        };
+        for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 q) {
+            const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+            if (VS::kCallerWeights) {
+                if (k != kcur) {
+                    if (kcur >= 0) flush_max();
+                    kcur = k;
+                    mx = 0u;
+                }
+                mx = __vmaxu2(mx, __vmaxu2(__vmaxu2(u[0], u[1]), __vmaxu2(u[2], u[3])));
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                if (u[e >> 1] == 0u) continue;
+                int w = static_cast<int>((u[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu);
+                if (!VS::kCallerWeights) w = pivot_weight(v, row_k, c * 8 + e, w);
+                if (VS::kCallerWeights && w > n - 2) {
+                    bad = true;
+                } else if (w > 0) {
+                    if (kSmem) atomicAdd(&sh[w], 1u);
+                    else atomicAdd(&v.hist[w], 1u);
+                }
+            }
+        });
+        if (VS::kCallerWeights) {
+            if (kcur >= 0) flush_max();
+            __syncthreads();
+            if (act && t < 16) v.rowmax[row] = static_cast<int>(smax[t]);
+        }
+    }
+    if (VS::kCallerWeights && bad) atomicOr(&v.ctl->err, TR_ERR_BAD_WEIGHT);
+    if (kSmem) {
+        __syncthreads();
+        for (int q = t; q <= n; q += kCountThreads)
+            if (sh[q]) atomicAdd(&v.hist[q], sh[q]);
+    }
+}
+
+__global__ void __launch_bounds__(1024) select_kernel(ManyViews vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_SELECT, blockIdx.x, lb);   // launch descriptors: before the wait
+    pdl_wait();
+    pdl_release();
+    __shared__ int sbuf[33];
+    select_alpha(v, sbuf);
+}
+
 // #{entries > alpha} and #{entries == alpha} of a chunk, as packed 16-bit
 // SIMD compares (weights and alpha < 2^16; a zeroed entry never counts, alpha >= 1).
 __device__ __forceinline__ void count_chunk(uint4 q, uint32_t a2, int& g, int& e)
@@ -168,19 +237,17 @@ __device__ __forceinline__ void count_chunk(uint4 q, uint32_t a2, int& g, int& e
 }
 
 // Per-row counts of the weight > alpha and weight == alpha edges.  A block
-// owns eight row pairs (w, n-1-w), whose upper-triangle parts hold about n/8
-// 16-byte chunks per pair, so every block has about the same span of rows.
-// Rows whose largest weight (recorded by the SC^2 pass) is below alpha hold
-// no such edge and are skipped without reading W (the learned pivot weight
-// floor(W p_i p_j) never exceeds W).  The chunks of the remaining rows are
-// spread over all the block's threads, eight 16-byte loads in flight each,
-// so a block with one or two such rows reads them in one round.  Rows
-// holding such edges are appended to the active list as (row, #gt, #eq), in
-// any order.
-// select_here (one problem whose histogram the SC^2 GEMM completed): every
-// block chooses the threshold itself from the histogram, staged in dynamic
-// shared memory while its row maxima load, and block 0 records it for the
-// later passes; otherwise it comes from the select launch.
+// owns a group of eight row pairs.  Rows whose largest weight (recorded by the
+// SC^2 pass or the histogram) is below alpha hold no such edge and are skipped
+// without reading W (the learned pivot weight floor(W p_i p_j) never exceeds
+// W).  The chunks of the remaining rows are spread over all the block's
+// threads, so a block with one or two such rows reads them in one round.
+// Rows holding such edges are appended to the active list as (row, #gt, #eq),
+// in any order.
+// select_here (one problem whose histogram is complete): every block chooses
+// the threshold itself from the histogram, staged in dynamic shared memory
+// while its row maxima load, and block 0 records it for the later passes;
+// otherwise it comes from the select launch.
 template <class VS>
 __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int select_here)
 {
@@ -189,27 +256,29 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     pdl_wait();
     pdl_release();
     extern __shared__ __align__(16) uint32_t shist_stage[];   // select_here: n + 4 words
-    __shared__ int srow[16], sc0[16], soff[17], sg[16], se[16];
+    __shared__ RowGroup sg;
+    __shared__ int sgt[16], seq[16];
     __shared__ int ssel[40];
     const int n = v.n;
     const int t = threadIdx.x;
-    // entry k = t (< 16): pair p = 8 lb + k / 2, side k % 2
-    const int p = lb * kCountPairs + (t >> 1);
-    const int row = (t & 1) ? n - 1 - p : p;
-    bool act = t < 16 && p < (n + 1) / 2 && !((t & 1) && row == p) && row + 1 < n;
+    int row;
+    bool act = group_row(lb, t, n, row);
     const int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
     int n_sel, alpha;
     if (select_here) {
+        const bool bad = VS::kCallerWeights && (__ldcg(&v.ctl->err) & TR_ERR_BAD_WEIGHT) != 0u;
         select_alpha(v, ssel, shist_stage, ssel + 33);
         __syncthreads();
-        n_sel = ssel[34];
-        alpha = ssel[35];
+        // out-of-range weights: nothing is selected, so that the emit and rank
+        // passes write no candidate (rank reports the error)
+        n_sel = bad ? 0 : ssel[34];
+        alpha = bad ? 0x7FFFFFFF : ssel[35];
         if (lb == 0 && t == 0) {
-            v.ctl->n_edges = ssel[33];
+            v.ctl->n_edges = bad ? 0 : ssel[33];
             v.ctl->n_sel = n_sel;
             v.ctl->alpha = alpha;
-            v.ctl->c_gt = ssel[36];
-            v.ctl->m_ties = ssel[37];
+            v.ctl->c_gt = bad ? 0 : ssel[36];
+            v.ctl->m_ties = bad ? 0 : ssel[37];
         }
     } else {
         n_sel = v.ctl->n_sel;
@@ -219,78 +288,40 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     if (t < 32) {
         if (act && v.rowmax != nullptr) act = rmax >= alpha;
         if (act && v.prob != nullptr) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
-        const int c0 = (row + 1) >> 3;
-        const int len = act ? ((n - 1) >> 3) - c0 + 1 : 0;
-        int incl = len;
-#pragma unroll
-        for (int off = 1; off < 16; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (t >= off) incl += y;
-        }
-        if (t < 16) {
-            srow[t] = row;
-            sc0[t] = c0;
-            soff[t] = incl - len;
-            sg[t] = 0;
-            se[t] = 0;
-        }
-        if (t == 15) soff[16] = incl;
+        group_offsets(sg, t, row, act, n);
+        if (t < 16) sgt[t] = seq[t] = 0;
     }
     __syncthreads();
-    const int tot = soff[16];
-    if (tot == 0) return;                     // uniform over the block
+    if (sg.off[16] == 0) return;              // uniform over the block
     const uint32_t a2 = static_cast<uint32_t>(alpha) * 0x10001u;
     const bool learned = v.prob != nullptr;
     int kcur = -1, g = 0, e = 0;              // running counts of entry kcur
-    for (int base = t; base < tot; base += 8 * kCountThreads) {
-        uint4 q[8];
-        int kk[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int x = base + u * kCountThreads;
-            int k = 0;
-#pragma unroll
-            for (int m = 1; m < 16; ++m) k += soff[m] <= x ? 1 : 0;
-            kk[u] = k;
-            q[u] = x < tot ? *reinterpret_cast<const uint4*>(v.w + (size_t)srow[k] * v.n_pad +
-                                                             (size_t)(sc0[k] + x - soff[k]) * 8)
-                           : make_uint4(0u, 0u, 0u, 0u);
+    auto flush = [&]() {
+        if (g) atomicAdd(&sgt[kcur], g);
+        if (e) atomicAdd(&seq[kcur], e);
+    };
+    for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 qm) {
+        if (k != kcur) {
+            if (kcur >= 0) flush();
+            kcur = k;
+            g = e = 0;
         }
+        if (!learned) {
+            count_chunk(qm, a2, g, e);
+        } else if ((qm.x | qm.y | qm.z | qm.w) != 0u) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int x = base + u * kCountThreads;
-            if (x >= tot) break;
-            const int k = kk[u];
-            const int row = srow[k], c = sc0[k] + x - soff[k];
-            if (k != kcur) {
-                if (kcur >= 0) {
-                    if (g) atomicAdd(&sg[kcur], g);
-                    if (e) atomicAdd(&se[kcur], e);
-                }
-                kcur = k;
-                g = e = 0;
-            }
-            const uint4 qm = mask_chunk(q[u], c, row, n);
-            if (!learned) {
-                count_chunk(qm, a2, g, e);
-            } else if ((qm.x | qm.y | qm.z | qm.w) != 0u) {
-#pragma unroll
-                for (int el = 0; el < 8; ++el) {
-                    const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
-                    const int pw = pivot_weight(v, row, c * 8 + el, static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu));
-                    g += pw > alpha;
-                    e += pw == alpha;
-                }
+            for (int el = 0; el < 8; ++el) {
+                const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
+                const int pw = pivot_weight(v, row_k, c * 8 + el, static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu));
+                g += pw > alpha;
+                e += pw == alpha;
             }
         }
-    }
-    if (kcur >= 0) {
-        if (g) atomicAdd(&sg[kcur], g);
-        if (e) atomicAdd(&se[kcur], e);
-    }
+    });
+    if (kcur >= 0) flush();
     __syncthreads();
-    if (t < 16 && (sg[t] | se[t]))
-        v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(srow[t], sg[t], se[t], 0);
+    if (t < 16 && (sgt[t] | seq[t]))
+        v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
 }
 
 // Blocks take the active rows in any order.  W > alpha edges take slots
@@ -417,11 +448,10 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
 
 // 32 candidates per block (one per lane); the 8 warps split the comparison
 // range; all n_sel keys of the problem are staged in shared memory.
-template <class VS>
-__global__ void __launch_bounds__(256) rank_kernel(VS vs)
+__global__ void __launch_bounds__(256) rank_kernel(OneView vs, int32_t* n_out)
 {
     int lb;
-    const ProbView v = vs.get(ST_RANK, blockIdx.x, lb);   // launch descriptors: before the wait
+    const ProbView v = vs.get(ST_RANK, blockIdx.x, lb);
     pdl_wait();
     pdl_release();
     extern __shared__ uint64_t sk[];
@@ -429,8 +459,7 @@ __global__ void __launch_bounds__(256) rank_kernel(VS vs)
     const int n_sel = v.ctl->n_sel;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lb == 0 && threadIdx.x == 0)
-        v.ctl->n_pivots = (VS::kCallerWeights && (v.ctl->err & TR_ERR_BAD_WEIGHT) != 0u) ? -TURBOREG_ERR_INVALID_ARG
-                                                                                         : n_sel;
+        *n_out = (v.ctl->err & TR_ERR_BAD_WEIGHT) != 0u ? -TURBOREG_ERR_INVALID_ARG : n_sel;
     if (lb * 32 >= n_sel) return;
     for (int q = threadIdx.x; q < n_sel; q += blockDim.x) sk[q] = v.cand[q];
     __syncthreads();
@@ -457,22 +486,12 @@ __global__ void __launch_bounds__(256) rank_kernel(VS vs)
 int g_num_sms = 0;
 
 template <class VS>
-cudaError_t set_attrs()
-{
-    cudaError_t e = cudaFuncSetAttribute(rank_kernel<VS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TURBOREG_K1_MAX * 8);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(hist_kernel<VS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kHistSmemMaxBins * 4);
-}
-
-template <class VS>
 void launch_hist_vs(const VS& vs, int total, int max_n, cudaStream_t s)
 {
     if (max_n + 1 <= kHistSmemMaxBins)
-        launch_pdl(hist_kernel<VS, true>, total, 256, (max_n + 1) * 4, s, vs);
+        launch_pdl(hist_kernel<VS, true>, total, kCountThreads, (max_n + 1) * 4, s, vs);
     else
-        launch_pdl(hist_kernel<VS, false>, total, 256, 0, s, vs);
+        launch_pdl(hist_kernel<VS, false>, total, kCountThreads, 0, s, vs);
 }
 
 }  // namespace
@@ -484,9 +503,13 @@ cudaError_t topk_setup()
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = set_attrs<ManyViews>();
+    e = cudaFuncSetAttribute(rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
     if (e != cudaSuccess) return e;
-    return set_attrs<OneView>();
+    e = cudaFuncSetAttribute(hist_kernel<ManyViews, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kHistSmemMaxBins * 4);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(hist_kernel<OneView, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kHistSmemMaxBins * 4);
 }
 
 void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s)
@@ -494,7 +517,7 @@ void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s)
     launch_hist_vs(ManyViews{b}, total, max_n, s);
 }
 
-void launch_select(const Batch& b, cudaStream_t s) { launch_pdl(select_kernel<ManyViews>, b.num, 1024, 0, s, ManyViews{b}); }
+void launch_select(const Batch& b, cudaStream_t s) { launch_pdl(select_kernel, b.num, 1024, 0, s, ManyViews{b}); }
 
 void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n,
                        cudaStream_t s)
@@ -505,15 +528,16 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
     launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
 }
 
-// One problem passed by value (no device-side problem table).
-void launch_topk_single(const ProbView& v, cudaStream_t s)
+// One problem passed by value (no device-side problem table); the count blocks
+// choose the threshold (n <= 8192: the histogram fits in 48 KB).
+void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s)
 {
     const OneView vs{v};
-    launch_hist_vs(vs, (v.n + kHistRowsPerBlock - 1) / kHistRowsPerBlock, v.n, s);
-    launch_pdl(select_kernel<OneView>, 1, 1024, 0, s, vs);
-    launch_pdl(count_kernel<OneView>, count_blocks(v.n), kCountThreads, 0, s, vs, 0);
+    launch_hist_vs(vs, hist_blocks(v.n), v.n, s);
+    launch_pdl(count_kernel<OneView>, count_blocks(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
+               vs, 1);
     launch_pdl(emit_kernel<OneView>, emit_blocks(v.n), 256, 0, s, vs);
-    launch_pdl(rank_kernel<OneView>, (v.k1 + 31) / 32, 256, v.k1 * 8, s, vs);
+    launch_pdl(rank_kernel, (v.k1 + 31) / 32, 256, v.k1 * 8, s, vs, n_out);
 }
 
 }  // namespace tr

@@ -69,6 +69,10 @@ enum Stage {
 // emit pass (active rows strided over the blocks).
 __host__ __device__ inline int count_blocks(int n) { return ((n + 1) / 2 + 7) / 8; }
 __host__ __device__ inline int emit_blocks(int n) { return (n + 7) / 8; }
+// Blocks of the histogram pass: one per group of eight row pairs; from n = 8192
+// on a fixed number that takes several groups each (a block clears and flushes
+// n bins: at n = 20000 that is 80 KB against the 320 KB of W a group holds).
+__host__ __device__ inline int hist_blocks(int n) { return count_blocks(n) <= 512 ? count_blocks(n) : 304; }
 
 struct Batch {
     const ProbView* views;   // [num] device
@@ -180,7 +184,8 @@ cudaError_t topk_setup();
 cudaError_t verify_pgs_setup();
 
 // single-problem pivot selection used by the allocation-free entry point
-void launch_topk_single(const ProbView& v, cudaStream_t s);
+// n_out (device): the pivot count, or -TURBOREG_ERR_INVALID_ARG
+void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s);
 
 constexpr int kSc2BM = 128;   // GEMM tile rows  (TMEM lanes)
 constexpr int kSc2BN = 256;   // GEMM tile cols  (TMEM columns)
