@@ -25,6 +25,7 @@
 //                  beside the histogram)
 //   warp 1 lane 0  MMA issuer: tcgen05.mma kind::mxf4, N=256 K=64, 4 per stage
 //   warps 2..17    epilogue of the previous block while the next one runs
+//   warp 18        scheduler: the next blocks' descriptors
 //
 // Tensor memory (512 columns): two 256-column accumulators and 16 columns of
 // block scales do not fit side by side, so the accumulators overlap in 16
@@ -46,9 +47,12 @@ namespace {
 constexpr int kHalf = kSc2BM * kSc2BK;     // 16 KB: 128 rows x 128 bytes of one operand
 constexpr int kEpiWarps = 16;              // 4 per TMEM lane quarter, each a quarter of the columns
 constexpr int kEpiCols = 4 * kSc2BN / kEpiWarps;   // 64 columns per epilogue warp
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kSchedWarp = 2 + kEpiWarps;  // hands out the blocks
+constexpr int kThreads = 32 * (kSchedWarp + 1);
 constexpr int kMaxStages = 5;
-constexpr int kBarBytes = 512;             // mbarriers, TMEM slot
+constexpr int kRing = 4;                   // block descriptors in flight
+constexpr int kBarBytes = 1024;            // mbarriers, TMEM slot, block descriptors
+constexpr int kColBytes = kEpiWarps * kEpiCols * 4;   // column sums of an epilogue warp's block
 constexpr int kStgBytes = kEpiWarps * 2048;   // W staging: 32 x 32 uint16 per epilogue warp
 constexpr int kSmemMax = 232448;           // 227 KB opt-in limit per block
 constexpr uint32_t kTmemCols = 512;
@@ -96,12 +100,26 @@ __device__ __forceinline__ int block_index(int k, int c, int C, int L)
     return (c + k / L * C) * L + k % L;
 }
 
-// The bitset words of an epilogue warp's columns, fetched before the
-// accumulator is waited for, so that their latency overlaps the MMAs.
-__device__ __forceinline__ uint2 epi_words(const ProbView& v, int row, int col)
+// One block as the scheduler warp hands it to the others: its problem (-1: no
+// more blocks), this CTA's part of it, and the problem's fields they need.
+struct BlockInfo {
+    int32_t p, nk, row0, colb;
+    int32_t n, n_pad, ldb, flush;   // flush: the worker's next block belongs to another problem
+    const uint32_t* bits;
+    uint16_t* w;
+    int32_t* rowscore;
+    int32_t* rowmax;
+    uint32_t* hist;
+    const CUtensorMap* map;         // 128-row boxes; + 1: 256-row boxes
+};
+static_assert(sizeof(BlockInfo) == 80 && kRing * sizeof(BlockInfo) + 256 <= kBarBytes, "block ring fits");
+
+// The bitset words of an epilogue warp's columns, fetched a block ahead, so
+// that their latency overlaps the previous block's epilogue and the MMAs.
+__device__ __forceinline__ uint2 epi_words(const BlockInfo& v, int row, int col)
 {
     static_assert(kEpiCols == 64, "one 8-byte bitset load per warp row");
-    return *reinterpret_cast<const uint2*>(v.bits + (size_t)row * v.ldb + (col >> 5));
+    return *reinterpret_cast<const uint2*>(v.bits + (size_t)(v.row0 + row) * v.ldb + ((v.colb + col) >> 5));
 }
 
 // The warp's 2 KB staging area holds its 32 x 32 block of W: row r as four
@@ -138,110 +156,129 @@ __device__ __forceinline__ void arrive_at(uint32_t bar)
     else mbar_arrive_addr(bar);
 }
 
+// Where an edge weight is counted: this CTA's bins, the pair's bins (a weight's
+// bin lies in the CTA of its parity, at half its index), or the global ones.
+enum HistForm { kHistGlobal, kHistCta, kHistPair };
+
 // Epilogue of one warp's 32 rows x 64 columns whose FP32 accumulator is at
 // TMEM address tacc: masks with the adjacency words and i < j, stores uint16
 // W, adds row and column sums to the SC^2 row scores, row maxima, and counts
-// the edge weights (shared or global histogram).
-//   integers      adding 2^23 leaves an accumulator's integer in its low 16
-//                 bits (exact: it is an integer below 2^16); a byte permute
-//                 packs two, and one that replicates sign bits turns two
-//                 adjacency bits into their mask
-//   W store       pass k writes rows 8k .. 8k + 7, lane l chunk l % 4 of row
-//                 8k + l / 4: each instruction covers 8 x 64 contiguous bytes
-//   column sums   lane l reads 8 bytes (4 columns) of rows 4k + l / 8; the
-//                 four row groups are added with two shuffles per column
-//   histogram     each lane visits only the set bits of its adjacency word
+// the edge weights.
+//   integers   adding 2^23 leaves an accumulator's integer in its low 16 bits
+//              (exact: it is an integer below 2^16); a byte permute packs two,
+//              and one that replicates sign bits turns two adjacency bits into
+//              their mask
+//   W store    pass k writes rows 8k .. 8k + 7, lane l chunk l % 4 of row
+//              8k + l / 4: each instruction covers 8 x 64 contiguous bytes
+//   the rest   each lane visits only the set bits of its adjacency word, two
+//              at a time: row sum and maximum in registers, column sum and bin
+//              by shared-memory additions.  (Sums over all 32 x 32 entries in
+//              packed halves took ~250 more instructions per chunk; the warps
+//              are bound by their own instruction chains, four per scheduler.)
 // first / over: the 32-column chunk to take first, and the barrier (or 0) to
-// report to once its accumulator columns are in registers.
-template <bool kPair, bool kHist>
-__device__ __forceinline__ void sc2_epilogue(const ProbView& v, uint32_t tacc, int row0, int col_w, int lane,
-                                             uint2 words, uint32_t* shist, uint4* stg, int first, uint32_t over)
+// report to once its accumulator columns are in registers; drained: the
+// barrier to report to once both chunks are.
+// bins0 / bins1: the bins of even and odd weights (kHistPair: cluster addresses).
+template <bool kPair, HistForm kHist>
+__device__ __forceinline__ void sc2_epilogue(const BlockInfo& v, uint32_t tacc, int row_off, int col_off, int lane,
+                                             uint2 words, uint32_t* shist, uint32_t bins0, uint32_t bins1, uint4* stg,
+                                             int* csum, int first, uint32_t over, uint32_t drained)
 {
-    const int row = row0 + lane;
-    uint32_t rsum = 0u, rmax2 = 0u;
-#pragma unroll 1
-    for (int k = 0; k < kEpiCols / 32; ++k) {
+    const int row0 = v.row0 + row_off, col_w = v.colb + col_off;
+    const int row = row0 + lane, n_pad = v.n_pad;
+    uint16_t* const w = v.w;
+    uint32_t rsum = 0u, rmax = 0u;
+    uint32_t acc[32];
+    tmem_ld32(tacc + static_cast<uint32_t>(first * 32), acc);
+    tmem_ld_wait32(acc);
+    if (over != 0u) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_at<kPair>(over);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        static_assert(kEpiCols == 64, "two 32-column chunks");
         const int c = k ^ first;
-        uint32_t acc[32];
-        tmem_ld32(tacc + static_cast<uint32_t>(c * 32), acc);
-        tmem_ld_wait();
-        if (k == 0 && over != 0u) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_at<kPair>(over);
-        }
         const int col0 = col_w + c * 32;
         uint32_t word = c == 0 ? words.x : words.y;
         if (col0 + 31 <= row) word = 0u;                       // keep only j > row
         else if (col0 <= row) word &= ~0u << (row - col0 + 1);
         const uint32_t ub = unshuffle16(word);
-        uint32_t h[16];
         const f2 magic = pk(8388608.f, 8388608.f);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const f2 s = add2(pk(__uint_as_float(acc[2 * e]), __uint_as_float(acc[2 * e + 1])), magic);
-            // columns 2e, 2e + 1: bit e % 8 of the two bytes of half e / 8, moved to the bytes' sign bits
-            const uint32_t m = sign_bytes(ub << (7 - (e & 7)), e < 8 ? 0x9988u : 0xBBAAu);
-            h[e] = __byte_perm(static_cast<uint32_t>(s.v), static_cast<uint32_t>(s.v >> 32), 0x5410u) & m;
-            rsum = __dp2a_lo(h[e], 0x0101u, rsum);
-            rmax2 = __vmaxu2(rmax2, h[e]);
-        }
+        for (int q = 0; q < 4; ++q) {
+            uint32_t h[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            stg[stg_slot(lane, q)] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+            for (int e4 = 0; e4 < 4; ++e4) {
+                const int e = 4 * q + e4;
+                const f2 s = add2(pk(__uint_as_float(acc[2 * e]), __uint_as_float(acc[2 * e + 1])), magic);
+                // columns 2e, 2e + 1: bit e % 8 of the two bytes of half e / 8, moved to the bytes' sign bits
+                const uint32_t m = sign_bytes(ub << (7 - (e & 7)), e < 8 ? 0x9988u : 0xBBAAu);
+                h[e4] = __byte_perm(static_cast<uint32_t>(s.v), static_cast<uint32_t>(s.v >> 32), 0x5410u) & m;
+            }
+            stg[stg_slot(lane, q)] = make_uint4(h[0], h[1], h[2], h[3]);
+        }
+        if (k == 0) tmem_ld32(tacc + static_cast<uint32_t>((first ^ 1) * 32), acc);   // in flight through chunk 0's stores
         __syncwarp();
         // W rows, as full 64-byte segments
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4) {
             const int r = 8 * k4 + (lane >> 2), q = lane & 3;
-            *reinterpret_cast<uint4*>(v.w + (size_t)(row0 + r) * v.n_pad + col0 + q * 8) = stg[stg_slot(r, q)];
+            *reinterpret_cast<uint4*>(w + (size_t)(row0 + r) * n_pad + col0 + q * 8) = stg[stg_slot(r, q)];
         }
-        // column sums: lane l adds columns 4 (l % 8) .. +3 over rows l / 8 + 4k
-        if (__any_sync(0xffffffffu, word != 0u)) {
-            static_assert(2 * (TURBOREG_MAX_N - 2) < 65536, "two weights add without a carry out of 16 bits");
-            const int m = lane & 7;
-            int cs[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int kk = 0; kk < 8; kk += 2) {
-                const uint2 d0 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * kk + (lane >> 3), m >> 1))[m & 1];
-                const uint2 d1 = reinterpret_cast<const uint2*>(stg + stg_slot(4 * kk + 4 + (lane >> 3), m >> 1))[m & 1];
-                const uint32_t x = d0.x + d1.x, y = d0.y + d1.y;   // two rows per 16-bit lane
-                cs[0] += static_cast<int>(x & 0xFFFFu);
-                cs[1] += static_cast<int>(x >> 16);
-                cs[2] += static_cast<int>(y & 0xFFFFu);
-                cs[3] += static_cast<int>(y >> 16);
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                cs[e] += __shfl_xor_sync(0xffffffffu, cs[e], 8);
-                cs[e] += __shfl_xor_sync(0xffffffffu, cs[e], 16);
-            }
-            // lane l reports column 4 (l % 8) + l / 8
-            const int e = lane >> 3;
-            const int sum = e == 0 ? cs[0] : e == 1 ? cs[1] : e == 2 ? cs[2] : cs[3];
-            if (sum != 0) atomicAdd(&v.rowscore[col0 + 4 * m + e], sum);
+        // this lane's edges
+        int* const cs = csum + c * 32;
+        auto edge_w = [&](int q) { return static_cast<uint32_t>(reinterpret_cast<const uint16_t*>(stg + stg_slot(lane, q >> 3))[q & 7]); };
+        auto count = [&](int q, uint32_t x) {
+            if (x == 0u) return;
+            atomicAdd(cs + q, static_cast<int>(x));
+            if (kHist == kHistCta) atomicAdd(&shist[x], 1u);
+            else if (kHist == kHistPair) red_add_cluster(((x & 1u) ? bins1 : bins0) + ((x >> 1) << 2), 1u);
+            else atomicAdd(&v.hist[x], 1u);
+        };
+        for (uint32_t bits = word; bits != 0u;) {
+            const int q0 = __ffs(bits) - 1;
+            bits &= bits - 1u;
+            const int q1 = bits != 0u ? __ffs(bits) - 1 : q0;
+            const uint32_t x0 = edge_w(q0), y = edge_w(q1);
+            const uint32_t x1 = bits != 0u ? y : 0u;
+            bits &= bits - 1u;
+            rsum += x0 + x1;
+            rmax = max(rmax, max(x0, x1));
+            count(q0, x0);
+            count(q1, x1);
         }
-        // histogram of the edge weights: only this lane's edges
-        for (uint32_t bits = word; bits != 0u; bits &= bits - 1u) {
-            const int q = __ffs(bits) - 1;
-            const int w = reinterpret_cast<const uint16_t*>(stg + stg_slot(lane, q >> 3))[q & 7];
-            if (w > 0) {
-                if (kHist) atomicAdd(&shist[w], 1u);
-                else atomicAdd(&v.hist[w], 1u);
-            }
+        if (k == 0) {
+            // the accumulator is read: its next block's MMAs may begin
+            tmem_ld_wait32(acc);
+            tc_fence_before();
         }
-        __syncwarp();   // the next chunk overwrites the staging area
+        __syncwarp();   // the next chunk overwrites the staging area; the column sums are complete
+        if (k == 0 && lane == 0) arrive_at<kPair>(drained);
     }
     if (rsum != 0u) atomicAdd(&v.rowscore[row], static_cast<int>(rsum));
-    const int rmax = static_cast<int>(max(rmax2 & 0xFFFFu, rmax2 >> 16));
-    if (rmax != 0 && v.rowmax) atomicMax(&v.rowmax[row], rmax);
+    if (rmax != 0u && v.rowmax) atomicMax(&v.rowmax[row], static_cast<int>(rmax));
+    static_assert(kEpiCols == 64, "two columns per lane");
+    const int2 cc = reinterpret_cast<const int2*>(csum)[lane];
+    if ((cc.x | cc.y) != 0) {
+        reinterpret_cast<int2*>(csum)[lane] = make_int2(0, 0);
+        if (cc.x) atomicAdd(&v.rowscore[col_w + 2 * lane], cc.x);
+        if (cc.y) atomicAdd(&v.rowscore[col_w + 2 * lane + 1], cc.y);
+    }
+    __syncwarp();   // the sums are cleared before the next block adds to them
 }
 
 // kPair: 2-CTA clusters with pair MMAs (M = 256 over both CTAs); else CTAs of
 // their own take 128-row halves of the blocks.  kHist: the edge-weight
-// histogram is kept in shared memory and added to the global one when the
-// worker leaves a problem (the count pass or the select launch then chooses
-// the pivot threshold from it); else every edge adds to the global bins.
+// histogram is kept in shared memory, per CTA or (one problem) split over the
+// pair, and added to the global one when the worker leaves a problem (the
+// count pass or the select launch then chooses the pivot threshold from it);
+// else every edge adds to the global bins.
+// The scheduler warp finds each block's problem and descriptor fields up to
+// four blocks ahead and hands them over through a ring in shared memory: read
+// by every role for itself, they were a chain of up to eight dependent loads
+// in front of each block's loads, MMAs and epilogue.
 //   pair: both CTAs' producers load their 128 rows of A and of B, counted on
 //         the leader's `full` barrier; the leader issues the MMAs, whose commits
 //         release the stage in both CTAs (`empty`) and hand each CTA its
@@ -251,7 +288,7 @@ __device__ __forceinline__ void sc2_epilogue(const ProbView& v, uint32_t tacc, i
 // releases and a cluster synchronises, so no arrival targets a finished CTA.
 // auto_mode: one problem whose SC^2 path the CUDA-core kernel before this one
 // chose; when it chose itself, every CTA returns at once (before any set-up).
-template <bool kPair, bool kHist>
+template <bool kPair, HistForm kHist>
 __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int total, int hist_bins, int nst, int chunk,
                                                               int auto_mode)
 {
@@ -275,12 +312,17 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
     uint64_t* tempty = tfull + 2;            // [2] accumulator drained
     uint64_t* tover = tempty + 2;            // the columns both accumulators share are read
     uint64_t* hsync = tover + 1;             // epilogue warps: a problem's bins complete / flushed
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(hsync + 1);
+    uint64_t* sfull = hsync + 1;             // [kRing] block descriptor written / consumed
+    uint64_t* sempty = sfull + kRing;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sempty + kRing);
+    static_assert((2 * kMaxStages + 6 + 2 * kRing) * 8 + 4 <= 256, "barriers before the block ring");
+    BlockInfo* ring = reinterpret_cast<BlockInfo*>(tail + 256);
     uint4* stg = reinterpret_cast<uint4*>(tail + kBarBytes);
-    uint32_t* shist = reinterpret_cast<uint32_t*>(tail + kBarBytes + kStgBytes);
+    int* csums = reinterpret_cast<int*>(tail + kBarBytes + kStgBytes);
+    uint32_t* shist = reinterpret_cast<uint32_t*>(tail + kBarBytes + kStgBytes + kColBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nbins = kHist ? hist_bins : 0;
+    const int nbins = kHist != kHistGlobal ? hist_bins : 0;   // words of this CTA's bins
     const uint32_t rank = kPair ? cluster_ctarank() : 0u;
     const bool leader = rank == 0;
 
@@ -295,10 +337,14 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         }
         mbar_init(tover, (kPair ? 2 : 1) * 4);
         mbar_init(hsync, kEpiWarps);
+        for (int b = 0; b < kRing; ++b) {
+            mbar_init(&sfull[b], 1);
+            mbar_init(&sempty[b], kEpiWarps + 1 + (leader ? 1 : 0));   // epilogue warps, producer, the leader's issuer
+        }
         fence_mbar_init();
     }
-    if (kHist)
-        for (int b = threadIdx.x; b < nbins; b += blockDim.x) shist[b] = 0u;
+    for (int b = threadIdx.x; b < nbins; b += blockDim.x) shist[b] = 0u;
+    for (int b = threadIdx.x; b < kEpiWarps * kEpiCols; b += blockDim.x) csums[b] = 0;
     if (warp == 0) {
         if (kPair) tmem_alloc_pair(tmem_slot, kTmemCols);
         else tmem_alloc(tmem_slot, kTmemCols);
@@ -323,17 +369,6 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
     const uint32_t full_l = kPair ? mapa_shared(&full[0], 0) : 0u;      // leader's barriers, cluster addresses
     const uint32_t tempty_l = kPair ? mapa_shared(&tempty[0], 0) : smem_u32(&tempty[0]);
     const uint32_t tover_l = kPair ? mapa_shared(tover, 0) : smem_u32(tover);
-    // block u of the launch -> problem, column blocks and this CTA's row / column offsets
-    auto place = [&](int u, int& p, int& nk, int& row0, int& colb) {
-        int lt;
-        p = locate(bt, ST_GEMM, kPair ? 2 * u : u, lt);
-        const int nb = bt.views[p].n_pad / kSc2BN;
-        int bm, bn;
-        block_of(lt >> 1, nb, bm, bn);
-        nk = nb;   // K stages of 256 columns
-        row0 = bm * kSc2BN + (kPair ? static_cast<int>(rank) : lt & 1) * kSc2BM;
-        colb = bn * kSc2BN;
-    };
     // the set-up above (barriers, tensor memory, shared histogram) overlaps the
     // previous stage; its outputs are read only from here on
     pdl_wait();
@@ -345,11 +380,12 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
             int s = 0;
             uint32_t ph = 0u;
             for (int k = 0; ok; ++k) {
-                const int u = block_index(k, c, C, chunk);
-                if (u >= nu) break;
-                int p, nk, row0, colb;
-                place(u, p, nk, row0, colb);
-                const CUtensorMap* mA = bt.maps + 2 * p;   // 128-row boxes; + 1: 256-row boxes
+                if (!mbar_wait(&sfull[k % kRing], (k / kRing) & 1)) { ok = false; break; }
+                const BlockInfo& bi = ring[k % kRing];
+                const int p = bi.p, nk = bi.nk, row0 = bi.row0, colb = bi.colb;
+                const CUtensorMap* mA = bi.map;
+                mbar_arrive(&sempty[k % kRing]);
+                if (p < 0) break;
                 for (int kb = 0; kb < nk; ++kb) {
                     if (!mbar_wait(&empty[s], ph ^ 1u)) { ok = false; break; }
                     if (kPair) {
@@ -380,10 +416,10 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
             int s = 0;
             uint32_t ph = 0u;
             for (int k = 0; ok; ++k) {
-                const int u = block_index(k, c, C, chunk);
-                if (u >= nu) break;
-                int p, nk, row0, colb;
-                place(u, p, nk, row0, colb);
+                if (!mbar_wait(&sfull[k % kRing], (k / kRing) & 1)) { ok = false; break; }
+                const int p = ring[k % kRing].p, nk = ring[k % kRing].nk;
+                mbar_arrive(&sempty[k % kRing]);
+                if (p < 0) break;
                 const int buf = k & 1;
                 const uint32_t use = static_cast<uint32_t>(k >> 1);
                 // this accumulator drained, and the previous one's shared columns read
@@ -410,49 +446,98 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
             }
         }
         __syncwarp();
+    } else if (warp == kSchedWarp) {
+        // ---------------- scheduler ----------------
+        const int32_t* pr = bt.pre + ST_GEMM * (bt.num + 1);
+        int p = 0;
+        for (int k = 0;; ++k) {
+            const int u = block_index(k, c, C, chunk);
+            const int slot = k % kRing;
+            if (k >= kRing && !__all_sync(0xffffffffu, mbar_wait(&sempty[slot], (k / kRing - 1) & 1))) {
+                ok = false;
+                break;
+            }
+            if (u >= nu) {
+                if (lane == 0) {
+                    ring[slot].p = -1;
+                    mbar_arrive(&sfull[slot]);
+                }
+                break;
+            }
+            // the last problem that begins at or before this block (blocks only move forward)
+            const int t = kPair ? 2 * u : u;
+            for (int step = 32; step == 32; p += step)
+                step = __popc(__ballot_sync(0xffffffffu, p + 1 + lane < bt.num && __ldg(pr + min(p + 1 + lane, bt.num)) <= t));
+            if (lane == 0) {
+                const ProbView& v = bt.views[p];
+                const int un = block_index(k + 1, c, C, chunk);
+                const int lt = t - __ldg(pr + p), nb = v.n_pad / kSc2BN;
+                int bm, bn;
+                block_of(lt >> 1, nb, bm, bn);
+                BlockInfo bi;
+                bi.p = p;
+                bi.nk = nb;   // K stages of 256 columns
+                bi.row0 = bm * kSc2BN + (kPair ? static_cast<int>(rank) : lt & 1) * kSc2BM;
+                bi.colb = bn * kSc2BN;
+                bi.n = v.n;
+                bi.n_pad = v.n_pad;
+                bi.ldb = v.ldb;
+                bi.flush = un < nu && (kPair ? 2 * un : un) >= __ldg(pr + p + 1) ? 1 : 0;
+                bi.bits = v.bits;
+                bi.w = v.w;
+                bi.rowscore = v.rowscore;
+                bi.rowmax = v.rowmax;
+                bi.hist = v.hist;
+                bi.map = bt.maps + 2 * p;
+                ring[slot] = bi;
+                mbar_arrive(&sfull[slot]);
+            }
+            __syncwarp();
+        }
     } else {
         // ---------------- epilogue warps ----------------
         const int quarter = warp & 3;              // TMEM lanes this warp may access
         const int part = (warp - 2) >> 2;          // column part of the block
         const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
-        for (int k = 0;; ++k) {
-            const int u = block_index(k, c, C, chunk);
-            if (u >= nu) break;
-            int p, nk, row0, colb;
-            place(u, p, nk, row0, colb);
-            const ProbView v = bt.views[p];
+        const int ro = quarter * 32, co = part * kEpiCols;
+        const uint32_t bins0 = kHist == kHistPair ? mapa_shared(shist, 0) : 0u;
+        const uint32_t bins1 = kHist == kHistPair ? mapa_shared(shist, 1) : 0u;
+        uint2 words = make_uint2(0u, 0u);
+        ok = __all_sync(0xffffffffu, mbar_wait(&sfull[0], 0u));
+        if (ok && ring[0].p >= 0) words = epi_words(ring[0], ro + lane, co);
+        for (int k = 0; ok; ++k) {
+            const BlockInfo& v = ring[k % kRing];
+            if (v.p < 0) break;
+            // the next block's descriptor and adjacency words
+            const BlockInfo& vn = ring[(k + 1) % kRing];
+            if (!__all_sync(0xffffffffu, mbar_wait(&sfull[(k + 1) % kRing], ((k + 1) / kRing) & 1))) { ok = false; break; }
+            uint2 words_n = make_uint2(0u, 0u);
+            if (vn.p >= 0) words_n = epi_words(vn, ro + lane, co);
             const int buf = k & 1;
-            const uint32_t use = static_cast<uint32_t>(k >> 1);
-            const int r0 = row0 + quarter * 32, cw = colb + part * kEpiCols;
-            const uint2 words = epi_words(v, r0 + lane, cw);
-            // a batch: whether this worker's next block belongs to another problem
-            bool flush_after = false;
-            const int un = block_index(k + 1, c, C, chunk);
-            if (kHist && un < nu) {
-                int ltn;
-                flush_after = locate(bt, ST_GEMM, kPair ? 2 * un : un, ltn) != p;
-            }
-            const bool got = mbar_wait(&tfull[buf], use & 1u);
+            const bool got = mbar_wait(&tfull[buf], static_cast<uint32_t>(k >> 1) & 1u);
             if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
             tc_fence_after();
             // the shared columns: the last 16 of accumulator 0, the first 16 of accumulator 1
             const bool owner = buf == 0 ? part == 3 : part == 0;
-            sc2_epilogue<kPair, kHist>(v, tmem + (buf ? kAcc1 : 0u) + static_cast<uint32_t>(part * kEpiCols) + lane_off, r0, cw,
-                                lane, words, shist, stg + (warp - 2) * 128, buf == 0 && part == 3 ? 1 : 0,
-                                owner ? tover_l : 0u);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_at<kPair>(tempty_l + static_cast<uint32_t>(buf * sizeof(uint64_t)));
-            if (flush_after) {
+            sc2_epilogue<kPair, kHist>(v, tmem + (buf ? kAcc1 : 0u) + static_cast<uint32_t>(co) + lane_off, ro, co, lane,
+                                       words, shist, bins0, bins1, stg + (warp - 2) * 128, csums + (warp - 2) * kEpiCols,
+                                       buf == 0 && part == 3 ? 1 : 0, owner ? tover_l : 0u,
+                                       tempty_l + static_cast<uint32_t>(buf * sizeof(uint64_t)));
+            const bool flush = kHist == kHistCta && v.flush != 0;
+            const int nf = v.n;
+            uint32_t* const ghist = v.hist;
+            __syncwarp();   // every lane's reads of the descriptor are done
+            if (lane == 0) mbar_arrive(&sempty[k % kRing]);
+            words = words_n;
+            if (flush) {
                 // the epilogue warps add this problem's bins to its global
                 // histogram and clear them (a rendezvous before and after)
-                const int nf = v.n;
                 if (lane == 0) mbar_arrive(hsync);
                 if (!__all_sync(0xffffffffu, mbar_wait(hsync, 0u))) { ok = false; break; }
                 for (int b = (warp - 2) * 32 + lane + 1; b <= nf; b += 32 * kEpiWarps) {
                     const uint32_t h = shist[b];
                     if (h) {
-                        atomicAdd(v.hist + b, h);
+                        atomicAdd(ghist + b, h);
                         shist[b] = 0u;
                     }
                 }
@@ -475,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         int lt;
         p_last = locate(bt, ST_GEMM, kPair ? 2 * ul : ul, lt);
     }
-    if (kPair && kHist && !leader && p_last >= 0) {
+    if (kPair && kHist == kHistCta && !leader && p_last >= 0) {
         // the peer's histogram into the leader's (distributed shared memory), so
         // that one CTA per cluster adds to the global bins
         const uint32_t lead_hist = mapa_shared(shist, 0);
@@ -491,12 +576,17 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         if (kPair) tmem_dealloc_pair(tmem, kTmemCols);
         else tmem_dealloc(tmem, kTmemCols);
     }
-    if (!kHist || !leader || p_last < 0) return;
+    if (kHist == kHistGlobal || p_last < 0 || (kHist == kHistCta && !leader)) return;
     // the worker's histogram into the global one, from which the count pass
     // (one problem) or the select launch (a batch) chooses the pivot threshold
     const ProbView vl = bt.views[p_last];
-    for (int b = threadIdx.x + 1; b <= vl.n; b += blockDim.x)
-        if (shist[b]) atomicAdd(&vl.hist[b], shist[b]);
+    if (kHist == kHistPair) {
+        for (int b = threadIdx.x; b < nbins; b += blockDim.x)
+            if (shist[b]) atomicAdd(&vl.hist[2 * b + static_cast<int>(rank)], shist[b]);
+    } else {
+        for (int b = threadIdx.x + 1; b <= vl.n; b += blockDim.x)
+            if (shist[b]) atomicAdd(&vl.hist[b], shist[b]);
+    }
 }
 
 int g_sc2_sms = 0;
@@ -505,7 +595,8 @@ int g_sc2_pair_clusters = 0;   // co-resident 2-CTA clusters of the pair kernels
 template <bool kPair>
 size_t smem_bytes(int nst, int bins)
 {
-    return static_cast<size_t>(nst) * stage_bytes<kPair>() + kBarBytes + kStgBytes + 1024 + static_cast<size_t>(bins) * 4;
+    return static_cast<size_t>(nst) * stage_bytes<kPair>() + kBarBytes + kStgBytes + kColBytes + 1024 +
+           static_cast<size_t>(bins) * 4;
 }
 
 // Ring stages beside `bins` histogram bins (at most kMaxStages; 0: fewer than two fit).
@@ -526,7 +617,7 @@ int chunk_for(const Batch& b, int units, int workers)
     return l < 1 ? 1 : l > 4 ? 4 : l;
 }
 
-template <bool kPair, bool kHist>
+template <bool kPair, HistForm kHist>
 cudaError_t launch_mma(const Batch& b, int total_tiles, int bins, cudaStream_t s, int auto_mode)
 {
     const int nst = stages_for<kPair>(bins);
@@ -551,7 +642,7 @@ cudaError_t launch_mma(const Batch& b, int total_tiles, int bins, cudaStream_t s
     return cudaLaunchKernelEx(&cfg, sc2_mma_kernel<kPair, kHist>, b, total_tiles, bins, nst, chunk, auto_mode);
 }
 
-template <bool kPair, bool kHist>
+template <bool kPair, HistForm kHist>
 cudaError_t mma_attr()
 {
     return cudaFuncSetAttribute(sc2_mma_kernel<kPair, kHist>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
@@ -568,9 +659,11 @@ cudaError_t sc2_tcgen05_setup()
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sc2_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = mma_attr<true, true>();
-    if (e == cudaSuccess) e = mma_attr<false, true>();
-    if (e == cudaSuccess) e = mma_attr<false, false>();
+    if (e == cudaSuccess) e = mma_attr<true, kHistCta>();
+    if (e == cudaSuccess) e = mma_attr<true, kHistPair>();
+    if (e == cudaSuccess) e = mma_attr<true, kHistGlobal>();
+    if (e == cudaSuccess) e = mma_attr<false, kHistCta>();
+    if (e == cudaSuccess) e = mma_attr<false, kHistGlobal>();
     if (e == cudaSuccess) {
         // how many 2-CTA clusters fit at once with the largest shared-memory request
         cudaLaunchConfig_t cfg = {};
@@ -585,7 +678,7 @@ cudaError_t sc2_tcgen05_setup()
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, sc2_mma_kernel<true, true>, &cfg) == cudaSuccess)
+        if (cudaOccupancyMaxActiveClusters(&nc, sc2_mma_kernel<true, kHistCta>, &cfg) == cudaSuccess)
             g_sc2_pair_clusters = nc;
         else
             cudaGetLastError();   // no cluster support: the single-CTA kernel is used
@@ -593,20 +686,31 @@ cudaError_t sc2_tcgen05_setup()
     return e;
 }
 
-// The bins of any problem the library takes fit beside two stages of the pair
-// form (131 KB at N = 32768); the single-CTA form's larger stages leave room
-// for N up to about 24 800, above which its edges add to the global bins.
+// The pair form keeps a CTA's bins beside its ring.  One problem whose bins
+// would cost the ring a stage splits them over the pair: at N = 20000 that
+// leaves four stages beside 40 KB of bins instead of three beside 80 KB (and
+// two stages at N = 32768).  A batch does not (its CTAs flush their bins by
+// themselves between problems): above N of about 31 800 its edges add to the
+// global bins, as the single-CTA form's do above about 24 000 (larger stages).
 bool launch_sc2_tcgen05(const Batch& b, int total_tiles, int max_n, bool pair_mma, cudaStream_t s, bool auto_mode)
 {
     const int bins = max_n + 1;
     if (pair_mma && g_sc2_pair_clusters > 0) {
-        static_assert(2 * stage_bytes<true>() + kBarBytes + kStgBytes + 1024 + (TURBOREG_MAX_N + 1) * 4 <= kSmemMax,
-                      "the largest histogram fits beside two stages");
-        launch_mma<true, true>(b, total_tiles, bins, s, auto_mode ? 1 : 0);
+        static_assert(2 * stage_bytes<true>() + kBarBytes + kStgBytes + kColBytes + 1024 +
+                      (TURBOREG_MAX_N / 2 + 2) * 4 <= kSmemMax, "half of the largest histogram fits beside two stages");
+        const int half = bins / 2 + 1;
+        if (b.num == 1 && stages_for<true>(half) > stages_for<true>(bins)) {
+            launch_mma<true, kHistPair>(b, total_tiles, half, s, auto_mode ? 1 : 0);
+        } else if (stages_for<true>(bins) > 0) {
+            launch_mma<true, kHistCta>(b, total_tiles, bins, s, auto_mode ? 1 : 0);
+        } else {
+            launch_mma<true, kHistGlobal>(b, total_tiles, 0, s, 0);
+            return false;
+        }
     } else if (stages_for<false>(bins) > 0) {
-        launch_mma<false, true>(b, total_tiles, bins, s, 0);
+        launch_mma<false, kHistCta>(b, total_tiles, bins, s, 0);
     } else {
-        launch_mma<false, false>(b, total_tiles, 0, s, 0);
+        launch_mma<false, kHistGlobal>(b, total_tiles, 0, s, 0);
         return false;
     }
     return b.num == 1;

@@ -296,10 +296,14 @@ __device__ __forceinline__ void red_add_cluster(uint32_t addr_cluster, uint32_t 
     asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(addr_cluster), "r"(v) : "memory");
 }
 
-// Arrive on an mbarrier given by its cluster-window address (possibly in the peer CTA).
+// Arrive on an mbarrier given by its cluster-window address (possibly in the
+// peer CTA).  Release at CTA scope: the arrivals report that tensor memory has
+// been read (ordered by tcgen05.wait::ld and the fence before them) and pass
+// no data to the peer; at cluster scope each one would wait until all earlier
+// global stores and additions of the thread have reached L2.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 
 // 2-D tiled load into this CTA's shared memory whose completion is counted on
@@ -435,6 +439,17 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, uint32_t x)
 }
 
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Wait for tmem_ld32 into v, whose values exist from here on.
+__device__ __forceinline__ void tmem_ld_wait32(uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
+                   "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]),
+                   "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]),
+                   "+r"(v[29]), "+r"(v[30]), "+r"(v[31])::"memory");
+}
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
