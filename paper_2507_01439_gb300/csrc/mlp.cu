@@ -8,16 +8,17 @@
 // Parameter vector (FP32 master copy, 17217 values, row-major [out][in]):
 //   W1[64][8] b1[64] W2[128][64] b2[128] W3[64][128] b3[64] W4[64] b4[1]
 //
-// Forward (inference and training): one CTA of 128 threads per 128 rows.
+// Forward (inference): one CTA of 128 threads per 128 rows.
 // Layer 1 (K = 8) and layer 4 (N = 1) run on CUDA cores; layers 2 and 3 run
 // on the tensor cores (tcgen05.mma kind::f16, BF16 operands, FP32 TMEM
 // accumulators) with operands written to shared memory in the 128-byte
 // swizzled K-major layout by the threads themselves.
-// Backward: the activation gradients of layers 3 and 2 and the weight
-// gradients of layers 2 and 3 on the tensor cores (BF16 operands, FP32
-// accumulation, the weight gradients accumulated in tensor memory over a
-// CTA's sample tiles); layers 1 and 4 and the biases on CUDA cores.  Adam on
-// CUDA cores.
+// Training: forward and backward of a 128-sample tile in one kernel, the
+// activations in shared memory only; the activation gradients of layers 3 and
+// 2 and the weight gradients of layers 2 and 3 on the tensor cores (BF16
+// operands, FP32 accumulation, the weight gradients accumulated in tensor
+// memory over a CTA's tiles); layers 1 and 4 and the biases on CUDA cores.
+// Adam on CUDA cores.
 #include <cuda_bf16.h>
 
 #include "tr_common.cuh"
@@ -53,15 +54,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 __device__ __forceinline__ float bf16r(float a) { return __bfloat162float(__float2bfloat16_rn(a)); }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// act (optional, training): per row h1[64] h2[128] h3[64] (bf16) and z4 (f32)
-struct FwdOut {
-    float* prob;               // [m] sigmoid(z4) (may be null)
-    float* z4;                 // [m] (may be null)
-    __nv_bfloat16* h1;         // [m][64]  (may be null)
-    __nv_bfloat16* h2;         // [m][128]
-    __nv_bfloat16* h3;         // [m][64]
-};
 
 // Set-up of a forward CTA: the weights into shared memory (B operands in the
 // swizzled layout), the mbarrier and 256 tensor-memory columns; returns the
@@ -115,7 +107,7 @@ __device__ uint32_t mlp_setup_cta(const float* __restrict__ wbf, uint8_t* smem)
 // One tile of 128 rows (row0 ..) after mlp_setup_cta: completes two phases of
 // the CTA's mbarrier (parities 0 then 1), so tiles can follow one another.
 // Returns this thread's probability (0 for rows past m).
-__device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, FwdOut out, uint8_t* smem, uint32_t tmem,
+__device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, float* prob, uint8_t* smem, uint32_t tmem,
                           uint32_t* err)
 {
     uint8_t* sH1 = smem + kOffH1;
@@ -151,11 +143,6 @@ __device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, FwdOu
             make_uint4(pack_bf16(h8[0], h8[1]), pack_bf16(h8[2], h8[3]), pack_bf16(h8[4], h8[5]),
                        pack_bf16(h8[6], h8[7]));
     }
-    if (out.h1 && row < m) {
-        uint4* d = reinterpret_cast<uint4*>(out.h1 + (size_t)row * 64);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) d[c] = *reinterpret_cast<const uint4*>(sH1 + sw128(t, c));
-    }
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -188,14 +175,6 @@ __device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, FwdOu
                 make_uint4(pack_bf16(hv[8 * c4 + 0], hv[8 * c4 + 1]), pack_bf16(hv[8 * c4 + 2], hv[8 * c4 + 3]),
                            pack_bf16(hv[8 * c4 + 4], hv[8 * c4 + 5]), pack_bf16(hv[8 * c4 + 6], hv[8 * c4 + 7]));
         }
-        if (out.h2 && row < m) {
-            uint4* d = reinterpret_cast<uint4*>(out.h2 + (size_t)row * 128 + cb * 32);
-#pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
-                const int k8 = cb * 4 + c4;
-                d[c4] = *reinterpret_cast<const uint4*>(sH2 + (k8 >> 3) * 16384 + sw128(t, k8 & 7));
-            }
-        }
     }
     fence_async_smem();
     tc_fence_before();
@@ -227,19 +206,11 @@ __device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, FwdOu
             hv[q] = bf16r(fmaxf(__uint_as_float(acc[q]) + sb3[cb * 32 + q], 0.f));
             z4 = fmaf(sW4[cb * 32 + q], hv[q], z4);
         }
-        if (out.h3 && row < m) {
-            uint4* d = reinterpret_cast<uint4*>(out.h3 + (size_t)row * 64 + cb * 32);
-#pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4)
-                d[c4] = make_uint4(pack_bf16(hv[8 * c4 + 0], hv[8 * c4 + 1]), pack_bf16(hv[8 * c4 + 2], hv[8 * c4 + 3]),
-                                   pack_bf16(hv[8 * c4 + 4], hv[8 * c4 + 5]), pack_bf16(hv[8 * c4 + 6], hv[8 * c4 + 7]));
-        }
     }
     float pr = 0.f;
     if (row < m) {
         pr = 1.f / (1.f + __expf(-z4));
-        if (out.z4) out.z4[row] = z4;
-        if (out.prob) out.prob[row] = pr;
+        prob[row] = pr;
     }
     // the tile's tensor-memory reads are complete before the next tile's MMAs
     tc_fence_before();
@@ -255,25 +226,20 @@ __device__ void mlp_teardown_cta(uint32_t tmem)
     }
 }
 
-__device__ void mlp_forward_tile(const float* __restrict__ feat, int m, int row0, const float* __restrict__ wbf,
-                                 FwdOut out, uint8_t* smem, uint32_t* err)
-{
-    const uint32_t tmem = mlp_setup_cta(wbf, smem);
-    mlp_tile(feat, m, row0, out, smem, tmem, err);
-    mlp_teardown_cta(tmem);
-}
-
 __device__ __forceinline__ uint8_t* aligned_smem(uint8_t* raw)
 {
     return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
 }
 
-// Standalone forward over an arbitrary feature array (training and tests).
-__global__ void __launch_bounds__(kRows, 1) mlp_fwd_kernel(const float* feat, int m, const float* wbf, FwdOut out,
+// Standalone forward over an arbitrary feature array.
+__global__ void __launch_bounds__(kRows, 1) mlp_fwd_kernel(const float* feat, int m, const float* wbf, float* prob,
                                                            uint32_t* err)
 {
     extern __shared__ uint8_t smem_raw[];
-    mlp_forward_tile(feat, m, blockIdx.x * kRows, wbf, out, aligned_smem(smem_raw), err);
+    uint8_t* smem = aligned_smem(smem_raw);
+    const uint32_t tmem = mlp_setup_cta(wbf, smem);
+    mlp_tile(feat, m, blockIdx.x * kRows, prob, smem, tmem, err);
+    mlp_teardown_cta(tmem);
 }
 
 // Registration path: persistent CTAs (weights, mbarrier and tensor memory set
@@ -291,8 +257,7 @@ __global__ void __launch_bounds__(kRows, 2) mlp_proposal_kernel(Batch bt, int to
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
         int lb;
         const ProbView v = bt.views[locate(bt, ST_MLP, tile, lb)];
-        FwdOut out = {v.prob, nullptr, nullptr, nullptr, nullptr};
-        float pm = mlp_tile(v.feat, v.n, lb * kRows, out, smem, tmem, &v.ctl->err);
+        float pm = mlp_tile(v.feat, v.n, lb * kRows, v.prob, smem, tmem, &v.ctl->err);
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, off));
         if ((threadIdx.x & 31) == 0 && pm > 0.f) atomicMax(&v.ctl->pmax_bits, __float_as_uint(pm));
@@ -368,11 +333,14 @@ __global__ void __launch_bounds__(1024) features_kernel(ManyViews vs)
     }
 }
 
-// ---------------- training: backward on the tensor cores ----------------
+// ---------------- training: forward and backward in one kernel ----------------
 //
-// Persistent CTAs of 128 threads take 128-sample tiles (thread t: sample
-// row0 + t).  Per sample:
-//   dz4 = (sigmoid(z4) - y) / m                  (mean binary cross-entropy)
+// Persistent CTAs of 512 threads take 128-sample tiles; thread t works for
+// sample t % 128 on a quarter of the columns (t / 128), which is also its
+// tensor-memory lane and column part.  Per tile:
+//   h1 = relu(W1 x + b1)                         (CUDA cores)
+//   h2 = relu(W2 h1 + b2), h3 = relu(W3 h2 + b3)  forward MMAs
+//   z4 = W4 h3 + b4,  dz4 = (sigmoid(z4) - y) / m   (mean binary cross-entropy)
 //   dz3 = W4 dz4 * [h3 > 0]                      (CUDA cores)
 //   dz2 = (dz3 W3) * [h2 > 0]                    MMA1: D1[128 x 128] = DZ3[128 x 64] W3
 //   dz1 = (dz2 W2) * [h1 > 0]                    MMA2: D2[128 x 64] = DZ2[128 x 128] W2
@@ -381,334 +349,456 @@ __global__ void __launch_bounds__(1024) features_kernel(ManyViews vs)
 //   dW3^T[128 in x 64 out] += H2^T[128 x 128 s] DZ3[128 s x 64]     MMA3 (G3)
 //   dW2[128 out x 64 in]    += DZ2^T[128 x 128 s] H1[128 s x 64]     MMA4 (G2)
 // dW1 = dz1^T x, dW4 = h3^T dz4 and the biases (sums of dz over the samples)
-// on CUDA cores, in registers over the tiles.  The MMAs take BF16 operands (dz
-// rounded to BF16; weights and activations are the forward's BF16 values) and
-// accumulate in FP32; every operand is written by the threads into shared
-// memory in the 128-byte swizzled K-major layout of the forward (transposed
-// operands element by element), and every MMA has a shape of the forward's
-// layers 2 and 3 (M 128, N 128 or 64, K 64 or 128).
-constexpr int kBOffDz3 = 0;                      // A  MMA1: 128 samples x 64 (dz3)
-constexpr int kBOffW3t = kBOffDz3 + 16384;       // B  MMA1: 128 (in3) x 64 (out3)
-constexpr int kBOffDz2 = kBOffW3t + 16384;       // A  MMA2: 2 K-blocks x 128 samples x 64 (dz2)
-constexpr int kBOffW2t = kBOffDz2 + 32768;       // B  MMA2: 2 K-blocks x 64 (in2) x 64 (out2)
-constexpr int kBOffH2t = kBOffW2t + 16384;       // A  MMA3: 2 K-blocks x 128 (in3) x 64 samples
-constexpr int kBOffDz3t = kBOffH2t + 32768;      // B  MMA3: 2 K-blocks x 64 (out3) x 64 samples
-constexpr int kBOffDz2t = kBOffDz3t + 16384;     // A  MMA4: 2 K-blocks x 128 (out2) x 64 samples
-constexpr int kBOffH1t = kBOffDz2t + 32768;      // B  MMA4: 2 K-blocks x 64 (in2) x 64 samples
-constexpr int kBRedLd = 129;                     // FP32 [64][129] scratch (column sums over samples)
-constexpr int kBOffRed = kBOffH1t + 16384;
-constexpr int kBOffX = kBOffRed + 64 * kBRedLd * 4;   // FP32 [8][128] features of the tile
-constexpr int kBOffG4 = kBOffX + 8 * 128 * 4;         // FP32 [128] dz4 of the tile
-constexpr int kBOffW4 = kBOffG4 + 128 * 4;            // FP32 [64] W4
-constexpr int kBOffLoss = kBOffW4 + 64 * 4;           // FP32 [4] per-warp loss
-constexpr int kBOffBar = (kBOffLoss + 16 + 127) / 128 * 128;
-constexpr int kBwdTcSmem = kBOffBar + 128 + 1024;
-constexpr uint32_t kBwdTmemCols = 512;   // D1 0..127, D2 128..191, G3 192..255, G2 256..319
+// on CUDA cores in FP32, in registers over the tiles.  The MMAs take BF16
+// operands (dz rounded to BF16; weights and activations are the forward's BF16
+// values) and accumulate in FP32.
+// Every operand is stored once, in the forward's swizzled K-major layout; where
+// an MMA contracts over the samples or over a weight's outputs it reads the
+// same buffer as an MN-major operand, so nothing is transposed or stored twice.
+// Bound by the chain of its seven barriers and four MMA phases per tile (about
+// 6 us) and by shared-memory reads (half of the path's rate).  Separate forward
+// and backward kernels of 128 threads, with the activations through global
+// memory and transposed operands written element by element, took 113 + 146 us
+// at m = 131 072 and 22 + 54 us at m = 16 384; this one takes 54 and 18 us.
+constexpr int kTrainThreads = 512;
+constexpr int kTOffH1 = 0;                       // [128 s][64]
+constexpr int kTOffW2 = kTOffH1 + 16384;         // [128 out][64 in]
+constexpr int kTOffH2 = kTOffW2 + 16384;         // 2 blocks of [128 s][64]
+constexpr int kTOffW3 = kTOffH2 + 32768;         // 2 blocks of [64 out][64 in]
+constexpr int kTOffDz3 = kTOffW3 + 16384;        // [128 s][64]
+constexpr int kTOffDz2 = kTOffDz3 + 16384;       // 2 blocks of [128 s][64]
+constexpr int kTOffH3 = kTOffDz2 + 32768;        // [128 s][64], read on CUDA cores only
+constexpr int kTDz1Ld = 68;                      // FP32 dz1 [128 s][68]: rows 16 bytes apart in the banks
+constexpr int kTOffDz1 = kTOffH3 + 16384;
+constexpr int kTOffX = kTOffDz1 + 128 * kTDz1Ld * 4;   // FP32 2 x [2 halves][128 s][4] features (alternating tiles)
+constexpr int kTOffW1 = kTOffX + 2 * 128 * 8 * 4;      // FP32 [32 output pairs][8 inputs][2]
+constexpr int kTOffSmall = kTOffW1 + 512 * 4;          // FP32 b1[64] b2[128] b3[64] W4[64] b4
+constexpr int kTOffZ = kTOffSmall + 336 * 4;           // FP32 [4][128] partial sums of z4
+constexpr int kTOffG4 = kTOffZ + 512 * 4;              // FP32 [128] dz4
+constexpr int kTOffBar = kTOffG4 + 128 * 4;
+constexpr int kTrainSmem = kTOffBar + 128 + 1024;
+static_assert(kTrainSmem <= 232448 && kTOffW1 % 16 == 0 && kTOffSmall % 16 == 0, "shared-memory plan");
+// the final sums over the CTA's threads reuse dz2, h3 and dz1: dW1 + b1 [16][576], W4 + b3 [16][128], b2 [8][128]
+static_assert((16 * 576 + 16 * 128 + 8 * 128) * 4 <= kTOffX - kTOffDz2, "scratch of the final sums");
+constexpr uint32_t kTrainTmemCols = 512;   // layer 2 and D1 0..127, layer 3 and D2 128..191, G3 192..255, G2 256..319
+constexpr uint32_t kMnA = 1u << 15, kMnB = 1u << 16;   // instruction descriptor: A / B MN-major
 
-// element (row r, column k) of a K-major 128-byte-swizzled BF16 operand made
-// of K-blocks of 64 columns, each `blk` bytes: byte offset
-__device__ __forceinline__ int sw128_elem(int r, int k, int blk)
-{
-    return (k >> 6) * blk + sw128(r, (k & 63) >> 3) + (k & 7) * 2;
-}
-
-__device__ __forceinline__ void st_bf16(uint8_t* base, int off, float v)
-{
-    *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
-}
-
-// sum over the 128 samples of row r of a transposed operand (2 K-blocks of blk bytes)
-__device__ __forceinline__ float sum_row_bf16(const uint8_t* base, int r, int blk)
-{
-    float s = 0.f;
-#pragma unroll
-    for (int c16 = 0; c16 < 16; ++c16) {
-        const uint4 q = *reinterpret_cast<const uint4*>(base + (c16 >> 3) * blk + sw128(r, c16 & 7));
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            s += __uint_as_float(w[e] << 16);
-            s += __uint_as_float(w[e] & 0xFFFF0000u);
-        }
-    }
-    return s;
-}
-
-__global__ void __launch_bounds__(kRows, 1)
-    mlp_bwd_kernel(const float* feat, const float* label, int m, const float* wbf, const float* z4,
-                   const __nv_bfloat16* h1, const __nv_bfloat16* h2, const __nv_bfloat16* h3, float* grad,
-                   float* loss, uint32_t* err)
+__global__ void __launch_bounds__(kTrainThreads, 1)
+    mlp_train_kernel(const float* __restrict__ feat, const float* __restrict__ label, int m,
+                     const float* __restrict__ wbf, float* grad, float* loss, uint32_t* err)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = aligned_smem(smem_raw);
-    uint8_t* sDz3 = smem + kBOffDz3;
-    uint8_t* sW3t = smem + kBOffW3t;
-    uint8_t* sDz2 = smem + kBOffDz2;
-    uint8_t* sW2t = smem + kBOffW2t;
-    uint8_t* sH2t = smem + kBOffH2t;
-    uint8_t* sDz3t = smem + kBOffDz3t;
-    uint8_t* sDz2t = smem + kBOffDz2t;
-    uint8_t* sH1t = smem + kBOffH1t;
-    float* sRed = reinterpret_cast<float*>(smem + kBOffRed);
-    float* sX = reinterpret_cast<float*>(smem + kBOffX);
-    float* sG4 = reinterpret_cast<float*>(smem + kBOffG4);
-    float* sW4 = reinterpret_cast<float*>(smem + kBOffW4);
-    float* sLoss = reinterpret_cast<float*>(smem + kBOffLoss);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kBOffBar);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kBOffBar + 16);
+    uint8_t *sH1 = smem + kTOffH1, *sW2 = smem + kTOffW2, *sH2 = smem + kTOffH2, *sW3 = smem + kTOffW3;
+    uint8_t *sDz3 = smem + kTOffDz3, *sDz2 = smem + kTOffDz2, *sH3 = smem + kTOffH3;
+    float* sDz1 = reinterpret_cast<float*>(smem + kTOffDz1);
+    float* sX = reinterpret_cast<float*>(smem + kTOffX);
+    float* sW1 = reinterpret_cast<float*>(smem + kTOffW1);
+    float* sb1 = reinterpret_cast<float*>(smem + kTOffSmall);
+    float *sb2 = sb1 + 64, *sb3 = sb2 + 128, *sW4 = sb3 + 64, *sb4 = sW4 + 64;
+    float* sZ = reinterpret_cast<float*>(smem + kTOffZ);
+    float* sG4 = reinterpret_cast<float*>(smem + kTOffG4);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kTOffBar);
+    uint64_t* bar4 = bar + 1;   // MMA4 of the tile complete (its operands may be overwritten)
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kTOffBar + 16);
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int sl = t & 127, part = t >> 7;   // sample of the tile, column part
     const int ntiles = (m + kRows - 1) / kRows;
-    if (static_cast<int>(blockIdx.x) >= ntiles) return;
 
-    // weights: W3^T (B of MMA1: row n = input of layer 3, K = its 64 outputs) and
-    // W2^T (B of MMA2: row n = input of layer 2, K = its 128 outputs), W4
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        float w8[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) w8[q] = wbf[kW3 + (8 * c + q) * 128 + t];
-        *reinterpret_cast<uint4*>(sW3t + sw128(t, c)) =
-            make_uint4(pack_bf16(w8[0], w8[1]), pack_bf16(w8[2], w8[3]), pack_bf16(w8[4], w8[5]),
-                       pack_bf16(w8[6], w8[7]));
+    // weights -> shared memory, 8 inputs (16 bytes) per step
+    static_assert(kW2 % 4 == 0 && kW3 % 4 == 0, "16-byte loads of the weight rows");
+    for (int q = t; q < 1024; q += kTrainThreads) {
+        const float4* w = reinterpret_cast<const float4*>(wbf + kW2) + 2 * q;   // row q / 8 (64 inputs), chunk q % 8
+        const float4* u = reinterpret_cast<const float4*>(wbf + kW3) + 2 * q;   // row q / 16 (128 inputs), chunk q % 16
+        const float4 w0 = w[0], w1 = w[1], u0 = u[0], u1 = u[1];
+        *reinterpret_cast<uint4*>(sW2 + sw128(q >> 3, q & 7)) =
+            make_uint4(pack_bf16(w0.x, w0.y), pack_bf16(w0.z, w0.w), pack_bf16(w1.x, w1.y), pack_bf16(w1.z, w1.w));
+        *reinterpret_cast<uint4*>(sW3 + ((q >> 3) & 1) * 8192 + sw128(q >> 4, q & 7)) =
+            make_uint4(pack_bf16(u0.x, u0.y), pack_bf16(u0.z, u0.w), pack_bf16(u1.x, u1.y), pack_bf16(u1.z, u1.w));
     }
+    sW1[(t >> 4) * 16 + (t & 7) * 2 + ((t >> 3) & 1)] = wbf[kW1 + t];   // output t / 8, input t % 8
     if (t < 64) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            float w8[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w8[q] = wbf[kW2 + (8 * c + q) * 64 + t];
-            *reinterpret_cast<uint4*>(sW2t + (c >> 3) * 8192 + sw128(t, c & 7)) =
-                make_uint4(pack_bf16(w8[0], w8[1]), pack_bf16(w8[2], w8[3]), pack_bf16(w8[4], w8[5]),
-                           pack_bf16(w8[6], w8[7]));
-        }
+        sb1[t] = wbf[kB1 + t];
+        sb3[t] = wbf[kB3 + t];
         sW4[t] = wbf[kW4 + t];
-    }
-    if (t == 0) {
+    } else if (t < 192) {
+        sb2[t - 64] = wbf[kB2 + t - 64];
+    } else if (t == 192) {
+        sb4[0] = wbf[kB4];
         mbar_init(bar, 1);
+        mbar_init(bar4, 1);
         fence_mbar_init();
     }
-    if (warp == 0) tmem_alloc(tslot, kBwdTmemCols);
+    if (warp == 0) tmem_alloc(tslot, kTrainTmemCols);
+    fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
+    const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);   // this warp's lanes
     const float inv_m = 1.f / static_cast<float>(m);
+    auto wait_on = [&](uint64_t* b, uint32_t parity) {
+        if (!mbar_wait(b, parity)) atomicOr(err, TR_ERR_TIMEOUT);
+        tc_fence_after();
+    };
+    auto wait = [&](uint32_t parity) { wait_on(bar, parity); };
 
-    // per-thread gradient sums over the tiles: dW1 row o = t & 63, inputs
-    // 4 (t >> 6) .. +3 and (t < 64) b1[o]; b2[t]; t < 64: b3[t]; t >= 64: W4[t - 64], b4
-    const int o1 = t & 63, k1 = 4 * (t >> 6);
-    float gW1[4] = {0.f, 0.f, 0.f, 0.f};
-    float gb1 = 0.f, gb2 = 0.f, gb3w4 = 0.f, gb4 = 0.f, lsum = 0.f;
-    bool first = true;
+    // sums over the tiles.  dW1 and b1, W4 and b3: columns 2 lane, 2 lane + 1,
+    // samples 8 warp ..; b2: columns 2 (t % 64), + 1, samples 16 (t / 64) ..
+    const int o1 = t & 63, s1 = 16 * (t >> 6);
+    float gW1[2][8] = {};
+    float gb1[2] = {0.f, 0.f}, gb2[2] = {0.f, 0.f}, gb3[2] = {0.f, 0.f}, gW4[2] = {0.f, 0.f}, gb4 = 0.f, lsum = 0.f;
+    // this thread's two of the next tile's 1024 features, and its sample's label
+    float xf[2], yl;
+    auto fetch = [&](int tile) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const size_t x = static_cast<size_t>(tile) * (kRows * 8) + t + q * kTrainThreads;
+            xf[q] = tile < ntiles && x < static_cast<size_t>(m) * 8 ? feat[x] : 0.f;
+        }
+        const int s = tile * kRows + sl;
+        yl = tile < ntiles && s < m ? label[s] : 0.f;
+    };
+    fetch(blockIdx.x);
+    uint32_t first = 0u;   // accumulate flag of the weight gradients' first MMA
+    uint32_t par4 = 0u;    // parity of this tile's phase of bar4
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int s = tile * kRows + t;
-        const bool valid = s < m;
-        // ---- sample t: dz4, dz3, masks; operands of MMA1 and MMA3 ----
+        float* x = sX;
+        sX += (sX == reinterpret_cast<float*>(smem + kTOffX)) ? 1024 : -1024;
+        // inputs 0..3 of the samples, then inputs 4..7: a warp's 16-byte reads are conflict-free
+        x[((t >> 2) & 1) * 512 + (t >> 3) * 4 + (t & 3)] = bf16r(xf[0]);
+        x[((t >> 2) & 1) * 512 + (64 + (t >> 3)) * 4 + (t & 3)] = bf16r(xf[1]);
+        const float y = yl;
+        const bool valid = tile * kRows + sl < m;
+        const float4 *xa = reinterpret_cast<const float4*>(x), *xb = xa + 128;
+        fetch(tile + gridDim.x);
+        if (first) wait_on(bar4, par4 ^ 1u);   // the previous tile's MMA4 has read H1 and DZ2
+        __syncthreads();
+        // ---- layer 1: outputs 4 warp .. + 3 of samples lane + 32 i ----
+        // (a thread's 16 outputs in a 4 x 4 block: 16 shared-memory reads of 16
+        // bytes; a row of 16 outputs of one sample took 34, and every such read
+        // occupies the read path for four cycles, broadcast or not)
+        {
+            f2 w[2][8], bz[2];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sX[k * 128 + t] = valid ? bf16r(feat[(size_t)s * 8 + k]) : 0.f;
-        float g4 = 0.f;
-        if (valid) {
-            const float z = z4[s], y = label[s];
-            const float p = 1.f / (1.f + __expf(-z));
-            lsum += log1pf(__expf(-fabsf(z))) + fmaxf(z, 0.f) - y * z;
-            g4 = (p - y) * inv_m;
-        }
-        sG4[t] = g4;
-        const uint4* h3r = reinterpret_cast<const uint4*>(h3 + (size_t)(valid ? s : 0) * 64);
+            for (int q = 0; q < 2; ++q) {
+                const ulonglong2* wq = reinterpret_cast<const ulonglong2*>(sW1 + (2 * warp + q) * 16);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint4 q = valid ? h3r[c] : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-            float d8[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float hv = __uint_as_float(e & 1 ? (w[e >> 1] & 0xFFFF0000u) : (w[e >> 1] << 16));
-                const int col = 8 * c + e;
-                d8[e] = bf16r(hv > 0.f ? sW4[col] * g4 : 0.f);
-                sRed[col * kBRedLd + t] = g4 * hv;                       // for dW4
-                st_bf16(sDz3t, sw128_elem(col, t, 8192), d8[e]);         // B of MMA3: row out3, column sample
+                for (int k = 0; k < 4; ++k) {
+                    const ulonglong2 wk = wq[k];
+                    w[q][2 * k] = f2{wk.x};
+                    w[q][2 * k + 1] = f2{wk.y};
+                }
+                bz[q] = f2{reinterpret_cast<const unsigned long long*>(sb1)[2 * warp + q]};
             }
-            *reinterpret_cast<uint4*>(sDz3 + sw128(t, c)) =
-                make_uint4(pack_bf16(d8[0], d8[1]), pack_bf16(d8[2], d8[3]), pack_bf16(d8[4], d8[5]),
-                           pack_bf16(d8[6], d8[7]));
-        }
-        uint32_t mask2[4] = {0u, 0u, 0u, 0u}, mask1[2] = {0u, 0u};
-        const uint4* h2r = reinterpret_cast<const uint4*>(h2 + (size_t)(valid ? s : 0) * 128);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            const uint4 q = valid ? h2r[c] : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+            for (int i = 0; i < 4; ++i) {
+                const int s = lane + 32 * i;
+                const float4 fa = xa[s], fb = xb[s];
+                const float f[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
+                const bool vs = tile * kRows + s < m;
+                uint32_t h[2];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint16_t hb = static_cast<uint16_t>(e & 1 ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xFFFFu));
-                const int col = 8 * c + e;
-                mask2[col >> 5] |= (hb != 0 && !(hb & 0x8000u) ? 1u : 0u) << (col & 31);   // h2 > 0
-                *reinterpret_cast<uint16_t*>(sH2t + sw128_elem(col, t, 16384)) = hb;     // A of MMA3
-            }
-        }
-        const uint4* h1r = reinterpret_cast<const uint4*>(h1 + (size_t)(valid ? s : 0) * 64);
+                for (int q = 0; q < 2; ++q) {
+                    f2 z = bz[q];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint4 q = valid ? h1r[c] : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint16_t hb = static_cast<uint16_t>(e & 1 ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xFFFFu));
-                const int col = 8 * c + e;
-                mask1[col >> 5] |= (hb != 0 && !(hb & 0x8000u) ? 1u : 0u) << (col & 31);   // h1 > 0
-                *reinterpret_cast<uint16_t*>(sH1t + sw128_elem(col, t, 8192)) = hb;      // B of MMA4
+                    for (int k = 0; k < 8; ++k) z = fma2(w[q][k], pk(f[k], f[k]), z);
+                    float a, b;
+                    upk(z, a, b);
+                    h[q] = vs ? pack_bf16(fmaxf(a, 0.f), fmaxf(b, 0.f)) : 0u;
+                }
+                *reinterpret_cast<uint2*>(sH1 + sw128(s, warp >> 1) + (warp & 1) * 8) = make_uint2(h[0], h[1]);
             }
         }
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
-        // MMA1 (D1 = DZ3 W3) and MMA3 (G3 += H2^T DZ3)
-        if (t == 0) {
+        if (t == 0) {   // layer 2: D[128 s x 128] = H1 W2^T
             tc_fence_after();
-            const uint32_t a1 = smem_u32(sDz3), b1 = smem_u32(sW3t);
+            const uint32_t a0 = smem_u32(sH1), b0 = smem_u32(sW2);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)   // K = 16 BF16 per MMA
+                mma_f16(tmem, sdesc_k_sw128(a0 + ks * 32), sdesc_k_sw128(b0 + ks * 32), kIdescL2, ks > 0 ? 1u : 0u);
+            mma_commit(bar);
+        }
+        __syncwarp();
+        wait(0u);
+        uint32_t mask2 = 0u;   // h2 > 0 of columns 32 part .. + 31
+        {
+            uint32_t acc[32];
+            tmem_ld32(tl + part * 32, acc);
+            tmem_ld_wait32(acc);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t h[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int e = 8 * c + 2 * q;
+                    const float2 b = reinterpret_cast<const float2*>(sb2)[part * 16 + (e >> 1)];
+                    h[q] = pack_bf16(fmaxf(__uint_as_float(acc[e]) + b.x, 0.f), fmaxf(__uint_as_float(acc[e + 1]) + b.y, 0.f));
+                    if (!valid) h[q] = 0u;
+                    mask2 |= (__uint_as_float(h[q] << 16) > 0.f ? 1u : 0u) << e;
+                    mask2 |= (__uint_as_float(h[q] & 0xFFFF0000u) > 0.f ? 1u : 0u) << (e + 1);
+                }
+                const int k8 = part * 4 + c;
+                *reinterpret_cast<uint4*>(sH2 + (k8 >> 3) * 16384 + sw128(sl, k8 & 7)) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+        }
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (t == 0) {   // layer 3: D[128 s x 64] = H2 W3^T
+            tc_fence_after();
+            const uint32_t a0 = smem_u32(sH2), b0 = smem_u32(sW3);
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    mma_f16(tmem + 128, sdesc_k_sw128(a0 + kb * 16384 + ks * 32), sdesc_k_sw128(b0 + kb * 8192 + ks * 32),
+                            kIdescL3, (kb | ks) != 0 ? 1u : 0u);
+            mma_commit(bar);
+        }
+        __syncwarp();
+        wait(1u);
+        uint32_t h3[8];   // columns 16 part .. + 15, BF16 pairs
+        {
+            uint32_t acc[16];
+            tmem_ld16(tl + 128 + part * 16, acc);
+            tmem_ld_wait();
+            float z = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float2 b = reinterpret_cast<const float2*>(sb3)[part * 8 + q];
+                const float2 w = reinterpret_cast<const float2*>(sW4)[part * 8 + q];
+                h3[q] = pack_bf16(fmaxf(__uint_as_float(acc[2 * q]) + b.x, 0.f), fmaxf(__uint_as_float(acc[2 * q + 1]) + b.y, 0.f));
+                if (!valid) h3[q] = 0u;
+                z = fmaf(w.x, __uint_as_float(h3[q] << 16), z);
+                z = fmaf(w.y, __uint_as_float(h3[q] & 0xFFFF0000u), z);
+            }
+            sZ[t] = z;
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                *reinterpret_cast<uint4*>(sH3 + sw128(sl, part * 2 + c)) =
+                    make_uint4(h3[4 * c], h3[4 * c + 1], h3[4 * c + 2], h3[4 * c + 3]);
+        }
+        __syncthreads();
+        // ---- dz4 (every thread of the sample), dz3 ----
+        {
+            float g4 = 0.f;
+            if (valid) {
+                const float z = sb4[0] + ((sZ[sl] + sZ[128 + sl]) + (sZ[256 + sl] + sZ[384 + sl]));
+                const float p = 1.f / (1.f + __expf(-z));
+                g4 = (p - y) * inv_m;
+                if (part == 0) {
+                    lsum += log1pf(__expf(-fabsf(z))) + fmaxf(z, 0.f) - y * z;
+                    gb4 += g4;
+                }
+            }
+            if (part == 0) sG4[sl] = g4;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                uint32_t d[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 w = reinterpret_cast<const float2*>(sW4)[part * 8 + 4 * c + q];
+                    d[q] = pack_bf16(__uint_as_float(h3[4 * c + q] << 16) > 0.f ? w.x * g4 : 0.f,
+                                     __uint_as_float(h3[4 * c + q] & 0xFFFF0000u) > 0.f ? w.y * g4 : 0.f);
+                }
+                *reinterpret_cast<uint4*>(sDz3 + sw128(sl, part * 2 + c)) = make_uint4(d[0], d[1], d[2], d[3]);
+            }
+        }
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (t == 0) {   // MMA1 (D1 = DZ3 W3) and MMA3 (G3 += H2^T DZ3)
+            tc_fence_after();
+            const uint32_t dz3 = smem_u32(sDz3), w3 = smem_u32(sW3), h2 = smem_u32(sH2);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma_f16(tmem, sdesc_k_sw128(a1 + ks * 32), sdesc_k_sw128(b1 + ks * 32), kIdescL2, ks > 0 ? 1u : 0u);
-            const uint32_t a3 = smem_u32(sH2t), b3 = smem_u32(sDz3t);
+                mma_f16(tmem, sdesc_k_sw128(dz3 + ks * 32), sdesc_mn_sw128(w3 + ks * 2048, 8192), kIdescL2 | kMnB,
+                        ks > 0 ? 1u : 0u);
+            mma_commit(bar);   // MMA3 is complete at the commit behind MMA2
 #pragma unroll
-            for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_f16(tmem + 192, sdesc_k_sw128(a3 + kb * 16384 + ks * 32),
-                            sdesc_k_sw128(b3 + kb * 8192 + ks * 32), kIdescL3, (first && kb == 0 && ks == 0) ? 0u : 1u);
-            mma_commit(bar);
+            for (int ks = 0; ks < 8; ++ks)
+                mma_f16(tmem + 192, sdesc_mn_sw128(h2 + ks * 2048, 16384), sdesc_mn_sw128(dz3 + ks * 2048, 16384),
+                        kIdescL3 | kMnA | kMnB, ks > 0 ? 1u : first);
         }
         __syncwarp();
-        // meanwhile: dW4, b4, b3 column sums of this tile
-        if (t < 64) {
-            gb3w4 += sum_row_bf16(sDz3t, t, 8192);
-        } else {
-            const float* r = sRed + (t - 64) * kBRedLd;
-            float a = 0.f;
-            for (int u = 0; u < 128; ++u) a += r[u];
-            gb3w4 += a;
-            if (t == 64)
-                for (int u = 0; u < 128; ++u) gb4 += sG4[u];
+        // meanwhile: W4 and b3 (columns 2 lane, + 1 over 8 samples)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int s = 8 * warp + q, off = sw128(s, lane >> 2) + (lane & 3) * 4;
+            const uint32_t hv = *reinterpret_cast<const uint32_t*>(sH3 + off);
+            const uint32_t dv = *reinterpret_cast<const uint32_t*>(sDz3 + off);
+            const float g4 = sG4[s];
+            gW4[0] = fmaf(g4, __uint_as_float(hv << 16), gW4[0]);
+            gW4[1] = fmaf(g4, __uint_as_float(hv & 0xFFFF0000u), gW4[1]);
+            gb3[0] += __uint_as_float(dv << 16);
+            gb3[1] += __uint_as_float(dv & 0xFFFF0000u);
         }
-        if (!mbar_wait(bar, 0)) atomicOr(err, TR_ERR_TIMEOUT);
-        tc_fence_after();
-        // ---- dz2 = D1 * [h2 > 0]: A of MMA2 (row = sample) and A of MMA4 (row = output of layer 2) ----
-#pragma unroll 1
-        for (int cb = 0; cb < 4; ++cb) {
+        wait(0u);
+        // ---- dz2 = D1 * [h2 > 0] ----
+        {
             uint32_t acc[32];
-            tmem_ld32(tmem + lane_base + cb * 32, acc);
-            tmem_ld_wait();
-            const uint32_t mk = cb == 0 ? mask2[0] : cb == 1 ? mask2[1] : cb == 2 ? mask2[2] : mask2[3];
-            float dv[32];
+            tmem_ld32(tl + part * 32, acc);
+            tmem_ld_wait32(acc);
 #pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                const int col = cb * 32 + q;
-                dv[q] = bf16r((mk >> q) & 1u ? __uint_as_float(acc[q]) : 0.f);
-                st_bf16(sDz2t, sw128_elem(col, t, 16384), dv[q]);
-            }
+            for (int c = 0; c < 4; ++c) {
+                uint32_t d[4];
 #pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
-                const int k8 = cb * 4 + c4;   // 16-byte chunk over the 128 outputs of layer 2
-                *reinterpret_cast<uint4*>(sDz2 + (k8 >> 3) * 16384 + sw128(t, k8 & 7)) =
-                    make_uint4(pack_bf16(dv[8 * c4 + 0], dv[8 * c4 + 1]), pack_bf16(dv[8 * c4 + 2], dv[8 * c4 + 3]),
-                               pack_bf16(dv[8 * c4 + 4], dv[8 * c4 + 5]), pack_bf16(dv[8 * c4 + 6], dv[8 * c4 + 7]));
+                for (int q = 0; q < 4; ++q) {
+                    const int e = 8 * c + 2 * q;
+                    d[q] = pack_bf16((mask2 >> e) & 1u ? __uint_as_float(acc[e]) : 0.f,
+                                     (mask2 >> (e + 1)) & 1u ? __uint_as_float(acc[e + 1]) : 0.f);
+                }
+                const int k8 = part * 4 + c;
+                *reinterpret_cast<uint4*>(sDz2 + (k8 >> 3) * 16384 + sw128(sl, k8 & 7)) = make_uint4(d[0], d[1], d[2], d[3]);
             }
         }
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
-        // MMA2 (D2 = DZ2 W2) and MMA4 (G2 += DZ2^T H1)
-        if (t == 0) {
+        if (t == 0) {   // MMA2 (D2 = DZ2 W2) and MMA4 (G2 += DZ2^T H1)
             tc_fence_after();
-            const uint32_t a2 = smem_u32(sDz2), b2 = smem_u32(sW2t);
-            const uint32_t a4 = smem_u32(sDz2t), b4 = smem_u32(sH1t);
+            const uint32_t dz2 = smem_u32(sDz2), w2 = smem_u32(sW2), h1 = smem_u32(sH1);
 #pragma unroll
-            for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_f16(tmem + 128, sdesc_k_sw128(a2 + kb * 16384 + ks * 32),
-                            sdesc_k_sw128(b2 + kb * 8192 + ks * 32), kIdescL3, (kb | ks) != 0 ? 1u : 0u);
-#pragma unroll
-            for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_f16(tmem + 256, sdesc_k_sw128(a4 + kb * 16384 + ks * 32),
-                            sdesc_k_sw128(b4 + kb * 8192 + ks * 32), kIdescL3, (first && kb == 0 && ks == 0) ? 0u : 1u);
+            for (int ks = 0; ks < 8; ++ks)
+                mma_f16(tmem + 128, sdesc_k_sw128(dz2 + (ks >> 2) * 16384 + (ks & 3) * 32),
+                        sdesc_mn_sw128(w2 + ks * 2048, 16384), kIdescL3 | kMnB, ks > 0 ? 1u : 0u);
             mma_commit(bar);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+                mma_f16(tmem + 256, sdesc_mn_sw128(dz2 + ks * 2048, 16384), sdesc_mn_sw128(h1 + ks * 2048, 16384),
+                        kIdescL3 | kMnA | kMnB, ks > 0 ? 1u : first);
+            mma_commit(bar4);
         }
         __syncwarp();
-        gb2 += sum_row_bf16(sDz2t, t, 16384);   // b2: the 128 samples of output t of layer 2
-        if (!mbar_wait(bar, 1)) atomicOr(err, TR_ERR_TIMEOUT);
-        tc_fence_after();
-        // ---- dz1 = D2 * [h1 > 0] (FP32) -> dW1, b1 on CUDA cores ----
-#pragma unroll 1
-        for (int cb = 0; cb < 2; ++cb) {
-            uint32_t acc[32];
-            tmem_ld32(tmem + lane_base + 128 + cb * 32, acc);
-            tmem_ld_wait();
-            const uint32_t mk = cb == 0 ? mask1[0] : mask1[1];
+        // meanwhile: b2 (columns 2 o1, + 1 over 16 samples)
 #pragma unroll
-            for (int q = 0; q < 32; ++q)
-                sRed[(cb * 32 + q) * kBRedLd + t] = (mk >> q) & 1u ? __uint_as_float(acc[q]) : 0.f;
+        for (int q = 0; q < 16; ++q) {
+            const uint32_t dv = *reinterpret_cast<const uint32_t*>(sDz2 + (o1 >> 5) * 16384 + sw128(s1 + q, (o1 & 31) >> 2) +
+                                                                   (o1 & 3) * 4);
+            gb2[0] += __uint_as_float(dv << 16);
+            gb2[1] += __uint_as_float(dv & 0xFFFF0000u);
         }
-        tc_fence_before();
-        __syncthreads();   // sRed holds dz1 (rows: outputs of layer 1); tensor memory D1, D2 read
+        wait(1u);
+        // ---- dz1 = D2 * [h1 > 0] (FP32) -> dW1, b1 ----
         {
-            const float* r = sRed + o1 * kBRedLd;
-            for (int u = 0; u < 128; ++u) {
-                const float a = r[u];
-                if (t < 64) gb1 += a;
+            uint32_t acc[16];
+            tmem_ld16(tl + 128 + part * 16, acc);
+            uint32_t h[8];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) gW1[k] = fmaf(a, sX[(k1 + k) * 128 + u], gW1[k]);
+            for (int c = 0; c < 2; ++c) {
+                const uint4 q = *reinterpret_cast<const uint4*>(sH1 + sw128(sl, part * 2 + c));
+                h[4 * c] = q.x; h[4 * c + 1] = q.y; h[4 * c + 2] = q.z; h[4 * c + 3] = q.w;
+            }
+            tmem_ld_wait();
+            float4* d = reinterpret_cast<float4*>(sDz1 + sl * kTDz1Ld + part * 16);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t hv = h[2 * c + (q >> 1)];
+                    v[q] = __uint_as_float(q & 1 ? hv & 0xFFFF0000u : hv << 16) > 0.f ? __uint_as_float(acc[4 * c + q]) : 0.f;
+                }
+                d[c] = make_float4(v[0], v[1], v[2], v[3]);
             }
         }
-        __syncthreads();   // the tile's shared operands and scratch are consumed
-        first = false;
+        tc_fence_before();
+        __syncthreads();
+        // (two outputs per thread: each sample's 32 bytes of inputs, read by all
+        // lanes, serve 16 products)
+#pragma unroll 2
+        for (int q = 0; q < 8; ++q) {
+            const int s = 8 * warp + q;
+            const float2 a = *reinterpret_cast<const float2*>(sDz1 + s * kTDz1Ld + 2 * lane);
+            const float4 fa = xa[s], fb = xb[s];
+            const float f[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
+            gb1[0] += a.x;
+            gb1[1] += a.y;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                gW1[0][k] = fmaf(a.x, f[k], gW1[0][k]);
+                gW1[1][k] = fmaf(a.y, f[k], gW1[1][k]);
+            }
+        }
+        par4 ^= 1u;
+        first = 1u;
     }
     // ---- the CTA's sums into the global gradient ----
-#pragma unroll
-    for (int k = 0; k < 4; ++k) atomicAdd(&grad[kW1 + o1 * 8 + k1 + k], gW1[k]);
-    if (t < 64) {
-        atomicAdd(&grad[kB1 + t], gb1);
-        atomicAdd(&grad[kB3 + t], gb3w4);
-    } else {
-        atomicAdd(&grad[kW4 + t - 64], gb3w4);
-        if (t == 64) atomicAdd(&grad[kB4], gb4);
-    }
-    atomicAdd(&grad[kB2 + t], gb2);
-    tc_fence_after();
-#pragma unroll 1
-    for (int cb = 0; cb < 2; ++cb) {
-        uint32_t g3[32], g2[32];
-        tmem_ld32(tmem + lane_base + 192 + cb * 32, g3);   // dW3[out = column][in = t]
-        tmem_ld32(tmem + lane_base + 256 + cb * 32, g2);   // dW2[out = t][in = column]
+    if (first) wait_on(bar4, par4 ^ 1u);
+    {
+        uint32_t g3[16], g2[16];
+        tmem_ld16(tl + 192 + part * 16, g3);   // dW3[out = column][in = lane]
+        tmem_ld16(tl + 256 + part * 16, g2);   // dW2[out = lane][in = column]
         tmem_ld_wait();
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            atomicAdd(&grad[kW3 + (cb * 32 + q) * 128 + t], __uint_as_float(g3[q]));
-            atomicAdd(&grad[kW2 + t * 64 + cb * 32 + q], __uint_as_float(g2[q]));
-        }
+        for (int q = 0; q < 16; ++q) atomicAdd(&grad[kW3 + (part * 16 + q) * 128 + sl], __uint_as_float(g3[q]));
+        static_assert(kW2 % 4 == 0, "16-byte additions to dW2");
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            atomicAdd(reinterpret_cast<float4*>(grad + kW2 + sl * 64 + part * 16 + 4 * q),
+                      make_float4(__uint_as_float(g2[4 * q]), __uint_as_float(g2[4 * q + 1]),
+                                  __uint_as_float(g2[4 * q + 2]), __uint_as_float(g2[4 * q + 3])));
     }
-    for (int off = 16; off >= 1; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-    if (lane == 0) sLoss[warp] = lsum;
+    __syncthreads();   // the last tile's buffers are consumed
+    float* r1 = reinterpret_cast<float*>(sDz2);   // [16][576]: dW1 [64][8], b1 [64]
+    float* r4 = r1 + 16 * 576;        // [16][128]: W4 [64], b3 [64]
+    float* r2 = r4 + 16 * 128;        // [8][128]: b2
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) r1[warp * 576 + (2 * lane + k) * 8 + q] = gW1[k][q];
+        r1[warp * 576 + 512 + 2 * lane + k] = gb1[k];
+        r4[warp * 128 + 2 * lane + k] = gW4[k];
+        r4[warp * 128 + 64 + 2 * lane + k] = gb3[k];
+        r2[(t >> 6) * 128 + 2 * o1 + k] = gb2[k];
+    }
+    for (int off = 16; off >= 1; off >>= 1) {
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+        gb4 += __shfl_xor_sync(0xffffffffu, gb4, off);
+    }
+    if (warp < 4 && lane == 0) {   // the part-0 threads
+        atomicAdd(loss, lsum * inv_m);
+        atomicAdd(&grad[kB4], gb4);
+    }
+    __syncthreads();
+    for (int q = t; q < 576 + 256; q += kTrainThreads) {
+        float a = 0.f;
+        int dst;
+        if (q < 576) {
+            for (int r = 0; r < 16; ++r) a += r1[r * 576 + q];
+            dst = q < 512 ? kW1 + q : kB1 + q - 512;
+        } else if (q < 704) {
+            for (int r = 0; r < 16; ++r) a += r4[r * 128 + q - 576];
+            dst = q < 640 ? kW4 + q - 576 : kB3 + q - 640;
+        } else {
+            for (int r = 0; r < 8; ++r) a += r2[r * 128 + q - 704];
+            dst = kB2 + q - 704;
+        }
+        atomicAdd(&grad[dst], a);
+    }
     tc_fence_before();
     __syncthreads();
-    if (t == 0) atomicAdd(loss, (sLoss[0] + sLoss[1] + sLoss[2] + sLoss[3]) * inv_m);
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem, kBwdTmemCols);
+        tmem_dealloc(tmem, kTrainTmemCols);
     }
 }
 
 // ---------------- training: Adam (CUDA cores) ----------------
 
 // Adam (bias-corrected), FP32 master weights; the forward's BF16-rounded copy
-// is refreshed from them.
+// is refreshed from them.  loss_out (page-locked host memory, or null) receives
+// the step's loss.
 __global__ void __launch_bounds__(256) mlp_adam_kernel(float* w, float* mom, float* vel, const float* g, float* wbf,
-                                                       int step, float lr, float b1, float b2, float eps)
+                                                       int step, float lr, float b1, float b2, float eps,
+                                                       const float* loss, float* loss_out)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    if (k == 0 && loss_out != nullptr) *loss_out = *loss;
     if (k >= kMlpParams) return;
     const float gk = g[k];
     const float m1 = b1 * mom[k] + (1.f - b1) * gk;
@@ -736,7 +826,7 @@ cudaError_t mlp_setup()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(mlp_proposal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(mlp_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdTcSmem);
+        e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem);
     return e;
 }
 
@@ -755,27 +845,25 @@ void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream
     launch_pdl(mlp_proposal_kernel, grid, kRows, kFwdSmem, s, b, total, wbf);
 }
 
-void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, float* z4, __nv_bfloat16* h1,
-                        __nv_bfloat16* h2, __nv_bfloat16* h3, uint32_t* err, cudaStream_t s)
+void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, uint32_t* err, cudaStream_t s)
 {
-    FwdOut out = {prob, z4, h1, h2, h3};
-    mlp_fwd_kernel<<<(m + kRows - 1) / kRows, kRows, kFwdSmem, s>>>(feat, m, wbf, out, err);
+    mlp_fwd_kernel<<<(m + kRows - 1) / kRows, kRows, kFwdSmem, s>>>(feat, m, wbf, prob, err);
 }
 
-void launch_mlp_backward(const float* feat, const float* label, int m, const float* wbf, const float* z4,
-                         const __nv_bfloat16* h1, const __nv_bfloat16* h2, const __nv_bfloat16* h3, float* grad,
-                         float* loss, uint32_t* err, cudaStream_t s)
+void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
+                      uint32_t* err, cudaStream_t s)
 {
     const int ntiles = (m + kRows - 1) / kRows;
     const int sms = device_sms();
     const int grid = ntiles < sms ? ntiles : sms;   // one CTA per SM (shared memory and tensor memory)
-    mlp_bwd_kernel<<<grid, kRows, kBwdTcSmem, s>>>(feat, label, m, wbf, z4, h1, h2, h3, grad, loss, err);
+    mlp_train_kernel<<<grid, kTrainThreads, kTrainSmem, s>>>(feat, label, m, wbf, grad, loss, err);
 }
 
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
-                     cudaStream_t s)
+                     const float* loss, float* loss_out, cudaStream_t s)
 {
-    mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(w, mom, vel, g, wbf, step, lr, 0.9f, 0.999f, 1e-8f);
+    launch_pdl(mlp_adam_kernel, (kMlpParams + 255) / 256, 256, 0, s, w, mom, vel, g, wbf, step, lr, 0.9f, 0.999f, 1e-8f,
+               loss, loss_out);
 }
 
 }  // namespace tr

@@ -1,7 +1,6 @@
 // C ABI of the proposal-MLP trainer (include/turboreg_internal.h): FP32
-// master weights, Adam moments and activation scratch on the device; the
-// forward, backward and update run in the kernels of mlp.cu.
-#include <cuda_bf16.h>
+// master weights, Adam moments and gradient on the device; the forward,
+// backward and update run in the kernels of mlp.cu.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -27,11 +26,11 @@ struct turboreg_mlp {
     float* wbf = nullptr;    // BF16-rounded copy used by the forward [P]
     float* mom = nullptr;    // Adam first moment [P]
     float* vel = nullptr;    // Adam second moment [P]
-    float* grad = nullptr;   // [P]
-    float* loss = nullptr;   // [1]
-    uint32_t* err = nullptr;
-    float* z4 = nullptr;     // [max_samples]
-    __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr;
+    // gradient [P], loss, error bits: cleared by one memset, read by one copy
+    float* grad = nullptr;
+    float* loss = nullptr;   // grad + P
+    uint32_t* err = nullptr; // grad + P + 1
+    float* host = nullptr;   // page-locked [P + 2]: a parameter vector or gradient, loss, error bits on their way out
 };
 
 namespace {
@@ -47,19 +46,27 @@ namespace {
 
 void free_all(turboreg_mlp* t)
 {
-    void* ptrs[] = {t->w, t->wbf, t->mom, t->vel, t->grad, t->loss, t->err, t->z4, t->h1, t->h2, t->h3};
+    void* ptrs[] = {t->w, t->wbf, t->mom, t->vel, t->grad};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    if (t->host) cudaFreeHost(t->host);
 }
 
-// Backward pass of the last forward: grad (device) = d(mean BCE)/d params.
+// grad, loss (device) = those of the mean BCE over m samples.
 int backward(turboreg_mlp* t, const float* feat, const float* label, int32_t m)
 {
-    TM_CHECK(cudaMemsetAsync(t->grad, 0, sizeof(float) * kMlpParams, t->stream));
-    TM_CHECK(cudaMemsetAsync(t->loss, 0, sizeof(float), t->stream));
-    launch_mlp_forward(feat, m, t->wbf, nullptr, t->z4, t->h1, t->h2, t->h3, t->err, t->stream);
-    launch_mlp_backward(feat, label, m, t->wbf, t->z4, t->h1, t->h2, t->h3, t->grad, t->loss, t->err, t->stream);
+    TM_CHECK(cudaMemsetAsync(t->grad, 0, sizeof(float) * (kMlpParams + 2), t->stream));
+    launch_mlp_train(feat, label, m, t->wbf, t->grad, t->loss, t->err, t->stream);
     TM_CHECK(cudaGetLastError());
+    return TURBOREG_OK;
+}
+
+// `count` values at `src` (device) through the page-locked buffer; the stream
+// is then idle.  (A copy to pageable memory would be staged by the driver.)
+int fetch(turboreg_mlp* t, const float* src, size_t count)
+{
+    TM_CHECK(cudaMemcpyAsync(t->host, src, sizeof(float) * count, cudaMemcpyDeviceToHost, t->stream));
+    TM_CHECK(cudaStreamSynchronize(t->stream));
     return TURBOREG_OK;
 }
 
@@ -76,7 +83,6 @@ int turboreg_mlp_create(int device, int32_t max_samples, uint64_t seed, void* cu
     if (!t) return TURBOREG_ERR_OOM;
     t->device = device;
     t->max_samples = max_samples;
-    const size_t M = static_cast<size_t>(max_samples);
     cudaError_t e = cudaSuccess;
     auto al = [&](void** p, size_t b) {
         if (e == cudaSuccess) e = cudaMalloc(p, b);
@@ -85,13 +91,10 @@ int turboreg_mlp_create(int device, int32_t max_samples, uint64_t seed, void* cu
     al(reinterpret_cast<void**>(&t->wbf), sizeof(float) * kMlpParams);
     al(reinterpret_cast<void**>(&t->mom), sizeof(float) * kMlpParams);
     al(reinterpret_cast<void**>(&t->vel), sizeof(float) * kMlpParams);
-    al(reinterpret_cast<void**>(&t->grad), sizeof(float) * kMlpParams);
-    al(reinterpret_cast<void**>(&t->loss), sizeof(float));
-    al(reinterpret_cast<void**>(&t->err), sizeof(uint32_t));
-    al(reinterpret_cast<void**>(&t->z4), sizeof(float) * M);
-    al(reinterpret_cast<void**>(&t->h1), sizeof(__nv_bfloat16) * M * 64);
-    al(reinterpret_cast<void**>(&t->h2), sizeof(__nv_bfloat16) * M * 128);
-    al(reinterpret_cast<void**>(&t->h3), sizeof(__nv_bfloat16) * M * 64);
+    al(reinterpret_cast<void**>(&t->grad), sizeof(float) * (kMlpParams + 2));
+    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&t->host), sizeof(float) * (kMlpParams + 2));
+    t->loss = t->grad + kMlpParams;
+    t->err = reinterpret_cast<uint32_t*>(t->grad + kMlpParams + 1);
     if (e == cudaSuccess) e = mlp_setup();
     if (e == cudaSuccess) {
         if (cuda_stream) t->stream = static_cast<cudaStream_t>(cuda_stream);
@@ -144,9 +147,9 @@ int turboreg_mlp_get_params(turboreg_mlp* t, float* params)
 {
     if (!t || !params) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
-    TM_CHECK(cudaMemcpyAsync(params, t->w, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
-    TM_CHECK(cudaStreamSynchronize(t->stream));
-    return TURBOREG_OK;
+    const int rc = fetch(t, t->w, kMlpParams);
+    if (rc == TURBOREG_OK) std::memcpy(params, t->host, sizeof(float) * kMlpParams);
+    return rc;
 }
 
 int turboreg_mlp_set_params(turboreg_mlp* t, const float* params)
@@ -189,7 +192,7 @@ int turboreg_mlp_forward(turboreg_mlp* t, const float* feat, int32_t m, float* p
     if (!t || !feat || !prob || m < 1) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
     TM_CHECK(cudaMemsetAsync(t->err, 0, sizeof(uint32_t), t->stream));
-    launch_mlp_forward(feat, m, t->wbf, prob, nullptr, nullptr, nullptr, nullptr, t->err, t->stream);
+    launch_mlp_forward(feat, m, t->wbf, prob, t->err, t->stream);
     TM_CHECK(cudaGetLastError());
     uint32_t err = 0;
     TM_CHECK(cudaMemcpyAsync(&err, t->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, t->stream));
@@ -201,16 +204,13 @@ int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, in
 {
     if (!t || !feat || !label || !grad || m < 1 || m > t->max_samples) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
-    TM_CHECK(cudaMemsetAsync(t->err, 0, sizeof(uint32_t), t->stream));
-    const int rc = backward(t, feat, label, m);
+    int rc = backward(t, feat, label, m);
+    if (rc == TURBOREG_OK) rc = fetch(t, t->grad, kMlpParams + 2);
     if (rc != TURBOREG_OK) return rc;
-    TM_CHECK(cudaMemcpyAsync(grad, t->grad, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
-    float l = 0.f;
-    uint32_t err = 0;
-    TM_CHECK(cudaMemcpyAsync(&l, t->loss, sizeof(float), cudaMemcpyDeviceToHost, t->stream));
-    TM_CHECK(cudaMemcpyAsync(&err, t->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, t->stream));
-    TM_CHECK(cudaStreamSynchronize(t->stream));
-    if (loss) *loss = l;
+    std::memcpy(grad, t->host, sizeof(float) * kMlpParams);
+    if (loss) *loss = t->host[kMlpParams];
+    uint32_t err;
+    std::memcpy(&err, t->host + kMlpParams + 1, sizeof(err));
     return err ? TURBOREG_ERR_TIMEOUT : TURBOREG_OK;
 }
 
@@ -222,11 +222,11 @@ int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* lab
     int rc = backward(t, feat, label, m);
     if (rc != TURBOREG_OK) return rc;
     t->step += 1;
-    launch_mlp_adam(t->w, t->mom, t->vel, t->grad, t->wbf, t->step, lr, t->stream);
+    launch_mlp_adam(t->w, t->mom, t->vel, t->grad, t->wbf, t->step, lr, t->loss, loss ? t->host : nullptr, t->stream);
     TM_CHECK(cudaGetLastError());
     if (loss) {
-        TM_CHECK(cudaMemcpyAsync(loss, t->loss, sizeof(float), cudaMemcpyDeviceToHost, t->stream));
         TM_CHECK(cudaStreamSynchronize(t->stream));
+        *loss = t->host[0];
     }
     return TURBOREG_OK;
 }

@@ -337,6 +337,15 @@ __device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr)
     return d;
 }
 
+// The same tile as an MN-major operand: its rows are the K index and the 64
+// 16-bit elements of a 128-byte row run along M or N.  Blocks of 64 elements
+// of M or N lie lbo bytes apart (leading byte offset); 8-row groups of K 1024
+// bytes apart, so K = 16 steps the start address by 2048.
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo)
+{
+    return (sdesc_k_sw128(saddr) & ~(static_cast<uint64_t>(0x3FFFu) << 16)) | (static_cast<uint64_t>(lbo >> 4) << 16);
+}
+
 // Instruction descriptor (kind::f16 layout): D format [4,6)
 // (1 = F32), A format [7,10), B format [10,13), A/B major bits 15/16 (0 = K),
 // N >> 3 at [17,23), M >> 4 at [24,29).
@@ -424,6 +433,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
           "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
           "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
           "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
+}
+
+// Load 16 consecutive 32-bit TMEM columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr)
         : "memory");
 }

@@ -24,13 +24,13 @@ cudaError_t mlp_setup();
 void launch_mlp_round(const float* w, float* wbf, cudaStream_t s);
 void launch_features(const Batch& b, cudaStream_t s);
 void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream_t s);
-void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, float* z4, __nv_bfloat16* h1,
-                        __nv_bfloat16* h2, __nv_bfloat16* h3, uint32_t* err, cudaStream_t s);
-void launch_mlp_backward(const float* feat, const float* label, int m, const float* wbf, const float* z4,
-                         const __nv_bfloat16* h1, const __nv_bfloat16* h2, const __nv_bfloat16* h3, float* grad,
-                         float* loss, uint32_t* err, cudaStream_t s);
+void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, uint32_t* err, cudaStream_t s);
+// adds d(mean BCE)/d params to grad[kMlpParams] and the loss to *loss (grad 16-byte aligned)
+void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
+                      uint32_t* err, cudaStream_t s);
+// loss_out: null, or page-locked host memory for a copy of *loss
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
-                     cudaStream_t s);
+                     const float* loss, float* loss_out, cudaStream_t s);
 void launch_learned_hist(const Batch& b, int total, int max_n, cudaStream_t s);
 
 }  // namespace tr
