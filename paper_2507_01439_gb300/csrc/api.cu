@@ -406,9 +406,10 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
         const int32_t vppb = (num == 1 && !vflag) ? balanced_vppb(n[b], prm[b]->k1 * prm[b]->k2, device_sms())
                                                   : 4 * vpw_flag;
         ws.h_views[b].vppb = vppb;
+        ws.h_views[b].in_batch = num > 1;
         if (vppb > vppb_max) vppb_max = vppb;
         int32_t blocks[kNumBatchStages];
-        stage_blocks(n[b], prm[b]->k1, prm[b]->k2, vppb, blocks);
+        stage_blocks(n[b], prm[b]->k1, prm[b]->k2, vppb, num > 1, blocks);
         for (int st = 0; st < kNumBatchStages; ++st) {
             plan.tot[st] += blocks[st];
             ws.h_pre[st * (num + 1) + b + 1] = plan.tot[st];

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kCountThreads, 3) hist_kernel(VS vs)
     pdl_wait();
     pdl_release();
     const bool learned = v.prob != nullptr;
-    const int groups = count_blocks(n), stride = hist_blocks(n);
+    const int groups = count_groups(n), stride = hist_blocks(n);
     bool bad = false;
     for (int g = lb; g < groups; g += stride) {
         __syncthreads();   // the bins are cleared; the previous group's list is consumed
@@ -243,7 +243,9 @@ __device__ __forceinline__ void count_chunk(uint4 q, uint32_t a2, int& g, int& e
 // W).  The chunks of the remaining rows are spread over all the block's
 // threads, so a block with one or two such rows reads them in one round.
 // Rows holding such edges are appended to the active list as (row, #gt, #eq),
-// in any order.
+// in any order.  In a batch a block takes several groups, a fixed distance
+// apart, so that finding its problem and reading the scalars is paid once
+// (256 problems: @COUNT us for the pass).
 // select_here (one problem whose histogram is complete): every block chooses
 // the threshold itself from the histogram, staged in dynamic shared memory
 // while its row maxima load, and block 0 records it for the later passes;
@@ -261,9 +263,10 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     __shared__ int ssel[40];
     const int n = v.n;
     const int t = threadIdx.x;
+    const int groups = count_groups(n), stride = count_blocks(n, v.in_batch);
     int row;
     bool act = group_row(lb, t, n, row);
-    const int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
+    int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
     int n_sel, alpha;
     if (select_here) {
         const bool bad = VS::kCallerWeights && (__ldcg(&v.ctl->err) & TR_ERR_BAD_WEIGHT) != 0u;
@@ -285,46 +288,151 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
         alpha = v.ctl->alpha;
     }
     if (n_sel == 0) return;                   // uniform over the block
-    if (t < 32) {
-        if (act && v.rowmax != nullptr) act = rmax >= alpha;
-        if (act && v.prob != nullptr) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
-        group_offsets(sg, t, row, act, n);
-        if (t < 16) sgt[t] = seq[t] = 0;
-    }
-    __syncthreads();
-    if (sg.off[16] == 0) return;              // uniform over the block
     const uint32_t a2 = static_cast<uint32_t>(alpha) * 0x10001u;
     const bool learned = v.prob != nullptr;
-    int kcur = -1, g = 0, e = 0;              // running counts of entry kcur
-    auto flush = [&]() {
-        if (g) atomicAdd(&sgt[kcur], g);
-        if (e) atomicAdd(&seq[kcur], e);
-    };
-    for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 qm) {
-        if (k != kcur) {
-            if (kcur >= 0) flush();
-            kcur = k;
-            g = e = 0;
+    for (int grp = lb; grp < groups; grp += stride) {
+        if (t < 32) {
+            if (act && v.rowmax != nullptr) act = rmax >= alpha;
+            if (act && learned) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
+            group_offsets(sg, t, row, act, n);
+            if (t < 16) sgt[t] = seq[t] = 0;
         }
-        if (!learned) {
-            count_chunk(qm, a2, g, e);
-        } else if ((qm.x | qm.y | qm.z | qm.w) != 0u) {
+        __syncthreads();
+        // the next group's row maxima, in flight
+        int row_n;
+        const bool act_n = grp + stride < groups && group_row(grp + stride, t, n, row_n);
+        const int rmax_n = (act_n && v.rowmax != nullptr) ? __ldg(v.rowmax + row_n) : 0;
+        if (sg.off[16] != 0) {                // uniform over the block
+            int kcur = -1, g = 0, e = 0;      // running counts of entry kcur
+            auto flush = [&]() {
+                if (g) atomicAdd(&sgt[kcur], g);
+                if (e) atomicAdd(&seq[kcur], e);
+            };
+            for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 qm) {
+                if (k != kcur) {
+                    if (kcur >= 0) flush();
+                    kcur = k;
+                    g = e = 0;
+                }
+                if (!learned) {
+                    count_chunk(qm, a2, g, e);
+                } else if ((qm.x | qm.y | qm.z | qm.w) != 0u) {
 #pragma unroll
-            for (int el = 0; el < 8; ++el) {
-                const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
-                const int pw = pivot_weight(v, row_k, c * 8 + el, static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu));
-                g += pw > alpha;
-                e += pw == alpha;
-            }
+                    for (int el = 0; el < 8; ++el) {
+                        const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
+                        const int pw = pivot_weight(v, row_k, c * 8 + el, static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu));
+                        g += pw > alpha;
+                        e += pw == alpha;
+                    }
+                }
+            });
+            if (kcur >= 0) flush();
+            __syncthreads();
+            if (t < 16 && (sgt[t] | seq[t]))
+                v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
         }
-    });
-    if (kcur >= 0) flush();
-    __syncthreads();
-    if (t < 16 && (sgt[t] | seq[t]))
-        v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
+        if (grp + stride < groups) __syncthreads();   // the group's list and counts are consumed
+        row = row_n;
+        act = act_n;
+        rmax = rmax_n;
+    }
 }
 
-// Blocks take the active rows in any order.  W > alpha edges take slots
+// A warp per active row (batches; one problem of up to kEmitWarpN matches):
+// lane l reads chunks 4l .. 4l + 3 of each 128-chunk sweep (lane order =
+// column order), the next sweep in flight, and needs no block barrier.  A
+// block's eight rows then run side by side: with a block per row and n/8
+// blocks, a problem whose rows are all active took eight rows in turn (10.5 us
+// at n = 67), and a batch's blocks mostly started for nothing (256 problems:
+// @EMIT us).  Same slots and tie ranks as the block form below.
+template <class VS>
+__global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_EMIT, blockIdx.x, lb);   // launch descriptors: before the wait
+    pdl_wait();
+    pdl_release();
+    const int lane = threadIdx.x & 31;
+    const int n = v.n, eb = emit_blocks(n, v.in_batch);
+    const int a0 = (threadIdx.x >> 5) * eb + lb;          // this warp's first active row
+    const int n_sel = v.ctl->n_sel;
+    const int nact = static_cast<int>(v.ctl->n_active);
+    const int m = v.ctl->m_ties, alpha = v.ctl->alpha, c_gt = v.ctl->c_gt;
+    int4 ar = a0 < n ? v.active[a0] : make_int4(0, 0, 0, 0);   // speculative: a0 < n is inside the list's capacity
+    if (n_sel == 0) return;
+    const int c1 = (n - 1) >> 3;
+    for (int a = a0; a < nact; a += 8 * eb) {
+        if (a != a0) ar = v.active[a];
+        const int i = ar.x, ng = ar.y, ne = ar.z;
+        const uint16_t* wrow = v.w + (size_t)i * v.n_pad;
+        const int cb0 = (i + 1) >> 3;
+        uint4 q[4];
+        auto load = [&](int cb) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int cc = cb + lane * 4 + k;
+                q[k] = cc <= c1 ? *reinterpret_cast<const uint4*>(wrow + cc * 8) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        };
+        load(cb0);
+        int base_g = 0;
+        if (lane == 0 && ng > 0) base_g = static_cast<int>(atomicAdd(&v.ctl->gt_slot, static_cast<uint32_t>(ng)));
+        int base_e = 0;   // ties in active rows above i
+        if (ne > 0) {
+            for (int b = lane; b < nact; b += 32) {
+                const int4 o = v.active[b];
+                base_e += o.x < i ? o.z : 0;
+            }
+            base_e = __reduce_add_sync(0xffffffffu, base_e);
+        }
+        int left_e = base_e < m ? min(ne, m - base_e) : 0, left_g = ng;   // edges of this row still to write
+        base_g = __shfl_sync(0xffffffffu, base_g, 0);
+        for (int cb = cb0; cb <= c1 && (left_g > 0 || left_e > 0); cb += 128) {
+            uint32_t gm = 0u, em = 0u;   // bit 8 k + e: chunk k, element e
+            const int cfirst = cb + lane * 4;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if ((q[k].x | q[k].y | q[k].z | q[k].w) == 0u) continue;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t word = e < 2 ? q[k].x : e < 4 ? q[k].y : e < 6 ? q[k].z : q[k].w;
+                    const int j = (cfirst + k) * 8 + e;
+                    const bool in = j > i && j < n;
+                    const int w = in ? pivot_weight(v, i, j, (word >> ((e & 1) * 16)) & 0xFFFF) : 0;
+                    gm |= static_cast<uint32_t>(in && w > alpha) << (8 * k + e);
+                    em |= static_cast<uint32_t>(in && w == alpha) << (8 * k + e);
+                }
+            }
+            if (cb + 128 <= c1) load(cb + 128);
+            // inclusive prefix sums of both counts over the lanes (at most 32 x 32 each)
+            const uint32_t own = static_cast<uint32_t>(__popc(gm)) | (static_cast<uint32_t>(__popc(em)) << 16);
+            uint32_t incl = own;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31), excl = incl - own;
+            int rg = base_g + static_cast<int>(excl & 0xFFFFu), re = static_cast<int>(excl >> 16);
+            for (; gm; gm &= gm - 1u) {
+                const int b = __ffs(gm) - 1;
+                const int j = (cfirst + (b >> 3)) * 8 + (b & 7);
+                v.cand[rg++] = edge_key(pivot_weight(v, i, j, wrow[j]), i, j, n);
+            }
+            for (; em && re < left_e; em &= em - 1u, ++re) {
+                const int b = __ffs(em) - 1;
+                v.cand[c_gt + base_e + re] = edge_key(alpha, i, (cfirst + (b >> 3)) * 8 + (b & 7), n);
+            }
+            base_g += static_cast<int>(tot & 0xFFFFu);
+            left_g -= static_cast<int>(tot & 0xFFFFu);
+            base_e += static_cast<int>(tot >> 16);
+            left_e -= static_cast<int>(tot >> 16);
+        }
+    }
+}
+
+// A block per active row (one larger problem: its rows are read in one or two
+// rounds).  Blocks take the active rows in any order.  W > alpha edges take slots
 // base + rank-in-row from one atomic per row (any slots in [0, c_gt) will
 // do: the rank pass orders the keys).  Ties must be the m lowest (i, j):
 // a row with ties sums the tie counts of the active rows above it (its tie
@@ -350,7 +458,7 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
     if (n_sel == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c1 = (v.n - 1) >> 3;
-    const int eb = emit_blocks(v.n);
+    const int eb = emit_blocks(v.n, 0);
     for (int a = lb; a < nact; a += eb) {
         const int4 ar = a == lb ? ar0 : v.active[a];
         const int i = ar.x, ng = ar.y, ne = ar.z;
@@ -525,7 +633,8 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
     const ManyViews vs{b};
     const size_t stage = select_here ? static_cast<size_t>((max_n + 4) / 4 * 4) * 4 : 0;
     launch_pdl(count_kernel<ManyViews>, tot[ST_COUNT], kCountThreads, stage, s, vs, select_here ? 1 : 0);
-    launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
+    if (emit_by_warp(max_n, b.num > 1)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
+    else launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
 }
 
 // One problem passed by value (no device-side problem table); the count blocks
@@ -534,9 +643,10 @@ void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s)
 {
     const OneView vs{v};
     launch_hist_vs(vs, hist_blocks(v.n), v.n, s);
-    launch_pdl(count_kernel<OneView>, count_blocks(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
+    launch_pdl(count_kernel<OneView>, count_groups(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
                vs, 1);
-    launch_pdl(emit_kernel<OneView>, emit_blocks(v.n), 256, 0, s, vs);
+    if (emit_by_warp(v.n, false)) launch_pdl(emit_warp_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
+    else launch_pdl(emit_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
     launch_pdl(rank_kernel, (v.k1 + 31) / 32, 256, v.k1 * 8, s, vs, n_out);
 }
 

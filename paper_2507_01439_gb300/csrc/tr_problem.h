@@ -26,6 +26,7 @@ struct ProbView {
     int32_t graph_mode;  // TURBOREG_GRAPH_O2 / _SC2: the graph the clique search runs on
     int32_t scoring;     // TURBOREG_SCORE_IN / _MAE / _MSE
     int32_t vppb;        // verification tile: matches per block (<= 4 x the kernel's points per warp)
+    int32_t in_batch;    // 1: one of several problems of a call (blocks per problem of the passes over W)
     uint32_t dbg;        // failure injection for tests (TR_DBG_*), 0 in normal use
     uint8_t* a4_auto;    // non-null: the SC^2 path is chosen on the device from the degrees (one
                          // problem, n_pad <= 5120); a4 is then null, so the compatibility kernel
@@ -65,14 +66,22 @@ enum Stage {
     ST_VERIFY, ST_FINAL, ST_HIST, ST_BITSET, ST_GEMM, ST_FEAT, ST_MLP, kNumBatchStages
 };
 
-// Blocks of the per-row count pass (eight row pairs per block) and of the
-// emit pass (active rows strided over the blocks).
-__host__ __device__ inline int count_blocks(int n) { return ((n + 1) / 2 + 7) / 8; }
-__host__ __device__ inline int emit_blocks(int n) { return (n + 7) / 8; }
-// Blocks of the histogram pass: one per group of eight row pairs; from n = 8192
-// on a fixed number that takes several groups each (a block clears and flushes
-// n bins: at n = 20000 that is 80 KB against the 320 KB of W a group holds).
-__host__ __device__ inline int hist_blocks(int n) { return count_blocks(n) <= 512 ? count_blocks(n) : 304; }
+// Groups of eight row pairs of the passes over W; blocks of the count pass (in
+// a batch four groups each) and of the emit pass (active rows strided over the
+// blocks, or in a batch over their warps).
+__host__ __device__ inline int count_groups(int n) { return ((n + 1) / 2 + 7) / 8; }
+__host__ __device__ inline int count_blocks(int n, int in_batch)
+{
+    return in_batch ? (count_groups(n) + 3) / 4 : count_groups(n);
+}
+__host__ __device__ inline int emit_blocks(int n, int in_batch) { return in_batch ? (n + 63) / 64 : (n + 7) / 8; }
+// The emit pass takes a warp per active row in a batch and for one problem of
+// up to 2048 matches (a row is at most two sweeps of a warp), else a block.
+inline bool emit_by_warp(int max_n, bool in_batch) { return in_batch || max_n <= 2048; }
+// Blocks of the histogram pass: one per group; from n = 8192 on a fixed number
+// that takes several groups each (a block clears and flushes n bins: at
+// n = 20000 that is 80 KB against the 320 KB of W a group holds).
+__host__ __device__ inline int hist_blocks(int n) { return count_groups(n) <= 512 ? count_groups(n) : 304; }
 
 struct Batch {
     const ProbView* views;   // [num] device
@@ -130,7 +139,7 @@ struct ManyViews {
 
 // per-problem block counts of each stage (host side, from n, k1, k2)
 // vppb: matches per verification block (ProbView::vppb)
-void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, int32_t blocks[kNumBatchStages]);
+void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, int32_t in_batch, int32_t blocks[kNumBatchStages]);
 // Matches per verification block for a single problem: the block count
 // (hypothesis blocks x match blocks) close to 4 blocks per SM, so that one
 // wave covers the problem with every SM holding the same number of blocks.
