@@ -116,9 +116,9 @@ __device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGro
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int x = base + u * kCountThreads;
-            int k = 0;
+            int k = 0;   // the last entry that begins at or before chunk x
 #pragma unroll
-            for (int m = 1; m < 16; ++m) k += sg.off[m] <= x ? 1 : 0;
+            for (int m = 8; m >= 1; m >>= 1) k += sg.off[k + m] <= x ? m : 0;
             kk[u] = k;
             q[u] = x < tot ? *reinterpret_cast<const uint4*>(v.w + (size_t)sg.row[k] * v.n_pad +
                                                              (size_t)(sg.c0[k] + x - sg.off[k]) * 8)
@@ -226,14 +226,13 @@ __global__ void __launch_bounds__(1024) select_kernel(ManyViews vs)
     select_alpha(v, sbuf);
 }
 
-// #{entries > alpha} and #{entries == alpha} of a chunk, as packed 16-bit
-// SIMD compares (weights and alpha < 2^16; a zeroed entry never counts, alpha >= 1).
-__device__ __forceinline__ void count_chunk(uint4 q, uint32_t a2, int& g, int& e)
+// Whether a chunk holds a weight of at least alpha (few do: the passes over the
+// active rows visit the entries of those only; a learned weight never exceeds
+// the plain one).
+__device__ __forceinline__ bool chunk_reaches(uint4 q, int alpha)
 {
-    g += (__popc(__vcmpgtu2(q.x, a2)) + __popc(__vcmpgtu2(q.y, a2)) + __popc(__vcmpgtu2(q.z, a2)) +
-          __popc(__vcmpgtu2(q.w, a2))) >> 4;
-    e += (__popc(__vcmpeq2(q.x, a2)) + __popc(__vcmpeq2(q.y, a2)) + __popc(__vcmpeq2(q.z, a2)) +
-          __popc(__vcmpeq2(q.w, a2))) >> 4;
+    const uint32_t m = __vmaxu2(__vmaxu2(q.x, q.y), __vmaxu2(q.z, q.w));
+    return static_cast<int>(m & 0xFFFFu) >= alpha || static_cast<int>(m >> 16) >= alpha;
 }
 
 // Per-row counts of the weight > alpha and weight == alpha edges.  A block
@@ -288,7 +287,6 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
         alpha = v.ctl->alpha;
     }
     if (n_sel == 0) return;                   // uniform over the block
-    const uint32_t a2 = static_cast<uint32_t>(alpha) * 0x10001u;
     const bool learned = v.prob != nullptr;
     for (int grp = lb; grp < groups; grp += stride) {
         if (t < 32) {
@@ -314,13 +312,12 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
                     kcur = k;
                     g = e = 0;
                 }
-                if (!learned) {
-                    count_chunk(qm, a2, g, e);
-                } else if ((qm.x | qm.y | qm.z | qm.w) != 0u) {
+                if (chunk_reaches(qm, alpha)) {
 #pragma unroll
                     for (int el = 0; el < 8; ++el) {
                         const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
-                        const int pw = pivot_weight(v, row_k, c * 8 + el, static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu));
+                        int pw = static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu);
+                        if (learned) pw = pivot_weight(v, row_k, c * 8 + el, pw);
                         g += pw > alpha;
                         e += pw == alpha;
                     }
@@ -392,7 +389,7 @@ __global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
             const int cfirst = cb + lane * 4;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                if ((q[k].x | q[k].y | q[k].z | q[k].w) == 0u) continue;
+                if (!chunk_reaches(q[k], alpha)) continue;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const uint32_t word = e < 2 ? q[k].x : e < 4 ? q[k].y : e < 6 ? q[k].z : q[k].w;
@@ -505,7 +502,7 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                if ((q[k].x | q[k].y | q[k].z | q[k].w) == 0u) continue;
+                if (!chunk_reaches(q[k], alpha)) continue;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const uint32_t word = e < 2 ? q[k].x : e < 4 ? q[k].y : e < 6 ? q[k].z : q[k].w;
@@ -552,6 +549,41 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
             if (base_g - pg >= ng && (!want_eq || base_e >= m || base_e - pe >= ne)) break;
         }
     }
+}
+
+// Batches: a problem's selected keys sorted in place, largest first (one block
+// per problem, bitonic in shared memory), so that the clique search takes
+// pivot c from key c.  Finding each key's rank there instead, one warp per key
+// over all K1 keys, was 380 of the search's 2100 warp instructions per pivot;
+// the sort takes 1/40 of that (but a launch more, so one problem keeps the
+// ranks).  A pass of stride 32 or less stays inside the 64 keys of a warp.
+__global__ void __launch_bounds__(1024) sort_kernel(ManyViews vs)
+{
+    const ProbView& v = vs.bt.views[blockIdx.x];   // launch descriptors: before the wait
+    extern __shared__ uint64_t sk[];
+    pdl_wait();
+    pdl_release();
+    const int cnt = v.ctl->n_sel;
+    int P = 64;
+    while (P < cnt) P <<= 1;
+    for (int q = threadIdx.x; q < P; q += blockDim.x) sk[q] = q < cnt ? __ldcg(v.cand + q) : 0ull;
+    __syncthreads();
+    for (int k = 2; k <= P; k <<= 1) {
+        for (int j = k >> 1; j >= 1; j >>= 1) {
+            for (int q = threadIdx.x; q < P / 2; q += blockDim.x) {
+                const int a = 2 * q - (q & (j - 1)), b = a + j;   // pair q of stride j
+                const uint64_t x = sk[a], y = sk[b];
+                if ((x < y) == ((a & k) == 0)) {
+                    sk[a] = y;
+                    sk[b] = x;
+                }
+            }
+            if (j > 32 || (j == 1 && k >= 64)) __syncthreads();   // the next pass leaves the warp's 64 keys
+            else __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < cnt; q += blockDim.x) v.cand[q] = sk[q];
 }
 
 // 32 candidates per block (one per lane); the 8 warps split the comparison
@@ -611,6 +643,8 @@ cudaError_t topk_setup()
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(hist_kernel<ManyViews, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -627,7 +661,7 @@ void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s)
 
 void launch_select(const Batch& b, cudaStream_t s) { launch_pdl(select_kernel, b.num, 1024, 0, s, ManyViews{b}); }
 
-void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n,
+void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n, int max_k1,
                        cudaStream_t s)
 {
     const ManyViews vs{b};
@@ -635,6 +669,11 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
     launch_pdl(count_kernel<ManyViews>, tot[ST_COUNT], kCountThreads, stage, s, vs, select_here ? 1 : 0);
     if (emit_by_warp(max_n, b.num > 1)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     else launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
+    if (b.num > 1) {
+        int cap = 64;
+        while (cap < max_k1) cap <<= 1;
+        launch_pdl(sort_kernel, b.num, cap / 2 < 1024 ? cap / 2 : 1024, static_cast<size_t>(cap) * 8, s, vs);
+    }
 }
 
 // One problem passed by value (no device-side problem table); the count blocks

@@ -165,10 +165,11 @@ int bitset_tiles(int n_pad);
 cudaError_t sc2_bitset_setup();
 void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s);
 void launch_select(const Batch& b, cudaStream_t s);
-// count and emit passes of the selection (the clique search ranks the pivots)
+// count and emit passes of the selection; in a batch the selected keys are then
+// sorted (for one problem the clique search ranks the pivots)
 // select_here: the count blocks choose the threshold from the histogram the
 // SC^2 GEMM completed (one problem of at most max_n matches)
-void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n,
+void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n, int max_k1,
                        cudaStream_t s);
 // The clique search also orders the pivots (each warp ranks its selected edge)
 void launch_pgs(const Batch& b, int total, int k2_max, int max_k1, cudaStream_t s);
