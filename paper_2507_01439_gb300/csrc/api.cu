@@ -503,7 +503,7 @@ int enqueue_plan(turboreg_ctx* c, const Plan& pl, const Batch& bt, const float* 
     }
     launch_count_emit(bt, pl.tot, sel_in_count, pl.max_n, pl.max_k1, s);
     TR_EV(5);
-    launch_pgs(bt, pl.tot[ST_PGS], pl.k2_common, pl.max_k1, s);   // also ranks the pivots and solves the cliques' Kabsch
+    launch_pgs(bt, pl.tot, pl.k2_common, pl.max_k1, s);   // also ranks the pivots and solves the cliques' Kabsch
     TR_EV(6);
     launch_verify(bt, pl.tot[ST_VERIFY], pl.vpw, pl.vcap != 0, s);
     TR_EV(7);

@@ -31,8 +31,9 @@
 // the warp computes the FP64 triangle normals with six lanes per clique
 // (triangle x or y, component 0..2) and the clique's lane redoes the closed
 // form with them.  One problem: each warp solves its own pivot's cliques at
-// once.  A batch, bound by issued instructions: the block's cliques are
-// collected and solved 32 to a warp.
+// once.  A batch: a kernel of its own solves 32 cliques to a warp, and the search,
+// bound by the latency of its gathers, keeps twice the warps per SM without
+// the closed form's registers.
 #include <type_traits>
 
 #include "tr_common.cuh"
@@ -43,8 +44,8 @@ namespace tr {
 
 namespace {
 
-constexpr int kCand = 1024;   // per-warp candidate list (z indices)
-constexpr int kListBytes = 8 * kCand * 4;   // the 8 warps' lists
+constexpr int kCand = 1024;   // per-warp candidate list (z indices, 16 bits)
+constexpr int kListBytes = 8 * kCand * 2;   // the 8 warps' lists
 constexpr int kWords = 8;     // bitset words per lane per load round
 constexpr int kBatch = 8;     // list entries per lane per scoring round (16 weight loads in flight)
 
@@ -103,18 +104,46 @@ __device__ __forceinline__ void solve_cliques(const ProbView& v, int4 cl, int h,
     if (has) store_hypothesis(v, h, present, o, need ? 2u : 0u);
 }
 
-// kDense: a batch (keys sorted, cliques solved by block, registers bounded for
-// three blocks per SM: many waves of blocks, latency hidden by occupancy);
-// otherwise two blocks, with more registers per warp (one problem: a single wave)
+// Kabsch of a batch's cliques, 32 to a warp, 128 to a block.  The block is kept
+// in the clique search's shape (256 threads, three to an SM, cliques handed to
+// the solving warps through shared memory): the assembler contracts products
+// and sums as its register budget suggests, and with a block of 128 threads a
+// batch's hypotheses came out one last bit away from one problem's.  (Equal in
+// every bit this way, which the tests check for every K2 form.)
+__global__ void __launch_bounds__(256, 3) solve_kernel(ManyViews vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_KABSCH, blockIdx.x, lb);   // launch descriptors: before the wait
+    pdl_wait();
+    pdl_release();
+    __shared__ int4 s_cl[128];
+    __shared__ int s_h[128];
+    const int t = threadIdx.x;
+    const int nh = v.ctl->n_pivots * v.k2;
+    if (t < 128) {
+        const int h = lb * 128 + t;
+        s_cl[t] = h < nh ? v.cliques[h] : make_int4(0, 0, 0, 0);
+        s_h[t] = h < nh ? h : -1;
+    }
+    __syncthreads();
+    const int lane = t & 31, warp = t >> 5;
+    if (warp >= 4) return;
+    const int e = warp * 32 + lane;
+    const bool has = s_h[e] >= 0;
+    solve_cliques(v, has ? s_cl[e] : make_int4(0, 0, 0, 0), has ? s_h[e] : 0, has, 32);
+}
+
+// kDense: a batch (keys sorted, cliques solved by solve_kernel, registers
+// bounded for four blocks per SM: many waves of blocks, latency hidden by
+// occupancy); otherwise two blocks, with more registers per warp (one problem:
+// a single wave)
 template <int K2C, bool kDense>
-__global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
+__global__ void __launch_bounds__(256, kDense ? 4 : 2) pgs_kernel(ManyViews vs)
 {
     // dynamic shared memory: per-warp candidate lists, then the selected edge keys (one problem)
     extern __shared__ __align__(16) uint8_t pgs_smem[];
-    int (*scand)[kCand] = reinterpret_cast<int (*)[kCand]>(pgs_smem);
+    uint16_t (*scand)[kCand] = reinterpret_cast<uint16_t (*)[kCand]>(pgs_smem);
     uint64_t* skey = reinterpret_cast<uint64_t*>(pgs_smem + kListBytes);
-    __shared__ int4 s_cl[kDense ? 8 * TURBOREG_K2_MAX : 1];
-    __shared__ int s_h[kDense ? 8 * TURBOREG_K2_MAX : 1];
     int lb;
     const ProbView v = vs.get(ST_PGS, blockIdx.x, lb);   // launch descriptors: before the wait
     pdl_wait();
@@ -166,7 +195,7 @@ __global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
     const int k2 = K2C > 0 ? K2C : v.k2;
     int p = c;
     if constexpr (kDense) {
-        if (lb * 8 >= np) return;             // uniform over the block
+        if (c >= np) return;
     } else {
         __syncthreads();
         if (c >= np) return;
@@ -174,7 +203,7 @@ __global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
         for (int q = lane; q < np; q += 32) p += skey[q] > mykey ? 1 : 0;
         p = __reduce_add_sync(0xffffffffu, p);
     }
-    int* cand = scand[warp];
+    uint16_t* cand = scand[warp];
     const uint16_t* wi = v.w + (size_t)i * v.n_pad;
     const uint16_t* wj = v.w + (size_t)j * v.n_pad;
 
@@ -245,7 +274,7 @@ __global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
 #pragma unroll
                 for (int t = 0; t < kWords; ++t) {
                     const int zb = (wb + lane + 32 * t) * 32;
-                    for (uint32_t m = mw[t]; m != 0u; m &= m - 1u) cand[pos++] = zb + __ffs(m) - 1;
+                    for (uint32_t m = mw[t]; m != 0u; m &= m - 1u) cand[pos++] = static_cast<uint16_t>(zb + __ffs(m) - 1);
                 }
                 nlist += total;
             } else {
@@ -268,7 +297,7 @@ __global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
                     }
                     int pos = nlist + in1 - c1;
                     const int zb = (wb + lane + 32 * t) * 32;
-                    for (uint32_t m = mw[t]; m != 0u; m &= m - 1u) cand[pos++] = zb + __ffs(m) - 1;
+                    for (uint32_t m = mw[t]; m != 0u; m &= m - 1u) cand[pos++] = static_cast<uint16_t>(zb + __ffs(m) - 1);
                     nlist += tot1;
                 }
             }
@@ -293,21 +322,8 @@ __global__ void __launch_bounds__(256, kDense ? 3 : 2) pgs_kernel(ManyViews vs)
         }
         return mine_cl;
     };
-    if constexpr (kDense) {
-        const bool live = c < np;             // the last block may hold fewer than eight pivots
-        const int4 mine_cl = live ? search() : make_int4(0, 0, 0, 0);
-        if (lane < k2) {
-            s_cl[warp * k2 + lane] = mine_cl;
-            s_h[warp * k2 + lane] = live ? lane * np + p : -1;
-        }
-        __syncthreads();
-        if (warp * 32 >= 8 * k2) return;
-        const int e = warp * 32 + lane;
-        const bool has = e < 8 * k2 && s_h[e] >= 0;
-        solve_cliques(v, has ? s_cl[e] : make_int4(0, 0, 0, 0), has ? s_h[e] : 0, has, 32);
-    } else {
-        solve_cliques(v, search(), lane * np + p, lane < k2, k2);
-    }
+    const int4 cl = search();
+    if (!kDense) solve_cliques(v, cl, lane * np + p, lane < k2, k2);
 }
 
 }  // namespace
@@ -333,8 +349,9 @@ cudaError_t pgs_setup()
 
 // k2 is the common K2 of the batch, or 0 when problems differ (generic list);
 // max_k1 sizes the shared copy of the selected keys
-void launch_pgs(const Batch& b, int total, int k2, int max_k1, cudaStream_t s)
+void launch_pgs(const Batch& b, const int32_t tot[kNumBatchStages], int k2, int max_k1, cudaStream_t s)
 {
+    const int total = tot[ST_PGS];
     auto go = [&](auto dense) {
         constexpr bool kD = decltype(dense)::value;
         const ManyViews vs{b};
@@ -347,8 +364,12 @@ void launch_pgs(const Batch& b, int total, int k2, int max_k1, cudaStream_t s)
             default: launch_pdl(pgs_kernel<0, kD>, total, 256, smem, s, vs); break;
         }
     };
-    if (b.num > 1) go(std::true_type{});
-    else go(std::false_type{});
+    if (b.num > 1) {
+        go(std::true_type{});
+        launch_pdl(solve_kernel, tot[ST_KABSCH], 256, 0, s, ManyViews{b});
+    } else {
+        go(std::false_type{});
+    }
 }
 
 cudaError_t verify_setup();

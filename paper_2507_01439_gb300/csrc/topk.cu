@@ -103,19 +103,19 @@ __device__ __forceinline__ void group_offsets(RowGroup& sg, int t, int row, bool
     if (t == 15) sg.off[16] = incl;
 }
 
-// The group's chunks spread over all the block's threads, eight 16-byte loads
-// in flight each: f(k, row, c, weights) for chunk c of entry k, entries outside
-// the upper part zeroed.
-template <typename F>
-__device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGroup& sg, F&& f)
+// The group's chunks spread over T threads (this one is number t), eight
+// 16-byte loads in flight each: f(k, row, c, weights) for chunk c of entry k,
+// entries outside the upper part zeroed.
+template <int T = kCountThreads, typename F>
+__device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGroup& sg, int t, F&& f)
 {
     const int tot = sg.off[16];
-    for (int base = threadIdx.x; base < tot; base += 8 * kCountThreads) {
+    for (int base = t; base < tot; base += 8 * T) {
         uint4 q[8];
         int kk[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int x = base + u * kCountThreads;
+            const int x = base + u * T;
             int k = 0;   // the last entry that begins at or before chunk x
 #pragma unroll
             for (int m = 8; m >= 1; m >>= 1) k += sg.off[k + m] <= x ? m : 0;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGro
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int x = base + u * kCountThreads;
+            const int x = base + u * T;
             if (x >= tot) break;
             const int k = kk[u];
             const int row = sg.row[k], c = sg.c0[k] + x - sg.off[k];
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kCountThreads, 3) hist_kernel(VS vs)
             const uint32_t m = max(mx & 0xFFFFu, mx >> 16);
             if (m) atomicMax(&smax[kcur], m);
         };
-        for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 q) {
+        for_group_chunks(v, sg, t, [&](int k, int row_k, int c, uint4 q) {
             const uint32_t u[4] = {q.x, q.y, q.z, q.w};
             if (VS::kCallerWeights) {
                 if (k != kcur) {
@@ -235,6 +235,21 @@ __device__ __forceinline__ bool chunk_reaches(uint4 q, int alpha)
     return static_cast<int>(m & 0xFFFFu) >= alpha || static_cast<int>(m >> 16) >= alpha;
 }
 
+// Adds a chunk's #{weight > alpha} and #{weight == alpha} to g and e.
+__device__ __forceinline__ void count_chunk(const ProbView& v, int row, int c, uint4 q, int alpha, bool learned, int& g,
+                                            int& e)
+{
+    if (!chunk_reaches(q, alpha)) return;
+#pragma unroll
+    for (int el = 0; el < 8; ++el) {
+        const uint32_t word = el < 2 ? q.x : el < 4 ? q.y : el < 6 ? q.z : q.w;
+        int pw = static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu);
+        if (learned) pw = pivot_weight(v, row, c * 8 + el, pw);
+        g += pw > alpha;
+        e += pw == alpha;
+    }
+}
+
 // Per-row counts of the weight > alpha and weight == alpha edges.  A block
 // owns a group of eight row pairs.  Rows whose largest weight (recorded by the
 // SC^2 pass or the histogram) is below alpha hold no such edge and are skipped
@@ -242,9 +257,7 @@ __device__ __forceinline__ bool chunk_reaches(uint4 q, int alpha)
 // W).  The chunks of the remaining rows are spread over all the block's
 // threads, so a block with one or two such rows reads them in one round.
 // Rows holding such edges are appended to the active list as (row, #gt, #eq),
-// in any order.  In a batch a block takes several groups, a fixed distance
-// apart, so that finding its problem and reading the scalars is paid once
-// (256 problems: @COUNT us for the pass).
+// in any order.
 // select_here (one problem whose histogram is complete): every block chooses
 // the threshold itself from the histogram, staged in dynamic shared memory
 // while its row maxima load, and block 0 records it for the later passes;
@@ -262,10 +275,9 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     __shared__ int ssel[40];
     const int n = v.n;
     const int t = threadIdx.x;
-    const int groups = count_groups(n), stride = count_blocks(n, v.in_batch);
     int row;
     bool act = group_row(lb, t, n, row);
-    int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
+    const int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
     int n_sel, alpha;
     if (select_here) {
         const bool bad = VS::kCallerWeights && (__ldcg(&v.ctl->err) & TR_ERR_BAD_WEIGHT) != 0u;
@@ -288,50 +300,71 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     }
     if (n_sel == 0) return;                   // uniform over the block
     const bool learned = v.prob != nullptr;
-    for (int grp = lb; grp < groups; grp += stride) {
-        if (t < 32) {
-            if (act && v.rowmax != nullptr) act = rmax >= alpha;
-            if (act && learned) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
-            group_offsets(sg, t, row, act, n);
-            if (t < 16) sgt[t] = seq[t] = 0;
-        }
-        __syncthreads();
-        // the next group's row maxima, in flight
-        int row_n;
-        const bool act_n = grp + stride < groups && group_row(grp + stride, t, n, row_n);
-        const int rmax_n = (act_n && v.rowmax != nullptr) ? __ldg(v.rowmax + row_n) : 0;
-        if (sg.off[16] != 0) {                // uniform over the block
-            int kcur = -1, g = 0, e = 0;      // running counts of entry kcur
-            auto flush = [&]() {
-                if (g) atomicAdd(&sgt[kcur], g);
-                if (e) atomicAdd(&seq[kcur], e);
-            };
-            for_group_chunks(v, sg, [&](int k, int row_k, int c, uint4 qm) {
-                if (k != kcur) {
-                    if (kcur >= 0) flush();
-                    kcur = k;
-                    g = e = 0;
-                }
-                if (chunk_reaches(qm, alpha)) {
-#pragma unroll
-                    for (int el = 0; el < 8; ++el) {
-                        const uint32_t word = el < 2 ? qm.x : el < 4 ? qm.y : el < 6 ? qm.z : qm.w;
-                        int pw = static_cast<int>((word >> ((el & 1) * 16)) & 0xFFFFu);
-                        if (learned) pw = pivot_weight(v, row_k, c * 8 + el, pw);
-                        g += pw > alpha;
-                        e += pw == alpha;
-                    }
-                }
-            });
+    if (t < 32) {
+        if (act && v.rowmax != nullptr) act = rmax >= alpha;
+        if (act && learned) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
+        group_offsets(sg, t, row, act, n);
+        if (t < 16) sgt[t] = seq[t] = 0;
+    }
+    __syncthreads();
+    if (sg.off[16] == 0) return;              // uniform over the block
+    int kcur = -1, g = 0, e = 0;              // running counts of entry kcur
+    auto flush = [&]() {
+        if (g) atomicAdd(&sgt[kcur], g);
+        if (e) atomicAdd(&seq[kcur], e);
+    };
+    for_group_chunks(v, sg, t, [&](int k, int row_k, int c, uint4 qm) {
+        if (k != kcur) {
             if (kcur >= 0) flush();
-            __syncthreads();
-            if (t < 16 && (sgt[t] | seq[t]))
-                v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
+            kcur = k;
+            g = e = 0;
         }
-        if (grp + stride < groups) __syncthreads();   // the group's list and counts are consumed
-        row = row_n;
-        act = act_n;
-        rmax = rmax_n;
+        count_chunk(v, row_k, c, qm, alpha, learned, g, e);
+    });
+    if (kcur >= 0) flush();
+    __syncthreads();
+    if (t < 16 && (sgt[t] | seq[t]))
+        v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
+}
+
+// The same counts in a batch: a warp per group, without block barriers; the
+// threshold comes from the select launch.  With a block per group the pass over
+// 256 problems took 345 us (blocks that start, find their problem and read
+// nothing), with four groups per block 254 us (bound by its barriers), now 98.
+__global__ void __launch_bounds__(kCountThreads, 4) count_warp_kernel(ManyViews vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_COUNT, blockIdx.x, lb);   // launch descriptors: before the wait
+    pdl_wait();
+    pdl_release();
+    __shared__ RowGroup sgs[kCountThreads / 32];
+    __shared__ int scnt[kCountThreads / 32][16];   // #gt | #eq << 16 (a row has fewer than 2^15 entries)
+    const int n = v.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    RowGroup& sg = sgs[warp];
+    int row;
+    bool act = group_row(lb * (kCountThreads / 32) + warp, lane, n, row);
+    const int rmax = act ? __ldg(v.rowmax + row) : 0;
+    const int alpha = v.ctl->alpha;
+    if (v.ctl->n_sel == 0) return;
+    const bool learned = v.prob != nullptr;
+    act = act && rmax >= alpha;
+    if (act && learned) act = learned_row_bound(v, row) >= static_cast<float>(alpha);
+    if (!__any_sync(0xffffffffu, act)) return;
+    group_offsets(sg, lane, row, act, n);
+    if (lane < 16) scnt[warp][lane] = 0;
+    __syncwarp();
+    for_group_chunks<32>(v, sg, lane, [&](int k, int row_k, int c, uint4 q) {
+        int g = 0, e = 0;
+        count_chunk(v, row_k, c, q, alpha, learned, g, e);
+        if ((g | e) != 0) atomicAdd(&scnt[warp][k], g | (e << 16));
+    });
+    __syncwarp();
+    static_assert(TURBOREG_MAX_N <= 32768, "a row's counts fit 16 bits each");
+    if (lane < 16) {
+        const uint32_t ge = static_cast<uint32_t>(scnt[warp][lane]);
+        if (ge != 0u)
+            v.active[atomicAdd(&v.ctl->n_active, 1u)] =
+                make_int4(sg.row[lane], static_cast<int>(ge & 0xFFFFu), static_cast<int>(ge >> 16), 0);
     }
 }
 
@@ -341,7 +374,7 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
 // block's eight rows then run side by side: with a block per row and n/8
 // blocks, a problem whose rows are all active took eight rows in turn (10.5 us
 // at n = 67), and a batch's blocks mostly started for nothing (256 problems:
-// @EMIT us).  Same slots and tie ranks as the block form below.
+// 562 us, now 124).  Same slots and tie ranks as the block form below.
 template <class VS>
 __global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
 {
@@ -665,8 +698,12 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
                        cudaStream_t s)
 {
     const ManyViews vs{b};
-    const size_t stage = select_here ? static_cast<size_t>((max_n + 4) / 4 * 4) * 4 : 0;
-    launch_pdl(count_kernel<ManyViews>, tot[ST_COUNT], kCountThreads, stage, s, vs, select_here ? 1 : 0);
+    if (b.num > 1) {
+        launch_pdl(count_warp_kernel, tot[ST_COUNT], 256, 0, s, vs);
+    } else {
+        const size_t stage = select_here ? static_cast<size_t>((max_n + 4) / 4 * 4) * 4 : 0;
+        launch_pdl(count_kernel<ManyViews>, tot[ST_COUNT], kCountThreads, stage, s, vs, select_here ? 1 : 0);
+    }
     if (emit_by_warp(max_n, b.num > 1)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     else launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     if (b.num > 1) {

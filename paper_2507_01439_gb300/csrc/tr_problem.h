@@ -67,12 +67,12 @@ enum Stage {
 };
 
 // Groups of eight row pairs of the passes over W; blocks of the count pass (in
-// a batch four groups each) and of the emit pass (active rows strided over the
+// a batch a warp per group) and of the emit pass (active rows strided over the
 // blocks, or in a batch over their warps).
 __host__ __device__ inline int count_groups(int n) { return ((n + 1) / 2 + 7) / 8; }
 __host__ __device__ inline int count_blocks(int n, int in_batch)
 {
-    return in_batch ? (count_groups(n) + 3) / 4 : count_groups(n);
+    return in_batch ? (count_groups(n) + 7) / 8 : count_groups(n);
 }
 __host__ __device__ inline int emit_blocks(int n, int in_batch) { return in_batch ? (n + 63) / 64 : (n + 7) / 8; }
 // The emit pass takes a warp per active row in a batch and for one problem of
@@ -171,8 +171,9 @@ void launch_select(const Batch& b, cudaStream_t s);
 // SC^2 GEMM completed (one problem of at most max_n matches)
 void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n, int max_k1,
                        cudaStream_t s);
-// The clique search also orders the pivots (each warp ranks its selected edge)
-void launch_pgs(const Batch& b, int total, int k2_max, int max_k1, cudaStream_t s);
+// Clique search and the cliques' Kabsch (for one problem the search also ranks
+// the pivots)
+void launch_pgs(const Batch& b, const int32_t tot[kNumBatchStages], int k2_max, int max_k1, cudaStream_t s);
 void launch_kabsch(const Batch& b, int total, cudaStream_t s);
 // out: results of the launch's problems in order (page-locked host or device
 // memory), or null for the workspace's result array
