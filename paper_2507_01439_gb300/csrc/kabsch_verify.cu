@@ -149,21 +149,46 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
     // hypothesis) is above every finite threshold
     const uint32_t th2b = __float_as_uint(th2);
     const float qs = kScore == TURBOREG_SCORE_MAE ? kScoreUnits / th : kScoreUnits / th2;
+    // Two of the three coordinates decide most matches: rounding is monotonic,
+    // so p = fl(e0^2 + fl(e1^2)) never exceeds d2, and a match whose p exceeds
+    // the threshold in all of the warp's 128 hypotheses counts nothing (a random
+    // pair passes with probability ~ pi theta^2 / area, 0.2 % at room scale).
+    // The margin of 2^-20 makes such a match's capped error exactly the cap
+    // (sqrt(d2) > theta after rounding), added once per skipped match.
+    const uint32_t skipb = __float_as_uint(th2 * (1.f + 9.5367431640625e-07f));
+    int skipped = 0;
     const int ppw = (vppb + kVWarps - 1) / kVWarps;     // matches per warp
     const int kb = warp * ppw;
     const int cnt = max(0, min(ppw, kn - kb));
     int in[4] = {0, 0, 0, 0};
     uint32_t sc[4] = {0u, 0u, 0u, 0u};
-#pragma unroll 2
-    for (int k = 0; k < cnt; ++k) {
-        const ulonglong2 q0 = sh.sp[kb + k][0], q1 = sh.sp[kb + k][1], q2 = sh.sp[kb + k][2];
-        const f2 X0{q0.x}, X1{q0.y}, X2{q1.x}, Y0{q1.y}, Y1{q2.x}, Y2{q2.y};
+    struct Partial {
+        f2 e0[2], e1[2];
+        bool any;
+    };
+    auto first_two = [&](int k) {
+        const ulonglong2 q0 = sh.sp[k][0], q1 = sh.sp[k][1], q2 = sh.sp[k][2];
+        const f2 X0{q0.x}, X1{q0.y}, X2{q1.x}, Y0{q1.y}, Y1{q2.x};
+        Partial r;
+        uint32_t mn = 0xFFFFFFFFu;
 #pragma unroll
         for (int pr = 0; pr < 2; ++pr) {
-            const f2 e0 = fma2(R[pr][0], X0, fma2(R[pr][1], X1, fma2(R[pr][2], X2, sub2(T[pr][0], Y0))));
-            const f2 e1 = fma2(R[pr][3], X0, fma2(R[pr][4], X1, fma2(R[pr][5], X2, sub2(T[pr][1], Y1))));
+            r.e0[pr] = fma2(R[pr][0], X0, fma2(R[pr][1], X1, fma2(R[pr][2], X2, sub2(T[pr][0], Y0))));
+            r.e1[pr] = fma2(R[pr][3], X0, fma2(R[pr][4], X1, fma2(R[pr][5], X2, sub2(T[pr][1], Y1))));
+            float lo, hi;
+            upk(fma2(r.e0[pr], r.e0[pr], mul2(r.e1[pr], r.e1[pr])), lo, hi);
+            mn = min(mn, min(__float_as_uint(lo), __float_as_uint(hi)));
+        }
+        r.any = __any_sync(0xffffffffu, mn <= skipb);
+        return r;
+    };
+    auto third = [&](int k, const Partial& r) {
+        const ulonglong2 q0 = sh.sp[k][0], q1 = sh.sp[k][1], q2 = sh.sp[k][2];
+        const f2 X0{q0.x}, X1{q0.y}, X2{q1.x}, Y2{q2.y};
+#pragma unroll
+        for (int pr = 0; pr < 2; ++pr) {
             const f2 e2 = fma2(R[pr][6], X0, fma2(R[pr][7], X1, fma2(R[pr][8], X2, sub2(T[pr][2], Y2))));
-            const f2 d2 = fma2(e0, e0, fma2(e1, e1, mul2(e2, e2)));
+            const f2 d2 = fma2(r.e0[pr], r.e0[pr], fma2(r.e1[pr], r.e1[pr], mul2(e2, e2)));
             float lo, hi;
             upk(d2, lo, hi);
             in[2 * pr] += static_cast<int>((__float_as_uint(lo) - th2b - 1u) >> 31);
@@ -177,6 +202,23 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
                 sc[2 * pr + 1] += __float2uint_rn(fminf(hi, th2) * qs);
             }
         }
+    };
+    int k = 0;
+    for (; k + 1 < cnt; k += 2) {
+        const Partial a = first_two(kb + k), b = first_two(kb + k + 1);
+        if (a.any) third(kb + k, a);
+        if (b.any) third(kb + k + 1, b);
+        if (kScore != TURBOREG_SCORE_IN) skipped += (a.any ? 0 : 1) + (b.any ? 0 : 1);
+    }
+    if (k < cnt) {
+        const Partial a = first_two(kb + k);
+        if (a.any) third(kb + k, a);
+        else ++skipped;
+    }
+    if (kScore != TURBOREG_SCORE_IN) {
+        const uint32_t cap = __float2uint_rn((kScore == TURBOREG_SCORE_MAE ? th : th2) * qs);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) sc[a] += static_cast<uint32_t>(skipped) * cap;
     }
     sh.scnt[warp][lane] = in[0];
     sh.scnt[warp][lane + 32] = in[1];
