@@ -138,13 +138,13 @@ __device__ __noinline__ bool compat_fp64(float xi0, float xi1, float xi2, float 
     return fabs(__dsub_rn(__dsqrt_rn(s), __dsqrt_rn(t))) <= (double)tau;
 }
 
-// FP32 decision for two columns at once (Phi <= 0, see the file header); n0/n1
-// are set when |Phi| is inside the guard band (or the arithmetic produced
-// NaN/Inf) and the FP64 evaluation must decide.  s = (ax^2 + ay^2) + az^2 by
+// FP32 decision for two columns at once (see the file header): the sign bit of
+// Phi; n is set when |Phi| is inside the guard band (Phi = 0 always is, as is
+// whatever produced NaN/Inf) and the FP64 evaluation must decide.  s = (ax^2 + ay^2) + az^2 by
 // mul then two fma; everything that can is a packed pair (add/sub/mul/fma
 // .rn.f32x2 round each half exactly like the scalar instructions).
-__device__ __forceinline__ void compat_fast2(const f2 (&XI)[6], const f2 (&XJ)[6], const Decide& k, bool& a0,
-                                             bool& a1, bool& n0, bool& n1)
+__device__ __forceinline__ void compat_fast2(const f2 (&XI)[6], const f2 (&XJ)[6], const Decide& k, float& P0,
+                                             float& P1, bool& n0, bool& n1)
 {
     const f2 ax = sub2(XI[0], XJ[0]), ay = sub2(XI[1], XJ[1]), az = sub2(XI[2], XJ[2]);
     const f2 bx = sub2(XI[3], XJ[3]), by = sub2(XI[4], XJ[4]), bz = sub2(XI[5], XJ[5]);
@@ -154,7 +154,7 @@ __device__ __forceinline__ void compat_fast2(const f2 (&XI)[6], const f2 (&XJ)[6
     float Q0, Q1;
     upk(add2(sX, sY), Q0, Q1);
     const f2 Qc = pk(fmaxf(Q0, k.t2), fmaxf(Q1, k.t2));
-    float P0, P1, D0, D1, w0, w1, g0, g1;
+    float D0, D1, w0, w1, g0, g1;
     upk(fma2(D, D, fma2(Qc, k.c1, k.c0)), P0, P1);        // Phi
     upk(D, D0, D1);
     upk(fma2(Qc, k.cq, k.ct), w0, w1);                     // 32u^2 Qc + 24u tau^2
@@ -163,8 +163,21 @@ __device__ __forceinline__ void compat_fast2(const f2 (&XI)[6], const f2 (&XJ)[6
     upk(mul2(Qc, pk(w0, w1)), g0, g1);                     // the band
     n0 = !(fabsf(P0) > g0);
     n1 = !(fabsf(P1) > g1);
-    a0 = P0 <= 0.f;
-    a1 = P1 <= 0.f;
+}
+
+// 32 x 32 bit matrix over the warp transposed: bit l of lane r's result is bit
+// r of lane l's x.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
+{
+#pragma unroll
+    for (int j = 16; j >= 1; j >>= 1) {
+        const uint32_t m = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        const bool up = (lane & j) != 0;
+        const uint32_t keep = up ? ~m : m;
+        x = (x & keep) | ((up ? y >> j : y << j) & ~keep);
+    }
+    return x;
 }
 
 // kAuto: the SC^2 path is chosen on the device (one problem): no FP4 matrix,
@@ -180,7 +193,6 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
     pdl_release();
     __shared__ __align__(128) float4 srow[kT][2];        // row points as copied (x0,x1,x2,y0 | y1,y2,w,0)
     __shared__ __align__(16) ulonglong2 srow2[kT][3];    // the same six values, each in both halves of a pair
-    __shared__ __align__(16) uint4 srbits[kT];           // row r's four bitset words (ballots of its warp)
     __shared__ __align__(16) uint32_t colpart[kT][4];    // column c: the 32-row masks of the 4 warps
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_wide;
@@ -240,29 +252,30 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
     if (!got && threadIdx.x == 0) atomicOr(&v.ctl->err, TR_ERR_TIMEOUT);
     const float tau = v.tau;
     const Decide K = decide_consts(tau, s_wide != 0 || !(tau >= kTauMin && tau <= kTauMax));
-    // bit r of cmask[q]: G(i0 + 32 warp + r, j_q), before the validity masks;
-    // bit r of nflag: row r has a pair inside the guard band
+    // bit r of cmask[q]: G(i0 + 32 warp + r, j_q), before the validity masks (the
+    // rows' sign bits shifted in one after the other: row 0 at the top until the
+    // reversal); bit r of nflag: row r has a pair inside the guard band.  The
+    // row words are the transposed masks, once per tile: a ballot per row and
+    // word, and the compares it needs, were a seventh of the instructions.
     uint32_t cmask[4] = {0u, 0u, 0u, 0u};
     uint32_t nflag = 0u;
     if (got) {
-#pragma unroll
+        // (half unrolled where many waves of blocks share the instruction cache)
+#pragma unroll kAuto ? kR : kR / 2
         for (int r = 0; r < kR; ++r) {
             const int rr = warp * kR + r;
             const ulonglong2 p0 = srow2[rr][0], p1 = srow2[rr][1], p2 = srow2[rr][2];
             const f2 XI[6] = {{p0.x}, {p0.y}, {p1.x}, {p1.y}, {p2.x}, {p2.y}};
-            bool a[4], nq[4];
-            compat_fast2(XI, XJ[0], K, a[0], a[1], nq[0], nq[1]);
-            compat_fast2(XI, XJ[1], K, a[2], a[3], nq[2], nq[3]);
+            float P[4];
+            bool nq[4];
+            compat_fast2(XI, XJ[0], K, P[0], P[1], nq[0], nq[1]);
+            compat_fast2(XI, XJ[1], K, P[2], P[3], nq[2], nq[3]);
             if (nq[0] | nq[1] | nq[2] | nq[3]) nflag |= 1u << r;
-            uint32_t word[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (a[q]) cmask[q] |= 1u << r;
-                word[q] = __ballot_sync(0xffffffffu, a[q]);
-            }
-            if (lane == 0) srbits[rr] = make_uint4(word[0], word[1], word[2], word[3]);
+            for (int q = 0; q < 4; ++q) cmask[q] = __funnelshift_l(__float_as_uint(P[q]), cmask[q], 1);
         }
-        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cmask[q] = __brev(cmask[q]);
         // rare: the pairs inside the band are decided again in FP64 with the
         // reference operation order, and their bits patched
         if (__any_sync(0xffffffffu, nflag != 0u)) {
@@ -272,11 +285,11 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
                 const int rr = warp * kR + r;
                 const ulonglong2 p0 = srow2[rr][0], p1 = srow2[rr][1], p2 = srow2[rr][2];
                 const f2 XI[6] = {{p0.x}, {p0.y}, {p1.x}, {p1.y}, {p2.x}, {p2.y}};
-                bool a[4], nq[4];
-                compat_fast2(XI, XJ[0], K, a[0], a[1], nq[0], nq[1]);
-                compat_fast2(XI, XJ[1], K, a[2], a[3], nq[2], nq[3]);
+                float P[4];
+                bool nq[4];
+                compat_fast2(XI, XJ[0], K, P[0], P[1], nq[0], nq[1]);
+                compat_fast2(XI, XJ[1], K, P[2], P[3], nq[2], nq[3]);
                 const float4 ra = srow[rr][0], rb = srow[rr][1];
-                uint32_t* wr = reinterpret_cast<uint32_t*>(&srbits[rr]);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (!nq[q]) continue;
@@ -285,42 +298,29 @@ __global__ void __launch_bounds__(kThreads, 8) compat_kernel(ManyViews vs)
                     const float4 ca = pj[0], cb = pj[1];
                     const bool e = compat_fp64(ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, ca.x, ca.y, ca.z, ca.w, cb.x, cb.y,
                                                tau);
-                    if (e) {
-                        cmask[q] |= 1u << r;
-                        atomicOr(wr + q, 1u << lane);
-                    } else {
-                        cmask[q] &= ~(1u << r);
-                        atomicAnd(wr + q, ~(1u << lane));
-                    }
+                    cmask[q] = e ? cmask[q] | (1u << r) : cmask[q] & ~(1u << r);
                 }
             }
         }
     }
     // validity: columns j < n, rows i < n, no diagonal entry
-    uint32_t colv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) colv[q] = __ballot_sync(0xffffffffu, jok[q]);
     const int nrow = min(max(v.n - (i0 + warp * kR), 0), kR);
     const uint32_t rowv = nrow >= 32 ? 0xFFFFFFFFu : (1u << nrow) - 1u;
 #pragma unroll
     for (int q = 0; q < 4; ++q) cmask[q] &= jok[q] ? rowv : 0u;
-    __syncwarp();
     // direct rows i0 + 32 warp + r (r = 0..31): lane r stores row r's bitset words (16 B)
-    uint32_t wrow_bits[4] = {0u, 0u, 0u, 0u};
+    uint32_t wrow_bits[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) wrow_bits[q] = transpose32(cmask[q], lane);
     {
         const int i = i0 + warp * kR + lane;
-        if (got && i < v.n) {
-            const uint4 w = srbits[warp * kR + lane];
-            wrow_bits[0] = w.x & colv[0]; wrow_bits[1] = w.y & colv[1];
-            wrow_bits[2] = w.z & colv[2]; wrow_bits[3] = w.w & colv[3];
-            if (diag) {   // column i - j0 = 32 warp + lane of this row: word warp, bit lane
-                const uint32_t off = ~(1u << lane);
-                const int qc = warp;
-                wrow_bits[0] &= qc == 0 ? off : 0xFFFFFFFFu;
-                wrow_bits[1] &= qc == 1 ? off : 0xFFFFFFFFu;
-                wrow_bits[2] &= qc == 2 ? off : 0xFFFFFFFFu;
-                wrow_bits[3] &= qc == 3 ? off : 0xFFFFFFFFu;
-            }
+        if (diag) {   // column i - j0 = 32 warp + lane of this row: word warp, bit lane
+            const uint32_t off = ~(1u << lane);
+            const int qc = warp;
+            wrow_bits[0] &= qc == 0 ? off : 0xFFFFFFFFu;
+            wrow_bits[1] &= qc == 1 ? off : 0xFFFFFFFFu;
+            wrow_bits[2] &= qc == 2 ? off : 0xFFFFFFFFu;
+            wrow_bits[3] &= qc == 3 ? off : 0xFFFFFFFFu;
         }
         *reinterpret_cast<uint4*>(v.bits + (size_t)i * v.ldb + (j0 >> 5)) =
             make_uint4(wrow_bits[0], wrow_bits[1], wrow_bits[2], wrow_bits[3]);

@@ -243,8 +243,12 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
     }
 }
 
+// Registers: five blocks per SM for the batch's tile (1077 -> 1038 us for 256
+// problems against 120 registers and four blocks); the single problem's balanced
+// launch holds four blocks per SM, and there the spills of that budget cost more
+// (N = 20000 44 -> 46 us).
 template <int PW>
-__global__ void __launch_bounds__(128) verify_kernel(ManyViews vs)
+__global__ void __launch_bounds__(128, PW == 64 ? 5 : 4) verify_kernel(ManyViews vs)
 {
     __shared__ __align__(16) VerifyShared<PW> sh;
     int lb;
