@@ -11,10 +11,11 @@
 // until the process exits).  The caller passes the weight matrix and the output buffers;
 // nothing is allocated or freed, by this code or by any library it calls.
 //
-// The scratch is shared by every call: the histogram and the control block
-// (which holds the active-row and slot counters) are cleared with
-// one cudaMemsetAsync at the start of each call, and two calls whose work overlaps on the GPU (different streams, or
-// different host threads) race on it.  Serialise calls per device.
+// The scratch is shared by every call: the histogram, the row maxima and the
+// control block (which holds the active-row and slot counters) are cleared with
+// one cudaMemsetAsync at the start of each call, and two calls whose work
+// overlaps on the GPU (different streams, or different host threads) race on
+// it.  Serialise calls per device.
 //
 // In host code the name g_pivot_scratch only stands in for the array; its
 // device address comes from cudaGetSymbolAddress, taken with the device
@@ -51,10 +52,10 @@ constexpr int32_t kMaxK1 = TURBOREG_K1_MAX;
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 constexpr size_t kOffCtl = 0;
 constexpr size_t kOffHist = align256(sizeof(Ctl));
-constexpr size_t kOffActive = kOffHist + align256(sizeof(uint32_t) * (kMaxN + 1));
+constexpr size_t kOffRowmax = kOffHist + align256(sizeof(uint32_t) * (kMaxN + 1));
+constexpr size_t kOffActive = kOffRowmax + align256(sizeof(int32_t) * kMaxN);
 constexpr size_t kOffCand = kOffActive + align256(sizeof(int4) * kMaxN);
-constexpr size_t kOffRowmax = kOffCand + align256(sizeof(uint64_t) * kMaxK1);
-constexpr size_t kScratchBytes = kOffRowmax + align256(sizeof(int32_t) * kMaxN);
+constexpr size_t kScratchBytes = kOffCand + align256(sizeof(uint64_t) * kMaxK1);
 
 static __device__ __align__(256) uint8_t g_pivot_scratch[kScratchBytes];
 
@@ -137,12 +138,12 @@ extern "C" int turboreg_select_pivots_noalloc(const uint16_t* w_dev, int32_t n, 
     v.hist = reinterpret_cast<uint32_t*>(scr + kOffHist);
     v.active = reinterpret_cast<int4*>(scr + kOffActive);
     v.cand = reinterpret_cast<uint64_t*>(scr + kOffCand);
-    v.rowmax = reinterpret_cast<int32_t*>(scr + kOffRowmax);   // rows with an edge: written by the histogram
+    v.rowmax = reinterpret_cast<int32_t*>(scr + kOffRowmax);
     v.piv = reinterpret_cast<int4*>(pivots_dev);
 
     // the previous call's contents stay in the array: clear what must start at
-    // zero (the control block and, behind it, the histogram)
-    cudaError_t e = cudaMemsetAsync(scr + kOffCtl, 0, kOffHist + sizeof(uint32_t) * (n + 1), s);
+    // zero (the control block and, behind it, the histogram and the row maxima)
+    cudaError_t e = cudaMemsetAsync(scr + kOffCtl, 0, kOffRowmax + sizeof(int32_t) * n, s);
     if (e != cudaSuccess) return TURBOREG_ERR_CUDA;
     launch_topk_single(v, n_pivots_dev, s);
     e = cudaGetLastError();

@@ -7,9 +7,9 @@
 //
 // Exact radix-style selection; the selected set, and so the pivots, do not
 // depend on the order in which blocks run:
-//   hist    histogram of edge weights (built by the SC^2 pass; by hist_kernel
-//           for the learned weights and for a caller's matrix, there with the
-//           row maxima)
+//   hist    histogram of edge weights (built by the SC^2 pass; by a pass of its
+//           own for the learned weights and for a caller's matrix, there with
+//           the row maxima)
 //   select  alpha = K1-th largest weight, c_gt = #{W > alpha}, m = K1' - c_gt
 //           ties still needed (K1' = min(K1, |E+|)): every count block for
 //           one problem, else one block per problem of the select launch
@@ -135,85 +135,139 @@ __device__ __forceinline__ void for_group_chunks(const ProbView& v, const RowGro
     }
 }
 
-// Histogram of edge weights, for the learned weights and for a caller's
-// matrix: the count pass's groups of row pairs (all rows read, in one or a few
-// rounds of eight loads per thread), shared-memory bins when they fit.  It
-// reads the upper triangle once; bound by the instructions on the non-zero
-// words.  One warp per row with two loads in flight and 64 rows per block (79
-// blocks, a chain of 80 load rounds per warp) took 196 us at n = 5000; the
-// whole selection call went from 231 to 49 us, a learned batch of 32 problems
-// from 1075 to 951 us.
-// A caller's weight above n - 2 (no SC^2 count can be larger; the bins end at
-// n) is not counted: it sets TR_ERR_BAD_WEIGHT, and nothing is selected then;
-// a caller's row maxima are recorded, so that the count pass skips rows.
-template <class VS, bool kSmem>
-__global__ void __launch_bounds__(kCountThreads, 3) hist_kernel(VS vs)
+// floor of a learned weight fl(fl(W p_i) p_j), the integer pivot_weight takes:
+// added to 2^23 toward zero, the floor is the low bits (0 <= W p_i p_j < 2^15;
+// a NaN counts as 0, as the conversion has it).
+__device__ __forceinline__ uint32_t learned_weight(uint32_t w, float pi, float pj)
+{
+    const float x = __fmul_rn(__fmul_rn(__uint_as_float(0x4B000000u | w) - 8388608.f, pi), pj);
+    return __float_as_uint(__fadd_rz(fmaxf(x, 0.f), 8388608.f)) & 0x7FFFFFu;
+}
+
+// Histogram of the learned weights: the groups of row pairs of the count pass.
+// Most rows hold only zeros (their bound is below 1) and are skipped, so the
+// chunks of the others are spread over the whole block (a warp per row pair
+// took 144 us instead of 99 for 32 problems: one or two warps of a block had
+// all its rows).
+template <bool kSmem>
+__global__ void __launch_bounds__(kCountThreads, 3) learned_hist_kernel(ManyViews vs)
 {
     int lb;
     const ProbView v = vs.get(ST_HIST, blockIdx.x, lb);   // launch descriptors: before the wait
     extern __shared__ uint32_t sh[];
     __shared__ RowGroup sg;
-    __shared__ uint32_t smax[16];
     const int n = v.n, t = threadIdx.x;
     if (kSmem)
         for (int q = t; q <= n; q += kCountThreads) sh[q] = 0;
     pdl_wait();
     pdl_release();
-    const bool learned = v.prob != nullptr;
+    uint32_t* const bins = kSmem ? sh : v.hist;
     const int groups = count_groups(n), stride = hist_blocks(n);
-    bool bad = false;
     for (int g = lb; g < groups; g += stride) {
         __syncthreads();   // the bins are cleared; the previous group's list is consumed
-        int row;
-        bool act = group_row(g, t, n, row);
         if (t < 32) {
-            // learned weights: a row whose bound is below 1 holds only zeros (not counted)
-            if (act && learned) act = learned_row_bound(v, row) >= 1.f;
+            int row;
+            const bool act = group_row(g, t, n, row) && learned_row_bound(v, row) >= 1.f;
             group_offsets(sg, t, row, act, n);
-            if (t < 16) smax[t] = 0u;
         }
         __syncthreads();
-        int kcur = -1;
-        uint32_t mx = 0u;   // running maximum of entry kcur's weights, two 16-bit halves
-        auto flush_max = [&]() {
-            const uint32_t m = max(mx & 0xFFFFu, mx >> 16);
-            if (m) atomicMax(&smax[kcur], m);
-        };
-        for_group_chunks(v, sg, t, [&](int k, int row_k, int c, uint4 q) {
-            const uint32_t u[4] = {q.x, q.y, q.z, q.w};
-            if (VS::kCallerWeights) {
-                if (k != kcur) {
-                    if (kcur >= 0) flush_max();
-                    kcur = k;
-                    mx = 0u;
-                }
-                mx = __vmaxu2(mx, __vmaxu2(__vmaxu2(u[0], u[1]), __vmaxu2(u[2], u[3])));
-            }
+        for_group_chunks(v, sg, t, [&](int, int row, int c, uint4 q) {
+            if ((q.x | q.y | q.z | q.w) == 0u) return;
+            const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
+            const float pi = __ldcg(v.prob + row);
+            // (n_pad is a multiple of 256: the probabilities of a whole chunk can be read)
+            const float4 pa = __ldcg(reinterpret_cast<const float4*>(v.prob + c * 8));
+            const float4 pb = __ldcg(reinterpret_cast<const float4*>(v.prob + c * 8 + 4));
+            const float pj[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                if (u[e >> 1] == 0u) continue;
-                int w = static_cast<int>((u[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu);
-                if (!VS::kCallerWeights) w = pivot_weight(v, row_k, c * 8 + e, w);
-                if (VS::kCallerWeights && w > n - 2) {
-                    bad = true;
-                } else if (w > 0) {
-                    if (kSmem) atomicAdd(&sh[w], 1u);
-                    else atomicAdd(&v.hist[w], 1u);
-                }
+                const uint32_t w = (wd[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu;
+                const uint32_t pw = w != 0u ? learned_weight(w, pi, pj[e]) : 0u;
+                if (pw != 0u) atomicAdd(bins + pw, 1u);
             }
         });
-        if (VS::kCallerWeights) {
-            if (kcur >= 0) flush_max();
-            __syncthreads();
-            if (act && t < 16) v.rowmax[row] = static_cast<int>(smax[t]);
-        }
     }
-    if (VS::kCallerWeights && bad) atomicOr(&v.ctl->err, TR_ERR_BAD_WEIGHT);
     if (kSmem) {
         __syncthreads();
         for (int q = t; q <= n; q += kCountThreads)
             if (sh[q]) atomicAdd(&v.hist[q], sh[q]);
     }
+}
+
+// Histogram of a caller's matrix (n <= 8192: the bins fit in shared memory),
+// one block per SM.  The chunks of a row pair (p, n-1-p), about n/8 together,
+// are cut into windows of 256, and the warps of the grid take windows, eight
+// 16-byte loads per lane in flight.  It reads the upper triangle once; the
+// entries of a chunk are counted by predicated additions without branches.  One
+// block per SM because every block adds its bins to the same few hundred
+// global ones.  At n = 5000: 15.0 us; with 313 blocks of a warp per pair 20.4, 625
+// of two 22.4; with the chunks of 16 rows spread over a block, each looking up
+// its row and checking every entry, 24.7; with a warp per row, two loads in
+// flight and 64 rows per block 196 (the whole selection then 231 us, now 35).
+// A weight above n - 2 (no SC^2 count can be larger; the bins end at n) is not
+// counted: it sets TR_ERR_BAD_WEIGHT, and nothing is selected then.  The row
+// maxima (cleared before) are recorded, so that the count pass skips rows.
+constexpr int kWindow = 256;
+__host__ __device__ inline int caller_windows(int n) { return (n / 8 + 2 + kWindow - 1) / kWindow; }   // per pair
+
+__global__ void __launch_bounds__(1024, 1) caller_hist_kernel(OneView vs)
+{
+    int lb;
+    const ProbView v = vs.get(ST_HIST, blockIdx.x, lb);
+    extern __shared__ uint32_t sh[];
+    const int n = v.n, t = threadIdx.x, lane = t & 31;
+    for (int q = t; q <= n; q += 1024) sh[q] = 0;
+    pdl_wait();
+    pdl_release();
+    __syncthreads();   // the bins are cleared
+    const int c1 = (n - 1) >> 3, nw = caller_windows(n), items = (n + 1) / 2 * nw;
+    const uint32_t wmax = static_cast<uint32_t>(max(n - 2, 0));
+    bool bad = false;
+    for (int it = (t >> 5) * static_cast<int>(gridDim.x) + lb; it < items; it += 32 * static_cast<int>(gridDim.x)) {
+        const int p = it / nw, x0 = (it - p * nw) * kWindow + lane;
+        const int ra = p, rb = n - 1 - p;   // (one row when they meet)
+        const int ca = (ra + 1) >> 3, cb = (rb + 1) >> 3;
+        const int la = ra + 1 < n ? c1 - ca + 1 : 0, lt = la + (rb > ra && rb + 1 < n ? c1 - cb + 1 : 0);
+        const uint16_t *wa = v.w + (size_t)ra * v.n_pad, *wb = v.w + (size_t)rb * v.n_pad;
+        uint4 q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int x = x0 + 32 * u;
+            q[u] = x < lt ? *reinterpret_cast<const uint4*>(x < la ? wa + (ca + x) * 8 : wb + (cb + x - la) * 8)
+                          : make_uint4(0u, 0u, 0u, 0u);
+        }
+        uint32_t ma = 0u, mb = 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int x = x0 + 32 * u;
+            const bool in_a = x < la;
+            const uint4 qm = mask_chunk(q[u], in_a ? ca + x : cb + x - la, in_a ? ra : rb, n);
+            const uint32_t wd[4] = {qm.x, qm.y, qm.z, qm.w};
+            const uint32_t m2 = __vmaxu2(__vmaxu2(wd[0], wd[1]), __vmaxu2(wd[2], wd[3]));
+            const uint32_t m = max(m2 & 0xFFFFu, m2 >> 16);
+            if (in_a) ma = max(ma, m);
+            else mb = max(mb, m);
+            if (m > wmax) {
+                bad = true;
+                continue;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const uint32_t w = (wd[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu;
+                if (w != 0u) atomicAdd(sh + w, 1u);
+            }
+        }
+        ma = __reduce_max_sync(0xffffffffu, ma);
+        mb = __reduce_max_sync(0xffffffffu, mb);
+        if (lane == 0) {
+            if (ma != 0u) atomicMax(v.rowmax + ra, static_cast<int>(ma));
+            if (mb != 0u) atomicMax(v.rowmax + rb, static_cast<int>(mb));
+        }
+    }
+    if (bad) atomicOr(&v.ctl->err, TR_ERR_BAD_WEIGHT);
+    __syncthreads();
+    for (int q = t; q <= n; q += 1024)
+        if (sh[q]) atomicAdd(&v.hist[q], sh[q]);
 }
 
 __global__ void __launch_bounds__(1024) select_kernel(ManyViews vs)
@@ -658,15 +712,6 @@ __global__ void __launch_bounds__(256) rank_kernel(OneView vs, int32_t* n_out)
 
 int g_num_sms = 0;
 
-template <class VS>
-void launch_hist_vs(const VS& vs, int total, int max_n, cudaStream_t s)
-{
-    if (max_n + 1 <= kHistSmemMaxBins)
-        launch_pdl(hist_kernel<VS, true>, total, kCountThreads, (max_n + 1) * 4, s, vs);
-    else
-        launch_pdl(hist_kernel<VS, false>, total, kCountThreads, 0, s, vs);
-}
-
 }  // namespace
 
 cudaError_t topk_setup()
@@ -680,16 +725,16 @@ cudaError_t topk_setup()
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(hist_kernel<ManyViews, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kHistSmemMaxBins * 4);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(hist_kernel<OneView, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(learned_hist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kHistSmemMaxBins * 4);
 }
 
 void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s)
 {
-    launch_hist_vs(ManyViews{b}, total, max_n, s);
+    if (max_n + 1 <= kHistSmemMaxBins)
+        launch_pdl(learned_hist_kernel<true>, total, kCountThreads, (max_n + 1) * 4, s, ManyViews{b});
+    else
+        launch_pdl(learned_hist_kernel<false>, total, kCountThreads, 0, s, ManyViews{b});
 }
 
 void launch_select(const Batch& b, cudaStream_t s) { launch_pdl(select_kernel, b.num, 1024, 0, s, ManyViews{b}); }
@@ -718,7 +763,8 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
 void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s)
 {
     const OneView vs{v};
-    launch_hist_vs(vs, hist_blocks(v.n), v.n, s);
+    const int warps = (v.n + 1) / 2 * caller_windows(v.n), sms = g_num_sms > 0 ? g_num_sms : 148;
+    launch_pdl(caller_hist_kernel, (warps + 31) / 32 < sms ? (warps + 31) / 32 : sms, 1024, (v.n + 1) * 4, s, vs);
     launch_pdl(count_kernel<OneView>, count_groups(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
                vs, 1);
     if (emit_by_warp(v.n, false)) launch_pdl(emit_warp_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
