@@ -208,7 +208,8 @@ __global__ void __launch_bounds__(kCountThreads, 3) learned_hist_kernel(ManyView
 // counted: it sets TR_ERR_BAD_WEIGHT, and nothing is selected then.  The row
 // maxima (cleared before) are recorded, so that the count pass skips rows.
 constexpr int kWindow = 256;
-__host__ __device__ inline int caller_windows(int n) { return (n / 8 + 2 + kWindow - 1) / kWindow; }   // per pair
+// windows per pair, whose two rows hold at most n / 8 + 3 chunks (both round outwards)
+__host__ __device__ inline int caller_windows(int n) { return (n / 8 + 3 + kWindow - 1) / kWindow; }
 
 __global__ void __launch_bounds__(1024, 1) caller_hist_kernel(OneView vs)
 {

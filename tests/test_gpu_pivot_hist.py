@@ -1,5 +1,6 @@
 """Weight histogram and row maxima of the pivot selection at the edges of its
-row-pair groups (16 rows) and 8-weight chunks, and, for the learned weights,
+row-pair groups (16 rows), 8-weight chunks and 256-chunk windows (at n = 2035 a
+pair of rows holds one chunk more than a window), and, for the learned weights,
 where a block takes several groups (n > 8192).  All results are whole numbers:
 equal, not close."""
 import numpy as np
@@ -12,8 +13,8 @@ from test_zz_no_alloc import _noalloc, _packed_w
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,wmax", [(3, 1), (15, 13), (16, 14), (17, 15), (31, 5), (33, 31), (257, 255), (8191, 60),
-                                    (8192, 8190)])
+@pytest.mark.parametrize("n,wmax", [(3, 1), (15, 13), (16, 14), (17, 15), (31, 5), (33, 31), (257, 255), (2033, 90),
+                                    (2035, 300), (4085, 60), (8179, 60), (8191, 60), (8192, 8190)])
 def test_caller_weights(n, wmax):
     import oracle
     k1 = min(8192, 3 * n)
