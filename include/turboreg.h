@@ -88,7 +88,8 @@ typedef enum {
                                              (cta_group::2), each CTA holding half of A and of B
                                              (same integers either way) */
 #define TURBOREG_FLAG_VERIFY_PTS32 0x10u   /* verification tile of 128 hypotheses x 128 matches per block */
-#define TURBOREG_FLAG_VERIFY_PTS128 0x20u  /* ... x 512 matches per block (default: 256); tile shapes are
+#define TURBOREG_FLAG_VERIFY_PTS128 0x20u  /* ... x 512 matches per block (default: 256, or 512 in a batch
+                                              with many blocks; one problem without tile flags: balanced);
                                               chosen by the autotuner (same results either way); in a
                                               batch the first problem's tile flags apply to all */
 

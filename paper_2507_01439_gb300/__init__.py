@@ -75,6 +75,7 @@ _RESULT_DTYPE = np.dtype([("R", np.float32, (3, 3)), ("t", np.float32, 3), ("cli
                           ("n_valid", np.int32), ("used_fp64", np.int32), ("used_fallback", np.int32),
                           ("status", np.int32), ("score", np.float32)])
 assert _RESULT_DTYPE.itemsize == ctypes.sizeof(turboreg_result)
+assert turboreg_result.clique.offset == 48 and turboreg_result.status.offset == 84
 
 _lib = None
 
@@ -220,10 +221,10 @@ class Result:
         """The results of a ctypes turboreg_result array, converted a field at a
         time (one by one, 256 results took 0.6 ms of a batched call)."""
         a = np.frombuffer(out, _RESULT_DTYPE)
-        cols = [a[f].tolist() for f in ("inlier_count", "hypothesis", "n_pivots", "n_valid", "used_fp64",
-                                        "used_fallback", "score")]
-        return [Result(*row) for row in zip(a["status"].tolist(), a["R"].copy(), a["t"].copy(),
-                                            map(tuple, a["clique"].tolist()), *cols)]
+        # words 12 .. 21: clique, inlier_count, hypothesis, n_pivots, n_valid, used_fp64, used_fallback, status
+        words = a.view(np.int32).reshape(len(a), -1)[:, 12:22].tolist()
+        return [Result(w[9], R, t, (w[0], w[1], w[2]), w[3], w[4], w[5], w[6], w[7], w[8], score)
+                for R, t, w, score in zip(a["R"].copy(), a["t"].copy(), words, a["score"].tolist())]
 
 
 class ResultSlots:

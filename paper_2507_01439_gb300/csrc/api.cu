@@ -391,8 +391,17 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
     // problem without tile flags the balanced width (one even wave); the
     // kernel's points per warp (plan.vpw) is the narrowest that holds them all
     const bool vflag = (prm[0]->flags & (TURBOREG_FLAG_VERIFY_PTS32 | TURBOREG_FLAG_VERIFY_PTS128)) != 0;
+    // a batch without tile flags: 512 matches per block while that leaves at
+    // least 16 blocks per SM (256 problems of N = 500 .. 5000 with the default
+    // pivots: 4668 -> 4599 us per call; with few blocks the wide tile loses: 64
+    // problems of N = 60 .. 600 take 122 us with 256 matches, 126 with 512, and
+    // 32 with 100 pivots 613 and 618)
+    int64_t wide = 0;   // blocks of the wide tile (128 hypotheses x 512 matches)
+    for (int32_t b = 0; b < num; ++b)
+        wide += static_cast<int64_t>((prm[b]->k1 * prm[b]->k2 + 127) / 128) * ((n[b] + 511) / 512);
     const int32_t vpw_flag = (prm[0]->flags & TURBOREG_FLAG_VERIFY_PTS32) ? 32
-                             : (prm[0]->flags & TURBOREG_FLAG_VERIFY_PTS128) ? 128 : 64;
+                             : (prm[0]->flags & TURBOREG_FLAG_VERIFY_PTS128) ? 128
+                             : num > 1 && !vflag && wide >= 16 * static_cast<int64_t>(device_sms()) ? 128 : 64;
     int32_t vppb_max = 0;
     plan.k2_common = prm[0]->k2;
     for (int st = 0; st < kNumBatchStages; ++st) ws.h_pre[st * (num + 1)] = 0;

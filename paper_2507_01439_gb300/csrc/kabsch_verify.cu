@@ -7,6 +7,8 @@
 //
 // The closed-form 3-point Kabsch itself is in tr_kabsch.cuh.
 //
+#include <type_traits>
+
 #include "tr_common.cuh"
 #include "tr_kabsch.cuh"
 #include "tr_problem.h"
@@ -243,12 +245,12 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
     }
 }
 
-// Registers: five blocks per SM for the batch's tile (1077 -> 1038 us for 256
-// problems against 120 registers and four blocks); the single problem's balanced
-// launch holds four blocks per SM, and there the spills of that budget cost more
+// Registers: five blocks per SM in a batch (kMany; 256 problems 1077 -> 1038 us
+// against 120 registers and four blocks); the single problem's balanced launch
+// holds four blocks per SM, and there the spills of that budget cost more
 // (N = 20000 44 -> 46 us).
-template <int PW>
-__global__ void __launch_bounds__(128, PW == 64 ? 5 : 4) verify_kernel(ManyViews vs)
+template <int PW, bool kMany>
+__global__ void __launch_bounds__(128, kMany ? 5 : 4) verify_kernel(ManyViews vs)
 {
     __shared__ __align__(16) VerifyShared<PW> sh;
     int lb;
@@ -430,14 +432,14 @@ void launch_kabsch(const Batch& b, int total, cudaStream_t s)
 
 cudaError_t verify_setup()
 {
-    cudaError_t e = cudaFuncSetAttribute(verify_kernel<32>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(verify_kernel<64>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(verify_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
+    const void* all[] = {
+        reinterpret_cast<const void*>(&verify_kernel<32, false>),  reinterpret_cast<const void*>(&verify_kernel<64, false>),
+        reinterpret_cast<const void*>(&verify_kernel<128, false>), reinterpret_cast<const void*>(&verify_kernel<32, true>),
+        reinterpret_cast<const void*>(&verify_kernel<64, true>),   reinterpret_cast<const void*>(&verify_kernel<128, true>)};
+    cudaError_t e = cudaSuccess;
+    for (const void* f : all)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     // padding that leaves room for kCapPerSm blocks per SM and no more: the
     // balanced single-problem tile launches exactly kCapPerSm blocks per SM, and
@@ -448,9 +450,7 @@ cudaError_t verify_setup()
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess) return e;
-    const void* fns[3] = {reinterpret_cast<const void*>(&verify_kernel<32>),
-                          reinterpret_cast<const void*>(&verify_kernel<64>),
-                          reinterpret_cast<const void*>(&verify_kernel<128>)};
+    const void* const* fns = all;   // the single problem's forms
     for (int k = 0; k < 3; ++k) {
         cudaFuncAttributes fa;
         if ((e = cudaFuncGetAttributes(&fa, fns[k])) != cudaSuccess) return e;
@@ -469,9 +469,14 @@ void launch_verify(const Batch& b, int total, int pw, bool capped, cudaStream_t 
 {
     const int k = pw == 32 ? 0 : pw == 128 ? 2 : 1;
     const size_t dyn = capped ? static_cast<size_t>(g_cap_dyn[k]) : 0;
-    if (pw == 32) launch_pdl(verify_kernel<32>, total, 128, dyn, s, ManyViews{b});
-    else if (pw == 128) launch_pdl(verify_kernel<128>, total, 128, dyn, s, ManyViews{b});
-    else launch_pdl(verify_kernel<64>, total, 128, dyn, s, ManyViews{b});
+    auto go = [&](auto many) {
+        constexpr bool kM = decltype(many)::value;
+        if (pw == 32) launch_pdl(verify_kernel<32, kM>, total, 128, dyn, s, ManyViews{b});
+        else if (pw == 128) launch_pdl(verify_kernel<128, kM>, total, 128, dyn, s, ManyViews{b});
+        else launch_pdl(verify_kernel<64, kM>, total, 128, dyn, s, ManyViews{b});
+    };
+    if (b.num > 1) go(std::true_type{});
+    else go(std::false_type{});
 }
 
 // Per-problem block counts of every stage.
