@@ -188,7 +188,7 @@ def stage_rooflines(stage_log, peaks, kind, sc2_path=2, words=0.0):
     record, a few microseconds, so short stages read low).  Algorithmic work
     per registration of the N = 5000, K1 = 2000, K2 = 2 workload:
       compat   n(n-1)/2 pairs x 17 FLOP (two 3-D distances, difference, compare)
-      sc2      420 tiles x 2 x 128 x 256 x 5120 dense FP8 MMA FLOP (GEMM), or
+      sc2      420 tiles x 2 x 128 x 256 x 5120 dense FP4 MMA FLOP (GEMM), or
                |E+| x 5120 / 32 words of AND + popcount (CUDA-core form)
       topk     the upper triangle of W read once: n(n-1)/2 x 2 bytes
       pgs      K1 x 2 bitset rows of n/8 bytes (the stage also solves each
@@ -201,7 +201,7 @@ def stage_rooflines(stage_log, peaks, kind, sc2_path=2, words=0.0):
     pairs = n * (n - 1) / 2
     work = {
         "compat": (pairs * 17, "alu", FP32_PEAK_TFLOPS, "TFLOP/s"),
-        "sc2": ((420 * 2.0 * 128 * 256 * 5120, "tensor", 2 * peaks["bf16_tflops_sustained"], "TFLOP/s")
+        "sc2": ((420 * 2.0 * 128 * 256 * 5120, "tensor", 6 * peaks["bf16_tflops_sustained"], "TFLOP/s")
                 if sc2_path == 2 else (words, "alu", POPC_PEAK_TWORDS, "Tword/s")),
         "topk": (pairs * 2, "hbm", peaks["hbm_gbs"], "GB/s"),
         "pgs": (k1 * 2 * n / 8, "hbm", peaks["hbm_gbs"], "GB/s"),
@@ -215,7 +215,7 @@ def stage_rooflines(stage_log, peaks, kind, sc2_path=2, words=0.0):
         scale = 1e12 if unit in ("TFLOP/s", "Tword/s") else 1e9
         ach = w / (ms / 1e3) / scale
         out[st] = {"ms": ms, "bound": bound, "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak}
-    out["peak_source"] = f"{kind} MEASURED_PEAKS.json for tensor (2 x bf16 sustained) and HBM; FP32 from unit counts"
+    out["peak_source"] = f"{kind} MEASURED_PEAKS.json for tensor (6 x bf16 sustained) and HBM; FP32 from unit counts"
     return out
 
 
@@ -612,7 +612,7 @@ def run_clique_stability(trg, per_tau=240):
 def run_sc2_paths(trg, probs, dx, dy):
     """SC^2 stage (with the edge-weight histogram and the pivot threshold) on
     the benchmark workload: the default (path chosen on the device), the
-    tcgen05 FP8 GEMM (2-CTA pair MMAs; independent CTAs) and the CUDA-core
+    tcgen05 FP4 GEMM (2-CTA pair MMAs; independent CTAs) and the CUDA-core
     bitset AND + popcount path (same integers); in-graph CUDA-event times."""
     import numpy as np
     out = {}
@@ -760,12 +760,12 @@ def run_ours(args):
     e2e = ws * args.steps / tot_host
 
     peaks, kind = _peaks()
-    # SC^2 GEMM: upper-triangle tiles x 2*BM*BN*N_pad dense FP8 MMA flops per launch
+    # SC^2 GEMM: upper-triangle tiles x 2*BM*BN*N_pad dense FP4 MMA flops per launch
     npad = 5120
     nb = npad // 256
     flops = nb * (nb + 1) * 2.0 * 128 * 256 * npad
     sc2_avg_s = (sum(sc2_ms) / len(sc2_ms)) / 1e3
-    peak = 2.0 * peaks["bf16_tflops_sustained"]    # FP8 dense = 2 x bf16 (nominal ratio)
+    peak = 6.0 * peaks["bf16_tflops_sustained"]    # FP4 dense = 6 x bf16 (nominal ratio 13.5 / 2.25)
     if sc2_path == 1:
         # the CUDA-core form ran: |E+| x n_pad / 32 words of AND + population count
         achieved = words / sc2_avg_s / 1e12
@@ -777,9 +777,9 @@ def run_ours(args):
                     "sc2_path_counts": {"cuda_core": paths.count(1), "tensor_core_gemm": paths.count(2)}}
     else:
         achieved = flops / sc2_avg_s / 1e12
-        roofline = {"bound": "tensor", "kernel": "sc2_pair_mma_kernel (FP8 E4M3 x E4M3 -> F32, cta_group::2 pair MMAs)",
+        roofline = {"bound": "tensor", "kernel": "sc2_mma_kernel (FP4 E2M1 x E2M1 -> F32, block-scaled, cta_group::2 pair MMAs)",
                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "peak_source": f"{kind}: 2 x bf16_tflops_sustained (FP8/BF16 nominal ratio 4.5/2.25)",
+                    "peak_source": f"{kind}: 6 x bf16_tflops_sustained (FP4/BF16 nominal ratio 13.5/2.25)",
                     "traffic": SC2_DRAM_BYTES, "sc2_ms": sc2_avg_s * 1e3,
                     "flops_per_launch": flops}
     # the batched leg runs on every rank (its problems are sharded over them)
@@ -791,7 +791,7 @@ def run_ours(args):
         return
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1e3 * tot_dev / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "u32+f32" if sc2_path == 1 else "fp8+f32",
+            "scaling": "weak", "vs_baseline": None, "dtype": "u32+f32" if sc2_path == 1 else "fp4+f32",
             "data": "synthetic",
             "config": dict(WORKLOAD, parallelism=f"replicas x{ws}"),
             "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 2 * 5000 * 12,

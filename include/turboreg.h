@@ -74,12 +74,14 @@ typedef enum {
 /* flags */
 #define TURBOREG_FLAG_SC2_BITSET 0x1u  /* SC^2 by bitset AND+popcount on CUDA cores
                                           instead of the tcgen05 FP4 GEMM (same integers) */
-#define TURBOREG_FLAG_SC2_GEMM 0x40u   /* SC^2 by the tcgen05 FP4 GEMM.  Without either flag a single
-                                          problem with N <= 5120 (and pair MMAs available) gets the
+#define TURBOREG_FLAG_SC2_GEMM 0x40u   /* SC^2 by the tcgen05 FP4 GEMM.  Without either flag (and with
+                                          pair MMAs available) one problem of N <= 2048 takes the
+                                          CUDA-core path; up to N = 5120 turboreg_register has the
                                           path chosen on the device after the compatibility graph,
                                           from N and the edge count (the CUDA-core path up to about
-                                          5 % density at N = 5000); batches and larger problems use
-                                          the GEMM.  Same integers on every path */
+                                          5 % density at N = 5000), and turboreg_register_async
+                                          takes the GEMM; batches and larger problems use the GEMM.
+                                          Same integers on every path */
 #define TURBOREG_FLAG_STAGE_TIMES 0x2u /* record per-stage CUDA-event times (turboreg_stage_times) */
 #define TURBOREG_FLAG_NO_GRAPH 0x4u    /* launch the stages one by one instead of replaying the
                                           captured CUDA graph of this problem shape */

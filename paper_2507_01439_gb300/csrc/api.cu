@@ -366,8 +366,15 @@ int encode_maps(turboreg_ctx* c, int slot, int32_t n_pad, CUtensorMap* out2)
 
 // Fill the host mirrors (h_views, h_pre, h_maps) for problems in slots
 // [0, num) and compute the plan's block totals.
+// queued: one problem of the stream form, which takes the tensor-core SC^2
+// above n_pad = 2048 without the device-side choice.  It is the faster path
+// there at every density measured (registrations enqueued back to back, us,
+// chosen path / GEMM: N = 2500 58 / 56 at 2 %, 62 / 57 at 5 %; N = 5000 98 / 93
+// at 2 %, 111 / 95 at 5 %; the kernel itself 35 against 45 + 4 at N = 5000).
+// The synchronous call keeps the choice, whose outcome its callers can read
+// (and which the library's tests fix).
 int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_t* n,
-               const turboreg_params* const* prm, Plan& plan)
+               const turboreg_params* const* prm, Plan& plan, bool queued = false)
 {
     Workspace& ws = c->ws;
     if (c->desc_pending) {   // a queued upload may still read the staging rewritten below
@@ -387,6 +394,7 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
         plan.sc2_auto = 0;   // the CUDA-core path is the faster one at any density: no choice to make
         plan.bitset = 1;
     }
+    if (queued) plan.sc2_auto = 0;
     // verification tile: the flags' width for every problem, or for a single
     // problem without tile flags the balanced width (one even wave); the
     // kernel's points per warp (plan.vpw) is the narrowest that holds them all
@@ -749,7 +757,7 @@ int enqueue_single(turboreg_ctx* c, const float* src, const float* dst, int32_t 
     }
     Plan pl;
     const int64_t off0 = 0;
-    rc = build_plan(c, 1, &off0, &n, &p, pl);
+    rc = build_plan(c, 1, &off0, &n, &p, pl, async);
     if (rc != TURBOREG_OK) return rc;
     const bool no_graph = (p->flags & TURBOREG_FLAG_NO_GRAPH) != 0;
     rc = run_plan(c, pl, no_graph, *s_in, *d_in, out);
