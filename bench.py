@@ -52,16 +52,17 @@ UNIT = "registrations/s"
 WORKLOAD = {"workload": "indoor-shaped single problem", "n": 5000, "inlier_ratio": 0.05, "sigma_m": 0.01,
             "tau_m": 0.1, "k1": 2000, "k2": 2, "inlier_thresh_m": 0.1, "problems_cycled": 8,
             "l2": "flushed between timed steps (256 MB write, outside the events)"}
-# kernels of ours launched per registration: pack, compat, sc2 (with the histogram and
-# the threshold choice; one problem without an SC^2 flag: the CUDA-core kernel, which
-# chooses the path, then the GEMM kernel, which runs or returns at once), count, emit,
-# pgs (with the pivot ranks and the cliques' Kabsch), verify, finalize
-LAUNCHES_PER_STEP = 9
+# kernels of ours launched per registration.  Stream form: pack, compat, SC^2 (the GEMM),
+# count, emit, pgs (with the pivot ranks and the cliques' Kabsch), verify, finalize; the
+# synchronous call without an SC^2 flag: the CUDA-core kernel, which chooses the path,
+# then the GEMM kernel, which runs or returns at once
+LAUNCHES_STREAM = 8
+LAUNCHES_SYNC = 9
 # DRAM bytes (read + write) of one launch of each SC^2 kernel on this workload, from one
-# ncu capture of the current kernel (profiles/sc2_pair_mma_indoor5000.txt,
+# ncu capture of the current kernel (profiles/sc2_mma_indoor5000.txt,
 # profiles/sc2_bitset_indoor5000.txt); None when the kernel has changed since, until
 # it has been captured again
-SC2_DRAM_BYTES = 28775424
+SC2_DRAM_BYTES = 229120
 SC2_BITSET_DRAM_BYTES = 3346176
 # the population count's rate: 16 per clock per SM on 152 SMs at the 2.07 GHz maximum clock
 POPC_PEAK_TWORDS = 16 * 152 * 2.07e9 / 1e12
@@ -389,7 +390,7 @@ def run_batched(trg, torch, stream, steps, warmup, flush, ws=1, rank=0):
             "mean_n": float(sum(p.n for p in allp) / len(allp)),
             "success": default["success"] + " (indoor RE<15deg TE<0.3m, outdoor RE<5deg TE<0.6m)",
             "default_k1": "2000 indoor-shaped, 1000 outdoor-shaped", "autotuned": tuned,
-            "stage_ms": stage_ms, "gpu_launches_per_call": 9}
+            "stage_ms": stage_ms, "gpu_launches_per_call": 11}
 
 
 def run_learned(trg, torch, stream, flush, ks=(1, 2, 4, 8, 100, 250, 500, 1000)):
@@ -677,7 +678,8 @@ def run_ours(args):
     prm = trg.default_params(0.1, 2000, 0.1)
     # roofline pass only: CUDA events inside the graph around every stage (they cost
     # ~40 us per registration, so the throughput passes run without them)
-    prm_ev = trg.default_params(0.1, 2000, 0.1, flags=trg.FLAG_STAGE_TIMES)
+    # (the synchronous call with the stream form's SC^2 path)
+    prm_ev = trg.default_params(0.1, 2000, 0.1, flags=trg.FLAG_STAGE_TIMES | trg.FLAG_SC2_GEMM)
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
     torch.cuda.synchronize()
 
@@ -685,13 +687,17 @@ def run_ours(args):
     import synth
     ok = 0
     first_results = []
-    edges, paths = [], []
+    edges, paths, sync_paths = [], [], []
+    guard = trg.ResultSlots(len(probs))
     for k, p in enumerate(probs):
         r = ctx.register(dx[k], dy[k], prm)
         first_results.append(r)
         ok += int(r.status == 0 and synth.rotation_error_deg(p.R_gt, r.R) < 15.0
                   and synth.translation_error(p.t_gt, r.t) < 0.3)
-        paths.append(ctx.sc2_path())   # the SC^2 path the device chose for this problem
+        sync_paths.append(ctx.sc2_path())   # the SC^2 path the device chose for this problem
+        ctx.register_async(dx[k], dy[k], prm, guard, k)
+        ctx.synchronize()
+        paths.append(ctx.sc2_path())        # the stream form's, which is timed
         edges.append(int(np.unpackbits(ctx.buffer(trg.BUF_ADJ_BITS).view(np.uint8)).sum()) // 2)
     sc2_path = max(set(paths), key=paths.count)
     words = (sum(edges) / len(edges)) * 5120 / 32   # |E+| x n_pad / 32 words of AND + popc
@@ -707,8 +713,14 @@ def run_ours(args):
         sc2 = []
         p_k = prm_ev if kind == "stages" else prm
         slots = trg.ResultSlots(steps)
-        for k in range(warmup):
-            ctx.register(dx[k % 8], dy[k % 8], p_k)
+        for k in range(warmup):   # the call that is timed (each form replays a graph of its own)
+            if kind == "device":
+                ctx.register_async(dx[k % 8], dy[k % 8], p_k, slots, 0)
+            elif kind == "host":
+                ctx.register_async(hx[k % 8], hy[k % 8], p_k, slots, 0)
+            else:
+                ctx.register(dx[k % 8], dy[k % 8], p_k)
+        ctx.synchronize()
         torch.cuda.synchronize()
         if ws > 1:
             dist.barrier()
@@ -796,9 +808,10 @@ def run_ours(args):
             "config": dict(WORKLOAD, parallelism=f"replicas x{ws}"),
             "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 2 * 5000 * 12,
                     "d2h_bytes_per_step": ctypes.sizeof(trg.turboreg_result)},
+            "sync_sc2_path_counts": {"cuda_core": sync_paths.count(1), "tensor_core_gemm": sync_paths.count(2)},
             "sync_call": {"ms_per_call": statistics.mean(ms_sync),
                           "value": 1e3 / statistics.mean(ms_sync), "unit": UNIT},
-            "gpu_launches": LAUNCHES_PER_STEP * (3 * args.steps + len(ms_stages)),
+            "gpu_launches": (2 * LAUNCHES_STREAM + LAUNCHES_SYNC) * args.steps + LAUNCHES_STREAM * len(ms_stages),
             "roofline": roofline, "clocks": clocks,
             "success_rate_check": f"{ok}/8 problems RE<15deg TE<0.3m"}
     if batched is not None:
