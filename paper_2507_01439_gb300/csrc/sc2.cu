@@ -690,8 +690,8 @@ cudaError_t sc2_tcgen05_setup()
 // would cost the ring a stage splits them over the pair: at N = 20000 that
 // leaves four stages beside 40 KB of bins instead of three beside 80 KB (and
 // two stages at N = 32768).  A batch does not (its CTAs flush their bins by
-// themselves between problems): above N of about 31 800 its edges add to the
-// global bins, as the single-CTA form's do above about 24 000 (larger stages).
+// themselves between problems): above N = 31 999 its edges add to the global
+// bins, as the single-CTA form's do above 23 807 (larger stages).
 bool launch_sc2_tcgen05(const Batch& b, int total_tiles, int max_n, bool pair_mma, cudaStream_t s, bool auto_mode)
 {
     const int bins = max_n + 1;
