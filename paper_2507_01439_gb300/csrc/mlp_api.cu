@@ -26,7 +26,7 @@ struct turboreg_mlp {
     float* wbf = nullptr;    // BF16-rounded copy used by the forward [P]
     float* mom = nullptr;    // Adam first moment [P]
     float* vel = nullptr;    // Adam second moment [P]
-    // gradient [P], loss, error bits: cleared by one memset, read by one copy
+    // gradient [P], loss, error bits: cleared by one kernel, read by one copy
     float* grad = nullptr;
     float* loss = nullptr;   // grad + P
     uint32_t* err = nullptr; // grad + P + 1
@@ -55,7 +55,6 @@ void free_all(turboreg_mlp* t)
 // grad, loss (device) = those of the mean BCE over m samples.
 int backward(turboreg_mlp* t, const float* feat, const float* label, int32_t m)
 {
-    TM_CHECK(cudaMemsetAsync(t->grad, 0, sizeof(float) * (kMlpParams + 2), t->stream));
     launch_mlp_train(feat, label, m, t->wbf, t->grad, t->loss, t->err, t->stream);
     TM_CHECK(cudaGetLastError());
     return TURBOREG_OK;

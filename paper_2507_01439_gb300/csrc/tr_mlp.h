@@ -25,7 +25,8 @@ void launch_mlp_round(const float* w, float* wbf, cudaStream_t s);
 void launch_features(const Batch& b, cudaStream_t s);
 void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream_t s);
 void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, uint32_t* err, cudaStream_t s);
-// adds d(mean BCE)/d params to grad[kMlpParams] and the loss to *loss (grad 16-byte aligned)
+// d(mean BCE)/d params into grad[kMlpParams] (16-byte aligned); loss and err, the
+// two words behind it, are cleared with it
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
                       uint32_t* err, cudaStream_t s);
 // loss_out: null, or page-locked host memory for a copy of *loss
