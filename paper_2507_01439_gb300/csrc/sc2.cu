@@ -560,9 +560,12 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         int lt;
         p_last = locate(bt, ST_GEMM, kPair ? 2 * ul : ul, lt);
     }
-    if (kPair && kHist == kHistCta && !leader && p_last >= 0) {
-        // the peer's histogram into the leader's (distributed shared memory), so
-        // that one CTA per cluster adds to the global bins
+    // One problem: the peer's histogram into the leader's (distributed shared
+    // memory), so that one CTA per cluster adds to the global bins.  Not in a
+    // batch: the leader may still be emptying its bins of an earlier problem
+    // (nothing orders its flush against the peer's end), so each CTA adds its own.
+    const bool merge = kPair && kHist == kHistCta && bt.num == 1;
+    if (merge && !leader && p_last >= 0) {
         const uint32_t lead_hist = mapa_shared(shist, 0);
         for (int b = threadIdx.x + 1; b < nbins; b += blockDim.x) {
             const uint32_t h = shist[b];
@@ -576,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         if (kPair) tmem_dealloc_pair(tmem, kTmemCols);
         else tmem_dealloc(tmem, kTmemCols);
     }
-    if (kHist == kHistGlobal || p_last < 0 || (kHist == kHistCta && !leader)) return;
+    if (kHist == kHistGlobal || p_last < 0 || (merge && !leader)) return;
     // the worker's histogram into the global one, from which the count pass
     // (one problem) or the select launch (a batch) chooses the pivot threshold
     const ProbView vl = bt.views[p_last];
