@@ -155,6 +155,12 @@ int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, in
 int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* label, int32_t m, float lr,
                             float* loss);
 
+/* Failure injection for tests: each of the next `calls` (>= 0) training passes
+ * (turboreg_mlp_grad, turboreg_mlp_train_step) waits for something that never
+ * comes; the bounded wait gives up after 20 ms and the pass reports it
+ * (TURBOREG_ERR_TIMEOUT).  No device fault and no hang. */
+int turboreg_mlp_debug_stall(turboreg_mlp* t, int32_t calls);
+
 /* Largest n accepted by turboreg_select_pivots_noalloc. */
 #define TURBOREG_NOALLOC_MAX_N 8192
 

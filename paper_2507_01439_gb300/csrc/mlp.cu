@@ -385,7 +385,8 @@ constexpr uint32_t kMnA = 1u << 15, kMnB = 1u << 16;   // instruction descriptor
 
 // Clears the gradient, the loss and the error bits.  It releases the training
 // kernel at once: that one's set-up (weights into shared memory, tensor memory)
-// and first tiles run meanwhile, and it waits only before it adds to them.  With a
+// and first tiles run meanwhile, and it waits before it writes any of them (a wait
+// that gave up is kept in a register until then).  With a
 // memset in front of it a step at m = 131 072 took 88 us and a gradient at
 // m = 16 384 42 us per call, so 87 and 38.
 __global__ void __launch_bounds__(256) mlp_clear_kernel(float* g, int count)
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(256) mlp_clear_kernel(float* g, int count)
 
 __global__ void __launch_bounds__(kTrainThreads, 1)
     mlp_train_kernel(const float* __restrict__ feat, const float* __restrict__ label, int m,
-                     const float* __restrict__ wbf, float* grad, float* loss, uint32_t* err)
+                     const float* __restrict__ wbf, float* grad, float* loss, uint32_t* err, uint32_t dbg)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = aligned_smem(smem_raw);
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kTOffBar);
     uint64_t* bar4 = bar + 1;   // MMA4 of the tile complete (its operands may be overwritten)
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kTOffBar + 16);
+    uint64_t* never = bar + 3;  // failure injection (tests only): nothing arrives here
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int sl = t & 127, part = t >> 7;   // sample of the tile, column part
     const int ntiles = (m + kRows - 1) / kRows;
@@ -439,6 +441,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
         sb4[0] = wbf[kB4];
         mbar_init(bar, 1);
         mbar_init(bar4, 1);
+        mbar_init(never, 1);
         fence_mbar_init();
     }
     if (warp == 0) tmem_alloc(tslot, kTrainTmemCols);
@@ -449,10 +452,12 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     const uint32_t tmem = *tslot;
     const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);   // this warp's lanes
     const float inv_m = 1.f / static_cast<float>(m);
+    bool expired = false;
     auto wait_on = [&](uint64_t* b, uint32_t parity) {
-        if (!mbar_wait(b, parity)) atomicOr(err, TR_ERR_TIMEOUT);
+        if (!mbar_wait(b, parity)) expired = true;
         tc_fence_after();
     };
+    if (dbg & TR_DBG_STALL_TRAIN) expired = !mbar_wait(never, 0u, kStallWaitNs);
     auto wait = [&](uint32_t parity) { wait_on(bar, parity); };
 
     // sums over the tiles.  dW1 and b1, W4 and b3: columns 2 lane, 2 lane + 1,
@@ -740,7 +745,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     }
     // ---- the CTA's sums into the global gradient ----
     if (first) wait_on(bar4, par4 ^ 1u);
-    pdl_wait();   // the gradient is cleared
+    pdl_wait();   // the gradient, the loss and the error bits are cleared
+    if (expired) atomicOr(err, TR_ERR_TIMEOUT);
     {
         uint32_t g3[16], g2[16];
         tmem_ld16(tl + 192 + part * 16, g3);   // dW3[out = column][in = lane]
@@ -864,13 +870,14 @@ void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob,
 }
 
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
-                      uint32_t* err, cudaStream_t s)
+                      uint32_t* err, uint32_t dbg, cudaStream_t s)
 {
     const int ntiles = (m + kRows - 1) / kRows;
     const int sms = device_sms();
     const int grid = ntiles < sms ? ntiles : sms;   // one CTA per SM (shared memory and tensor memory)
     mlp_clear_kernel<<<(kMlpParams + 2 + 255) / 256, 256, 0, s>>>(grad, kMlpParams + 2);
-    launch_pdl(mlp_train_kernel, grid, kTrainThreads, kTrainSmem, s, feat, label, m, wbf, grad, loss, err);
+    launch_pdl(mlp_train_kernel, grid, kTrainThreads, kTrainSmem, s, feat, label, m, wbf, grad, loss, err,
+               dbg);
 }
 
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,

@@ -30,6 +30,7 @@ struct turboreg_mlp {
     float* grad = nullptr;
     float* loss = nullptr;   // grad + P
     uint32_t* err = nullptr; // grad + P + 1
+    int32_t stalls = 0;      // failure injection: training passes left that stall
     float* host = nullptr;   // page-locked [P + 2]: a parameter vector or gradient, loss, error bits on their way out
 };
 
@@ -55,7 +56,9 @@ void free_all(turboreg_mlp* t)
 // grad, loss (device) = those of the mean BCE over m samples.
 int backward(turboreg_mlp* t, const float* feat, const float* label, int32_t m)
 {
-    launch_mlp_train(feat, label, m, t->wbf, t->grad, t->loss, t->err, t->stream);
+    const uint32_t dbg = t->stalls > 0 ? TR_DBG_STALL_TRAIN : 0u;
+    if (t->stalls > 0) --t->stalls;
+    launch_mlp_train(feat, label, m, t->wbf, t->grad, t->loss, t->err, dbg, t->stream);
     TM_CHECK(cudaGetLastError());
     return TURBOREG_OK;
 }
@@ -140,6 +143,13 @@ void turboreg_mlp_destroy(turboreg_mlp* t)
     free_all(t);
     if (t->own_stream && t->stream) cudaStreamDestroy(t->stream);
     delete t;
+}
+
+int turboreg_mlp_debug_stall(turboreg_mlp* t, int32_t calls)
+{
+    if (!t || calls < 0) return TURBOREG_ERR_INVALID_ARG;
+    t->stalls = calls;
+    return TURBOREG_OK;
 }
 
 int turboreg_mlp_get_params(turboreg_mlp* t, float* params)

@@ -20,10 +20,11 @@ constexpr uint32_t TR_ERR_OVERFLOW = 4u;
 constexpr uint32_t TR_ERR_BAD_WEIGHT = 8u;   // a caller's weight outside 0..n-2 (allocation-free selection)
 
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound on any device wait
-// bound of the one wait that the failure-injection hook (ProbView::dbg) leaves
-// without an arrival, so that a test sees it expire quickly
+// bound of the one wait that a failure-injection hook (TR_DBG_*) leaves without
+// an arrival, so that a test sees it expire quickly
 constexpr unsigned long long kStallWaitNs = 20000000ull;   // 20 ms
 constexpr uint32_t TR_DBG_STALL_COMPAT = 1u;
+constexpr uint32_t TR_DBG_STALL_TRAIN = 2u;
 
 // Scalars that flow between stages on the device (no host round trip).
 struct Ctl {

@@ -26,9 +26,9 @@ void launch_features(const Batch& b, cudaStream_t s);
 void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream_t s);
 void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, uint32_t* err, cudaStream_t s);
 // d(mean BCE)/d params into grad[kMlpParams] (16-byte aligned); loss and err, the
-// two words behind it, are cleared with it
+// two words behind it, are cleared with it; dbg: TR_DBG_STALL_TRAIN or 0
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
-                      uint32_t* err, cudaStream_t s);
+                      uint32_t* err, uint32_t dbg, cudaStream_t s);
 // loss_out: null, or page-locked host memory for a copy of *loss
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
                      const float* loss, float* loss_out, cudaStream_t s);
