@@ -151,7 +151,12 @@ int turboreg_mlp_forward(turboreg_mlp* t, const float* feat, int32_t m, float* p
 int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, int32_t m, float* grad,
                       float* loss);
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8) on the mean BCE of the
- * mini-batch; loss (host, may be NULL) receives the loss before the step. */
+ * mini-batch; loss (host, may be NULL) receives the loss before the step.  With
+ * loss the call waits for the step, without it the step is only enqueued.  A
+ * step whose gradient is incomplete (a bounded device wait gave up) changes
+ * neither the weights nor the Adam state nor the step count; this call reports
+ * it as TIMEOUT, or, for a step that was not waited for, the next call that
+ * waits (a step with loss, grad, forward, get_params, get_state), once. */
 int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* label, int32_t m, float lr,
                             float* loss);
 

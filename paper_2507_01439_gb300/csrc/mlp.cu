@@ -810,23 +810,30 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
 
 // Adam (bias-corrected), FP32 master weights; the forward's BF16-rounded copy
 // is refreshed from them.  loss_out (page-locked host memory, or null) receives
-// the step's loss.
+// the step's loss.  A gradient whose kernel gave up on a wait (err) is left out:
+// nothing is updated, and skipped (page-locked host memory) counts the step.
 __global__ void __launch_bounds__(256) mlp_adam_kernel(float* w, float* mom, float* vel, const float* g, float* wbf,
                                                        int step, float lr, float b1, float b2, float eps,
-                                                       const float* loss, float* loss_out)
+                                                       const float* loss, float* loss_out, const uint32_t* err,
+                                                       uint32_t* skipped)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (k == 0 && loss_out != nullptr) *loss_out = *loss;
+    const uint32_t bad = *err;   // in flight with the loads below
     if (k >= kMlpParams) return;
-    const float gk = g[k];
-    const float m1 = b1 * mom[k] + (1.f - b1) * gk;
-    const float v1 = b2 * vel[k] + (1.f - b2) * gk * gk;
+    const float gk = g[k], m0 = mom[k], v0 = vel[k], w0 = w[k];
+    if (bad != 0u) {
+        if (k == 0) *skipped += 1u;
+        return;
+    }
+    const float m1 = b1 * m0 + (1.f - b1) * gk;
+    const float v1 = b2 * v0 + (1.f - b2) * gk * gk;
     mom[k] = m1;
     vel[k] = v1;
     const float mh = m1 / (1.f - powf(b1, static_cast<float>(step)));
     const float vh = v1 / (1.f - powf(b2, static_cast<float>(step)));
-    const float nw = w[k] - lr * mh / (sqrtf(vh) + eps);
+    const float nw = w0 - lr * mh / (sqrtf(vh) + eps);
     w[k] = nw;
     wbf[k] = bf16r(nw);
 }
@@ -881,10 +888,10 @@ void launch_mlp_train(const float* feat, const float* label, int m, const float*
 }
 
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
-                     const float* loss, float* loss_out, cudaStream_t s)
+                     const float* loss, float* loss_out, const uint32_t* err, uint32_t* skipped, cudaStream_t s)
 {
     launch_pdl(mlp_adam_kernel, (kMlpParams + 255) / 256, 256, 0, s, w, mom, vel, g, wbf, step, lr, 0.9f, 0.999f, 1e-8f,
-               loss, loss_out);
+               loss, loss_out, err, skipped);
 }
 
 }  // namespace tr

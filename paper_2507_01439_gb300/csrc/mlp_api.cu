@@ -31,7 +31,11 @@ struct turboreg_mlp {
     float* loss = nullptr;   // grad + P
     uint32_t* err = nullptr; // grad + P + 1
     int32_t stalls = 0;      // failure injection: training passes left that stall
-    float* host = nullptr;   // page-locked [P + 2]: a parameter vector or gradient, loss, error bits on their way out
+    // page-locked [P + 4]: a parameter vector or gradient, loss, error bits on their
+    // way out; then a step's loss, and the steps left out that no call has reported yet
+    float* host = nullptr;
+    float* step_loss = nullptr;    // host + P + 2
+    uint32_t* skipped = nullptr;   // host + P + 3
 };
 
 namespace {
@@ -61,6 +65,16 @@ int backward(turboreg_mlp* t, const float* feat, const float* label, int32_t m)
     launch_mlp_train(feat, label, m, t->wbf, t->grad, t->loss, t->err, dbg, t->stream);
     TM_CHECK(cudaGetLastError());
     return TURBOREG_OK;
+}
+
+// With the stream idle: TIMEOUT if steps were left out since the last report
+// (once; they do not count as steps).
+int report_skipped(turboreg_mlp* t)
+{
+    const uint32_t k = *t->skipped;
+    *t->skipped = 0u;
+    t->step -= static_cast<int32_t>(k);
+    return k != 0u ? TURBOREG_ERR_TIMEOUT : TURBOREG_OK;
 }
 
 // `count` values at `src` (device) through the page-locked buffer; the stream
@@ -94,7 +108,12 @@ int turboreg_mlp_create(int device, int32_t max_samples, uint64_t seed, void* cu
     al(reinterpret_cast<void**>(&t->mom), sizeof(float) * kMlpParams);
     al(reinterpret_cast<void**>(&t->vel), sizeof(float) * kMlpParams);
     al(reinterpret_cast<void**>(&t->grad), sizeof(float) * (kMlpParams + 2));
-    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&t->host), sizeof(float) * (kMlpParams + 2));
+    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&t->host), sizeof(float) * (kMlpParams + 4));
+    if (e == cudaSuccess) {
+        t->step_loss = t->host + kMlpParams + 2;
+        t->skipped = reinterpret_cast<uint32_t*>(t->host + kMlpParams + 3);
+        *t->skipped = 0u;
+    }
     t->loss = t->grad + kMlpParams;
     t->err = reinterpret_cast<uint32_t*>(t->grad + kMlpParams + 1);
     if (e == cudaSuccess) e = mlp_setup();
@@ -157,8 +176,9 @@ int turboreg_mlp_get_params(turboreg_mlp* t, float* params)
     if (!t || !params) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
     const int rc = fetch(t, t->w, kMlpParams);
-    if (rc == TURBOREG_OK) std::memcpy(params, t->host, sizeof(float) * kMlpParams);
-    return rc;
+    if (rc != TURBOREG_OK) return rc;
+    std::memcpy(params, t->host, sizeof(float) * kMlpParams);
+    return report_skipped(t);
 }
 
 int turboreg_mlp_set_params(turboreg_mlp* t, const float* params)
@@ -181,8 +201,9 @@ int turboreg_mlp_get_state(turboreg_mlp* t, float* m, float* v, int32_t* step)
     TM_CHECK(cudaMemcpyAsync(m, t->mom, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaMemcpyAsync(v, t->vel, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
+    const int rc = report_skipped(t);
     *step = t->step;
-    return TURBOREG_OK;
+    return rc;
 }
 
 int turboreg_mlp_set_state(turboreg_mlp* t, const float* m, const float* v, int32_t step)
@@ -192,6 +213,7 @@ int turboreg_mlp_set_state(turboreg_mlp* t, const float* m, const float* v, int3
     TM_CHECK(cudaMemcpyAsync(t->mom, m, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, t->stream));
     TM_CHECK(cudaMemcpyAsync(t->vel, v, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
+    *t->skipped = 0u;   // the steps are counted from here
     t->step = step;
     return TURBOREG_OK;
 }
@@ -206,7 +228,8 @@ int turboreg_mlp_forward(turboreg_mlp* t, const float* feat, int32_t m, float* p
     uint32_t err = 0;
     TM_CHECK(cudaMemcpyAsync(&err, t->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
-    return err ? TURBOREG_ERR_TIMEOUT : TURBOREG_OK;
+    const int rc = report_skipped(t);
+    return err ? TURBOREG_ERR_TIMEOUT : rc;
 }
 
 int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, int32_t m, float* grad, float* loss)
@@ -220,7 +243,8 @@ int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, in
     if (loss) *loss = t->host[kMlpParams];
     uint32_t err;
     std::memcpy(&err, t->host + kMlpParams + 1, sizeof(err));
-    return err ? TURBOREG_ERR_TIMEOUT : TURBOREG_OK;
+    rc = report_skipped(t);
+    return err ? TURBOREG_ERR_TIMEOUT : rc;
 }
 
 int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* label, int32_t m, float lr,
@@ -231,11 +255,13 @@ int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* lab
     int rc = backward(t, feat, label, m);
     if (rc != TURBOREG_OK) return rc;
     t->step += 1;
-    launch_mlp_adam(t->w, t->mom, t->vel, t->grad, t->wbf, t->step, lr, t->loss, loss ? t->host : nullptr, t->stream);
+    launch_mlp_adam(t->w, t->mom, t->vel, t->grad, t->wbf, t->step, lr, t->loss, loss ? t->step_loss : nullptr,
+                    t->err, t->skipped, t->stream);
     TM_CHECK(cudaGetLastError());
     if (loss) {
         TM_CHECK(cudaStreamSynchronize(t->stream));
-        *loss = t->host[0];
+        *loss = *t->step_loss;
+        return report_skipped(t);
     }
     return TURBOREG_OK;
 }

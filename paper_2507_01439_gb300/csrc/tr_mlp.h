@@ -29,9 +29,10 @@ void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob,
 // two words behind it, are cleared with it; dbg: TR_DBG_STALL_TRAIN or 0
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
                       uint32_t* err, uint32_t dbg, cudaStream_t s);
-// loss_out: null, or page-locked host memory for a copy of *loss
+// loss_out: null, or page-locked host memory for a copy of *loss; *err != 0: no
+// update, and *skipped (page-locked host memory) counts the step
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
-                     const float* loss, float* loss_out, cudaStream_t s);
+                     const float* loss, float* loss_out, const uint32_t* err, uint32_t* skipped, cudaStream_t s);
 void launch_learned_hist(const Batch& b, int total, int max_n, cudaStream_t s);
 
 }  // namespace tr
