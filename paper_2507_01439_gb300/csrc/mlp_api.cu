@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <random>
 #include <vector>
@@ -34,6 +35,7 @@ struct turboreg_mlp {
     // page-locked [P + 4]: a parameter vector or gradient, loss, error bits on their
     // way out; then a step's loss, and the steps left out that no call has reported yet
     float* host = nullptr;
+    std::mutex host_mu;            // one call at a time between its copy into `host` and its reading of it
     float* step_loss = nullptr;    // host + P + 2
     uint32_t* skipped = nullptr;   // host + P + 3
 };
@@ -67,7 +69,7 @@ int backward(turboreg_mlp* t, const float* feat, const float* label, int32_t m)
     return TURBOREG_OK;
 }
 
-// With the stream idle: TIMEOUT if steps were left out since the last report
+// With the stream idle and host_mu held: TIMEOUT if steps were left out since the last report
 // (once; they do not count as steps).
 int report_skipped(turboreg_mlp* t)
 {
@@ -78,7 +80,8 @@ int report_skipped(turboreg_mlp* t)
 }
 
 // `count` values at `src` (device) through the page-locked buffer; the stream
-// is then idle.  (A copy to pageable memory would be staged by the driver.)
+// is then idle; the caller holds host_mu until it has read the buffer, so that
+// several threads may read one trainer.  (A copy to pageable memory would be staged by the driver.)
 int fetch(turboreg_mlp* t, const float* src, size_t count)
 {
     TM_CHECK(cudaMemcpyAsync(t->host, src, sizeof(float) * count, cudaMemcpyDeviceToHost, t->stream));
@@ -175,6 +178,7 @@ int turboreg_mlp_get_params(turboreg_mlp* t, float* params)
 {
     if (!t || !params) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
+    std::lock_guard<std::mutex> lk(t->host_mu);
     const int rc = fetch(t, t->w, kMlpParams);
     if (rc != TURBOREG_OK) return rc;
     std::memcpy(params, t->host, sizeof(float) * kMlpParams);
@@ -201,6 +205,7 @@ int turboreg_mlp_get_state(turboreg_mlp* t, float* m, float* v, int32_t* step)
     TM_CHECK(cudaMemcpyAsync(m, t->mom, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaMemcpyAsync(v, t->vel, sizeof(float) * kMlpParams, cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
+    std::lock_guard<std::mutex> lk(t->host_mu);
     const int rc = report_skipped(t);
     *step = t->step;
     return rc;
@@ -213,6 +218,7 @@ int turboreg_mlp_set_state(turboreg_mlp* t, const float* m, const float* v, int3
     TM_CHECK(cudaMemcpyAsync(t->mom, m, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, t->stream));
     TM_CHECK(cudaMemcpyAsync(t->vel, v, sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
+    std::lock_guard<std::mutex> lk(t->host_mu);
     *t->skipped = 0u;   // the steps are counted from here
     t->step = step;
     return TURBOREG_OK;
@@ -228,6 +234,7 @@ int turboreg_mlp_forward(turboreg_mlp* t, const float* feat, int32_t m, float* p
     uint32_t err = 0;
     TM_CHECK(cudaMemcpyAsync(&err, t->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, t->stream));
     TM_CHECK(cudaStreamSynchronize(t->stream));
+    std::lock_guard<std::mutex> lk(t->host_mu);
     const int rc = report_skipped(t);
     return err ? TURBOREG_ERR_TIMEOUT : rc;
 }
@@ -237,7 +244,9 @@ int turboreg_mlp_grad(turboreg_mlp* t, const float* feat, const float* label, in
     if (!t || !feat || !label || !grad || m < 1 || m > t->max_samples) return TURBOREG_ERR_INVALID_ARG;
     TM_CHECK(cudaSetDevice(t->device));
     int rc = backward(t, feat, label, m);
-    if (rc == TURBOREG_OK) rc = fetch(t, t->grad, kMlpParams + 2);
+    if (rc != TURBOREG_OK) return rc;
+    std::lock_guard<std::mutex> lk(t->host_mu);
+    rc = fetch(t, t->grad, kMlpParams + 2);
     if (rc != TURBOREG_OK) return rc;
     std::memcpy(grad, t->host, sizeof(float) * kMlpParams);
     if (loss) *loss = t->host[kMlpParams];
@@ -260,6 +269,7 @@ int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* lab
     TM_CHECK(cudaGetLastError());
     if (loss) {
         TM_CHECK(cudaStreamSynchronize(t->stream));
+        std::lock_guard<std::mutex> lk(t->host_mu);
         *loss = *t->step_loss;
         return report_skipped(t);
     }
