@@ -164,7 +164,7 @@ __device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, float
     for (int cb = 0; cb < 4; ++cb) {
         uint32_t acc[32];
         tmem_ld32(tmem + lane_base + cb * 32, acc);
-        tmem_ld_wait();
+        tmem_ld_wait32(acc);
         float hv[32];
 #pragma unroll
         for (int q = 0; q < 32; ++q) hv[q] = bf16r(fmaxf(__uint_as_float(acc[q]) + sb2[cb * 32 + q], 0.f));
@@ -199,7 +199,7 @@ __device__ float mlp_tile(const float* __restrict__ feat, int m, int row0, float
     for (int cb = 0; cb < 2; ++cb) {
         uint32_t acc[32];
         tmem_ld32(tmem + lane_base + 128 + cb * 32, acc);
-        tmem_ld_wait();
+        tmem_ld_wait32(acc);
         float hv[32];
 #pragma unroll
         for (int q = 0; q < 32; ++q) {
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
         {
             uint32_t acc[16];
             tmem_ld16(tl + 128 + part * 16, acc);
-            tmem_ld_wait();
+            tmem_ld_wait16(acc);
             float z = 0.f;
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
                 const uint4 q = *reinterpret_cast<const uint4*>(sH1 + sw128(sl, part * 2 + c));
                 h[4 * c] = q.x; h[4 * c + 1] = q.y; h[4 * c + 2] = q.z; h[4 * c + 3] = q.w;
             }
-            tmem_ld_wait();
+            tmem_ld_wait16(acc);
             float4* d = reinterpret_cast<float4*>(sDz1 + sl * kTDz1Ld + part * 16);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -751,7 +751,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
         uint32_t g3[16], g2[16];
         tmem_ld16(tl + 192 + part * 16, g3);   // dW3[out = column][in = lane]
         tmem_ld16(tl + 256 + part * 16, g2);   // dW2[out = lane][in = column]
-        tmem_ld_wait();
+        tmem_ld_wait16(g3);
+        tmem_ld_wait16(g2);
 #pragma unroll
         for (int q = 0; q < 16; ++q) atomicAdd(&grad[kW3 + (part * 16 + q) * 128 + sl], __uint_as_float(g3[q]));
         static_assert(kW2 % 4 == 0, "16-byte additions to dW2");

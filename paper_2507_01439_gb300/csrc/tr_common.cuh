@@ -462,7 +462,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, uint32_t x)
 
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Wait for tmem_ld32 into v, whose values exist from here on.
+// Wait for tmem_ld32 / tmem_ld16 into v, whose values exist from here on.  (There
+// is no wait without the registers: nothing would keep the compiler from using
+// them before it.)
 __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&v)[32])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -473,6 +475,12 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&v)[32])
                    "+r"(v[29]), "+r"(v[30]), "+r"(v[31])::"memory");
 }
 
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld_wait16(uint32_t (&v)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
+                   "+r"(v[15])::"memory");
+}
 
 }  // namespace tr
