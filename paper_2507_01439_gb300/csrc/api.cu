@@ -1064,15 +1064,21 @@ int turboreg_register_batched(turboreg_ctx* c, const float* src_cat, const float
 namespace {
 
 // The packed FP4 adjacency as one FP8 E4M3 byte per entry (0x38 = 1.0): the
-// inspection format of TURBOREG_BUF_ADJ_FP8.
+// inspection format of TURBOREG_BUF_ADJ_FP8.  The packed bytes (up to 512 MB) go
+// to the end of the caller's buffer and are expanded from there: byte j becomes
+// bytes 2j and 2j + 1, which never reach the packed bytes still to be read.
 int64_t copy_adj_bytes(const uint8_t* a4, size_t count, void* dst, int64_t max_bytes)
 {
     if (count > static_cast<size_t>(max_bytes)) count = static_cast<size_t>(max_bytes);
-    std::vector<uint8_t> packed((count + 1) / 2);
-    if (count && cudaMemcpy(packed.data(), a4, packed.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return -TURBOREG_ERR_CUDA;
     uint8_t* out = static_cast<uint8_t*>(dst);
-    for (size_t k = 0; k < count; ++k) out[k] = ((packed[k / 2] >> (4 * (k & 1))) & 0xFu) ? 0x38 : 0x00;
+    const uint8_t* packed = out + count / 2;
+    if (count && cudaMemcpy(out + count / 2, a4, (count + 1) / 2, cudaMemcpyDeviceToHost) != cudaSuccess)
+        return -TURBOREG_ERR_CUDA;
+    for (size_t k = 0; k < count; k += 2) {
+        const uint8_t b = packed[k / 2];
+        out[k] = (b & 0x0Fu) ? 0x38 : 0x00;
+        if (k + 1 < count) out[k + 1] = (b & 0xF0u) ? 0x38 : 0x00;
+    }
     return static_cast<int64_t>(count);
 }
 
