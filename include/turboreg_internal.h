@@ -166,6 +166,9 @@ int turboreg_mlp_train_step(turboreg_mlp* t, const float* feat, const float* lab
  * (TURBOREG_ERR_TIMEOUT).  No device fault and no hang. */
 int turboreg_mlp_debug_stall(turboreg_mlp* t, int32_t calls);
 
+/* Thread blocks a training pass over m samples takes (one per SM at most), or -status. */
+int turboreg_mlp_debug_blocks(turboreg_mlp* t, int32_t m);
+
 /* Largest n accepted by turboreg_select_pivots_noalloc. */
 #define TURBOREG_NOALLOC_MAX_N 8192
 

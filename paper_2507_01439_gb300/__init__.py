@@ -50,7 +50,7 @@ EXPORTED = (
     "turboreg_set_proposal_model", "turboreg_features", "turboreg_mlp_create", "turboreg_mlp_destroy",
     "turboreg_mlp_get_params", "turboreg_mlp_set_params", "turboreg_mlp_get_state", "turboreg_mlp_set_state",
     "turboreg_mlp_forward", "turboreg_mlp_grad", "turboreg_mlp_train_step", "turboreg_mlp_debug_stall",
-    "turboreg_score_transforms",
+    "turboreg_mlp_debug_blocks", "turboreg_score_transforms",
     "turboreg_kabsch_cliques", "turboreg_register_async", "turboreg_synchronize",
 )
 TURBOREG_MLP_PARAMS = 17217
@@ -140,10 +140,11 @@ def load_library(path: str = LIB_PATH):
     lib.turboreg_mlp_grad.argtypes = [P, P, P, i32, P, F]
     lib.turboreg_mlp_train_step.argtypes = [P, P, P, i32, ctypes.c_float, F]
     lib.turboreg_mlp_debug_stall.argtypes = [P, i32]
+    lib.turboreg_mlp_debug_blocks.argtypes = [P, i32]
     for nm in ("turboreg_set_proposal_model", "turboreg_features", "turboreg_mlp_create", "turboreg_mlp_get_params",
                "turboreg_mlp_set_params", "turboreg_mlp_get_state", "turboreg_mlp_set_state",
                "turboreg_mlp_forward", "turboreg_mlp_grad", "turboreg_mlp_train_step",
-               "turboreg_mlp_debug_stall"):
+               "turboreg_mlp_debug_stall", "turboreg_mlp_debug_blocks"):
         getattr(lib, nm).restype = ctypes.c_int
     _lib = lib
     return lib

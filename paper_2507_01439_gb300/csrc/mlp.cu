@@ -866,8 +866,7 @@ void launch_features(const Batch& b, cudaStream_t s) { launch_pdl(features_kerne
 
 void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream_t s)
 {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     const int grid = total < 2 * sms ? total : 2 * sms;
     launch_pdl(mlp_proposal_kernel, grid, kRows, kFwdSmem, s, b, total, wbf);
 }
@@ -877,12 +876,16 @@ void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob,
     mlp_fwd_kernel<<<(m + kRows - 1) / kRows, kRows, kFwdSmem, s>>>(feat, m, wbf, prob, err);
 }
 
+int mlp_train_blocks(int m)
+{
+    const int ntiles = (m + kRows - 1) / kRows, sms = device_sms();
+    return ntiles < sms ? ntiles : sms;   // one CTA per SM (shared memory and tensor memory)
+}
+
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
                       uint32_t* err, uint32_t dbg, cudaStream_t s)
 {
-    const int ntiles = (m + kRows - 1) / kRows;
-    const int sms = device_sms();
-    const int grid = ntiles < sms ? ntiles : sms;   // one CTA per SM (shared memory and tensor memory)
+    const int grid = mlp_train_blocks(m);
     mlp_clear_kernel<<<(kMlpParams + 2 + 255) / 256, 256, 0, s>>>(grad, kMlpParams + 2);
     launch_pdl(mlp_train_kernel, grid, kTrainThreads, kTrainSmem, s, feat, label, m, wbf, grad, loss, err,
                dbg);

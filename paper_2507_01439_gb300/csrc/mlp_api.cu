@@ -174,6 +174,13 @@ int turboreg_mlp_debug_stall(turboreg_mlp* t, int32_t calls)
     return TURBOREG_OK;
 }
 
+int turboreg_mlp_debug_blocks(turboreg_mlp* t, int32_t m)
+{
+    if (!t || m < 1 || m > t->max_samples) return -TURBOREG_ERR_INVALID_ARG;
+    if (cudaSetDevice(t->device) != cudaSuccess) return -TURBOREG_ERR_CUDA;
+    return mlp_train_blocks(m);
+}
+
 int turboreg_mlp_get_params(turboreg_mlp* t, float* params)
 {
     if (!t || !params) return TURBOREG_ERR_INVALID_ARG;

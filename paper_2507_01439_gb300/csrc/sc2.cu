@@ -36,6 +36,8 @@
 //
 // Alternative (sc2_bitset.cu): the same integers from the adjacency bitset
 // with AND + popcount on CUDA cores, work only on the edges.
+#include <atomic>
+
 #include "tr_common.cuh"
 #include "tr_problem.h"
 #include "tr_select.cuh"
@@ -592,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
     }
 }
 
-int g_sc2_sms = 0;
+std::atomic<int> g_sc2_sms{0};
 int g_sc2_pair_clusters = 0;   // co-resident 2-CTA clusters of the pair kernels (0: use single CTAs)
 
 template <bool kPair>
@@ -653,15 +655,27 @@ cudaError_t mma_attr()
 
 }  // namespace
 
-int device_sms() { return g_sc2_sms > 0 ? g_sc2_sms : 148; }
+// Asked of the current device on first use: a trainer, the allocation-free
+// selection and a context each may be the only part of the library in a process.
+int device_sms()
+{
+    int n = g_sc2_sms.load(std::memory_order_relaxed), dev = 0;
+    if (n > 0) return n;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+        return 148;   // no device to ask
+    g_sc2_sms.store(n, std::memory_order_relaxed);
+    return n;
+}
 
 int sc2_pair_clusters() { return g_sc2_pair_clusters; }
 
 cudaError_t sc2_tcgen05_setup()
 {
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sc2_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) g_sc2_sms.store(sms, std::memory_order_relaxed);
     if (e == cudaSuccess) e = mma_attr<true, kHistCta>();
     if (e == cudaSuccess) e = mma_attr<true, kHistPair>();
     if (e == cudaSuccess) e = mma_attr<true, kHistGlobal>();

@@ -711,18 +711,11 @@ __global__ void __launch_bounds__(256) rank_kernel(OneView vs, int32_t* n_out)
     }
 }
 
-int g_num_sms = 0;
-
 }  // namespace
 
 cudaError_t topk_setup()
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
+    cudaError_t e = cudaFuncSetAttribute(sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TURBOREG_K1_MAX * 8);
     if (e != cudaSuccess) return e;
@@ -764,7 +757,7 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
 void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s)
 {
     const OneView vs{v};
-    const int warps = (v.n + 1) / 2 * caller_windows(v.n), sms = g_num_sms > 0 ? g_num_sms : 148;
+    const int warps = (v.n + 1) / 2 * caller_windows(v.n), sms = device_sms();
     launch_pdl(caller_hist_kernel, (warps + 31) / 32 < sms ? (warps + 31) / 32 : sms, 1024, (v.n + 1) * 4, s, vs);
     launch_pdl(count_kernel<OneView>, count_groups(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
                vs, 1);

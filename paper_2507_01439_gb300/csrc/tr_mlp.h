@@ -25,6 +25,8 @@ void launch_mlp_round(const float* w, float* wbf, cudaStream_t s);
 void launch_features(const Batch& b, cudaStream_t s);
 void launch_mlp_proposal(const Batch& b, int total, const float* wbf, cudaStream_t s);
 void launch_mlp_forward(const float* feat, int m, const float* wbf, float* prob, uint32_t* err, cudaStream_t s);
+// blocks of the training kernel for m samples
+int mlp_train_blocks(int m);
 // d(mean BCE)/d params into grad[kMlpParams] (16-byte aligned); loss and err, the
 // two words behind it, are cleared with it; dbg: TR_DBG_STALL_TRAIN or 0
 void launch_mlp_train(const float* feat, const float* label, int m, const float* wbf, float* grad, float* loss,
