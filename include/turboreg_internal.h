@@ -46,6 +46,12 @@ typedef enum {
  * and the result's status is TURBOREG_ERR_TIMEOUT.  No device fault and no
  * hang: the context stays usable and the next registration is unaffected. */
 #define TURBOREG_FLAG_DEBUG_STALL_COMPAT 0x10000u
+/* The same for the SC^2 GEMM (in a batch, the first problem's flag): its first
+ * worker never learns of its second block, so that worker's roles give up after
+ * the normal 2 s, and blocks of any problem of the call may be missing.  Every
+ * result of the call carries TURBOREG_ERR_TIMEOUT, and nothing is selected from
+ * the incomplete weights. */
+#define TURBOREG_FLAG_DEBUG_STALL_SC2 0x20000u
 
 /* Allocation-failure injection for tests: when the environment variable
  * TURBOREG_DEBUG_FAIL_ALLOC holds k >= 1, the k-th memory allocation made by

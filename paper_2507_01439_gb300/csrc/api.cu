@@ -307,7 +307,8 @@ ProbView make_view(turboreg_ctx* c, int slot, int64_t in_off, int32_t n, const t
     v.kappa_fp64 = p->kappa_fp64 > 0.f ? p->kappa_fp64 : 100.f;
     v.graph_mode = p->graph_mode;
     v.scoring = p->scoring;
-    v.dbg = (p->flags & TURBOREG_FLAG_DEBUG_STALL_COMPAT) ? TR_DBG_STALL_COMPAT : 0u;
+    v.dbg = ((p->flags & TURBOREG_FLAG_DEBUG_STALL_COMPAT) ? TR_DBG_STALL_COMPAT : 0u) |
+            ((p->flags & TURBOREG_FLAG_DEBUG_STALL_SC2) ? TR_DBG_STALL_SC2 : 0u);
     v.pts = ws.pts + s * 6 * np;
     v.pts8 = ws.pts8 + s * 8 * np;
     v.a4 = ws.a4 + s * n2 / 2;

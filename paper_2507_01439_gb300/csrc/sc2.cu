@@ -455,6 +455,11 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
         for (int k = 0;; ++k) {
             const int u = block_index(k, c, C, chunk);
             const int slot = k % kRing;
+            // failure injection (tests only): the first worker's second block is never handed out
+            if (k == 1 && c == 0 && (bt.views[0].dbg & TR_DBG_STALL_SC2) != 0u) {
+                ok = false;
+                break;
+            }
             if (k >= kRing && !__all_sync(0xffffffffu, mbar_wait(&sempty[slot], (k / kRing - 1) & 1))) {
                 ok = false;
                 break;
@@ -549,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) sc2_mma_kernel(Batch bt, int tota
             }
         }
     }
-    if (!ok && lane == 0) atomicOr(&bt.views[0].ctl->err, TR_ERR_TIMEOUT);
+    if (!ok && lane == 0) mark_timeout(bt);
     tc_fence_before();
     __syncthreads();
     // the problem of this worker's last block (both CTAs of a cluster take the

@@ -20,6 +20,7 @@
 // histogram in shared memory, with the same results as the GEMM's epilogue.
 #include "tr_common.cuh"
 #include "tr_problem.h"
+#include "tr_select.cuh"
 
 namespace tr {
 
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(kLThreads, 1)
     }
     __syncthreads();
     flush_rows(prev, true);   // the last row block and problem
-    if (!ok && lane == 0) atomicOr(&bt.views[0].ctl->err, TR_ERR_TIMEOUT);
+    if (!ok && lane == 0) mark_timeout(bt);
 }
 
 // ---------------------------------------------------------------------------

@@ -335,19 +335,16 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
     const int rmax = (act && v.rowmax != nullptr) ? __ldg(v.rowmax + row) : 0;
     int n_sel, alpha;
     if (select_here) {
-        const bool bad = VS::kCallerWeights && (__ldcg(&v.ctl->err) & TR_ERR_BAD_WEIGHT) != 0u;
         select_alpha(v, ssel, shist_stage, ssel + 33);
         __syncthreads();
-        // out-of-range weights: nothing is selected, so that the emit and rank
-        // passes write no candidate (rank reports the error)
-        n_sel = bad ? 0 : ssel[34];
-        alpha = bad ? 0x7FFFFFFF : ssel[35];
+        n_sel = ssel[34];
+        alpha = ssel[35];
         if (lb == 0 && t == 0) {
-            v.ctl->n_edges = bad ? 0 : ssel[33];
+            v.ctl->n_edges = ssel[33];
             v.ctl->n_sel = n_sel;
             v.ctl->alpha = alpha;
-            v.ctl->c_gt = bad ? 0 : ssel[36];
-            v.ctl->m_ties = bad ? 0 : ssel[37];
+            v.ctl->c_gt = ssel[36];
+            v.ctl->m_ties = ssel[37];
         }
     } else {
         n_sel = v.ctl->n_sel;

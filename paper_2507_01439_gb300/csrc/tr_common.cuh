@@ -25,6 +25,7 @@ constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound on any devic
 constexpr unsigned long long kStallWaitNs = 20000000ull;   // 20 ms
 constexpr uint32_t TR_DBG_STALL_COMPAT = 1u;
 constexpr uint32_t TR_DBG_STALL_TRAIN = 2u;
+constexpr uint32_t TR_DBG_STALL_SC2 = 4u;
 
 // Scalars that flow between stages on the device (no host round trip).
 struct Ctl {

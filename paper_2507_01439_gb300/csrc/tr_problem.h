@@ -118,7 +118,6 @@ __device__ __forceinline__ int pivot_weight(const ProbView& v, int i, int j, int
 // allocation-free selection on a caller's weight matrix, whose weights are
 // checked against the range 0..n-2 of an SC^2 count) ...
 struct OneView {
-    static constexpr bool kCallerWeights = true;
     ProbView v;
     __device__ __forceinline__ ProbView get(int, int b, int& local) const
     {
@@ -128,7 +127,6 @@ struct OneView {
 };
 // ... or a group of problems, located per block.
 struct ManyViews {
-    static constexpr bool kCallerWeights = false;   // weights come from the library's own SC^2 pass
     Batch bt;
     __device__ __forceinline__ ProbView get(int st, int b, int& local) const
     {

@@ -1,11 +1,19 @@
 // Threshold step of the exact top-K1 pivot selection (Eq. 4), shared by the
-// standalone select kernel and the count kernel's blocks.
+// standalone select kernel and the count kernel's blocks, and how an SC^2 pass
+// that gave up is kept out of it.
 #pragma once
 
 #include "tr_common.cuh"
 #include "tr_problem.h"
 
 namespace tr {
+
+// A worker of an SC^2 pass gave up: the blocks it leaves out, and the bins it
+// keeps, may be any problem's of the launch.
+__device__ __forceinline__ void mark_timeout(const Batch& bt)
+{
+    for (int p = 0; p < bt.num; ++p) atomicOr(&bt.views[p].ctl->err, TR_ERR_TIMEOUT);
+}
 
 // Block-wide inclusive scan of one int per thread (blockDim.x a multiple of
 // 32, at most 1024); sbuf holds 33 ints of shared memory.
@@ -43,11 +51,15 @@ __device__ __forceinline__ int block_incl_scan(int x, int* sbuf)
 // both passes below read it from there.  res: optional shared memory of five
 // words that receives (|E+|, n_sel, alpha, c_gt, m) instead of the problem's
 // control block; the caller synchronises the block before reading it.
+// Nothing is selected (n_sel = 0) when the histogram may not be W's: a wait of an
+// earlier stage gave up, or a caller's weight was out of range.  The passes over
+// W would otherwise find more edges above alpha than the key list holds.
 __device__ __forceinline__ void select_alpha(const ProbView& v, int* sbuf, uint32_t* stage = nullptr,
                                              int* res = nullptr)
 {
     const int nb = v.n;                       // weights 1..n (W <= n - 2)
     const uint32_t* H = v.hist;
+    const bool usable = (__ldcg(&v.ctl->err) & (TR_ERR_TIMEOUT | TR_ERR_BAD_WEIGHT)) == 0u;
     if (stage != nullptr && (reinterpret_cast<uintptr_t>(v.hist) & 15u) == 0u) {
         const int nq = (nb + 4) >> 2;         // 16-byte words covering bins 0..n
         const uint4* H4 = reinterpret_cast<const uint4*>(v.hist);
@@ -100,7 +112,7 @@ __device__ __forceinline__ void select_alpha(const ProbView& v, int* sbuf, uint3
     const int incl = block_incl_scan(mine, sbuf);
     if (threadIdx.x == blockDim.x - 1) sbuf[32] = incl;
     __syncthreads();
-    const int n_edges = sbuf[32];
+    const int n_edges = usable ? sbuf[32] : 0;
     const int n_sel = n_edges < v.k1 ? n_edges : v.k1;
     // result k of (n_edges, n_sel, alpha, c_gt, m_ties)
     auto put = [&](int k, int val) {
