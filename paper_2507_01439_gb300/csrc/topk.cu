@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) count_warp_kernel(ManyViews 
     }
 }
 
-// A warp per active row (batches; one problem of up to kEmitWarpN matches):
+// A warp per active row (batches; one problem of up to 1024 matches):
 // lane l reads chunks 4l .. 4l + 3 of each 128-chunk sweep (lane order =
 // column order), the next sweep in flight, and needs no block barrier.  A
 // block's eight rows then run side by side: with a block per row and n/8

@@ -76,8 +76,11 @@ __host__ __device__ inline int count_blocks(int n, int in_batch)
 }
 __host__ __device__ inline int emit_blocks(int n, int in_batch) { return in_batch ? (n + 63) / 64 : (n + 7) / 8; }
 // The emit pass takes a warp per active row in a batch and for one problem of
-// up to 2048 matches (a row is at most two sweeps of a warp), else a block.
-inline bool emit_by_warp(int max_n, bool in_batch) { return in_batch || max_n <= 2048; }
+// up to 1024 matches (a row is one sweep of a warp), else a block.  One
+// registration, warp / block (us): N = 67 30.8 / 32.9, 200 35.0 / 35.0, 1000
+// 42.8 / 43.1, 1400 45.3 / 45.0, 2000 51.4 / 49.9, 2048 53.1 / 51.3; N = 5000 (the
+// pass alone) 12 / 7.0.
+inline bool emit_by_warp(int max_n, bool in_batch) { return in_batch || max_n <= 1024; }
 // Blocks of the histogram pass: one per group; from n = 8192 on a fixed number
 // that takes several groups each (a block clears and flushes n bins: at
 // n = 20000 that is 80 KB against the 320 KB of W a group holds).
