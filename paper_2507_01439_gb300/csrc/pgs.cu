@@ -13,9 +13,9 @@
 // (z != i, j follows from the zero diagonal) and W read symmetrically,
 // W_ab = W_min(a,b),max(a,b) (only the upper triangle is stored).
 //
-// One warp per selected edge (Eq. 4).  One problem: in the order the selection
-// wrote them; the warp first finds the edge's pivot index, its rank among the
-// selected keys (staged once per block in shared memory).  A batch: the keys
+// One warp per selected edge (Eq. 4).  One problem or a small batch: in the order
+// the selection wrote them; the warp first finds the edge's pivot index, its rank
+// among the selected keys (staged once per block in shared memory).  A large batch: the keys
 // are sorted, so edge c is pivot c.  All outputs go to the pivot index.
 // Candidates: every lane loads its share of both rows' bitset words at once
 // (eight words of each per lane in flight), and the warp compacts the set bits
@@ -30,8 +30,8 @@
 // Kabsch (Sec. 3.5): one lane per clique in FP32; for ill-conditioned cliques
 // the warp computes the FP64 triangle normals with six lanes per clique
 // (triangle x or y, component 0..2) and the clique's lane redoes the closed
-// form with them.  One problem: each warp solves its own pivot's cliques at
-// once.  A batch: a kernel of its own solves 32 cliques to a warp, and the search,
+// form with them.  One problem or a small batch: each warp solves its own pivot's
+// cliques at once.  A large batch: a kernel of its own solves 32 cliques to a warp, and the search,
 // bound by the latency of its gathers, keeps twice the warps per SM without
 // the closed form's registers.
 #include <type_traits>
@@ -104,7 +104,7 @@ __device__ __forceinline__ void solve_cliques(const ProbView& v, int4 cl, int h,
     if (has) store_hypothesis(v, h, present, o, need ? 2u : 0u);
 }
 
-// Kabsch of a batch's cliques, 32 to a warp, 128 to a block.  The block is kept
+// Kabsch of a large batch's cliques, 32 to a warp, 128 to a block.  The block is kept
 // in the clique search's shape (256 threads, three to an SM, cliques handed to
 // the solving warps through shared memory): the assembler contracts products
 // and sums as its register budget suggests, and with a block of 128 threads a
@@ -133,14 +133,14 @@ __global__ void __launch_bounds__(256, 3) solve_kernel(ManyViews vs)
     solve_cliques(v, has ? s_cl[e] : make_int4(0, 0, 0, 0), has ? s_h[e] : 0, has, 32);
 }
 
-// kDense: a batch (keys sorted, cliques solved by solve_kernel, registers
+// kDense: a large batch (keys sorted, cliques solved by solve_kernel, registers
 // bounded for four blocks per SM: many waves of blocks, latency hidden by
 // occupancy); otherwise two blocks, with more registers per warp (one problem:
 // a single wave)
 template <int K2C, bool kDense>
 __global__ void __launch_bounds__(256, kDense ? 4 : 2) pgs_kernel(ManyViews vs)
 {
-    // dynamic shared memory: per-warp candidate lists, then the selected edge keys (one problem)
+    // dynamic shared memory: per-warp candidate lists, then the selected edge keys (unless dense)
     extern __shared__ __align__(16) uint8_t pgs_smem[];
     uint16_t (*scand)[kCand] = reinterpret_cast<uint16_t (*)[kCand]>(pgs_smem);
     uint64_t* skey = reinterpret_cast<uint64_t*>(pgs_smem + kListBytes);
@@ -152,12 +152,12 @@ __global__ void __launch_bounds__(256, kDense ? 4 : 2) pgs_kernel(ManyViews vs)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the selected edges (Eq. 4); keys W << 32 | ~(i n + j) are unique, larger =
     // heavier, then lower (i, j), and a pivot's index is its rank, the number of
-    // larger keys.  One problem: all K1 key slots are staged in the same round of
+    // larger keys.  Unless dense, all K1 key slots are staged in the same round of
     // loads as the number of selected edges (the selection fills the first
     // n_sel; the rest are ignored).
     const int np = v.ctl->n_sel;   // through L1: every warp of every block reads it
     const int kcap = v.k1;
-    // one problem: warp w of block b takes selected edge w * blocks + b; a batch
+    // warp w of block b takes selected edge w * blocks + b; dense:
     // 8 b + w, so that a block's pivots share rows more often
     const int c = kDense ? lb * 8 + warp : warp * ((kcap + 7) / 8) + lb;
     const uint64_t mykey = c < kcap ? __ldcg(v.cand + c) : 0ull;
@@ -409,7 +409,7 @@ void launch_pgs(const Batch& b, const int32_t tot[kNumBatchStages], int k2, int 
             default: launch_pdl(pgs_kernel<0, kD>, total, 256, smem, s, vs); break;
         }
     };
-    if (b.num > 1) {
+    if (pgs_dense(b.num, total, device_sms())) {
         go(std::true_type{});
         launch_pdl(solve_kernel, tot[ST_KABSCH], 256, 0, s, ManyViews{b});
     } else {

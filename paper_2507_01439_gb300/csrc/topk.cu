@@ -636,12 +636,11 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
     }
 }
 
-// Batches: a problem's selected keys sorted in place, largest first (one block
+// Large batches: a problem's selected keys sorted in place, largest first (one block
 // per problem, bitonic in shared memory), so that the clique search takes
 // pivot c from key c.  Finding each key's rank there instead, one warp per key
 // over all K1 keys, was 380 of the search's 2100 warp instructions per pivot;
-// the sort takes 1/40 of that (but a launch more, so one problem keeps the
-// ranks).  A pass of stride 32 or less stays inside the 64 keys of a warp.
+// the sort takes 1/40 of that (but a launch more: pgs_dense has the line).  A pass of stride 32 or less stays inside the 64 keys of a warp.
 __global__ void __launch_bounds__(1024) sort_kernel(ManyViews vs)
 {
     const ProbView& v = vs.bt.views[blockIdx.x];   // launch descriptors: before the wait
@@ -742,7 +741,7 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
     }
     if (emit_by_warp(max_n, b.num > 1)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     else launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
-    if (b.num > 1) {
+    if (pgs_dense(b.num, tot[ST_PGS], device_sms())) {
         int cap = 64;
         while (cap < max_k1) cap <<= 1;
         launch_pdl(sort_kernel, b.num, cap / 2 < 1024 ? cap / 2 : 1024, static_cast<size_t>(cap) * 8, s, vs);

@@ -81,6 +81,17 @@ __host__ __device__ inline int emit_blocks(int n, int in_batch) { return in_batc
 // 42.8 / 43.1, 1400 45.3 / 45.0, 2000 51.4 / 49.9, 2048 53.1 / 51.3; N = 5000 (the
 // pass alone) 12 / 7.0.
 inline bool emit_by_warp(int max_n, bool in_batch) { return in_batch || max_n <= 1024; }
+// Whether a batch's clique search takes its dense form: keys sorted by a launch
+// of their own, cliques solved by another, twice the warps per SM.  The two
+// launches and the sort (one block per problem) pay from some eight blocks of
+// the search per SM on, and with few problems, whose sorts occupy few SMs, later.
+// A call, dense / in the search itself (us, default graph): 2 problems of N = 300
+// with 300 pivots 70 / 62, 16 of 700 with 300 104 / 89, 64 of 300 with 100 117 /
+// 108, 32 of 300 with 300 (1216 blocks) 117 / 107, 64 of 1000 with 200 (1600) 197 /
+// 201, 256 of 100 with 50 (1792) 144 / 154, 16 of 3000 with 2000 (4000) 413 / 436;
+// 2 of 5000 with 8192 (2048) 387 / 305, 3 (3072) 469 / 418, 4 (4096) 550 / 528, 8 of
+// 2000 with 4096 (4096) 270 / 282, 8 of 5000 with 8192 879 / 970.
+inline bool pgs_dense(int num, int blocks, int sms) { return num > 1 && blocks > (num > 12 ? 8 : 26) * sms; }
 // Blocks of the histogram pass: one per group; from n = 8192 on a fixed number
 // that takes several groups each (a block clears and flushes n bins: at
 // n = 20000 that is 80 KB against the 320 KB of W a group holds).
@@ -166,14 +177,13 @@ int bitset_tiles(int n_pad);
 cudaError_t sc2_bitset_setup();
 void launch_hist(const Batch& b, int total, int max_n, cudaStream_t s);
 void launch_select(const Batch& b, cudaStream_t s);
-// count and emit passes of the selection; in a batch the selected keys are then
-// sorted (for one problem the clique search ranks the pivots)
+// count and emit passes of the selection; the selected keys are then sorted where
+// the clique search takes its dense form (else it ranks the pivots itself)
 // select_here: the count blocks choose the threshold from the histogram the
 // SC^2 GEMM completed (one problem of at most max_n matches)
 void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool select_here, int max_n, int max_k1,
                        cudaStream_t s);
-// Clique search and the cliques' Kabsch (for one problem the search also ranks
-// the pivots)
+// Clique search and the cliques' Kabsch
 void launch_pgs(const Batch& b, const int32_t tot[kNumBatchStages], int k2_max, int max_k1, cudaStream_t s);
 void launch_kabsch(const Batch& b, int total, cudaStream_t s);
 // out: results of the launch's problems in order (page-locked host or device

@@ -1,0 +1,49 @@
+"""Batches on both sides of the lines at which their passes change form, against
+single calls: equal bit for bit, for mixed K2, graph and scoring too."""
+import numpy as np
+import pytest
+
+import paper_2507_01439_gb300 as trg
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(sizes, params):
+    probs = [synth.make_problem("indoor", n, 0.05 + 0.02 * (b % 12), 3000 + 31 * b) for b, n in enumerate(sizes)]
+    offs = np.cumsum([0] + list(sizes)).astype(np.int64)
+    xs, ys = (np.concatenate([getattr(p, k) for p in probs]) for k in "xy")
+    which = (trg.BUF_PIVOTS, trg.BUF_CLIQUES, trg.BUF_RT, trg.BUF_INLIERS)
+    with trg.TurboReg(max_n=max(sizes), max_batch=len(sizes)) as c:
+        one = [c.register(p.x, p.y, q) for p, q in zip(probs, params)]
+        c.register(probs[0].x, probs[0].y, params[0])
+        first = [c.buffer(w) for w in which]
+        out = c.register_batched(xs, ys, offs, params)
+        many = [c.buffer(w) for w in which]
+    for a, b in zip(first, many):
+        assert a.shape == b.shape and np.array_equal(a.view(np.uint32), b.view(np.uint32))
+    for a, b in zip(one, out):
+        assert (a.status, a.hypothesis, a.n_pivots, a.n_valid, a.inlier_count, a.clique, a.score) == \
+            (b.status, b.hypothesis, b.n_pivots, b.n_valid, b.inlier_count, b.clique, b.score)
+        assert np.array_equal(a.R, b.R) and np.array_equal(a.t, b.t)
+
+
+def _sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+# the clique search's blocks (eight pivots each) at 8 per SM with 13 problems and more, at 26 with fewer
+@pytest.mark.parametrize("num,per_sm", [(2, 26), (12, 26), (13, 8), (64, 8)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_clique_search_forms(num, per_sm, more):
+    k1 = 8 * (per_sm * _sms() // num + more)
+    k1 = min(k1, trg.TURBOREG_K1_MAX)
+    _check([900 + 7 * b for b in range(num)], [trg.default_params(0.1, k1, 0.1) for _ in range(num)])
+
+
+@pytest.mark.parametrize("num", [3, 20])
+def test_mixed_parameters(num):
+    prm = [trg.default_params(0.1 + 0.05 * (b % 3), 50 + 400 * (b % 4), 0.1, k2=1 + b % 5,
+                              graph_mode=trg.GRAPH_SC2 if b % 2 else trg.GRAPH_O2, scoring=b % 3) for b in range(num)]
+    _check([150 + 97 * b for b in range(num)], prm)
