@@ -411,7 +411,9 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
     const int32_t vpw_flag = (prm[0]->flags & TURBOREG_FLAG_VERIFY_PTS32) ? 32
                              : (prm[0]->flags & TURBOREG_FLAG_VERIFY_PTS128) ? 128
                              : num > 1 && !vflag && wide >= 16 * static_cast<int64_t>(device_sms()) ? 128 : 64;
-    int32_t vppb_max = 0;
+    int32_t vppb_max = 0, n_max = 0;
+    for (int32_t b = 0; b < num; ++b) n_max = n[b] > n_max ? n[b] : n_max;
+    const bool emit_few = num > 1 && emit_by_warp(num, n_max);
     plan.k2_common = prm[0]->k2;
     for (int st = 0; st < kNumBatchStages; ++st) ws.h_pre[st * (num + 1)] = 0;
     for (int32_t b = 0; b < num; ++b) {
@@ -424,10 +426,10 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
         const int32_t vppb = (num == 1 && !vflag) ? balanced_vppb(n[b], prm[b]->k1 * prm[b]->k2, device_sms())
                                                   : 4 * vpw_flag;
         ws.h_views[b].vppb = vppb;
-        ws.h_views[b].in_batch = num > 1;
+        ws.h_views[b].emit_few = emit_few;
         if (vppb > vppb_max) vppb_max = vppb;
         int32_t blocks[kNumBatchStages];
-        stage_blocks(n[b], prm[b]->k1, prm[b]->k2, vppb, num > 1, blocks);
+        stage_blocks(n[b], prm[b]->k1, prm[b]->k2, vppb, count_by_warp(num), emit_few, blocks);
         for (int st = 0; st < kNumBatchStages; ++st) {
             plan.tot[st] += blocks[st];
             ws.h_pre[st * (num + 1) + b + 1] = plan.tot[st];

@@ -491,7 +491,8 @@ int32_t balanced_vppb(int32_t n, int32_t nh, int32_t num_sms)
     return vppb < 64 ? 64 : vppb;                                      // at least 16 matches per warp
 }
 
-void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, int32_t in_batch, int32_t blocks[kNumBatchStages])
+void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, bool count_warp, bool emit_few,
+                  int32_t blocks[kNumBatchStages])
 {
     const int32_t vpts = vppb;
     const int32_t n_pad = (n + kSc2BN - 1) / kSc2BN * kSc2BN;
@@ -501,9 +502,9 @@ void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, int32_t in_ba
     blocks[ST_PACK] = n_pad / 256;
     blocks[ST_COMPAT] = T * (T + 1) / 2;
     blocks[ST_SELECT] = 1;
-    blocks[ST_COUNT] = count_blocks(n, in_batch);
+    blocks[ST_COUNT] = count_blocks(n, count_warp);
     blocks[ST_SCAN] = 0;   // no separate row-scan pass
-    blocks[ST_EMIT] = emit_blocks(n, in_batch);
+    blocks[ST_EMIT] = emit_blocks(n, emit_few);
     blocks[ST_RANK] = (k1 + 31) / 32;
     blocks[ST_PGS] = (k1 + 7) / 8;
     blocks[ST_KABSCH] = (nh + 127) / 128;

@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
         v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
 }
 
-// The same counts in a batch: a warp per group, without block barriers; the
+// The same counts in a batch of many problems: a warp per group, without block barriers; the
 // threshold comes from the select launch.  With a block per group the pass over
 // 256 problems took 345 us (blocks that start, find their problem and read
 // nothing), with four groups per block 254 us (bound by its barriers), now 98.
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) count_warp_kernel(ManyViews 
     }
 }
 
-// A warp per active row (batches; one problem of up to 1024 matches):
+// A warp per active row (most batches; one problem of up to 1024 matches):
 // lane l reads chunks 4l .. 4l + 3 of each 128-chunk sweep (lane order =
 // column order), the next sweep in flight, and needs no block barrier.  A
 // block's eight rows then run side by side: with a block per row and n/8
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
     pdl_wait();
     pdl_release();
     const int lane = threadIdx.x & 31;
-    const int n = v.n, eb = emit_blocks(n, v.in_batch);
+    const int n = v.n, eb = emit_blocks(n, v.emit_few);
     const int a0 = (threadIdx.x >> 5) * eb + lb;          // this warp's first active row
     const int n_sel = v.ctl->n_sel;
     const int nact = static_cast<int>(v.ctl->n_active);
@@ -513,8 +513,8 @@ __global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
     }
 }
 
-// A block per active row (one larger problem: its rows are read in one or two
-// rounds).  Blocks take the active rows in any order.  W > alpha edges take slots
+// A block per active row (one or a few larger problems: a row is read in one or
+// two rounds).  Blocks take the active rows in any order.  W > alpha edges take slots
 // base + rank-in-row from one atomic per row (any slots in [0, c_gt) will
 // do: the rank pass orders the keys).  Ties must be the m lowest (i, j):
 // a row with ties sums the tie counts of the active rows above it (its tie
@@ -733,13 +733,13 @@ void launch_count_emit(const Batch& b, const int32_t tot[kNumBatchStages], bool 
                        cudaStream_t s)
 {
     const ManyViews vs{b};
-    if (b.num > 1) {
+    if (count_by_warp(b.num)) {
         launch_pdl(count_warp_kernel, tot[ST_COUNT], 256, 0, s, vs);
     } else {
         const size_t stage = select_here ? static_cast<size_t>((max_n + 4) / 4 * 4) * 4 : 0;
         launch_pdl(count_kernel<ManyViews>, tot[ST_COUNT], kCountThreads, stage, s, vs, select_here ? 1 : 0);
     }
-    if (emit_by_warp(max_n, b.num > 1)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
+    if (emit_by_warp(b.num, max_n)) launch_pdl(emit_warp_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     else launch_pdl(emit_kernel<ManyViews>, tot[ST_EMIT], 256, 0, s, vs);
     if (pgs_dense(b.num, tot[ST_PGS], device_sms())) {
         int cap = 64;
@@ -757,7 +757,7 @@ void launch_topk_single(const ProbView& v, int32_t* n_out, cudaStream_t s)
     launch_pdl(caller_hist_kernel, (warps + 31) / 32 < sms ? (warps + 31) / 32 : sms, 1024, (v.n + 1) * 4, s, vs);
     launch_pdl(count_kernel<OneView>, count_groups(v.n), kCountThreads, static_cast<size_t>((v.n + 4) / 4 * 4) * 4, s,
                vs, 1);
-    if (emit_by_warp(v.n, false)) launch_pdl(emit_warp_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
+    if (emit_by_warp(1, v.n)) launch_pdl(emit_warp_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
     else launch_pdl(emit_kernel<OneView>, emit_blocks(v.n, 0), 256, 0, s, vs);
     launch_pdl(rank_kernel, (v.k1 + 31) / 32, 256, v.k1 * 8, s, vs, n_out);
 }

@@ -26,7 +26,7 @@ struct ProbView {
     int32_t graph_mode;  // TURBOREG_GRAPH_O2 / _SC2: the graph the clique search runs on
     int32_t scoring;     // TURBOREG_SCORE_IN / _MAE / _MSE
     int32_t vppb;        // verification tile: matches per block (<= 4 x the kernel's points per warp)
-    int32_t in_batch;    // 1: one of several problems of a call (blocks per problem of the passes over W)
+    int32_t emit_few;    // 1: the emit pass takes n / 64 blocks for this problem, else n / 8
     uint32_t dbg;        // failure injection for tests (TR_DBG_*), 0 in normal use
     uint8_t* a4_auto;    // non-null: the SC^2 path is chosen on the device from the degrees (one
                          // problem, n_pad <= 5120); a4 is then null, so the compatibility kernel
@@ -66,21 +66,31 @@ enum Stage {
     ST_VERIFY, ST_FINAL, ST_HIST, ST_BITSET, ST_GEMM, ST_FEAT, ST_MLP, kNumBatchStages
 };
 
-// Groups of eight row pairs of the passes over W; blocks of the count pass (in
-// a batch a warp per group) and of the emit pass (active rows strided over the
-// blocks, or in a batch over their warps).
+// Groups of eight row pairs of the passes over W; blocks of the count pass (a
+// block or a warp per group) and of the emit pass (active rows strided over the
+// blocks, or with few blocks over their warps).
 __host__ __device__ inline int count_groups(int n) { return ((n + 1) / 2 + 7) / 8; }
-__host__ __device__ inline int count_blocks(int n, int in_batch)
+__host__ __device__ inline int count_blocks(int n, bool by_warp)
 {
-    return in_batch ? (count_groups(n) + 7) / 8 : count_groups(n);
+    return by_warp ? (count_groups(n) + 7) / 8 : count_groups(n);
 }
-__host__ __device__ inline int emit_blocks(int n, int in_batch) { return in_batch ? (n + 63) / 64 : (n + 7) / 8; }
-// The emit pass takes a warp per active row in a batch and for one problem of
-// up to 1024 matches (a row is one sweep of a warp), else a block.  One
+__host__ __device__ inline int emit_blocks(int n, int few) { return few ? (n + 63) / 64 : (n + 7) / 8; }
+// The count pass takes a warp per group from 17 problems on (blocks that start
+// and read nothing), else a block (a group's rows read by eight warps).  A call,
+// warp / block (us): 2 problems of N = 5000 with 2000 pivots 174 / 161, 4 of 1500
+// with 300 75 / 71, 16 of 700 with 1000 133 / 118, 16 of 3000 with 1000 340 / 339; 24
+// of 1000 with 100 103 / 105, 48 of 400 with 200 116 / 120, 64 of 1000 with 200 196 /
+// 211.
+inline bool count_by_warp(int num) { return num > 16; }
+// The emit pass takes a warp per active row for one problem of up to 1024
+// matches (a row is one sweep of a warp), from five problems on, and for fewer
+// with short rows, else a block.  A call, warp / block (us): 2 problems of N =
+// 5000 with 2000 pivots 174 / 170, with 8192 387 / 319; 4 of 1500 with 300 75 / 75, 8
+// of 3000 with 1000 200 / 206, 64 of 1000 with 200 196 / 221.  One
 // registration, warp / block (us): N = 67 30.8 / 32.9, 200 35.0 / 35.0, 1000
 // 42.8 / 43.1, 1400 45.3 / 45.0, 2000 51.4 / 49.9, 2048 53.1 / 51.3; N = 5000 (the
 // pass alone) 12 / 7.0.
-inline bool emit_by_warp(int max_n, bool in_batch) { return in_batch || max_n <= 1024; }
+inline bool emit_by_warp(int num, int max_n) { return num > 4 || max_n <= (num == 1 ? 1024 : 2048); }
 // Whether a batch's clique search takes its dense form: keys sorted by a launch
 // of their own, cliques solved by another, twice the warps per SM.  The two
 // launches and the sort (one block per problem) pay from some eight blocks of
@@ -151,7 +161,8 @@ struct ManyViews {
 
 // per-problem block counts of each stage (host side, from n, k1, k2)
 // vppb: matches per verification block (ProbView::vppb)
-void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, int32_t in_batch, int32_t blocks[kNumBatchStages]);
+void stage_blocks(int32_t n, int32_t k1, int32_t k2, int32_t vppb, bool count_warp, bool emit_few,
+                  int32_t blocks[kNumBatchStages]);
 // Matches per verification block for a single problem: the block count
 // (hypothesis blocks x match blocks) close to 4 blocks per SM, so that one
 // wave covers the problem with every SM holding the same number of blocks.

@@ -47,3 +47,17 @@ def test_mixed_parameters(num):
     prm = [trg.default_params(0.1 + 0.05 * (b % 3), 50 + 400 * (b % 4), 0.1, k2=1 + b % 5,
                               graph_mode=trg.GRAPH_SC2 if b % 2 else trg.GRAPH_O2, scoring=b % 3) for b in range(num)]
     _check([150 + 97 * b for b in range(num)], prm)
+
+
+# the count pass: a block per group up to 16 problems, then a warp
+@pytest.mark.parametrize("num", [16, 17])
+@pytest.mark.parametrize("k1", [10, 3000])
+def test_count_forms(num, k1):
+    _check([200 + 61 * b for b in range(num)], [trg.default_params(0.1, k1, 0.1) for _ in range(num)])
+
+
+# the emit pass: up to four problems of more than 2048 matches a block per active row, else a warp
+@pytest.mark.parametrize("sizes", [[2048, 2047], [2049, 40], [2500, 300, 2049, 1000], [2500, 300, 2049, 1000, 64]])
+@pytest.mark.parametrize("k1", [10, 3000])
+def test_emit_forms(sizes, k1):
+    _check(sizes, [trg.default_params(0.1 if n > 500 else 9.0, k1, 0.1) for n in sizes])   # 9.0: complete graphs, all ties
