@@ -245,10 +245,12 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
     }
 }
 
-// Registers: five blocks per SM in a batch (kMany; 256 problems 1077 -> 1038 us
-// against 120 registers and four blocks); the single problem's balanced launch
-// holds four blocks per SM, and there the spills of that budget cost more
-// (N = 20000 44 -> 46 us).
+// Registers: five blocks per SM (kMany) in a batch of at least 16 blocks per SM
+// (256 problems 1077 -> 1038 us against 120 registers and four blocks).  In less
+// than a few waves the spills of that budget cost more than the fifth block
+// gives (a call of 8 problems of N = 700 71 us, with four blocks 68; 64 of 300 110,
+// 108; equal from 64 of 1000 on), as they do in the single problem's balanced
+// launch of four blocks per SM (N = 20000 44 -> 46 us).
 template <int PW, bool kMany>
 __global__ void __launch_bounds__(128, kMany ? 5 : 4) verify_kernel(ManyViews vs)
 {
@@ -475,7 +477,7 @@ void launch_verify(const Batch& b, int total, int pw, bool capped, cudaStream_t 
         else if (pw == 128) launch_pdl(verify_kernel<128, kM>, total, 128, dyn, s, ManyViews{b});
         else launch_pdl(verify_kernel<64, kM>, total, 128, dyn, s, ManyViews{b});
     };
-    if (b.num > 1) go(std::true_type{});
+    if (b.num > 1 && total >= 16 * device_sms()) go(std::true_type{});
     else go(std::false_type{});
 }
 

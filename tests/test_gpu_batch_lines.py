@@ -61,3 +61,10 @@ def test_count_forms(num, k1):
 @pytest.mark.parametrize("k1", [10, 3000])
 def test_emit_forms(sizes, k1):
     _check(sizes, [trg.default_params(0.1 if n > 500 else 9.0, k1, 0.1) for n in sizes])   # 9.0: complete graphs, all ties
+
+
+# verification: from 16 blocks per SM on (128 hypotheses x 256 matches each, then x 512) another register budget
+@pytest.mark.parametrize("num,k1", [(8, 1152), (19, 1000), (20, 1024), (40, 1024)])
+@pytest.mark.parametrize("scoring", [trg.SCORE_IN, trg.SCORE_MAE, trg.SCORE_MSE])
+def test_verification_forms(num, k1, scoring):
+    _check([2040 + b for b in range(num)], [trg.default_params(0.1, k1, 0.1, scoring=scoring) for _ in range(num)])
