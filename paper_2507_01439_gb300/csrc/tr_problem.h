@@ -99,9 +99,13 @@ inline bool emit_by_warp(int num, int max_n) { return num > 4 || max_n <= (num =
 // with 300 pivots 70 / 62, 16 of 700 with 300 104 / 89, 64 of 300 with 100 117 /
 // 108, 32 of 300 with 300 (1216 blocks) 117 / 107, 64 of 1000 with 200 (1600) 197 /
 // 201, 256 of 100 with 50 (1792) 144 / 154, 16 of 3000 with 2000 (4000) 413 / 436;
-// 2 of 5000 with 8192 (2048) 387 / 305, 3 (3072) 469 / 418, 4 (4096) 550 / 528, 8 of
-// 2000 with 4096 (4096) 270 / 282, 8 of 5000 with 8192 879 / 970.
-inline bool pgs_dense(int num, int blocks, int sms) { return num > 1 && blocks > (num > 12 ? 8 : 26) * sms; }
+// 12 of 2000 with 1000 (1500) 189 / 177, 8 of 2000 with 2000 (2000) 187 / 181, 12 of
+// 500 with 2000 (3000) 133 / 157, 8 of 2000 with 4096 (4096) 270 / 282; 2 of 5000
+// with 8192 (2048) 387 / 305, 3 (3072) 469 / 418, 4 (4096) 550 / 528.
+inline bool pgs_dense(int num, int blocks, int sms)
+{
+    return num > 1 && blocks > (num > 12 ? 8 : num > 4 ? 16 : 26) * sms;
+}
 // Blocks of the histogram pass: one per group; from n = 8192 on a fixed number
 // that takes several groups each (a block clears and flushes n bins: at
 // n = 20000 that is 80 KB against the 320 KB of W a group holds).

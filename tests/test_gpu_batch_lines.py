@@ -33,8 +33,8 @@ def _sms():
     return torch.cuda.get_device_properties(0).multi_processor_count
 
 
-# the clique search's blocks (eight pivots each) at 8 per SM with 13 problems and more, at 26 with fewer
-@pytest.mark.parametrize("num,per_sm", [(2, 26), (12, 26), (13, 8), (64, 8)])
+# the clique search's blocks (eight pivots each): 8 per SM with 13 problems and more, 16 with five, 26 with fewer
+@pytest.mark.parametrize("num,per_sm", [(2, 26), (4, 26), (5, 16), (12, 16), (13, 8), (64, 8)])
 @pytest.mark.parametrize("more", [0, 1])
 def test_clique_search_forms(num, per_sm, more):
     k1 = 8 * (per_sm * _sms() // num + more)
