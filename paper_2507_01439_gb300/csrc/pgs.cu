@@ -55,13 +55,13 @@ __device__ __forceinline__ void solve_cliques(const ProbView& v, int4 cl, int h,
 {
     const int lane = threadIdx.x & 31;
     float P[3][3], Q[3][3];
-    KabschOut<float> o;
+    KabschOut o;
     o.ok = false;
     bool need = false;
     const bool present = has && cl.w != 0;
     if (present) {
         load_clique(v, cl, P, Q);
-        kabsch3<float>(P, Q, o);
+        kabsch3(P, Q, o);
         need = !(o.ok && o.kappa <= v.kappa_fp64);
     }
     const uint32_t needm = __ballot_sync(0xffffffffu, need);
@@ -99,38 +99,22 @@ __device__ __forceinline__ void solve_cliques(const ProbView& v, int4 cl, int h,
                 }
             }
         }
-        if (need) kabsch3<float, true>(P, Q, o, nx, ny);
+        if (need) kabsch3<true>(P, Q, o, nx, ny);
     }
     if (has) store_hypothesis(v, h, present, o, need ? 2u : 0u);
 }
 
-// Kabsch of a large batch's cliques, 32 to a warp, 128 to a block.  The block is kept
-// in the clique search's shape (256 threads, three to an SM, cliques handed to
-// the solving warps through shared memory): the assembler contracts products
-// and sums as its register budget suggests, and with a block of 128 threads a
-// batch's hypotheses came out one last bit away from one problem's.  (Equal in
-// every bit this way, which the tests check for every K2 form.)
-__global__ void __launch_bounds__(256, 3) solve_kernel(ManyViews vs)
+// Kabsch of a large batch's cliques, a lane each.
+__global__ void __launch_bounds__(128) solve_kernel(ManyViews vs)
 {
     int lb;
     const ProbView v = vs.get(ST_KABSCH, blockIdx.x, lb);   // launch descriptors: before the wait
     pdl_wait();
     pdl_release();
-    __shared__ int4 s_cl[128];
-    __shared__ int s_h[128];
-    const int t = threadIdx.x;
-    const int nh = v.ctl->n_pivots * v.k2;
-    if (t < 128) {
-        const int h = lb * 128 + t;
-        s_cl[t] = h < nh ? v.cliques[h] : make_int4(0, 0, 0, 0);
-        s_h[t] = h < nh ? h : -1;
-    }
-    __syncthreads();
-    const int lane = t & 31, warp = t >> 5;
-    if (warp >= 4) return;
-    const int e = warp * 32 + lane;
-    const bool has = s_h[e] >= 0;
-    solve_cliques(v, has ? s_cl[e] : make_int4(0, 0, 0, 0), has ? s_h[e] : 0, has, 32);
+    const int h = lb * 128 + static_cast<int>(threadIdx.x);
+    const bool has = h < v.ctl->n_pivots * v.k2;
+    if (!__any_sync(0xffffffffu, has)) return;
+    solve_cliques(v, has ? v.cliques[h] : make_int4(0, 0, 0, 0), h, has, 32);
 }
 
 // kDense: a large batch (keys sorted, cliques solved by solve_kernel, registers
@@ -411,7 +395,7 @@ void launch_pgs(const Batch& b, const int32_t tot[kNumBatchStages], int k2, int 
     };
     if (pgs_dense(b.num, total, device_sms())) {
         go(std::true_type{});
-        launch_pdl(solve_kernel, tot[ST_KABSCH], 256, 0, s, ManyViews{b});
+        launch_pdl(solve_kernel, tot[ST_KABSCH], 128, 0, s, ManyViews{b});
     } else {
         go(std::false_type{});
     }

@@ -27,6 +27,13 @@
 // FP64 components with six lanes per clique (one per triangle and component),
 // so a warp issues a dozen FP64 instructions instead of a hundred.  A clique
 // with sigma2 <= 1e-12 sigma1 (collinear or repeated points) is invalid.
+//
+// Every product and sum names its rounding (__fmaf_rn, __fmul_rn, __fadd_rn), so
+// that a clique's R, t and kappa are the same bits in every kernel that solves
+// it: one problem's search, a batch's solve kernel, the clique-Kabsch entry.  Left
+// to the compiler, which products it contracts changed with the kernel's shape
+// and register budget.  (The order of the operations is the one the search's
+// kernels had been given: the results are the earlier ones.)
 #pragma once
 
 #include "tr_common.cuh"
@@ -36,31 +43,32 @@ namespace tr {
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ T inv_sqrt(T x);
-template <>
-__device__ __forceinline__ float inv_sqrt<float>(float x) { return 1.0f / sqrtf(x); }
-template <typename T>
+__device__ __forceinline__ float inv_sqrt(float x) { return 1.0f / sqrtf(x); }
+
 struct KabschOut {
-    T R[9];
-    T t[3];
-    T kappa;
+    float R[9];
+    float t[3];
+    float kappa;
     bool ok;    // frames defined and sigma1 > 0
-    T s1, s2;
+    float s1, s2;
 };
 
-template <typename T>
-__device__ __forceinline__ void cross3(const T a[3], const T b[3], T c[3])
+// a b - c d
+__device__ __forceinline__ float diff_prod(float a, float b, float c, float d)
 {
-    c[0] = a[1] * b[2] - a[2] * b[1];
-    c[1] = a[2] * b[0] - a[0] * b[2];
-    c[2] = a[0] * b[1] - a[1] * b[0];
+    return __fmaf_rn(a, b, -__fmul_rn(c, d));
 }
 
-template <typename T>
-__device__ __forceinline__ T dot3(const T a[3], const T b[3])
+__device__ __forceinline__ void cross3(const float a[3], const float b[3], float c[3])
 {
-    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+    c[0] = diff_prod(a[1], b[2], a[2], b[1]);
+    c[1] = diff_prod(a[2], b[0], a[0], b[2]);
+    c[2] = diff_prod(a[0], b[1], a[1], b[0]);
+}
+
+__device__ __forceinline__ float dot3(const float a[3], const float b[3])
+{
+    return __fmaf_rn(a[2], b[2], __fmaf_rn(a[0], b[0], __fmul_rn(a[1], b[1])));
 }
 
 // Component c of the normal (p1 - p0) x (p2 - p0) in FP64 from exact FP64
@@ -79,32 +87,35 @@ __device__ __forceinline__ float exact_normal_comp(const float (&p)[3][3], int c
 // n = unit normal of (p1 - p0) x (p2 - p0), e2 = n x e1.  ng: the normal's
 // components given by the caller (FP64 cross product rounded to FP32), and
 // then *nlen receives their length |(p1 - p0) x (p2 - p0)| (twice the area).
-template <typename T, bool kGiven>
-__device__ __forceinline__ bool frame3(const T p[3][3], T e1[3], T e2[3], T nrm[3], const T* ng, T* nlen)
+template <bool kGiven>
+__device__ __forceinline__ bool frame3(const float p[3][3], float e1[3], float e2[3], float nrm[3], const float* ng,
+                                       float* nlen)
 {
-    T d01[3], d02[3], d12[3];
+    float d01[3], d02[3], d12[3];
     for (int c = 0; c < 3; ++c) {
-        d01[c] = p[1][c] - p[0][c];
-        d02[c] = p[2][c] - p[0][c];
-        d12[c] = p[2][c] - p[1][c];
+        d01[c] = __fsub_rn(p[1][c], p[0][c]);
+        d02[c] = __fsub_rn(p[2][c], p[0][c]);
+        d12[c] = __fsub_rn(p[2][c], p[1][c]);
     }
+    float nn;
     if (kGiven) {
         nrm[0] = ng[0]; nrm[1] = ng[1]; nrm[2] = ng[2];
+        nn = __fmaf_rn(nrm[2], nrm[2], __fmaf_rn(nrm[1], nrm[1], __fmul_rn(nrm[0], nrm[0])));
+        *nlen = sqrtf(nn);
     } else {
         cross3(d01, d02, nrm);
+        nn = dot3(nrm, nrm);
     }
-    const T nn = dot3(nrm, nrm);
-    if (kGiven) *nlen = sqrt(nn);
-    const T l01 = dot3(d01, d01), l02 = dot3(d02, d02), l12 = dot3(d12, d12);
+    const float l01 = dot3(d01, d01), l02 = dot3(d02, d02), l12 = dot3(d12, d12);
     int sel = 0;   // longest edge, selected by value (no pointer into local arrays)
-    T le = l01;
+    float le = l01;
     if (l02 > le) { sel = 1; le = l02; }
     if (l12 > le) { sel = 2; le = l12; }
-    if (!(nn > T(0)) || !(le > T(0))) return false;
-    const T in = inv_sqrt(nn), ie = inv_sqrt(le);
+    if (!(nn > 0.f) || !(le > 0.f)) return false;
+    const float in = inv_sqrt(nn), ie = inv_sqrt(le);
     for (int c = 0; c < 3; ++c) {
-        nrm[c] *= in;
-        e1[c] = (sel == 0 ? d01[c] : sel == 1 ? d02[c] : d12[c]) * ie;
+        nrm[c] = __fmul_rn(nrm[c], in);
+        e1[c] = __fmul_rn(sel == 0 ? d01[c] : sel == 1 ? d02[c] : d12[c], ie);
     }
     cross3(nrm, e1, e2);
     return true;
@@ -112,72 +123,77 @@ __device__ __forceinline__ bool frame3(const T p[3][3], T e1[3], T e2[3], T nrm[
 
 // kGiven: the two triangles' normals nxg, nyg are given by the caller (the
 // FP64 path); otherwise they are the FP32 cross products.
-template <typename T, bool kGiven = false>
-__device__ __forceinline__ void kabsch3(const T p[3][3], const T q[3][3], KabschOut<T>& o, const T* nxg = nullptr,
-                                        const T* nyg = nullptr)
+template <bool kGiven = false>
+__device__ __forceinline__ void kabsch3(const float p[3][3], const float q[3][3], KabschOut& o,
+                                        const float* nxg = nullptr, const float* nyg = nullptr)
 {
-    T cx[3], cy[3];
+    constexpr float kThird = static_cast<float>(1.0 / 3.0);
+    float cx[3], sy[3];   // mean of the p, sum of the q
     for (int c = 0; c < 3; ++c) {
-        cx[c] = (p[0][c] + p[1][c] + p[2][c]) * T(1.0 / 3.0);
-        cy[c] = (q[0][c] + q[1][c] + q[2][c]) * T(1.0 / 3.0);
+        cx[c] = __fmul_rn(__fadd_rn(__fadd_rn(p[0][c], p[1][c]), p[2][c]), kThird);
+        sy[c] = __fadd_rn(__fadd_rn(q[0][c], q[1][c]), q[2][c]);
     }
-    T e1[3], e2[3], nx[3], f1[3], f2[3], ny[3];
-    T lx = T(0), ly = T(0);
-    o.ok = frame3<T, kGiven>(p, e1, e2, nx, nxg, &lx) && frame3<T, kGiven>(q, f1, f2, ny, nyg, &ly);
+    float e1[3], e2[3], nx[3], f1[3], f2[3], ny[3];
+    float lx = 0.f, ly = 0.f;
+    o.ok = frame3<kGiven>(p, e1, e2, nx, nxg, &lx) && frame3<kGiven>(q, f1, f2, ny, nyg, &ly);
     if (!o.ok) {
-        o.kappa = T(INFINITY);
-        o.s1 = o.s2 = T(0);
+        o.kappa = INFINITY;
+        o.s1 = o.s2 = 0.f;
         return;
     }
-    T m11 = 0, m12 = 0, m21 = 0, m22 = 0;
+    float m11 = 0.f, m12 = 0.f, m21 = 0.f, m22 = 0.f;
     for (int k = 0; k < 3; ++k) {
-        T a[3], b[3];
+        float a[3], b[3];
         for (int c = 0; c < 3; ++c) {
-            a[c] = p[k][c] - cx[c];
-            b[c] = q[k][c] - cy[c];
+            a[c] = __fsub_rn(p[k][c], cx[c]);
+            b[c] = __fmaf_rn(-sy[c], kThird, q[k][c]);
         }
-        const T P1 = dot3(a, e1), P2 = dot3(a, e2);
-        const T Q1 = dot3(b, f1), Q2 = dot3(b, f2);
-        m11 += P1 * Q1; m12 += P1 * Q2;
-        m21 += P2 * Q1; m22 += P2 * Q2;
+        const float P1 = dot3(a, e1), P2 = dot3(a, e2);
+        const float Q1 = dot3(b, f1), Q2 = dot3(b, f2);
+        m11 = __fmaf_rn(P1, Q1, m11); m12 = __fmaf_rn(P1, Q2, m12);
+        m21 = __fmaf_rn(P2, Q1, m21); m22 = __fmaf_rn(P2, Q2, m22);
     }
-    const T rx = m11 + m22, ry = m12 - m21;   // rotation candidate
-    const T fx = m11 - m22, fy = m12 + m21;   // reflection candidate
-    const T r2 = rx * rx + ry * ry, q2 = fx * fx + fy * fy;
-    if (!(r2 > T(0) || q2 > T(0))) {
+    const float rx = __fadd_rn(m11, m22), ry = __fsub_rn(m12, m21);   // rotation candidate
+    const float fx = __fsub_rn(m11, m22), fy = __fadd_rn(m12, m21);   // reflection candidate
+    const float r2 = __fmaf_rn(ry, ry, __fmul_rn(rx, rx)), q2 = __fmaf_rn(fy, fy, __fmul_rn(fx, fx));
+    if (!(r2 > 0.f || q2 > 0.f)) {
         o.ok = false;
-        o.kappa = T(INFINITY);
-        o.s1 = o.s2 = T(0);
+        o.kappa = INFINITY;
+        o.s1 = o.s2 = 0.f;
         return;
     }
     const bool rot = r2 >= q2;
-    const T ih = inv_sqrt(rot ? r2 : q2);               // 1 / (sigma1 + sigma2)
-    const T hi = (rot ? r2 : q2) * ih;
-    const T lo2 = rot ? q2 : r2;
-    const T lo = lo2 > T(0) ? lo2 * inv_sqrt(lo2) : T(0);
-    o.s1 = (hi + lo) * T(0.5);
-    o.s2 = (hi - lo) * T(0.5);
-    if (kGiven && o.s1 > T(0)) {
+    const float hi2 = rot ? r2 : q2, lo2 = rot ? q2 : r2;
+    const float ih = inv_sqrt(hi2);                     // 1 / (sigma1 + sigma2)
+    const float lo = lo2 > 0.f ? __fmul_rn(lo2, inv_sqrt(lo2)) : 0.f;
+    o.s1 = __fmul_rn(__fmaf_rn(hi2, ih, lo), 0.5f);
+    o.s2 = __fmul_rn(__fmaf_rn(hi2, ih, -lo), 0.5f);
+    if (kGiven && o.s1 > 0.f) {
         // sigma2 of a thin clique from sigma1 sigma2 = |det M| = |n_x| |n_y| / 3
         // (Cauchy-Binet over three centred points), with the lengths of the
         // accurate normals, instead of the cancelling difference (hi - lo) / 2
-        o.s2 = lx * ly / (T(3) * o.s1);
+        o.s2 = __fmul_rn(lx, ly) / __fmul_rn(3.f, o.s1);
     }
-    o.kappa = o.s2 > T(0) ? static_cast<T>(static_cast<float>(o.s1) / static_cast<float>(o.s2)) : T(INFINITY);
-    T X00, X01, X10, X11, sg;
+    o.kappa = o.s2 > 0.f ? o.s1 / o.s2 : INFINITY;
+    float X00, X01, X10, X11, sg;
     if (rot) {
-        const T c = rx * ih, s = ry * ih;
-        X00 = c; X01 = -s; X10 = s; X11 = c; sg = T(1);
+        const float c = __fmul_rn(rx, ih), s = __fmul_rn(ry, ih);
+        X00 = c; X01 = -s; X10 = s; X11 = c; sg = 1.f;
     } else {
-        const T c = fx * ih, s = fy * ih;
-        X00 = c; X01 = s; X10 = s; X11 = -c; sg = T(-1);
+        const float c = __fmul_rn(fx, ih), s = __fmul_rn(fy, ih);
+        X00 = c; X01 = s; X10 = s; X11 = -c; sg = -1.f;
     }
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c)
-            o.R[r * 3 + c] = X00 * f1[r] * e1[c] + X01 * f1[r] * e2[c] + X10 * f2[r] * e1[c] +
-                             X11 * f2[r] * e2[c] + sg * ny[r] * nx[c];
-    for (int r = 0; r < 3; ++r)
-        o.t[r] = cy[r] - (o.R[r * 3 + 0] * cx[0] + o.R[r * 3 + 1] * cx[1] + o.R[r * 3 + 2] * cx[2]);
+    for (int r = 0; r < 3; ++r) {
+        const float xa = __fmul_rn(X00, f1[r]), xb = __fmul_rn(X01, f1[r]);
+        const float xc = __fmul_rn(X10, f2[r]), xd = __fmul_rn(X11, f2[r]), xe = __fmul_rn(sg, ny[r]);
+        for (int c = 0; c < 3; ++c) {
+            float v = __fmaf_rn(xa, e1[c], __fmul_rn(xb, e2[c]));
+            v = __fmaf_rn(xc, e1[c], v);
+            v = __fmaf_rn(xd, e2[c], v);
+            o.R[r * 3 + c] = __fmaf_rn(xe, nx[c], v);
+        }
+    }
+    for (int r = 0; r < 3; ++r) o.t[r] = __fmaf_rn(sy[r], kThird, -dot3(&o.R[r * 3], cx));
 }
 
 __device__ __forceinline__ void load_clique(const ProbView& v, const int4 cl, float p[3][3], float q[3][3])
@@ -194,7 +210,7 @@ __device__ __forceinline__ void load_clique(const ProbView& v, const int4 cl, fl
 // Writes hypothesis h: R, t and kappa of a solved clique (flags: 1 valid,
 // 2 the FP64 normals were used), zero for an empty slot; the inlier count
 // and score are cleared.
-__device__ __forceinline__ void store_hypothesis(const ProbView& v, int h, bool present, const KabschOut<float>& o,
+__device__ __forceinline__ void store_hypothesis(const ProbView& v, int h, bool present, const KabschOut& o,
                                                  uint32_t flags)
 {
     v.inl[h] = 0;
@@ -225,12 +241,12 @@ __device__ __forceinline__ void store_hypothesis(const ProbView& v, int h, bool 
 // when needed, computed by the same thread).
 __device__ __forceinline__ void kabsch_hypothesis(const ProbView& v, int h, int4 cl)
 {
-    KabschOut<float> o;
+    KabschOut o;
     uint32_t flags = 0;
     if (cl.w) {
         float p[3][3], q[3][3];
         load_clique(v, cl, p, q);
-        kabsch3<float>(p, q, o);
+        kabsch3(p, q, o);
         if (!(o.ok && o.kappa <= v.kappa_fp64)) {   // ill-conditioned: FP64 normals
             float nx[3], ny[3];
 #pragma unroll
@@ -238,7 +254,7 @@ __device__ __forceinline__ void kabsch_hypothesis(const ProbView& v, int h, int4
                 nx[c] = exact_normal_comp(p, c);
                 ny[c] = exact_normal_comp(q, c);
             }
-            kabsch3<float, true>(p, q, o, nx, ny);
+            kabsch3<true>(p, q, o, nx, ny);
             flags = 2u;
         }
     }
