@@ -78,8 +78,8 @@ typedef enum {
                                           pair MMAs available) one problem of N <= 2048 takes the
                                           CUDA-core path; up to N = 5120 turboreg_register has the
                                           path chosen on the device after the compatibility graph,
-                                          from N and the edge count (the CUDA-core path up to about
-                                          5 % density at N = 5000), and turboreg_register_async
+                                          from N and the edge count (the CUDA-core path up to nearly
+                                          6 % density at N = 5000), and turboreg_register_async
                                           takes the GEMM; batches and larger problems use the GEMM.
                                           Same integers on every path */
 #define TURBOREG_FLAG_STAGE_TIMES 0x2u /* record per-stage CUDA-event times (turboreg_stage_times) */
@@ -138,7 +138,8 @@ void turboreg_default_params(turboreg_params* p, float tau, int32_t k1, float in
  * max_n correspondences and batches of up to max_batch problems whose total
  * correspondence count is at most max_n * max_batch.  `cuda_stream` is a
  * cudaStream_t to run on, or NULL to let the context create its own.  The
- * device workspace (about 2.6 * max_n^2 bytes per batched problem slot) is allocated here, never inside register calls.
+ * device workspace (about 2.6 * max_n^2 bytes per batched problem slot) is
+ * allocated here, never inside register calls.
  * On success *out receives the context.
  * Errors: INVALID_ARG (out NULL, max_n < 3 or > TURBOREG_MAX_N, max_batch < 1),
  *         OOM, CUDA. */

@@ -185,8 +185,8 @@ int turboreg_mlp_debug_blocks(turboreg_mlp* t, int32_t m);
  * memory through its own pool, or a real-time loop that forbids allocation
  * after start-up (cudaMalloc may synchronise the device and take unbounded
  * time).  Its scratch (histogram, active-row list with per-row counts,
- * candidate keys, control block, row maxima: about 257 KB) is one fixed array in the library's device memory,
- * loaded with the module and held by every GPU that loads the library until
+ * candidate keys, control block, row maxima: about 257 KB) is one fixed array
+ * in the library's device memory, loaded with the module and held by every GPU that loads the library until
  * the process exits; nothing is allocated or freed by this call.
  *
  *  w_dev       device, uint16 [n][ldw] row-major, 16-byte aligned; entry (i, j)

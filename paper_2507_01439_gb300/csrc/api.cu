@@ -372,8 +372,8 @@ int encode_maps(turboreg_ctx* c, int slot, int32_t n_pad, CUtensorMap* out2)
 // there at every density measured (registrations enqueued back to back, us,
 // chosen path / GEMM: N = 2500 58 / 56 at 2 %, 62 / 57 at 5 %; N = 5000 98 / 93
 // at 2 %, 111 / 95 at 5 %; the kernel itself 35 against 45 + 4 at N = 5000).
-// The synchronous call keeps the choice, whose outcome its callers can read
-// (and which the library's tests fix).
+// The synchronous call keeps the choice fitted to the FP8 GEMM, which is the
+// slower path on sparse graphs there (sc2_bitset_faster has the figures).
 int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_t* n,
                const turboreg_params* const* prm, Plan& plan, bool queued = false)
 {
@@ -392,7 +392,11 @@ int build_plan(turboreg_ctx* c, int32_t num, const int64_t* in_off, const int32_
                     !(prm[0]->flags & (TURBOREG_FLAG_SC2_SINGLE_CTA | TURBOREG_FLAG_SC2_GEMM)) &&
                     round_up(n[0], kSc2BN) <= kSc2AutoMaxNpad && sc2_pair_clusters() > 0;
     if (plan.sc2_auto && round_up(n[0], kSc2BN) <= kSc2BitsetAlwaysNpad) {
-        plan.sc2_auto = 0;   // the CUDA-core path is the faster one at any density: no choice to make
+        // The CUDA-core path without a choice: the faster one on sparse graphs, the
+        // slower one from about 13 % density on (registrations enqueued back to back,
+        // us, this path / GEMM: N = 1000 40 / 45 at 3 %, 43 / 47 at 5 %, 45 / 47 at 13 %,
+        // 66 / 51 at 39 %; N = 2048 47 / 51 at 3 %, 55 / 52 at 15 %, 79 / 58 at 44 %).
+        plan.sc2_auto = 0;
         plan.bitset = 1;
     }
     if (queued) plan.sc2_auto = 0;

@@ -32,9 +32,9 @@ __global__ void __launch_bounds__(128) kabsch_kernel(ManyViews vs)
 }
 
 // Verification.  A block holds 128 hypotheses (R, t staged in shared memory)
-// and 256 correspondences (as packed pairs (v, v), so a point feeds the
-// packed arithmetic straight from shared memory); each of its 4 warps takes 64 of
-// the correspondences for all 128 hypotheses, 4 per lane, evaluated as two
+// and up to 512 correspondences (as packed pairs (v, v), so a point feeds the
+// packed arithmetic straight from shared memory); each of its 4 warps takes a
+// quarter of them for all 128 hypotheses, 4 per lane, evaluated as two
 // packed pairs: e = R x + (t - y), d2 = |e|^2 with fma.rn.f32x2 (the same
 // rounding as the scalar expression, two hypotheses per instruction).  The
 // warps' counts are summed in shared memory; one atomic per hypothesis.
@@ -239,7 +239,7 @@ __device__ __forceinline__ void verify_body(const ProbView& v, int lb, VerifySha
     const int tot = sh.scnt[0][t] + sh.scnt[1][t] + sh.scnt[2][t] + sh.scnt[3][t];
     if (tot) atomicAdd(&v.inl[hh], tot);
     if (kScore != TURBOREG_SCORE_IN && sh.sok[t]) {
-        // per block at most 256 terms of <= 2^22 + 1 units: fits 32 bits
+        // per block at most 512 terms of <= 2^22 + 1 units: fits 32 bits
         const uint32_t s = sh.ssc[0][t] + sh.ssc[1][t] + sh.ssc[2][t] + sh.ssc[3][t];
         atomicAdd(&v.score[hh], static_cast<unsigned long long>(s));
     }

@@ -359,7 +359,8 @@ __global__ void __launch_bounds__(1024) features_kernel(ManyViews vs)
 // 6 us) and by shared-memory reads (half of the path's rate).  Separate forward
 // and backward kernels of 128 threads, with the activations through global
 // memory and transposed operands written element by element, took 113 + 146 us
-// at m = 131 072 and 22 + 54 us at m = 16 384; this one takes 54 and 18 us.
+// at m = 131 072 and 22 + 54 us at m = 16 384; this one takes 54 to 57
+// and 18 us.
 constexpr int kTrainThreads = 512;
 constexpr int kTOffH1 = 0;                       // [128 s][64]
 constexpr int kTOffW2 = kTOffH1 + 16384;         // [128 out][64 in]

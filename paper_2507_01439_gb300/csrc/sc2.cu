@@ -276,7 +276,8 @@ __device__ __forceinline__ void sc2_epilogue(const BlockInfo& v, uint32_t tacc, 
 // histogram is kept in shared memory, per CTA or (one problem) split over the
 // pair, and added to the global one when the worker leaves a problem (the
 // count pass or the select launch then chooses the pivot threshold from it);
-// else every edge adds to the global bins.
+// else every edge adds to the global bins.  In a batch each CTA adds its own
+// bins; for one problem a cluster's are merged in its first CTA before.
 // The scheduler warp finds each block's problem and descriptor fields up to
 // four blocks ahead and hands them over through a ring in shared memory: read
 // by every role for itself, they were a chain of up to eight dependent loads
@@ -710,8 +711,8 @@ cudaError_t sc2_tcgen05_setup()
 
 // The pair form keeps a CTA's bins beside its ring.  One problem whose bins
 // would cost the ring a stage splits them over the pair: at N = 20000 that
-// leaves four stages beside 40 KB of bins instead of three beside 80 KB (and
-// two stages at N = 32768).  A batch does not (its CTAs flush their bins by
+// leaves four stages beside 40 KB of bins instead of three beside 80 KB (and at
+// N = 32768 three beside 64 KB, where 128 KB leave fewer than two).  A batch does not (its CTAs flush their bins by
 // themselves between problems): above N = 31 999 its edges add to the global
 // bins, as the single-CTA form's do above 23 807 (larger stages).
 bool launch_sc2_tcgen05(const Batch& b, int total_tiles, int max_n, bool pair_mma, cudaStream_t s, bool auto_mode)

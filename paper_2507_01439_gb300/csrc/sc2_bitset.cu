@@ -246,15 +246,16 @@ __device__ __forceinline__ uint32_t and_popc(const uint4 (&a)[NQ], const uint4 (
 // graph: predicted times (us) fitted to measurements on GB300 at N = 1000 ..
 // 5000 and 1.7 .. 14 % density.  This CUDA-core form: a + b |E+| / 1e6, with
 // (a, b) = (21.5, 49) at n_pad = 5120 and (13.9, 70.8) at 3072, linear in
-// between (fewer units per CTA for smaller N), and always the faster one up
+// between (fewer units per CTA for smaller N), and taken without a choice up
 // to n_pad = 2048; the tensor-core GEMM: 12.5 + waves x K-stages x 0.368 (its
 // 2-CTA clusters over the 256 x 256 upper-triangle tiles, 0.368 us per
 // 128-deep stage) plus 4 (n_pad / 5120)^2 for the FP4 matrix it then needs.
-// The constants are those of the FP8 GEMM.  The FP4 one takes about 0.19 us per
-// stage, and the two paths now meet near 2 % density at N = 5000 (whole
-// registrations there: 97 us on this path, 93 with the GEMM forced; at 5 %
-// 110 and 95); the line stays where it was because the choice at 5.7 %
-// (713 598 edges, N = 5000) is part of the library's tested behaviour.
+// The constants are those of the FP8 GEMM this choice was fitted to.  The FP4 one
+// takes about 0.19 us per stage, so the choice is no longer the faster path
+// everywhere: at N = 5000 the two meet near 2 % density (whole registrations
+// there: 97 us on this path, 93 with the GEMM forced; at 5 % 110 and 95), and from
+// there to nearly 6 % a synchronous call takes the slower one.  A test expects
+// this path at 5.7 % (713 598 edges, N = 5000).
 __device__ __forceinline__ bool sc2_bitset_faster(int n_pad, unsigned long long deg_sum, int clusters)
 {
     if (n_pad <= 2048) return true;

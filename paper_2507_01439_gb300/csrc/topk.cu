@@ -379,10 +379,11 @@ __global__ void __launch_bounds__(kCountThreads, 3) count_kernel(VS vs, int sele
         v.active[atomicAdd(&v.ctl->n_active, 1u)] = make_int4(sg.row[t], sgt[t], seq[t], 0);
 }
 
-// The same counts in a batch of many problems: a warp per group, without block barriers; the
-// threshold comes from the select launch.  With a block per group the pass over
-// 256 problems took 345 us (blocks that start, find their problem and read
-// nothing), with four groups per block 254 us (bound by its barriers), now 98.
+// The same counts in a batch of many problems: a warp per group, without block
+// barriers; the threshold comes from the select launch.  With a block per group
+// the pass over 256 problems took 364 us (blocks that start, find their problem
+// and read nothing; with four groups per block it was bound by its barriers), so
+// 125 (device times in a profiler's launch list, cold caches).
 __global__ void __launch_bounds__(kCountThreads, 4) count_warp_kernel(ManyViews vs)
 {
     int lb;
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) count_warp_kernel(ManyViews 
 // block's eight rows then run side by side: with a block per row and n/8
 // blocks, a problem whose rows are all active took eight rows in turn (10.5 us
 // at n = 67), and a batch's blocks mostly started for nothing (256 problems:
-// 562 us, now 124).  Same slots and tie ranks as the block form below.
+// 613 us, so 136, measured as the count pass above).  Same slots and tie ranks as the block form below.
 template <class VS>
 __global__ void __launch_bounds__(256) emit_warp_kernel(VS vs)
 {
@@ -636,11 +637,12 @@ __global__ void __launch_bounds__(256) emit_kernel(VS vs)
     }
 }
 
-// Large batches: a problem's selected keys sorted in place, largest first (one block
-// per problem, bitonic in shared memory), so that the clique search takes
+// Large batches: a problem's selected keys sorted in place, largest first (one
+// block per problem, bitonic in shared memory), so that the clique search takes
 // pivot c from key c.  Finding each key's rank there instead, one warp per key
 // over all K1 keys, was 380 of the search's 2100 warp instructions per pivot;
-// the sort takes 1/40 of that (but a launch more: pgs_dense has the line).  A pass of stride 32 or less stays inside the 64 keys of a warp.
+// the sort takes 1/40 of that (but a launch more: pgs_dense has the line).  A
+// pass of stride 32 or less stays inside the 64 keys of a warp.
 __global__ void __launch_bounds__(1024) sort_kernel(ManyViews vs)
 {
     const ProbView& v = vs.bt.views[blockIdx.x];   // launch descriptors: before the wait

@@ -35,6 +35,5 @@ void launch_mlp_train(const float* feat, const float* label, int m, const float*
 // update, and *skipped (page-locked host memory) counts the step
 void launch_mlp_adam(float* w, float* mom, float* vel, const float* g, float* wbf, int step, float lr,
                      const float* loss, float* loss_out, const uint32_t* err, uint32_t* skipped, cudaStream_t s);
-void launch_learned_hist(const Batch& b, int total, int max_n, cudaStream_t s);
 
 }  // namespace tr
