@@ -9,12 +9,14 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-def _check(sizes, params):
+def _check(sizes, params, model=None):
     probs = [synth.make_problem("indoor", n, 0.05 + 0.02 * (b % 12), 3000 + 31 * b) for b, n in enumerate(sizes)]
     offs = np.cumsum([0] + list(sizes)).astype(np.int64)
     xs, ys = (np.concatenate([getattr(p, k) for p in probs]) for k in "xy")
     which = (trg.BUF_PIVOTS, trg.BUF_CLIQUES, trg.BUF_RT, trg.BUF_INLIERS)
     with trg.TurboReg(max_n=max(sizes), max_batch=len(sizes)) as c:
+        if model is not None:
+            c.set_proposal_model(model)
         one = [c.register(p.x, p.y, q) for p, q in zip(probs, params)]
         c.register(probs[0].x, probs[0].y, params[0])
         first = [c.buffer(w) for w in which]
@@ -68,3 +70,12 @@ def test_emit_forms(sizes, k1):
 @pytest.mark.parametrize("scoring", [trg.SCORE_IN, trg.SCORE_MAE, trg.SCORE_MSE])
 def test_verification_forms(num, k1, scoring):
     _check([2040 + b for b in range(num)], [trg.default_params(0.1, k1, 0.1, scoring=scoring) for _ in range(num)])
+
+
+# the learned proposal's weights through every form of the count and emit passes
+@pytest.mark.parametrize("sizes", [[2100, 60, 3000], [300, 900, 2049, 70, 1500], [150 + 90 * b for b in range(18)]])
+@pytest.mark.parametrize("k1", [20, 2000])
+def test_learned_forms(sizes, k1):
+    from paper_2507_01439_gb300.train_proposal import load_model
+    prm = [trg.default_params(0.1, k1, 0.1, proposal=trg.PROPOSAL_LEARNED, learned_min_inliers=1) for _ in sizes]
+    _check(sizes, prm, load_model())
